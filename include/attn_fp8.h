@@ -174,8 +174,8 @@ typedef struct {
  *   workspace  device, >= ATTN_STATUS_WORKSPACE_BYTES, 16-byte aligned: its status word reports a
  *              copy that never completed (attn_fp8_read_status -> ATTN_ERR_TIMEOUT), as for the
  *              attention entry points; a workspace of those calls may be passed
- * attn_fp8_quantize is this call with one job; its status word lands in the library's built-in
- * scratch of the current device, which attn_fp8_read_status(NULL, stream) reads.                 */
+ * attn_fp8_quantize is this call with one job; its status word (and attn_fp8_quantize_fused's) lands in
+ * the library's built-in scratch of the current device, which attn_fp8_read_status(NULL, stream) reads. */
 attn_status_t attn_fp8_quantize_batch(const attn_quantize_job_t* jobs, int32_t n_jobs, void* workspace,
                                       size_t workspace_bytes, void* stream);
 

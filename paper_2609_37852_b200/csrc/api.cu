@@ -234,9 +234,13 @@ attn_status_t attn_fp8_quantize_fused(const void* src, int32_t src_dtype, int32_
     return fail(ATTN_ERR_INVALID_ARG, "codes and scales of an orientation must be given together");
   if (out.row_codes) { CHECK(check_ptr(out.row_codes, "row_codes")); CHECK(check_ptr(out.row_scales, "row_scales")); }
   if (out.col_codes) { CHECK(check_ptr(out.col_codes, "col_codes")); CHECK(check_ptr(out.col_scales, "col_scales")); }
+  if (static_cast<long long>(B) * H * (N / 128) > 0x7fffffffLL)
+    return fail(ATTN_ERR_UNSUPPORTED, "tensor of more than 2^31 - 1 tiles of 128 tokens");
   CHECK(check_device());
-  return launch_quantize_fused(src, src_dtype, B, H, N, d, rope_cos, rope_sin, scale, mean, out,
-                               static_cast<cudaStream_t>(stream));
+  void* scratch = nullptr;                            // as in attn_fp8_quantize: the status word of the kernel
+  CHECK(builtin_scratch_for_current_device(&scratch));
+  const attn_quantize_job_t job = {src, src_dtype, B, H, N, d, out};
+  return launch_quantize_fused(job, rope_cos, rope_sin, scale, mean, static_cast<int*>(scratch), static_cast<cudaStream_t>(stream));
 }
 
 attn_status_t attn_fp8_prepare_bf16(const void* src, int32_t src_dtype, int32_t B, int32_t H, int32_t N, int32_t d,

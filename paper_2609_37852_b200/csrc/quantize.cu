@@ -1,16 +1,7 @@
-// The quantiser with the operand producer fused in front (rotary embedding, key centering, scale
-// folding), the token-mean kernel it needs, and the operand copies of BF16 mode.  The plain
-// quantiser (no producer steps) lives in quantize_batch.cu.
-//
-// One CTA owns a tile of 128 tokens x d channels of one (batch, head) slab, so it owns whole
-// 512-byte scale tiles of both orientations.  Pass 1 reads the tile from HBM once with 16-byte
-// coalesced loads, applies the producer steps in FP32, quantises along channels (4 lanes share a
-// block of 32) and parks the FP32 values in shared memory; pass 2 walks the parked tile along
-// tokens.  Codes of the transposed copy are staged in shared memory so that they leave as full
-// 128-byte rows.
+// The token mean that key centering subtracts, and the operand copies of BF16 mode.  The quantiser, with
+// and without the producer steps in front, lives in quantize_batch.cu.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
-
-#include <type_traits>
 
 #include "common.cuh"
 #include "mxfp8_device.cuh"
@@ -19,220 +10,125 @@
 namespace attnfp8 {
 namespace {
 
-constexpr int kTokens = 128;
+namespace cg = cooperative_groups;
+
 constexpr int kThreads = 256;
 
 __device__ __forceinline__ float to_f32(__nv_bfloat16 x) { return __bfloat162float(x); }
 __device__ __forceinline__ float to_f32(float x) { return x; }
 
-// Producer steps fused in front of the quantiser (paper Appendix "Operands, Scaling, and
-// Accumulation"): rotary embedding in FP32 with the rotated channels rounded to BF16, subtraction
-// of the FP32 token mean (key centering), FP32 multiplication by a scale (tau folded into Q).
-struct Producer {
-  const float* cos;     // [N, d/2] or nullptr
-  const float* sin;
-  const float* mean;    // [B*H, d] or nullptr
-  float scale;
-  int use_scale;
-};
+// Four consecutive values as FP32.
+__device__ __forceinline__ void load4(const __nv_bfloat16* p, float* x) {
+  const uint2 raw = *reinterpret_cast<const uint2*>(p);
+  x[0] = __uint_as_float(raw.x << 16); x[1] = __uint_as_float(raw.x & 0xFFFF0000u);
+  x[2] = __uint_as_float(raw.y << 16); x[3] = __uint_as_float(raw.y & 0xFFFF0000u);
+}
+__device__ __forceinline__ void load4(const float* p, float* x) {
+  const float4 a = *reinterpret_cast<const float4*>(p);
+  x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w;
+}
 
-// One rotated channel: x*cos -+ partner*sin with one rounding for the product and a fused
-// multiply-add, then BF16 (the order the header of attn_fp8_quantize_fused states).
+// One rotated channel, as the quantiser forms it (quantize_batch.cu).
 __device__ __forceinline__ float rotate_bf16(float x, float partner, float c, float s, bool upper) {
   const float t = __fmul_rn(partner, s);
   const float r = __fmaf_rn(x, c, upper ? t : -t);
   return __bfloat162float(__float2bfloat16_rn(r));
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kThreads) quantize_fused_kernel(const T* __restrict__ src, int N, int d,
-                                                            uint8_t* __restrict__ row_codes,
-                                                            uint8_t* __restrict__ row_scales,
-                                                            uint8_t* __restrict__ col_codes,
-                                                            uint8_t* __restrict__ col_scales, const Producer prod) {
-  extern __shared__ __align__(16) uint8_t smem[];
-  using TT = float;                                                  // what the parked tile holds
-  const int pitch = d + 16 / static_cast<int>(sizeof(TT)) * 1;      // elements; +16 bytes per row
-  TT* tile = reinterpret_cast<TT*>(smem);
-  const int n_ct = (d / 32 + 3) / 4;                                 // row-copy scale tiles of this CTA
-  const int n_rt = (d + 127) / 128;                                  // col-copy scale tiles of this CTA
-  uint8_t* s_row_sf = smem + static_cast<size_t>(kTokens) * pitch * sizeof(TT);
-  uint8_t* s_col_sf = s_row_sf + n_ct * 512;
-  uint8_t* s_col_codes = s_col_sf + n_rt * 512;                      // [d][128 + 16]
-  constexpr int kColPitch = kTokens + 16;
-
-  const int tid = threadIdx.x;
-  const int tok_tile = blockIdx.x;
-  const size_t slab = blockIdx.y;
-  const size_t tok0 = static_cast<size_t>(tok_tile) * kTokens;
-  const T* g_src = src + (slab * N + tok0) * d;
-  const bool want_row = row_codes != nullptr;
-  const bool want_col = col_codes != nullptr;
-
-  for (int i = tid; i < (n_ct + n_rt) * 512 / 4; i += kThreads) reinterpret_cast<uint32_t*>(s_row_sf)[i] = 0;
-  __syncthreads();
-
-  // ---- pass 1: rows.  8 elements per thread per step, 4 lanes per block of 32 channels.
-  const int steps = kTokens * d / (8 * kThreads);
-  // unrolled so that the loads of several steps are in flight together (a CTA is short-lived:
-  // the latency of its own loads is most of its life)
-#pragma unroll 8
-  for (int s = 0; s < steps; ++s) {
-    const int ci = s * kThreads + tid;
-    const int e0 = ci * 8;
-    const int tok = e0 / d, ch = e0 - tok * d;
-    float x[8];
-    if constexpr (sizeof(T) == 2) {
-      const uint4 raw = *reinterpret_cast<const uint4*>(g_src + e0);
-      const __nv_bfloat16* h = reinterpret_cast<const __nv_bfloat16*>(&raw);
-#pragma unroll
-      for (int i = 0; i < 8; ++i) x[i] = to_f32(h[i]);
-    } else {
-      const float4 a = *reinterpret_cast<const float4*>(g_src + e0);
-      const float4 b = *reinterpret_cast<const float4*>(g_src + e0 + 4);
-      x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w; x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
-    }
-    {
-      if (prod.cos != nullptr) {
-        const int half = d >> 1;
-        const bool upper = ch >= half;
-        const int pc = upper ? ch - half : ch;                       // pair index; 8 consecutive pairs per thread
-        const T* g_partner = g_src + e0 + (upper ? -half : half);
-        const size_t tab = (tok0 + tok) * half + pc;
-#pragma unroll
-        for (int i = 0; i < 8; ++i)
-          x[i] = rotate_bf16(x[i], to_f32(g_partner[i]), prod.cos[tab + i], prod.sin[tab + i], upper);
-      }
-      if (prod.mean != nullptr) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) x[i] = __fsub_rn(x[i], prod.mean[slab * d + ch + i]);
-      }
-      if (prod.use_scale) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) x[i] = __fmul_rn(x[i], prod.scale);
-      }
-      if (want_col) {
-        *reinterpret_cast<float4*>(tile + tok * pitch + ch) = make_float4(x[0], x[1], x[2], x[3]);
-        *reinterpret_cast<float4*>(tile + tok * pitch + ch + 4) = make_float4(x[4], x[5], x[6], x[7]);
-      }
-    }
-    if (want_row) {
-      float amax = 0.f;
-#pragma unroll
-      for (int i = 0; i < 8; ++i) amax = fmaxf(amax, fabsf(x[i]));
-      amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 1));
-      amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 2));
-      uint32_t byte; float inv;
-      block_scale(amax, byte, inv);
-      uint2 codes;
-      codes.x = sm100::cvt_e4m3x4(x[0] * inv, x[1] * inv, x[2] * inv, x[3] * inv);
-      codes.y = sm100::cvt_e4m3x4(x[4] * inv, x[5] * inv, x[6] * inv, x[7] * inv);
-      *reinterpret_cast<uint2*>(row_codes + (slab * N + tok0) * d + e0) = codes;
-      if ((tid & 3) == 0) {
-        const int blk = ch >> 5;
-        s_row_sf[(blk >> 2) * 512 + sf_tile_offset(tok, blk & 3)] = static_cast<uint8_t>(byte);
-      }
-    }
-  }
-  __syncthreads();
-  if (want_row) {
-    uint8_t* g = row_scales + (slab * (N / kTokens) + tok_tile) * n_ct * 512;
-    for (int i = tid; i < n_ct * 512 / 16; i += kThreads)
-      reinterpret_cast<uint4*>(g)[i] = reinterpret_cast<const uint4*>(s_row_sf)[i];
-  }
-  if (!want_col) return;
-
-  // ---- pass 2: columns.  One (channel, block of 32 tokens) per thread per step.
-  for (int item = tid; item < d * 4; item += kThreads) {
-    const int c = item % d, tb = item / d;
-    float x[32];
-    float amax = 0.f;
-#pragma unroll
-    for (int t = 0; t < 32; ++t) {
-      x[t] = to_f32(tile[(tb * 32 + t) * pitch + c]);
-      amax = fmaxf(amax, fabsf(x[t]));
-    }
-    uint32_t byte; float inv;
-    block_scale(amax, byte, inv);
-    uint32_t w[8];
-#pragma unroll
-    for (int t = 0; t < 8; ++t)
-      w[t] = sm100::cvt_e4m3x4(x[4 * t] * inv, x[4 * t + 1] * inv, x[4 * t + 2] * inv, x[4 * t + 3] * inv);
-    uint4* dst = reinterpret_cast<uint4*>(s_col_codes + c * kColPitch + tb * 32);
-    dst[0] = make_uint4(w[0], w[1], w[2], w[3]);
-    dst[1] = make_uint4(w[4], w[5], w[6], w[7]);
-    s_col_sf[(c >> 7) * 512 + sf_tile_offset(c & 127, tb)] = static_cast<uint8_t>(byte);
-  }
-  __syncthreads();
-  for (int i = tid; i < d * 8; i += kThreads) {
-    const int c = i >> 3, chunk = i & 7;
-    *reinterpret_cast<uint4*>(col_codes + (slab * d + c) * N + tok0 + chunk * 16) =
-        *reinterpret_cast<const uint4*>(s_col_codes + c * kColPitch + chunk * 16);
-  }
-  for (int rt = 0; rt < n_rt; ++rt) {
-    uint8_t* g = col_scales + ((slab * n_rt + rt) * (N / kTokens) + tok_tile) * 512;
-    for (int i = tid; i < 512 / 16; i += kThreads)
-      reinterpret_cast<uint4*>(g)[i] = reinterpret_cast<const uint4*>(s_col_sf + rt * 512)[i];
-  }
-}
-
-template <typename T>
-attn_status_t launch_t(const void* src, int B, int H, int N, int d, attn_qtensor_t out, const Producer& prod,
-                       cudaStream_t stream) {
-  const int tile_elem = 4;                                           // the parked tile is FP32
-  const int pitch = d + 16 / tile_elem;
-  const int n_ct = (d / 32 + 3) / 4, n_rt = (d + 127) / 128;
-  const size_t smem = static_cast<size_t>(kTokens) * pitch * tile_elem + (n_ct + n_rt) * 512 +
-                      static_cast<size_t>(d) * (kTokens + 16);
-  cudaError_t e = cudaFuncSetAttribute(quantize_fused_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
-  if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "quantize: cudaFuncSetAttribute: %s", cudaGetErrorString(e));
-  dim3 grid(N / kTokens, B * H);
-  quantize_fused_kernel<T><<<grid, kThreads, smem, stream>>>(static_cast<const T*>(src), N, d, out.row_codes,
-                                                              out.row_scales, out.col_codes, out.col_scales, prod);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "quantize: launch: %s", cudaGetErrorString(e));
-  return ATTN_OK;
-}
-
 // FP32 mean over tokens of the (rotated, BF16-rounded) tensor, per (batch, head, channel).  The
 // terms are BF16 values, so a double-precision sum is exact whatever its order, and the result is
-// the correctly rounded quotient: bitwise reproducible.  One CTA per (batch, head).
-constexpr int kMeanThreads = 1024;
+// the correctly rounded quotient: bitwise reproducible.
+//
+// Memory-bound work (the key tensor once, the tables from L2) on few slabs: a grouped-query layer has 4 to
+// 8, so a slab is shared by a cluster of up to eight CTAs, each summing a range of the tokens with vector
+// loads; the first CTA adds the others' sums from their shared memory.  With rotary embedding, BF16:
+// 4 x 4096 x 128 values 135 -> 13 us, 48 x 2816 x 128 97 -> 24 us against one CTA per slab with scalar loads
+// (four pairs per thread and 64 registers: with eight pairs and 88 registers the second took 40 us).
+constexpr int kMaxCluster = 8;
+constexpr int kMeanThreads = 512;
 
 template <typename T>
-__global__ void __launch_bounds__(kMeanThreads) token_mean_kernel(const T* __restrict__ src, int N, int d,
-                                                                  const float* __restrict__ cos,
-                                                                  const float* __restrict__ sin,
-                                                                  float* __restrict__ mean) {
+__global__ void __launch_bounds__(kMeanThreads, 2) token_mean_kernel(const T* __restrict__ src, int N, int d,
+                                                              const float* __restrict__ cos, const float* __restrict__ sin,
+                                                              float* __restrict__ mean) {
   extern __shared__ __align__(16) uint8_t smem[];
-  double* part = reinterpret_cast<double*>(smem);                   // [phases][d]
-  const int half = d >> 1;
-  const int phases = kMeanThreads / half;
-  const int pc = threadIdx.x % half, ph = threadIdx.x / half;
-  const size_t slab = blockIdx.x;
-  const T* g = src + slab * N * d;
-  double a1 = 0.0, a2 = 0.0;
+  double* part = reinterpret_cast<double*>(smem);                   // [phases][d], then the CTA's sums in row 0
+  cg::cluster_group cluster = cg::this_cluster();
+  const int rank = static_cast<int>(cluster.block_rank()), ranks = static_cast<int>(cluster.num_blocks());
+  const int half = d >> 1, chunks = half >> 2, phases = kMeanThreads / chunks;   // a thread sums four pairs (c, c + d / 2)
+  const int ph = threadIdx.x / chunks, pc = (threadIdx.x - ph * chunks) * 4;
+  const size_t slab = blockIdx.x / ranks;
+  const T* g = src + slab * N * d + pc;
+  const int per = N / ranks;                                         // N is a multiple of 128
+  const int n0 = rank * per, n1 = rank == ranks - 1 ? N : n0 + per;
   if (ph < phases) {
-    for (int n = ph; n < N; n += phases) {
-      float x1 = to_f32(g[static_cast<size_t>(n) * d + pc]), x2 = to_f32(g[static_cast<size_t>(n) * d + half + pc]);
+    double lo[4], hi[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) lo[k] = hi[k] = 0.0;
+#pragma unroll 4
+    for (int n = n0 + ph; n < n1; n += phases) {
+      float x1[4], x2[4];
+      load4(g + static_cast<size_t>(n) * d, x1);
+      load4(g + static_cast<size_t>(n) * d + half, x2);
       if (cos != nullptr) {
-        const float c = cos[static_cast<size_t>(n) * half + pc], s = sin[static_cast<size_t>(n) * half + pc];
-        const float r1 = rotate_bf16(x1, x2, c, s, false), r2 = rotate_bf16(x2, x1, c, s, true);
-        x1 = r1; x2 = r2;
+        float c[4], s[4];
+        load4(cos + static_cast<size_t>(n) * half + pc, c);
+        load4(sin + static_cast<size_t>(n) * half + pc, s);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const float r = rotate_bf16(x1[k], x2[k], c[k], s[k], false);
+          x2[k] = rotate_bf16(x2[k], x1[k], c[k], s[k], true);
+          x1[k] = r;
+        }
       }
-      a1 += static_cast<double>(x1);
-      a2 += static_cast<double>(x2);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        lo[k] += static_cast<double>(x1[k]);
+        hi[k] += static_cast<double>(x2[k]);
+      }
     }
-    part[ph * d + pc] = a1;
-    part[ph * d + half + pc] = a2;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      part[ph * d + pc + k] = lo[k];
+      part[ph * d + half + pc + k] = hi[k];
+    }
   }
   __syncthreads();
-  for (int c = threadIdx.x; c < d; c += kMeanThreads) {
+  const int c = threadIdx.x;                                         // d <= 256: one channel per thread
+  if (c < d) {
     double sum = 0.0;
     for (int i = 0; i < phases; ++i) sum += part[i * d + c];
+    part[c] = sum;                                                   // only this thread reads column c
+  }
+  cluster.sync();
+  if (rank == 0 && c < d) {
+    double sum = part[c];
+    for (int r = 1; r < ranks; ++r) sum += *cluster.map_shared_rank(part + c, r);
     mean[slab * d + c] = static_cast<float>(sum / static_cast<double>(N));
   }
+  cluster.sync();                                                    // the sums stay until they have been read
+}
+
+template <typename T>
+attn_status_t launch_mean_t(const void* src, int slabs, int N, int d, const float* cos, const float* sin, float* mean,
+                            cudaStream_t stream) {
+  // enough CTAs for two on every SM of the largest part, no fewer than 128 tokens each
+  int ranks = 1;
+  while (ranks < kMaxCluster && slabs * ranks < 296 && 2 * ranks <= N / 128) ranks *= 2;
+  const int chunks = d / 8;
+  const size_t smem = static_cast<size_t>(kMeanThreads / chunks) * d * sizeof(double);   // 32 KB
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(slabs) * ranks);
+  cfg.blockDim = dim3(kMeanThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = ranks; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr; cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, token_mean_kernel<T>, static_cast<const T*>(src), N, d, cos, sin, mean);
+  if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "token mean: launch: %s", cudaGetErrorString(e));
+  return ATTN_OK;
 }
 
 // BF16 mode: the operands are the tensors themselves, rounded to BF16, in both orientations.
@@ -287,21 +183,10 @@ attn_status_t launch_bf16_copies(const void* src, int src_dtype, int B, int H, i
   return launch_copies_t<float>(src, B, H, N, d, row_out, col_out, stream);
 }
 
-attn_status_t launch_quantize_fused(const void* src, int src_dtype, int B, int H, int N, int d, const float* cos,
-                                    const float* sin, float scale, float* mean, attn_qtensor_t out,
-                                    cudaStream_t stream) {
-  if (mean != nullptr) {
-    const size_t smem = static_cast<size_t>(kMeanThreads / (d / 2)) * d * sizeof(double);
-    if (src_dtype == ATTN_SRC_BF16)
-      token_mean_kernel<__nv_bfloat16><<<B * H, kMeanThreads, smem, stream>>>(static_cast<const __nv_bfloat16*>(src), N, d, cos, sin, mean);
-    else
-      token_mean_kernel<float><<<B * H, kMeanThreads, smem, stream>>>(static_cast<const float*>(src), N, d, cos, sin, mean);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "token mean: launch: %s", cudaGetErrorString(e));
-  }
-  const Producer prod{cos, sin, mean, scale, scale != 1.f ? 1 : 0};
-  if (src_dtype == ATTN_SRC_BF16) return launch_t<__nv_bfloat16>(src, B, H, N, d, out, prod, stream);
-  return launch_t<float>(src, B, H, N, d, out, prod, stream);
+attn_status_t launch_token_mean(const void* src, int src_dtype, int slabs, int N, int d, const float* cos, const float* sin,
+                                float* mean, cudaStream_t stream) {
+  if (src_dtype == ATTN_SRC_BF16) return launch_mean_t<__nv_bfloat16>(src, slabs, N, d, cos, sin, mean, stream);
+  return launch_mean_t<float>(src, slabs, N, d, cos, sin, mean, stream);
 }
 
 }  // namespace attnfp8

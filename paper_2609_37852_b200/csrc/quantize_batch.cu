@@ -1,6 +1,7 @@
 // Block-scaling quantiser: E4M3 codes with one E8M0 scale per 32 consecutive elements, written
 // in both orientations (blocks along channels; blocks along tokens, stored transposed), for one
-// tensor or for several in one launch (the four operands of a step: Q, K, V, dO).
+// tensor or for several in one launch (the four operands of a step: Q, K, V, dO), and for one tensor
+// with the producer steps in front (rotary embedding, key centering, scale folding).
 //
 // The tiles (128 tokens x d channels, contiguous in the source) of all tensors form one list.  A
 // persistent grid (two CTAs per SM) walks it; each CTA keeps a ring of two source tiles in shared
@@ -10,6 +11,13 @@
 // disappear and every SM always has loads outstanding.
 // Pass 1 walks the tile along channels (row copy), pass 2 along tokens (column copy, staged in
 // shared memory so that it leaves as full 128-byte rows).
+//
+// Producer steps (kProd).  A pass ahead of the other two rotates the tile in place: a rotated channel is
+// a BF16 value, so it goes back into the slot it came from whatever the source type.  The FP32 steps
+// (minus the token mean, times the scale) are repeated by both passes, two packed operations per pair,
+// instead of parking an FP32 tile.  The kernel this replaced (one tile per CTA, scalar loads of partner
+// and tables, an FP32 tile parked in shared memory) took 17.4 us on average over Q and K of a layer with
+// 16 + 4 heads of 4096 x 128 BF16 values, this one 12.7 us.
 #include <cuda_bf16.h>
 
 #include "common.cuh"
@@ -33,6 +41,13 @@ struct BatchJob {
   int first_tile;        // index of this tensor's first tile in the list
 };
 
+// The producer of a one-tensor launch (paper Appendix "Operands, Scaling, and Accumulation").
+struct Producer {
+  const float *cos, *sin;  // [N, d / 2], or both null: no rotary embedding
+  const float* mean;       // [B * H, d], or null: no centering
+  float scale;             // 1: no scaling (an exact multiplication)
+};
+
 struct BatchParams {
   BatchJob job[ATTN_QUANTIZE_MAX_JOBS];
   int n_jobs;
@@ -40,6 +55,7 @@ struct BatchParams {
   int d_max;
   int ring;              // source tiles a CTA keeps in shared memory (1 or 2)
   int* status;
+  Producer prod;         // kProd only
 };
 
 // |a| max |b| per 16-bit lane; a NaN lane yields the other operand, as fmaxf does
@@ -51,13 +67,79 @@ __device__ __forceinline__ float2 unpack_bf16x2(uint32_t raw) {
   return make_float2(__uint_as_float(raw << 16), __uint_as_float(raw & 0xFFFF0000u));
 }
 
+// One rotated channel: x*cos -+ partner*sin with one rounding for the product and a fused
+// multiply-add, then BF16 (the order the header of attn_fp8_quantize_fused states).
+__device__ __forceinline__ float rotate_bf16(float x, float partner, float c, float s, bool upper) {
+  const float t = __fmul_rn(partner, s);
+  const float r = __fmaf_rn(x, c, upper ? t : -t);
+  return __bfloat162float(__float2bfloat16_rn(r));
+}
+// Eight consecutive values as FP32, and back (the values of a BF16 row are BF16-representable).
+__device__ __forceinline__ void load8(const __nv_bfloat16* p, float* x) {
+  const uint4 raw = *reinterpret_cast<const uint4*>(p);
+  const float2 a = unpack_bf16x2(raw.x), b = unpack_bf16x2(raw.y), c = unpack_bf16x2(raw.z), e = unpack_bf16x2(raw.w);
+  x[0] = a.x; x[1] = a.y; x[2] = b.x; x[3] = b.y; x[4] = c.x; x[5] = c.y; x[6] = e.x; x[7] = e.y;
+}
+__device__ __forceinline__ void load8(const float* p, float* x) {
+  const float4 a = reinterpret_cast<const float4*>(p)[0], b = reinterpret_cast<const float4*>(p)[1];
+  x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w; x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
+}
+__device__ __forceinline__ void store8(__nv_bfloat16* p, const float* x) {
+  *reinterpret_cast<uint4*>(p) = make_uint4(cvt_bf16x2(x[0], x[1]), cvt_bf16x2(x[2], x[3]), cvt_bf16x2(x[4], x[5]), cvt_bf16x2(x[6], x[7]));
+}
+__device__ __forceinline__ void store8(float* p, const float* x) {
+  reinterpret_cast<float4*>(p)[0] = make_float4(x[0], x[1], x[2], x[3]);
+  reinterpret_cast<float4*>(p)[1] = make_float4(x[4], x[5], x[6], x[7]);
+}
+
+// Rotary embedding of a tile in place: eight pairs (c, c + d / 2) of one token per thread and step.
+template <typename T>
+__device__ __forceinline__ void rotate_tile(T* tile, int d, const Producer& prod, size_t tok0, int tid) {
+  const int half = d >> 1, chunks = half >> 3;
+#pragma unroll 2
+  for (int i = tid; i < kTokens * chunks; i += kThreads) {
+    const int tok = i / chunks, pc = (i - tok * chunks) * 8;
+    float c[8], s[8], lo[8], hi[8];
+    load8(prod.cos + (tok0 + tok) * half + pc, c);
+    load8(prod.sin + (tok0 + tok) * half + pc, s);
+    T* row = tile + tok * d + pc;
+    load8(row, lo);
+    load8(row + half, hi);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const float r = rotate_bf16(lo[k], hi[k], c[k], s[k], false);
+      hi[k] = rotate_bf16(hi[k], lo[k], c[k], s[k], true);
+      lo[k] = r;
+    }
+    store8(row, lo);
+    store8(row + half, hi);
+  }
+  fence_proxy_async_smem();        // the slot is refilled by a bulk copy later
+}
+
+// The FP32 steps behind the rotation.  Without centering the subtrahend is +0 and without scaling the
+// factor is 1: both exact.
+__device__ __forceinline__ float2 affine2(float2 x, float2 neg_mean, float2 scale) { return __fmul2_rn(__fadd2_rn(x, neg_mean), scale); }
+__device__ __forceinline__ float2 neg_mean2(const float* mean) {        // mean: of two neighbouring channels, or null
+  if (mean == nullptr) return make_float2(-0.f, -0.f);
+  const float2 m = *reinterpret_cast<const float2*>(mean);
+  return make_float2(-m.x, -m.y);
+}
+
 // Both passes over one source tile in shared memory ([128 tokens][d], unpadded).  kD is the head
 // dim when it is one of the built ones (0: use the run-time value).
-template <typename T, int kD>
-__device__ __forceinline__ void quantize_tile(const T* tile, int d_rt, const BatchJob& job, size_t slab, size_t tok0,
-                                              uint8_t* s_row_sf, uint8_t* s_col_sf, uint8_t* s_col_codes, int tid) {
+template <typename T, int kD, bool kProd>
+__device__ __forceinline__ void quantize_tile(T* tile, int d_rt, const BatchJob& job, const Producer& prod, size_t slab,
+                                              size_t tok0, uint8_t* s_row_sf, uint8_t* s_col_sf, uint8_t* s_col_codes,
+                                              int tid) {
   const int d = kD ? kD : d_rt;
   const int N = job.N;
+  const float* mean = kProd && prod.mean != nullptr ? prod.mean + slab * d : nullptr;
+  const float2 scale2 = make_float2(prod.scale, prod.scale);
+  if (kProd && prod.cos != nullptr) {
+    rotate_tile(tile, d, prod, tok0, tid);
+    __syncthreads();
+  }
   // ---- pass 1: rows.  8 elements per thread per step, 4 lanes per block of 32 channels.
   if (job.row_codes != nullptr) {
     uint8_t* g_codes = job.row_codes + (slab * N + tok0) * d;
@@ -71,7 +153,7 @@ __device__ __forceinline__ void quantize_tile(const T* tile, int d_rt, const Bat
       if constexpr (sizeof(T) == 2) {
         const uint4 raw = *reinterpret_cast<const uint4*>(tile + e0);
         __nv_bfloat162 m = __float2bfloat162_rn(0.f);
-        m = absmax2(m, raw.x); m = absmax2(m, raw.y); m = absmax2(m, raw.z); m = absmax2(m, raw.w);
+        if (!kProd) { m = absmax2(m, raw.x); m = absmax2(m, raw.y); m = absmax2(m, raw.z); m = absmax2(m, raw.w); }
         amax = fmaxf(__low2float(m), __high2float(m));
         v[0] = unpack_bf16x2(raw.x); v[1] = unpack_bf16x2(raw.y); v[2] = unpack_bf16x2(raw.z); v[3] = unpack_bf16x2(raw.w);
       } else {
@@ -79,6 +161,12 @@ __device__ __forceinline__ void quantize_tile(const T* tile, int d_rt, const Bat
         const float4 b = *reinterpret_cast<const float4*>(tile + e0 + 4);
         v[0] = make_float2(a.x, a.y); v[1] = make_float2(a.z, a.w); v[2] = make_float2(b.x, b.y); v[3] = make_float2(b.z, b.w);
         amax = 0.f;
+      }
+      if (kProd) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = affine2(v[k], neg_mean2(mean ? mean + ch + 2 * k : nullptr), scale2);
+      }
+      if (kProd || sizeof(T) == 4) {
 #pragma unroll
         for (int k = 0; k < 4; ++k) amax = fmaxf(amax, fmaxf(fabsf(v[k].x), fabsf(v[k].y)));
       }
@@ -110,20 +198,29 @@ __device__ __forceinline__ void quantize_tile(const T* tile, int d_rt, const Bat
         const uint32_t* col = reinterpret_cast<const uint32_t*>(tile + tb * 32 * d + c);
         uint32_t raw[32];
         __nv_bfloat162 m = __float2bfloat162_rn(0.f);
+        float2 amax2 = make_float2(0.f, 0.f);
+        const float2 nm = kProd ? neg_mean2(mean ? mean + c : nullptr) : make_float2(0.f, 0.f);
+        auto value = [&](uint32_t w) { return kProd ? affine2(unpack_bf16x2(w), nm, scale2) : unpack_bf16x2(w); };
 #pragma unroll
         for (int t = 0; t < 32; ++t) {
           raw[t] = col[t * pairs];
-          m = absmax2(m, raw[t]);
+          if (kProd) {
+            const float2 x = value(raw[t]);
+            amax2 = make_float2(fmaxf(amax2.x, fabsf(x.x)), fmaxf(amax2.y, fabsf(x.y)));
+          } else {
+            m = absmax2(m, raw[t]);
+          }
         }
+        if (!kProd) amax2 = make_float2(__low2float(m), __high2float(m));
         uint32_t byte_lo, byte_hi;
         float2 inv2;
-        block_scale(__low2float(m), byte_lo, inv2.x);
-        block_scale(__high2float(m), byte_hi, inv2.y);
+        block_scale(amax2.x, byte_lo, inv2.x);
+        block_scale(amax2.y, byte_hi, inv2.y);
         uint32_t w_lo[8], w_hi[8];
 #pragma unroll
         for (int t = 0; t < 8; ++t) {
-          const float2 a = __fmul2_rn(unpack_bf16x2(raw[4 * t]), inv2), b = __fmul2_rn(unpack_bf16x2(raw[4 * t + 1]), inv2);
-          const float2 e = __fmul2_rn(unpack_bf16x2(raw[4 * t + 2]), inv2), f = __fmul2_rn(unpack_bf16x2(raw[4 * t + 3]), inv2);
+          const float2 a = __fmul2_rn(value(raw[4 * t]), inv2), b = __fmul2_rn(value(raw[4 * t + 1]), inv2);
+          const float2 e = __fmul2_rn(value(raw[4 * t + 2]), inv2), f = __fmul2_rn(value(raw[4 * t + 3]), inv2);
           w_lo[t] = cvt_e4m3x4(a.x, b.x, e.x, f.x);
           w_hi[t] = cvt_e4m3x4(a.y, b.y, e.y, f.y);
         }
@@ -142,9 +239,11 @@ __device__ __forceinline__ void quantize_tile(const T* tile, int d_rt, const Bat
         const int c = item % d, tb = item / d;
         float x[32];
         float amax = 0.f;
+        const float m = mean ? mean[c] : 0.f;
 #pragma unroll
         for (int t = 0; t < 32; ++t) {
           x[t] = tile[(tb * 32 + t) * d + c];
+          if (kProd) x[t] = __fmul_rn(__fsub_rn(x[t], m), prod.scale);
           amax = fmaxf(amax, fabsf(x[t]));
         }
         uint32_t byte; float inv;
@@ -162,7 +261,7 @@ __device__ __forceinline__ void quantize_tile(const T* tile, int d_rt, const Bat
   }
 }
 
-template <typename T>
+template <typename T, bool kProd>
 __global__ void __launch_bounds__(kThreads, 2) quantize_batch_kernel(const __grid_constant__ BatchParams p) {
   extern __shared__ __align__(128) uint8_t smem[];
   const int tile_bytes_max = kTokens * p.d_max * static_cast<int>(sizeof(T));
@@ -215,7 +314,7 @@ __global__ void __launch_bounds__(kThreads, 2) quantize_batch_kernel(const __gri
     const size_t tok0 = static_cast<size_t>(tok_tile) * kTokens;
     const int n_ct = (d / 32 + 3) / 4, n_rt = (d + 127) / 128;
     const bool want_row = job.row_codes != nullptr, want_col = job.col_codes != nullptr;
-    const T* tile = ring(i % n_ring);
+    T* tile = ring(i % n_ring);
 
     for (int w = tid; w < (n_ct_max + n_rt_max) * 512 / 4; w += kThreads) reinterpret_cast<uint32_t*>(s_row_sf)[w] = 0;
     // bounded wait: a copy that never lands ends the CTA with the time-out status, not a hang
@@ -223,11 +322,11 @@ __global__ void __launch_bounds__(kThreads, 2) quantize_batch_kernel(const __gri
     if (__syncthreads_or(!landed)) break;        // all threads take the same way out
 
     switch (d) {                      // compile-time head dims: no integer division, constant strides
-      case 64:  quantize_tile<T, 64>(tile, d, job, slab, tok0, s_row_sf, s_col_sf, s_col_codes, tid); break;
-      case 128: quantize_tile<T, 128>(tile, d, job, slab, tok0, s_row_sf, s_col_sf, s_col_codes, tid); break;
-      case 192: quantize_tile<T, 192>(tile, d, job, slab, tok0, s_row_sf, s_col_sf, s_col_codes, tid); break;
-      case 256: quantize_tile<T, 256>(tile, d, job, slab, tok0, s_row_sf, s_col_sf, s_col_codes, tid); break;
-      default:  quantize_tile<T, 0>(tile, d, job, slab, tok0, s_row_sf, s_col_sf, s_col_codes, tid); break;
+      case 64:  quantize_tile<T, 64, kProd>(tile, d, job, p.prod, slab, tok0, s_row_sf, s_col_sf, s_col_codes, tid); break;
+      case 128: quantize_tile<T, 128, kProd>(tile, d, job, p.prod, slab, tok0, s_row_sf, s_col_sf, s_col_codes, tid); break;
+      case 192: quantize_tile<T, 192, kProd>(tile, d, job, p.prod, slab, tok0, s_row_sf, s_col_sf, s_col_codes, tid); break;
+      case 256: quantize_tile<T, 256, kProd>(tile, d, job, p.prod, slab, tok0, s_row_sf, s_col_sf, s_col_codes, tid); break;
+      default:  quantize_tile<T, 0, kProd>(tile, d, job, p.prod, slab, tok0, s_row_sf, s_col_sf, s_col_codes, tid); break;
     }
     __syncthreads();
     // the source tile is consumed: refill its slot while the staged outputs leave
@@ -263,7 +362,7 @@ static size_t batch_smem_bytes(size_t elem, int d_max, int ring) {
          static_cast<size_t>(d_max) * kColPitch + 64;
 }
 
-template <typename T>
+template <typename T, bool kProd>
 attn_status_t launch_batch_t(BatchParams& p, cudaStream_t stream) {
   // two CTAs per SM come first (each covers the other's stalls), the deeper ring second: measured
   // at d = 192 one tile x two CTAs 0.078 ms against two tiles x one CTA 0.098 ms
@@ -272,27 +371,24 @@ attn_status_t launch_batch_t(BatchParams& p, cudaStream_t stream) {
   else if (batch_smem_bytes(sizeof(T), p.d_max, 1) <= half_sm) p.ring = 1;
   else p.ring = batch_smem_bytes(sizeof(T), p.d_max, kMaxRing) <= whole_sm ? kMaxRing : 1;
   const size_t smem = batch_smem_bytes(sizeof(T), p.d_max, p.ring);
-  cudaError_t e = cudaFuncSetAttribute(quantize_batch_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaError_t e = cudaFuncSetAttribute(quantize_batch_kernel<T, kProd>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(smem));
   if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "quantize: cudaFuncSetAttribute: %s", cudaGetErrorString(e));
   int dev = 0, sms = 0, per_sm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, quantize_batch_kernel<T>, kThreads, smem);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, quantize_batch_kernel<T, kProd>, kThreads, smem);
   if (e != cudaSuccess || per_sm < 1 || sms < 1)
     return fail(ATTN_ERR_CUDA, "quantize: occupancy query: %s", cudaGetErrorString(e));
   const int resident = sms * per_sm;
   const int grid = p.total_tiles < resident ? p.total_tiles : resident;
-  quantize_batch_kernel<T><<<grid, kThreads, smem, stream>>>(p);
+  quantize_batch_kernel<T, kProd><<<grid, kThreads, smem, stream>>>(p);
   e = cudaGetLastError();
   if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "quantize: launch: %s", cudaGetErrorString(e));
   return ATTN_OK;
 }
 
-}  // namespace
-
-attn_status_t launch_quantize_batch(const attn_quantize_job_t* jobs, int n_jobs, int* status, cudaStream_t stream) {
-  BatchParams p = {};
+void fill_params(BatchParams& p, const attn_quantize_job_t* jobs, int n_jobs, int* status) {
   p.n_jobs = n_jobs;
   p.status = status;
   int tiles = 0, d_max = 0;
@@ -309,8 +405,29 @@ attn_status_t launch_quantize_batch(const attn_quantize_job_t* jobs, int n_jobs,
   }
   p.total_tiles = tiles;
   p.d_max = d_max;
-  if (jobs[0].src_dtype == ATTN_SRC_BF16) return launch_batch_t<__nv_bfloat16>(p, stream);
-  return launch_batch_t<float>(p, stream);
+}
+
+}  // namespace
+
+attn_status_t launch_quantize_batch(const attn_quantize_job_t* jobs, int n_jobs, int* status, cudaStream_t stream) {
+  BatchParams p = {};
+  fill_params(p, jobs, n_jobs, status);
+  if (jobs[0].src_dtype == ATTN_SRC_BF16) return launch_batch_t<__nv_bfloat16, false>(p, stream);
+  return launch_batch_t<float, false>(p, stream);
+}
+
+attn_status_t launch_quantize_fused(const attn_quantize_job_t& job, const float* cos, const float* sin, float scale,
+                                    float* mean, int* status, cudaStream_t stream) {
+  if (cos == nullptr && mean == nullptr && scale == 1.f) return launch_quantize_batch(&job, 1, status, stream);
+  if (mean != nullptr) {
+    const attn_status_t st = launch_token_mean(job.src, job.src_dtype, job.B * job.H, job.N, job.d, cos, sin, mean, stream);
+    if (st != ATTN_OK) return st;
+  }
+  BatchParams p = {};
+  fill_params(p, &job, 1, status);
+  p.prod = Producer{cos, sin, mean, scale};
+  if (job.src_dtype == ATTN_SRC_BF16) return launch_batch_t<__nv_bfloat16, true>(p, stream);
+  return launch_batch_t<float, true>(p, stream);
 }
 
 }  // namespace attnfp8

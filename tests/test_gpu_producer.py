@@ -50,6 +50,25 @@ def test_fused_producer_bit_exact(d):
         assert torch.equal(a, b)
 
 
+@pytest.mark.parametrize("H,N,d", [(1, 128, 32), (2, 1152, 96), (300, 128, 64), (1, 1024, 256)])
+def test_fused_producer_shares_a_slab_between_ctas(H, N, d):
+    """One CTA per slab (N = 128, or many slabs), and clusters of two to eight with a token count they do
+    not divide into whole tiles; head dims without a compile-time kernel; centering without rotation."""
+    from paper_2609_37852_b200 import binding
+    g = torch.Generator().manual_seed(H + N + d)
+    x = (torch.randn((1, H, N, d), generator=g) - 1.5).to(torch.bfloat16)
+    cos, sin = P.rope_tables(N, d)
+    tc, ts = torch.from_numpy(cos).cuda(), torch.from_numpy(sin).cuda()
+    for rope in (True, False):
+        kt, mean = binding.attn_fp8_quantize_fused(x.cuda(), tc if rope else None, ts if rope else None, scale=0.3, center=True)
+        y, m = P.fused_operand(to_np(x), cos if rope else None, sin if rope else None, scale=np.float32(0.3), center=True)
+        assert np.array_equal(to_np(mean), m)
+        _codes_match(kt, y, 1, H, N, d)
+    qt, _ = binding.attn_fp8_quantize_fused(x.float().cuda(), tc, ts)                   # FP32 source
+    y, _ = P.fused_operand(to_np(x), cos, sin)
+    _codes_match(qt, y, 1, H, N, d)
+
+
 def test_attention_from_fused_operands():
     """q, k before rotary embedding -> fused producer (tau folded, keys centered) -> forward and
     backward with softmax_scale = 1, against the oracle run on the producer oracle's tensors."""
