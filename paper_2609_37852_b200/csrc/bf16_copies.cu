@@ -1,0 +1,86 @@
+// Operands of BF16 mode: the tensors themselves, rounded to BF16, in both orientations.
+#include <cuda_bf16.h>
+
+#include "common.cuh"
+#include "sm100_ptx.cuh"
+
+namespace attnfp8 {
+namespace {
+
+constexpr int kThreads = 256;
+constexpr int kTokens = 64;
+
+// Eight consecutive values as four words of two BF16 values.
+__device__ __forceinline__ uint4 load8(const __nv_bfloat16* p) { return *reinterpret_cast<const uint4*>(p); }
+__device__ __forceinline__ uint4 load8(const float* p) {
+  const float4 a = reinterpret_cast<const float4*>(p)[0], b = reinterpret_cast<const float4*>(p)[1];
+  return make_uint4(sm100::cvt_bf16x2(a.x, a.y), sm100::cvt_bf16x2(a.z, a.w), sm100::cvt_bf16x2(b.x, b.y), sm100::cvt_bf16x2(b.z, b.w));
+}
+
+// Memory-bound: each value read once and written once or twice.  One CTA transposes 64 tokens x d channels
+// through shared memory, 16 bytes per access on both sides: a thread loads eight channels of a token, and
+// stores eight tokens of two neighbouring channels, eight threads of a warp covering one 128-byte line of
+// a channel.  The 16-byte groups of token t sit at group ^ (t / 8), so that the words the lanes of a warp
+// read (eight token groups x four channel pairs) fall into 32 different banks.  The four operands of a
+// layer with 2 x (16 + 4 + 4 + 16) heads of 4096 x 128 BF16 values: 54 us with 4-byte accesses and strided
+// 2-byte shared-memory reads, 32 us now (168 MB: 5.2 TB/s, 0.80 of the measured copy bandwidth).
+template <typename T>
+__global__ void __launch_bounds__(kThreads) bf16_copies_kernel(const T* __restrict__ src, int N, int d,
+                                                               __nv_bfloat16* __restrict__ row_out,
+                                                               __nv_bfloat16* __restrict__ col_out) {
+  extern __shared__ __align__(16) uint8_t smem[];
+  uint4* tile = reinterpret_cast<uint4*>(smem);                       // [64][d / 8]
+  const uint32_t* words = reinterpret_cast<const uint32_t*>(smem);
+  const int groups = d >> 3;
+  const int mask = (groups & 7) ? 3 : 7;                              // d is a multiple of 32
+  const size_t slab = blockIdx.y;
+  const size_t tok0 = static_cast<size_t>(blockIdx.x) * kTokens;
+  const size_t first = (slab * N + tok0) * d;
+#pragma unroll 4
+  for (int i = threadIdx.x; i < kTokens * groups; i += kThreads) {
+    const int tok = i / groups, ch = i - tok * groups;
+    const uint4 v = load8(src + first + static_cast<size_t>(i) * 8);
+    tile[tok * groups + (ch ^ ((tok >> 3) & mask))] = v;
+    if (row_out) *reinterpret_cast<uint4*>(row_out + first + static_cast<size_t>(i) * 8) = v;
+  }
+  if (!col_out) return;
+  __syncthreads();
+  const int lane = threadIdx.x & 31, tg = lane & 7, cw = lane >> 3;   // token group, channel pair of the 16-byte group
+  for (int ch = threadIdx.x >> 5; ch < groups; ch += kThreads / 32) {
+    uint32_t w[8];
+#pragma unroll
+    for (int t = 0; t < 8; ++t) w[t] = words[((8 * tg + t) * groups + (ch ^ (tg & mask))) * 4 + cw];
+    uint32_t lo[4], hi[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      lo[k] = __byte_perm(w[2 * k], w[2 * k + 1], 0x5410);
+      hi[k] = __byte_perm(w[2 * k], w[2 * k + 1], 0x7632);
+    }
+    __nv_bfloat16* dst = col_out + (slab * d + 8 * ch + 2 * cw) * N + tok0 + 8 * tg;
+    *reinterpret_cast<uint4*>(dst) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+    *reinterpret_cast<uint4*>(dst + N) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+  }
+}
+
+template <typename T>
+attn_status_t launch_copies_t(const void* src, int B, int H, int N, int d, void* row_out, void* col_out,
+                              cudaStream_t stream) {
+  const size_t smem = static_cast<size_t>(kTokens) * d * sizeof(__nv_bfloat16);        // at most 32 KB
+  dim3 grid(N / kTokens, B * H);
+  bf16_copies_kernel<T><<<grid, kThreads, smem, stream>>>(static_cast<const T*>(src), N, d,
+                                                         static_cast<__nv_bfloat16*>(row_out),
+                                                         static_cast<__nv_bfloat16*>(col_out));
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "bf16 copies: launch: %s", cudaGetErrorString(e));
+  return ATTN_OK;
+}
+
+}  // namespace
+
+attn_status_t launch_bf16_copies(const void* src, int src_dtype, int B, int H, int N, int d, void* row_out, void* col_out,
+                                 cudaStream_t stream) {
+  if (src_dtype == ATTN_SRC_BF16) return launch_copies_t<__nv_bfloat16>(src, B, H, N, d, row_out, col_out, stream);
+  return launch_copies_t<float>(src, B, H, N, d, row_out, col_out, stream);
+}
+
+}  // namespace attnfp8

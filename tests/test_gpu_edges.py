@@ -221,6 +221,18 @@ def test_prepare_bf16_is_an_exact_rounding_and_transpose(dtype):
     assert torch.equal(t.col_codes, want.transpose(2, 3).contiguous())
 
 
+@pytest.mark.parametrize("d", [32, 64, 96, 160, 192, 256])
+def test_prepare_bf16_transposes_every_head_dim(d):
+    """Head dims of an odd and an even number of 64-channel groups, one CTA column of 64 tokens and several."""
+    from paper_2609_37852_b200 import binding as B
+    g = torch.Generator().manual_seed(d)
+    for n in (128, 640):
+        x = torch.randn((1, 2, n, d), generator=g).cuda()
+        t = B.attn_fp8_prepare_bf16(x)
+        assert torch.equal(t.row_codes, x.to(torch.bfloat16))
+        assert torch.equal(t.col_codes, x.to(torch.bfloat16).transpose(2, 3).contiguous())
+
+
 @pytest.mark.parametrize("d", [192, 256])
 def test_quantize_wide_heads_bit_exact(d):
     """Two 512-byte scale tiles per 128-row tile in both orientations."""
