@@ -50,15 +50,28 @@ attn_status_t encode_tmap_u8_sw128(CUtensorMap* out, const void* base, uint64_t 
 
 static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
-static attn_status_t check_device() {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
+attn_status_t current_device(int* dev, int* sms) {
+  constexpr int kKept = 64;
+  static std::atomic<uint32_t> kept[kKept];           // major << 16 | SM count; 0: not asked yet
+  cudaError_t e = cudaGetDevice(dev);
   if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "cudaGetDevice: %s", cudaGetErrorString(e));
-  int major = 0;
-  e = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
-  if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "cudaDeviceGetAttribute: %s", cudaGetErrorString(e));
-  if (major != 10) return fail(ATTN_ERR_ARCH, "device compute capability %d.x is not 10.x (sm_100a)", major);
+  uint32_t info = *dev < kKept ? kept[*dev].load(std::memory_order_relaxed) : 0;
+  if (!info) {
+    int major = 0, n = 0;
+    e = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, *dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, *dev);
+    if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "cudaDeviceGetAttribute: %s", cudaGetErrorString(e));
+    info = static_cast<uint32_t>(major) << 16 | static_cast<uint32_t>(n);
+    if (*dev < kKept) kept[*dev].store(info, std::memory_order_relaxed);
+  }
+  if (info >> 16 != 10) return fail(ATTN_ERR_ARCH, "device compute capability %d.x is not 10.x (sm_100a)", static_cast<int>(info >> 16));
+  *sms = static_cast<int>(info & 0xFFFF);
   return ATTN_OK;
+}
+
+static attn_status_t check_device() {
+  int dev = 0, sms = 0;
+  return current_device(&dev, &sms);
 }
 
 enum Entry { kEntryFwd = 0, kEntryDelta = 1, kEntryDq = 2, kEntryDkdv = 3 };
@@ -338,12 +351,6 @@ static attn_status_t bwd_impl(const attn_params_t* p, attn_qtensor_t q, attn_qte
   int* status = nullptr;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   CHECK(prepare_workspace(workspace, workspace_bytes, attn_fp8_workspace_bytes(p, ATTN_WS_BWD), st, &status));
-  if (want_dq) {
-    // the ticket counter of the persistent dQ kernel (bytes 16..31 of the header) starts at zero; cleared
-    // here, ahead of both kernels, so that nothing sits between the key-major launch and the dQ launch
-    cudaError_t e = cudaMemsetAsync(static_cast<char*>(workspace) + 16, 0, 16, st);
-    if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "bwd: cudaMemsetAsync(ticket counter): %s", cudaGetErrorString(e));
-  }
   // Key-major kernel first: its CTAs are few and long, so its last wave leaves SMs idle, which
   // the many short CTAs of the query-major kernel, launched behind it, fill.
   if (want_dkdv) CHECK(launch_bwd_dkdv(s, q, k, v, dO, lse, delta, dk_bf16, dv_bf16, status, st));

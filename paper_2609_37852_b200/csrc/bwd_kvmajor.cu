@@ -759,9 +759,9 @@ attn_status_t launch_kvmajor_t(const AttnShape& s, attn_qtensor_t q, attn_qtenso
   p.scale = s.scale; p.scale_log2 = s.scale * kLog2e;
   p.tail_wait = behind ? 1 : 0;
   const size_t smem = sizeof(KvSmem<C>) + 1024;
-  cudaError_t e = cudaFuncSetAttribute(kvmajor_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-  if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "bwd kv-major: cudaFuncSetAttribute: %s", cudaGetErrorString(e));
+  if ((st = allow_smem<kvmajor_kernel<C>>(smem, "bwd kv-major")) != ATTN_OK) return st;
   dim3 grid(s.Hkv, s.Nk / kTile, s.B);
+  cudaError_t e;
   if (behind) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid; cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = smem; cfg.stream = stream;

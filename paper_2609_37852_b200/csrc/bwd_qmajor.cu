@@ -159,7 +159,7 @@ struct QmParams {
   float* post_rowabs;
   float* p_abs_dp;          // optional (with rowsum): sum_j P_ij |dP^_ij|, the scale of the rounding dust of a row sum
   int* status;
-  int* sched;               // ticket mode: the next item number; the host zeroes it ahead of the launch
+  int* sched;               // ticket mode: the next item number; zero between calls (the last draw puts it back)
   int N, Nk, q0t, Hq, Hkv, dqk, dv, causal;   // N query rows, Nk keys, q0t: tile offset of the causal diagonal
   int kv_lim;               // without the causal mask: last real key of the last key tile (127: all real)
   int gx, gy, gz;           // the (head x column tile, query tile, batch) grid the work items are numbered in
@@ -281,7 +281,11 @@ qmajor_kernel(const QmParams p, const __grid_constant__ CUtensorMap tm_q, const 
           const int l = ticket < total_items ? ticket : -1;
           sm.item_l[i & 3] = l;
           mbar_arrive(&sm.item_full[i & 3]);
-          if (l < 0) break;
+          if (l < 0) {
+            // every CTA draws until it is refused: with this ticket all draws have been made
+            if (ticket == total_items + n_cta - 1) atomicExch(p.sched, 0);
+            break;
+          }
           it = decode_linear(l);
           ticket = atomicAdd(p.sched, 1);
         } else {
@@ -792,21 +796,19 @@ attn_status_t launch_qmajor_t(const AttnShape& s, attn_qtensor_t q, attn_qtensor
   p.tail_wait = behind_dkdv ? 1 : 0;
   p.sched = status + 4;                             // bytes 16..23 of the workspace header
   const size_t smem = sizeof(QmSmem<C>) + 1024;
-  cudaError_t e = cudaFuncSetAttribute(qmajor_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-  if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "bwd q-major: cudaFuncSetAttribute: %s", cudaGetErrorString(e));
+  if ((st = allow_smem<qmajor_kernel<C>>(smem, "bwd q-major")) != ATTN_OK) return st;
   const int rq = (kDQ && !C::kWhole) ? (s.dqk + 127) / 128 : 1;
   dim3 grid(s.Hq * rq, s.N / kTile, s.B);
   p.gx = static_cast<int>(grid.x); p.gy = static_cast<int>(grid.y); p.gz = static_cast<int>(grid.z);
   if (C::kPersist) {
     // one CTA per SM (the kernel takes a whole SM's shared memory) walks the item list
     int dev = 0, sms = 0;
-    e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess || sms < 1) return fail(ATTN_ERR_CUDA, "bwd q-major: SM count: %s", cudaGetErrorString(e));
+    if ((st = current_device(&dev, &sms)) != ATTN_OK) return st;
     const long long items = static_cast<long long>(p.gx) * p.gy * p.gz;
     if (items > 0x7fffffffLL) return fail(ATTN_ERR_UNSUPPORTED, "bwd q-major: %lld work items exceed 2^31 - 1", items);
     grid = dim3(static_cast<unsigned>(items < sms ? items : sms), 1, 1);
   }
+  cudaError_t e;
   if (behind_dkdv) {
     // the key-major kernel ahead in the stream reads what this one reads and writes other buffers:
     // this grid may take the SMs that kernel's last wave leaves idle

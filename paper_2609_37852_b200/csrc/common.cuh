@@ -1,5 +1,6 @@
 // Declarations shared by the kernels' translation units and the C-ABI layer.
 #pragma once
+#include <atomic>
 #include <cstddef>
 #include <cstdint>
 #include <cuda.h>
@@ -11,6 +12,25 @@ namespace attnfp8 {
 
 // Records a message for attn_fp8_last_error() and returns `code`.
 attn_status_t fail(attn_status_t code, const char* fmt, ...);
+
+// The current device's ordinal and SM count; fails when it is not compute capability 10.x.  What the runtime
+// says of a device is kept per ordinal: asked for on every call it was a quarter of a small call's host time.
+attn_status_t current_device(int* dev, int* sms);
+
+// Lets `kernel` ask for up to `bytes` of dynamic shared memory: one runtime call per kernel and device.
+template <auto kernel>
+attn_status_t allow_smem(size_t bytes, const char* who) {
+  static std::atomic<uint64_t> done{0};               // bit per device ordinal
+  int dev = 0, sms = 0;
+  const attn_status_t st = current_device(&dev, &sms);
+  if (st != ATTN_OK) return st;
+  const uint64_t bit = dev < 64 ? uint64_t{1} << dev : 0;
+  if (done.load(std::memory_order_acquire) & bit) return ATTN_OK;
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+  if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "%s: cudaFuncSetAttribute: %s", who, cudaGetErrorString(e));
+  done.fetch_or(bit, std::memory_order_release);
+  return ATTN_OK;
+}
 
 // Bytes at the head of every workspace reserved for the device status word.
 constexpr size_t kWorkspaceHeaderBytes = ATTN_STATUS_WORKSPACE_BYTES;

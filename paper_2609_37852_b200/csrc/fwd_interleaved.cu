@@ -617,19 +617,16 @@ attn_status_t launch_fwd_il_t(const AttnShape& s, attn_qtensor_t q, attn_qtensor
   p.N = s.N; p.Nk = s.Nk; p.q0t = s.q0t; p.kv_lim = s.kv_lim; p.Hq = s.Hq; p.Hkv = s.Hkv; p.dqk = s.dqk; p.dv = s.dv; p.causal = s.causal;
   p.scale_log2 = s.scale * kLog2e;
   const size_t smem = sizeof(IlSmem<C>) + 1024;
-  cudaError_t e = cudaFuncSetAttribute(fwd_il_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-  if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "fwd: cudaFuncSetAttribute: %s", cudaGetErrorString(e));
+  if ((st = allow_smem<fwd_il_kernel<C>>(smem, "fwd")) != ATTN_OK) return st;
   p.gx = s.Hq; p.gy = s.N / kTile; p.gz = s.B;
   const long long items = static_cast<long long>(p.gx) * p.gy * p.gz;
   if (items > 0x7fffffffLL) return fail(ATTN_ERR_UNSUPPORTED, "fwd: %lld work items exceed 2^31 - 1", items);
   // one CTA per SM (the kernel takes all of an SM's tensor memory) walks the item list
   int dev = 0, sms = 0;
-  e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e != cudaSuccess || sms < 1) return fail(ATTN_ERR_CUDA, "fwd: SM count: %s", cudaGetErrorString(e));
+  if ((st = current_device(&dev, &sms)) != ATTN_OK) return st;
   dim3 grid(static_cast<unsigned>(items < sms ? items : sms), 1, 1);
   fwd_il_kernel<C><<<grid, C::kThreads, smem, stream>>>(p, tm_q, tm_k, tm_v);
-  e = cudaGetLastError();
+  const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "fwd: launch: %s", cudaGetErrorString(e));
   return ATTN_OK;
 }

@@ -371,19 +371,15 @@ attn_status_t launch_batch_t(BatchParams& p, cudaStream_t stream) {
   else if (batch_smem_bytes(sizeof(T), p.d_max, 1) <= half_sm) p.ring = 1;
   else p.ring = batch_smem_bytes(sizeof(T), p.d_max, kMaxRing) <= whole_sm ? kMaxRing : 1;
   const size_t smem = batch_smem_bytes(sizeof(T), p.d_max, p.ring);
-  cudaError_t e = cudaFuncSetAttribute(quantize_batch_kernel<T, kProd>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
-  if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "quantize: cudaFuncSetAttribute: %s", cudaGetErrorString(e));
-  int dev = 0, sms = 0, per_sm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, quantize_batch_kernel<T, kProd>, kThreads, smem);
-  if (e != cudaSuccess || per_sm < 1 || sms < 1)
-    return fail(ATTN_ERR_CUDA, "quantize: occupancy query: %s", cudaGetErrorString(e));
+  int dev = 0, sms = 0;
+  attn_status_t st = current_device(&dev, &sms);
+  if (st == ATTN_OK) st = allow_smem<quantize_batch_kernel<T, kProd>>(whole_sm, "quantize");
+  if (st != ATTN_OK) return st;
+  const int per_sm = smem <= half_sm ? 2 : 1;        // two CTAs fit by registers (launch bounds): shared memory decides
   const int resident = sms * per_sm;
   const int grid = p.total_tiles < resident ? p.total_tiles : resident;
   quantize_batch_kernel<T, kProd><<<grid, kThreads, smem, stream>>>(p);
-  e = cudaGetLastError();
+  const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "quantize: launch: %s", cudaGetErrorString(e));
   return ATTN_OK;
 }
