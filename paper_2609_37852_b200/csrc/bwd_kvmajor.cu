@@ -186,6 +186,7 @@ struct KvParams {
   int N, Nk, q0t, Hq, Hkv, dqk, dv, causal;   // N query rows, Nk keys, q0t: tile offset of the causal diagonal
   int kv_lim;               // without the causal mask: last real key of the last key tile (127: all real)
   int tail_wait;            // launched behind another key-major pass of the same call (see launch_kvmajor_t)
+  int* tickets;             // the dQ kernel's ticket counter, to be cleared ahead of it; or null
   float scale, scale_log2;
 };
 
@@ -249,6 +250,12 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
     mbar_init(&sm.done, 1);
     sm.abort_flag = 0;
     fence_mbar_init();
+    // The dQ kernel behind this grid starts once every CTA here has passed griddepcontrol.launch_dependents
+    // (below): it finds its counter cleared, without a memset of its own between the two launches.
+    if (p.tickets != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) {
+      atomicExch(p.tickets, 0);
+      __threadfence();
+    }
   }
   if (warp == 0) {
     tmem_alloc(&sm.tmem_base, kTmemCols);
@@ -737,7 +744,7 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
 template <class C>
 attn_status_t launch_kvmajor_t(const AttnShape& s, attn_qtensor_t q, attn_qtensor_t k, attn_qtensor_t v, attn_qtensor_t dO,
                                const float* lse, const float* delta, void* dk, void* dv, int* status,
-                               cudaStream_t stream, bool behind = false) {
+                               cudaStream_t stream, bool behind = false, bool clear_tickets = false) {
   static_assert(sizeof(KvSmem<C>) + 1024 <= kSmemLimit, "shared memory exceeded");
   CUtensorMap tm_k, tm_v, tm_q, tm_dO, tm_qc, tm_dOc;
   attn_status_t st;
@@ -758,6 +765,7 @@ attn_status_t launch_kvmajor_t(const AttnShape& s, attn_qtensor_t q, attn_qtenso
   p.N = s.N; p.Nk = s.Nk; p.q0t = s.q0t; p.kv_lim = s.kv_lim; p.Hq = s.Hq; p.Hkv = s.Hkv; p.dqk = s.dqk; p.dv = s.dv; p.causal = s.causal;
   p.scale = s.scale; p.scale_log2 = s.scale * kLog2e;
   p.tail_wait = behind ? 1 : 0;
+  p.tickets = clear_tickets ? ticket_counter(status) : nullptr;
   const size_t smem = sizeof(KvSmem<C>) + 1024;
   if ((st = allow_smem<kvmajor_kernel<C>>(smem, "bwd kv-major")) != ATTN_OK) return st;
   dim3 grid(s.Hkv, s.Nk / kTile, s.B);
@@ -783,35 +791,35 @@ attn_status_t launch_kvmajor_t(const AttnShape& s, attn_qtensor_t q, attn_qtenso
 
 attn_status_t launch_bwd_dkdv(const AttnShape& s, attn_qtensor_t q, attn_qtensor_t k, attn_qtensor_t v, attn_qtensor_t dO,
                               const float* lse, const float* delta, void* dk, void* dv, int* status,
-                              cudaStream_t stream) {
+                              cudaStream_t stream, bool clear_tickets) {
   const int cq = (s.dqk * s.eb + 127) / 128, cv = (s.dv * s.ebv + 127) / 128;
   if (s.eb == 1 && s.ebv == 2) {                     // protected dP: BF16 row copies of V and dO
     if (cq == 1 && cv == 1)
-      return launch_kvmajor_t<KvCfg<1, 1, 1, kBoth, 2>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream);
+      return launch_kvmajor_t<KvCfg<1, 1, 1, kBoth, 2>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream, false, clear_tickets);
     if (cq == 1 && cv == 2)
-      return launch_kvmajor_t<KvCfg<1, 1, 2, kBoth, 2>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream);
+      return launch_kvmajor_t<KvCfg<1, 1, 2, kBoth, 2>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream, false, clear_tickets);
     return fail(ATTN_ERR_UNSUPPORTED, "bwd kv-major: protected dP is built for head dims (64,64) and (128,128)");
   }
   if (s.eb == 1 && cq == 1 && cv == 1)
-    return launch_kvmajor_t<KvCfg<1, 1, 1, kBoth>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream);
+    return launch_kvmajor_t<KvCfg<1, 1, 1, kBoth>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream, false, clear_tickets);
   if (s.eb == 2 && cq == 1 && cv == 1)
-    return launch_kvmajor_t<KvCfg<2, 1, 1, kBoth>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream);
+    return launch_kvmajor_t<KvCfg<2, 1, 1, kBoth>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream, false, clear_tickets);
   if (s.eb == 2 && cq == 2 && cv == 2)
-    return launch_kvmajor_t<KvCfg<2, 2, 2, kBoth>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream);
+    return launch_kvmajor_t<KvCfg<2, 2, 2, kBoth>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream, false, clear_tickets);
   // qk head dim above 128: dV and dK do not fit in tensor memory together; one pass each, the
   // heavier dK pass first and the dV pass launched behind it (see launch_kvmajor_t)
   // (at (192,128) both fit when every operand buffer and scale slot is single: KvCfg::kTight)
   if (s.eb == 1 && cq == 2 && cv == 1)
-    return launch_kvmajor_t<KvCfg<1, 2, 1, kBoth>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream);
+    return launch_kvmajor_t<KvCfg<1, 2, 1, kBoth>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream, false, clear_tickets);
   if (s.eb == 1 && cq == 2 && cv == 2) {
-    attn_status_t st = launch_kvmajor_t<KvCfg<1, 2, 2, kDkOnly>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream);
+    attn_status_t st = launch_kvmajor_t<KvCfg<1, 2, 2, kDkOnly>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream, false, clear_tickets);
     if (st != ATTN_OK) return st;
     return launch_kvmajor_t<KvCfg<1, 2, 2, kDvOnly>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream, true);
   }
   if (s.eb == 2 && cq == 3 && cv == 2)
-    return launch_kvmajor_t<KvCfg<2, 3, 2, kBoth>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream);
+    return launch_kvmajor_t<KvCfg<2, 3, 2, kBoth>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream, false, clear_tickets);
   if (s.eb == 2 && cq == 4 && cv == 4) {
-    attn_status_t st = launch_kvmajor_t<KvCfg<2, 4, 4, kDkOnly, 2, 0>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream);
+    attn_status_t st = launch_kvmajor_t<KvCfg<2, 4, 4, kDkOnly, 2, 0>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream, false, clear_tickets);
     if (st != ATTN_OK) return st;
     st = launch_kvmajor_t<KvCfg<2, 4, 4, kDkOnly, 2, 1>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream, true);
     if (st != ATTN_OK) return st;

@@ -159,7 +159,7 @@ struct QmParams {
   float* post_rowabs;
   float* p_abs_dp;          // optional (with rowsum): sum_j P_ij |dP^_ij|, the scale of the rounding dust of a row sum
   int* status;
-  int* sched;               // ticket mode: the next item number; zero between calls (the last draw puts it back)
+  int* sched;               // ticket mode: the next item number; the call zeroes it ahead of this kernel
   int N, Nk, q0t, Hq, Hkv, dqk, dv, causal;   // N query rows, Nk keys, q0t: tile offset of the causal diagonal
   int kv_lim;               // without the causal mask: last real key of the last key tile (127: all real)
   int gx, gy, gz;           // the (head x column tile, query tile, batch) grid the work items are numbered in
@@ -281,11 +281,7 @@ qmajor_kernel(const QmParams p, const __grid_constant__ CUtensorMap tm_q, const 
           const int l = ticket < total_items ? ticket : -1;
           sm.item_l[i & 3] = l;
           mbar_arrive(&sm.item_full[i & 3]);
-          if (l < 0) {
-            // every CTA draws until it is refused: with this ticket all draws have been made
-            if (ticket == total_items + n_cta - 1) atomicExch(p.sched, 0);
-            break;
-          }
+          if (l < 0) break;
           it = decode_linear(l);
           ticket = atomicAdd(p.sched, 1);
         } else {
@@ -794,7 +790,7 @@ attn_status_t launch_qmajor_t(const AttnShape& s, attn_qtensor_t q, attn_qtensor
   p.N = s.N; p.Nk = s.Nk; p.q0t = s.q0t; p.kv_lim = s.kv_lim; p.Hq = s.Hq; p.Hkv = s.Hkv; p.dqk = s.dqk; p.dv = s.dv; p.causal = s.causal;
   p.scale = s.scale; p.scale_log2 = s.scale * kLog2e;
   p.tail_wait = behind_dkdv ? 1 : 0;
-  p.sched = status + 4;                             // bytes 16..23 of the workspace header
+  p.sched = ticket_counter(status);
   const size_t smem = sizeof(QmSmem<C>) + 1024;
   if ((st = allow_smem<qmajor_kernel<C>>(smem, "bwd q-major")) != ATTN_OK) return st;
   const int rq = (kDQ && !C::kWhole) ? (s.dqk + 127) / 128 : 1;

@@ -35,6 +35,9 @@ attn_status_t allow_smem(size_t bytes, const char* who) {
 // Bytes at the head of every workspace reserved for the device status word.
 constexpr size_t kWorkspaceHeaderBytes = ATTN_STATUS_WORKSPACE_BYTES;
 
+// The ticket counter of the persistent dQ kernel: bytes 16..19 of the workspace header, whose first word is `status`.
+inline int* ticket_counter(int* status) { return status + 4; }
+
 // cuTensorMapEncodeTiled fetched through the runtime (no link-time dependency on libcuda).
 // Encodes a 2-D uint8 tensor [rows, row_bytes] (row pitch == row_bytes) with a
 // (box_rows x 128-byte) box and the 128-byte swizzle.
@@ -75,7 +78,7 @@ attn_status_t launch_bwd_dq(const AttnShape& s, attn_qtensor_t q, attn_qtensor_t
                             bool behind_dkdv = false, float* p_abs_dp = nullptr);
 attn_status_t launch_bwd_dkdv(const AttnShape& s, attn_qtensor_t q, attn_qtensor_t k, attn_qtensor_t v,
                               attn_qtensor_t dO, const float* lse, const float* delta, void* dk, void* dv,
-                              int* status, cudaStream_t stream);
+                              int* status, cudaStream_t stream, bool clear_tickets);
 
 attn_status_t measure_mma_peak(double* tflops_out, int* status, cudaStream_t stream);
 attn_status_t measure_dq_reduction(const AttnShape& s, float* dq_f32, double* ms_out, double* bytes_out, cudaStream_t stream);
