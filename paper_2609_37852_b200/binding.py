@@ -1,10 +1,11 @@
-"""ctypes binding of ``libattnfp8.so`` -- same entry-point names as ``include/attn_fp8.h``.
+"""Binding of ``libattnfp8.so`` -- same entry-point names as ``include/attn_fp8.h``.
 
 Argument marshalling only: tensors are torch CUDA tensors whose device pointers
 are handed to the C ABI; every step of the attention path runs in the
-library's kernels.  Importing this module fails loudly when the library has
-not been built (``python -m paper_2609_37852_b200.build``): there is no
-fallback path.
+library's kernels.  The calls of a training or inference step go through
+``_marshal`` (csrc/marshal.cpp), the rest through ctypes.  Importing this module
+fails loudly when the library has not been built
+(``python -m paper_2609_37852_b200.build``): there is no fallback path.
 """
 import ctypes
 import os
@@ -22,6 +23,7 @@ if not os.path.exists(LIB_PATH):
         f"{LIB_PATH} is missing: build the CUDA library first (python -m paper_2609_37852_b200.build); "
         "this package has no CPU or eager fallback")
 _lib = ctypes.CDLL(LIB_PATH)
+from . import _marshal  # noqa: E402  (links against the library loaded above; built with it)
 
 ATTN_OK = 0
 STATUS_NAMES = {0: "ATTN_OK", 1: "ATTN_ERR_INVALID_ARG", 2: "ATTN_ERR_UNSUPPORTED", 3: "ATTN_ERR_ALIGNMENT",
@@ -189,31 +191,20 @@ def unpack_scales(scales: torch.Tensor, B: int, H: int, rows: int, cols: int) ->
     return slab[:, idx].reshape(B, H, rows, nb)
 
 
+def _new_operand(src, want_row, want_col) -> QTensor:
+    """Buffers for the quantised ``src`` in the orientations asked for."""
+    return QTensor(tuple(src.shape), *_marshal.new_operand(src, want_row, want_col))
+
+
 def attn_fp8_quantize(src: torch.Tensor, want_row: bool = True, want_col: bool = True, stream=None,
                       out: Optional[QTensor] = None) -> QTensor:
     """Quantise ``src`` [B, H, N, d] (BF16 or FP32, CUDA, contiguous) into the requested orientations.
     ``out`` reuses the buffers of an earlier call of the same shape (its non-None orientations are written)."""
-    if not src.is_cuda or not src.is_contiguous() or src.dim() != 4:
-        raise ValueError("src must be a contiguous CUDA tensor [B, H, N, d]")
-    if src.dtype == torch.bfloat16:
-        dt = ATTN_SRC_BF16
-    elif src.dtype == torch.float32:
-        dt = ATTN_SRC_FP32
-    else:
-        raise ValueError("src must be bfloat16 or float32")
-    B, H, N, d = src.shape
     if out is None:
-        out = QTensor(shape=(B, H, N, d))
-        u8 = dict(dtype=torch.uint8, device=src.device)
-        if want_row:
-            out.row_codes = torch.empty((B, H, N, d), **u8)
-            out.row_scales = torch.empty(attn_fp8_scale_bytes(B, H, N, d), **u8)
-        if want_col:
-            out.col_codes = torch.empty((B, H, d, N), **u8)
-            out.col_scales = torch.empty(attn_fp8_scale_bytes(B, H, d, N), **u8)
-    elif tuple(out.shape) != (B, H, N, d):
-        raise ValueError("out was allocated for another shape")
-    _check(_lib.attn_fp8_quantize(_ptr(src), dt, B, H, N, d, out.c_struct(), _stream(stream)))
+        out = _new_operand(src, want_row, want_col)
+    status = _marshal.quantize(src, out, stream)
+    if status:
+        _check(status)
     return out
 
 
@@ -235,33 +226,14 @@ def attn_fp8_quantize_batch(srcs, outs=None, want=None, workspace=None, stream=N
     srcs = list(srcs)
     if outs is None:
         want = want or [(True, True)] * len(srcs)
-        outs = []
-        for x, (wr, wc) in zip(srcs, want):
-            B, H, N, d = x.shape
-            q = QTensor(shape=(B, H, N, d))
-            u8 = dict(dtype=torch.uint8, device=x.device)
-            if wr:
-                q.row_codes = torch.empty((B, H, N, d), **u8)
-                q.row_scales = torch.empty(attn_fp8_scale_bytes(B, H, N, d), **u8)
-            if wc:
-                q.col_codes = torch.empty((B, H, d, N), **u8)
-                q.col_scales = torch.empty(attn_fp8_scale_bytes(B, H, d, N), **u8)
-            outs.append(q)
-    jobs = (_QuantizeJob * len(srcs))()
-    for j, (x, q) in enumerate(zip(srcs, outs)):
-        if not x.is_cuda or not x.is_contiguous() or x.dim() != 4:
-            raise ValueError("every source must be a contiguous CUDA tensor [B, H, N, d]")
-        if x.dtype not in (torch.bfloat16, torch.float32):
-            raise ValueError("sources must be bfloat16 or float32")
-        if tuple(q.shape) != tuple(x.shape):
-            raise ValueError("an output was allocated for another shape")
-        B, H, N, d = x.shape
-        jobs[j] = _QuantizeJob(_ptr(x), ATTN_SRC_BF16 if x.dtype == torch.bfloat16 else ATTN_SRC_FP32, B, H, N, d,
-                               q.c_struct())
+        outs = [_new_operand(x, wr, wc) for x, (wr, wc) in zip(srcs, want)]
     if workspace is None:
         workspace = new_workspace(ATTN_STATUS_WORKSPACE_BYTES, srcs[0].device)
-    _check(_lib.attn_fp8_quantize_batch(jobs, len(srcs), _ptr(workspace), workspace.numel(), _stream(stream)))
-    return list(outs), workspace
+    outs = list(outs)
+    status = _marshal.quantize_batch(srcs, outs, workspace, stream)
+    if status:
+        _check(status)
+    return outs, workspace
 
 
 _lib.attn_fp8_quantize_fused.restype = _i32
@@ -273,26 +245,12 @@ def attn_fp8_quantize_fused(src: torch.Tensor, rope_cos: Optional[torch.Tensor] 
                             want_row: bool = True, want_col: bool = True, stream=None):
     """Quantiser with the producer fused in front: optional rotary embedding (FP32 tables [N, d/2]),
     optional key centering, optional FP32 scale.  Returns (QTensor, mean [B, H, d] fp32 or None)."""
-    if not src.is_cuda or not src.is_contiguous() or src.dim() != 4:
-        raise ValueError("src must be a contiguous CUDA tensor [B, H, N, d]")
-    if src.dtype not in (torch.bfloat16, torch.float32):
-        raise ValueError("src must be bfloat16 or float32")
-    dt = ATTN_SRC_BF16 if src.dtype == torch.bfloat16 else ATTN_SRC_FP32
-    B, H, N, d = src.shape
-    out = QTensor(shape=(B, H, N, d))
-    u8 = dict(dtype=torch.uint8, device=src.device)
-    if want_row:
-        out.row_codes = torch.empty((B, H, N, d), **u8)
-        out.row_scales = torch.empty(attn_fp8_scale_bytes(B, H, N, d), **u8)
-    if want_col:
-        out.col_codes = torch.empty((B, H, d, N), **u8)
-        out.col_scales = torch.empty(attn_fp8_scale_bytes(B, H, d, N), **u8)
+    out = _new_operand(src, want_row, want_col)
+    B, H, _, d = src.shape
     mean = torch.empty((B, H, d), dtype=torch.float32, device=src.device) if center else None
-    for t in (rope_cos, rope_sin):
-        if t is not None and (t.dtype != torch.float32 or not t.is_contiguous() or tuple(t.shape) != (N, d // 2)):
-            raise ValueError("rotary tables must be contiguous float32 [N, d/2]")
-    _check(_lib.attn_fp8_quantize_fused(_ptr(src), dt, B, H, N, d, _ptr(rope_cos), _ptr(rope_sin), float(scale),
-                                        _ptr(mean), out.c_struct(), _stream(stream)))
+    status = _marshal.quantize_fused(src, rope_cos, rope_sin, scale, mean, out, stream)
+    if status:
+        _check(status)
     return out, mean
 
 
@@ -305,7 +263,6 @@ def attn_fp8_prepare_bf16(src: torch.Tensor, want_row: bool = True, want_col: bo
         raise ValueError("src must be a contiguous CUDA tensor [B, H, N, d]")
     if src.dtype not in (torch.bfloat16, torch.float32):
         raise ValueError("src must be bfloat16 or float32")
-    dt = ATTN_SRC_BF16 if src.dtype == torch.bfloat16 else ATTN_SRC_FP32
     B, H, N, d = src.shape
     alias_row = src.dtype == torch.bfloat16      # the row operand is the source itself
     if out is None:
@@ -319,9 +276,9 @@ def attn_fp8_prepare_bf16(src: torch.Tensor, want_row: bool = True, want_col: bo
         raise ValueError("out was allocated for another shape")
     row_buf = None if alias_row else out.row_codes
     if row_buf is not None or out.col_codes is not None:
-        c = _QTensor(None if row_buf is None else row_buf.data_ptr(), None,
-                     None if out.col_codes is None else out.col_codes.data_ptr(), None)
-        _check(_lib.attn_fp8_prepare_bf16(_ptr(src), dt, B, H, N, d, c, _stream(stream)))
+        status = _marshal.prepare_bf16(src, row_buf, out.col_codes, stream)
+        if status:
+            _check(status)
     if alias_row and (want_row or out.row_codes is not None):
         out.row_codes = src
     return out
@@ -399,53 +356,53 @@ def attn_fp8_measure_mma_peak(workspace: torch.Tensor, stream=None) -> float:
 def attn_fp8_fwd(params: AttnParams, q: QTensor, k: QTensor, v: QTensor, o=None, lse=None, workspace=None,
                  stream=None):
     """Returns (O [B,Hq,N,dv] bf16, LSE [B,Hq,N] fp32, workspace)."""
-    dev = q.row_codes.device
     if o is None:
-        o = torch.empty((params.batch, params.heads_q, params.seqlen, params.head_dim_v), dtype=torch.bfloat16, device=dev)
+        o = torch.empty((params.batch, params.heads_q, params.seqlen, params.head_dim_v), dtype=torch.bfloat16,
+                        device=q.row_codes.device)
     if lse is None:
-        lse = torch.empty((params.batch, params.heads_q, params.seqlen), dtype=torch.float32, device=dev)
-    workspace = _workspace(params, ATTN_WS_FWD, workspace, dev)
-    c = params.c_struct()
-    _check(_lib.attn_fp8_fwd(ctypes.byref(c), q.c_struct(), k.c_struct(), v.c_struct(), _ptr(o), _ptr(lse),
-                             _ptr(workspace), workspace.numel(), _stream(stream)))
+        lse = torch.empty((params.batch, params.heads_q, params.seqlen), dtype=torch.float32, device=q.row_codes.device)
+    if workspace is None:
+        workspace = _workspace(params, ATTN_WS_FWD, None, q.row_codes.device)
+    status = _marshal.fwd(params, q, k, v, o, lse, workspace, stream)
+    if status:
+        _check(status)
     return o, lse, workspace
 
 
 def attn_fp8_bwd_delta(params: AttnParams, q: QTensor, k: QTensor, v: QTensor, dO: QTensor, lse, dO_bf16=None,
                        o_bf16=None, delta=None, workspace=None, stream=None):
     """Returns (delta [B,Hq,N] fp32, workspace).  ``params.delta_mode`` selects matched / stale."""
-    dev = lse.device
     if delta is None:
-        delta = torch.empty((params.batch, params.heads_q, params.seqlen), dtype=torch.float32, device=dev)
-    workspace = _workspace(params, ATTN_WS_BWD_DELTA, workspace, dev)
-    c = params.c_struct()
-    _check(_lib.attn_fp8_bwd_delta(ctypes.byref(c), q.c_struct(), k.c_struct(), v.c_struct(), dO.c_struct(),
-                                   _ptr(dO_bf16), _ptr(o_bf16), _ptr(lse), _ptr(delta), _ptr(workspace),
-                                   workspace.numel(), _stream(stream)))
+        delta = torch.empty((params.batch, params.heads_q, params.seqlen), dtype=torch.float32, device=lse.device)
+    if workspace is None:
+        workspace = _workspace(params, ATTN_WS_BWD_DELTA, None, lse.device)
+    status = _marshal.bwd_delta(params, q, k, v, dO, dO_bf16, o_bf16, lse, delta, workspace, stream)
+    if status:
+        _check(status)
     return delta, workspace
 
 
 def attn_fp8_bwd(params: AttnParams, q: QTensor, k: QTensor, v: QTensor, dO: QTensor, lse, delta, dq=None, dk=None,
                  dv=None, diagnostics: bool = False, workspace=None, stream=None):
     """Returns (dQ, dK, dV, rowsum_dS or None, rowsum_abs_dS or None, workspace)."""
-    dev = lse.device
-    bf = dict(dtype=torch.bfloat16, device=dev)
-    B, N = params.batch, params.seqlen
-    if dq is None:
-        dq = torch.empty((B, params.heads_q, N, params.head_dim_qk), **bf)
-    if dk is None:
-        dk = torch.empty((B, params.heads_kv, params.keys, params.head_dim_qk), **bf)
-    if dv is None:
-        dv = torch.empty((B, params.heads_kv, params.keys, params.head_dim_v), **bf)
+    if dq is None or dk is None or dv is None or diagnostics or workspace is None:
+        dev = lse.device
+        bf = dict(dtype=torch.bfloat16, device=dev)
+        B, N = params.batch, params.seqlen
+        if dq is None:
+            dq = torch.empty((B, params.heads_q, N, params.head_dim_qk), **bf)
+        if dk is None:
+            dk = torch.empty((B, params.heads_kv, params.keys, params.head_dim_qk), **bf)
+        if dv is None:
+            dv = torch.empty((B, params.heads_kv, params.keys, params.head_dim_v), **bf)
+        workspace = _workspace(params, ATTN_WS_BWD, workspace, dev)
     rs = ra = None
     if diagnostics:
         rs = torch.empty((B, params.heads_q, N), dtype=torch.float32, device=dev)
         ra = torch.empty((B, params.heads_q, N), dtype=torch.float32, device=dev)
-    workspace = _workspace(params, ATTN_WS_BWD, workspace, dev)
-    c = params.c_struct()
-    _check(_lib.attn_fp8_bwd(ctypes.byref(c), q.c_struct(), k.c_struct(), v.c_struct(), dO.c_struct(), _ptr(lse),
-                             _ptr(delta), _ptr(dq), _ptr(dk), _ptr(dv), _ptr(rs), _ptr(ra), _ptr(workspace),
-                             workspace.numel(), _stream(stream)))
+    status = _marshal.bwd(params, q, k, v, dO, lse, delta, dq, dk, dv, rs, ra, workspace, stream)
+    if status:
+        _check(status)
     return dq, dk, dv, rs, ra, workspace
 
 
@@ -461,10 +418,7 @@ def attn_fp8_bwd_dq(params: AttnParams, q: QTensor, k: QTensor, v: QTensor, dO: 
         rs = torch.empty((B, params.heads_q, N), dtype=torch.float32, device=dev)
         ra = torch.empty((B, params.heads_q, N), dtype=torch.float32, device=dev)
     workspace = _workspace(params, ATTN_WS_BWD, workspace, dev)
-    c = params.c_struct()
-    _check(_lib.attn_fp8_bwd_dq(ctypes.byref(c), q.c_struct(), k.c_struct(), v.c_struct(), dO.c_struct(), _ptr(lse),
-                                _ptr(delta), _ptr(dq), _ptr(rs), _ptr(ra), _ptr(workspace), workspace.numel(),
-                                _stream(stream)))
+    _check(_marshal.bwd_dq(params, q, k, v, dO, lse, delta, dq, rs, ra, workspace, stream))
     return dq, rs, ra, workspace
 
 
@@ -523,10 +477,7 @@ def attn_fp8_bwd_dkdv(params: AttnParams, q: QTensor, k: QTensor, v: QTensor, dO
     if dv is None:
         dv = torch.empty((B, params.heads_kv, params.keys, params.head_dim_v), **bf)
     workspace = _workspace(params, ATTN_WS_BWD, workspace, dev)
-    c = params.c_struct()
-    _check(_lib.attn_fp8_bwd_dkdv(ctypes.byref(c), q.c_struct(), k.c_struct(), v.c_struct(), dO.c_struct(),
-                                  _ptr(lse), _ptr(delta), _ptr(dk), _ptr(dv), _ptr(workspace), workspace.numel(),
-                                  _stream(stream)))
+    _check(_marshal.bwd_dkdv(params, q, k, v, dO, lse, delta, dk, dv, workspace, stream))
     return dk, dv, workspace
 
 
@@ -540,6 +491,4 @@ def attn_fp8_fwd_noalloc(params: AttnParams, q: QTensor, k: QTensor, v: QTensor,
     (already allocated, like the inputs) and no workspace; the library uses its built-in 4096-byte
     scratch array.  This wrapper allocates nothing either.  Calls that overlap on the GPU share that
     array and race; see the header for the remaining rules."""
-    c = params.c_struct()
-    _check(_lib.attn_fp8_fwd_noalloc(ctypes.byref(c), q.c_struct(), k.c_struct(), v.c_struct(), _ptr(o), _ptr(lse),
-                                     _stream(stream)))
+    _check(_marshal.fwd_noalloc(params, q, k, v, o, lse, stream))

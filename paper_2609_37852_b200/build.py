@@ -1,4 +1,5 @@
-"""Builds the C-ABI library ``libattnfp8.so`` in-tree with nvcc for sm_100a.
+"""Builds the C-ABI library ``libattnfp8.so`` in-tree with nvcc for sm_100a, and beside it ``_marshal.so``,
+the C++ side of ``binding`` (argument marshalling, compiled against the installed torch).
 
 Usage: ``python -m paper_2609_37852_b200.build`` (or ``build()`` from Python).
 Sources are compiled to objects in parallel and linked into
@@ -13,6 +14,7 @@ import sys
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "libattnfp8.so")
+MARSHAL = os.path.join(HERE, "_marshal.so")
 OBJ_DIR = os.path.join(HERE, "build")
 
 NVCC_FLAGS = [
@@ -70,7 +72,32 @@ def build(force=False, verbose=False):
         if r.returncode:
             sys.stderr.write(r.stdout + r.stderr)
             raise RuntimeError("link failed")
+    build_marshal(force, verbose)
     return OUT
+
+
+def build_marshal(force=False, verbose=False):
+    """Compile csrc/marshal.cpp into an extension module linked against the library and torch's own."""
+    src = os.path.join(CSRC, "marshal.cpp")
+    if not force and not _stale(MARSHAL, [src, os.path.join(os.path.dirname(HERE), "include", "attn_fp8.h")]):
+        return
+    import sysconfig
+    import torch
+    from torch.utils import cpp_extension
+    inc = cpp_extension.include_paths() + [sysconfig.get_paths()["include"],
+                                           os.path.join(os.path.dirname(os.path.dirname(_nvcc())), "include")]
+    lib = os.path.join(os.path.dirname(torch.__file__), "lib")
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch.compiled_with_cxx11_abi())]
+    for d in inc:
+        cmd += ["-isystem", d]
+    cmd += [src, "-o", MARSHAL, "-L" + HERE, "-lattnfp8", "-L" + lib, "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python",
+            "-Wl,-rpath,$ORIGIN", "-Wl,-rpath," + lib]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if verbose or r.returncode:
+        sys.stderr.write(" ".join(cmd) + "\n" + r.stdout + r.stderr)
+    if r.returncode:
+        raise RuntimeError("the marshalling module did not compile")
 
 
 if __name__ == "__main__":
