@@ -203,6 +203,12 @@ attn_status_t attn_fp8_quantize_fused(const void* src, int32_t src_dtype, int32_
 attn_status_t attn_fp8_prepare_bf16(const void* src, int32_t src_dtype, int32_t B, int32_t H, int32_t N,
                                     int32_t d, attn_qtensor_t out, void* stream);
 
+/* The padded form of a ragged sequence (see keys_valid): dst [B, H, n_padded, d] = src [B, H, n, d] followed by
+ * zero rows.  Any element type of `elem_bytes` bytes whose rows are a multiple of 16 bytes; src and dst 16-byte
+ * aligned, not overlapping.                                                                     */
+attn_status_t attn_fp8_pad_tokens(const void* src, int32_t elem_bytes, int32_t B, int32_t H, int32_t n, int32_t d,
+                                  int32_t n_padded, void* dst, void* stream);
+
 /* Forward (paper Appendix "Forward Probability Encoding"): per query row, online softmax of
  * S = scale * Q^ K^^T over key tiles with a running INTEGER power-of-two shift, normaliser l
  * taken from the exponentials BEFORE the FP8 cast, probabilities quantised in-register in

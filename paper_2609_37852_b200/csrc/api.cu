@@ -271,6 +271,17 @@ attn_status_t attn_fp8_prepare_bf16(const void* src, int32_t src_dtype, int32_t 
   return launch_bf16_copies(src, src_dtype, B, H, N, d, out.row_codes, out.col_codes, static_cast<cudaStream_t>(stream));
 }
 
+attn_status_t attn_fp8_pad_tokens(const void* src, int32_t elem_bytes, int32_t B, int32_t H, int32_t n, int32_t d,
+                                  int32_t n_padded, void* dst, void* stream) {
+  if (B <= 0 || H <= 0 || n <= 0 || d <= 0 || elem_bytes <= 0) return fail(ATTN_ERR_INVALID_ARG, "sizes must be positive");
+  if (n_padded < n) return fail(ATTN_ERR_INVALID_ARG, "n_padded (%d) is smaller than n (%d)", n_padded, n);
+  const long long row_bytes = static_cast<long long>(d) * elem_bytes;
+  if (row_bytes % 16) return fail(ATTN_ERR_UNSUPPORTED, "pad_tokens needs rows of a multiple of 16 bytes (%lld)", row_bytes);
+  CHECK(check_ptr(src, "src")); CHECK(check_ptr(dst, "dst"));
+  CHECK(check_device());
+  return launch_pad_tokens(src, static_cast<long long>(B) * H, row_bytes, n, n_padded, dst, static_cast<cudaStream_t>(stream));
+}
+
 size_t attn_fp8_workspace_bytes(const attn_params_t* p, int32_t which) {
   (void)p;
   (void)which;

@@ -8,6 +8,7 @@
 #include <torch/csrc/autograd/python_variable.h>
 
 #include <ATen/ops/empty.h>
+#include <c10/cuda/CUDAFunctions.h>
 #include <c10/cuda/CUDAStream.h>
 
 #include "../../include/attn_fp8.h"
@@ -328,10 +329,30 @@ PyObject* new_operand(PyObject*, PyObject* const* a, Py_ssize_t n) {
   });
 }
 
+// (x, n_padded): the padded tensor, or None where the kernel does not apply (the caller pads with torch then)
+PyObject* pad_tokens(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  return guarded(n, 2, [&]() -> PyObject* {
+    if (!THPVariable_Check(a[0])) Py_RETURN_NONE;
+    const at::Tensor& x = THPVariable_Unpack(a[0]);
+    const int64_t rows = integer(a[1]);
+    if (!x.is_cuda() || !x.is_contiguous() || x.dim() != 4 || x.requires_grad() || x.numel() == 0 || x.is_conj() || x.is_neg() ||
+        (x.size(3) * x.element_size()) % 16 || reinterpret_cast<uintptr_t>(x.data_ptr()) % 16 || x.size(0) * x.size(1) > INT32_MAX ||
+        x.get_device() != c10::cuda::current_device())
+      Py_RETURN_NONE;
+    at::Tensor out = at::empty({x.size(0), x.size(1), rows, x.size(3)}, x.options());
+    const attn_status_t st = attn_fp8_pad_tokens(x.data_ptr(), static_cast<int32_t>(x.element_size()), static_cast<int32_t>(x.size(0)),
+                                                 static_cast<int32_t>(x.size(1)), static_cast<int32_t>(x.size(2)),
+                                                 static_cast<int32_t>(x.size(3)), static_cast<int32_t>(rows), out.data_ptr(),
+                                                 c10::cuda::getCurrentCUDAStream().stream());
+    if (st != ATTN_OK) fail(PyExc_RuntimeError, attn_fp8_last_error());
+    return THPVariable_Wrap(out);
+  });
+}
+
 PyMethodDef methods[] = {
 #define ENTRY(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(name)), METH_FASTCALL, nullptr}
     ENTRY(fwd), ENTRY(fwd_noalloc), ENTRY(bwd_delta), ENTRY(bwd), ENTRY(bwd_dq), ENTRY(bwd_dkdv), ENTRY(quantize),
-    ENTRY(quantize_batch), ENTRY(quantize_fused), ENTRY(prepare_bf16), ENTRY(new_operand),
+    ENTRY(quantize_batch), ENTRY(quantize_fused), ENTRY(prepare_bf16), ENTRY(new_operand), ENTRY(pad_tokens),
 #undef ENTRY
     {nullptr, nullptr, 0, nullptr}};
 

@@ -73,6 +73,20 @@ def test_ragged_lengths_match_the_unpadded_oracle(name, kw, n_real, bf16):
     assert float(np.median(r)) <= 1e-5
 
 
+@pytest.mark.parametrize("shape,dtype", [((1, 1, 1, 64), torch.bfloat16), ((2, 3, 129, 96), torch.float32), ((1, 2, 511, 256), torch.bfloat16),
+                                         ((2, 2, 100, 4), torch.bfloat16)])      # rows of 8 bytes: not the kernel's
+def test_pad_tokens_appends_zero_rows(shape, dtype):
+    from paper_2609_37852_b200 import binding as B
+    x = torch.randn(shape, device="cuda").to(dtype)
+    for t in (x, x.transpose(1, 2).contiguous().transpose(1, 2)):                # contiguous, and strided
+        y = B.pad_tokens(t)
+        n = shape[2]
+        assert y.shape == (shape[0], shape[1], -(-n // 128) * 128, shape[3]) and y.dtype == dtype
+        assert torch.equal(y[:, :, :n], x) and not y[:, :, n:].any()
+    y = B.pad_tokens(x.clone().requires_grad_(True))                             # stays differentiable
+    y.sum().backward()
+
+
 def test_keys_valid_is_validated():
     from paper_2609_37852_b200 import binding as B
     w = workloads.WORKLOADS["gqa4k"].scaled(batch=1, heads_q=2, heads_kv=1, seqlen=256)
