@@ -25,9 +25,8 @@ __device__ __forceinline__ uint4 load8(const float* p) {
 // layer with 2 x (16 + 4 + 4 + 16) heads of 4096 x 128 BF16 values: 54 us with 4-byte accesses and strided
 // 2-byte shared-memory reads, 32 us now (168 MB: 5.2 TB/s, 0.80 of the measured copy bandwidth).
 template <typename T>
-__global__ void __launch_bounds__(kThreads) bf16_copies_kernel(const T* __restrict__ src, int N, int d,
-                                                               __nv_bfloat16* __restrict__ row_out,
-                                                               __nv_bfloat16* __restrict__ col_out) {
+__global__ void __launch_bounds__(kThreads) bf16_copies_kernel(const T* src, int N, int d, __nv_bfloat16* row_out,
+                                                               __nv_bfloat16* col_out) {
   extern __shared__ __align__(16) uint8_t smem[];
   uint4* tile = reinterpret_cast<uint4*>(smem);                       // [64][d / 8]
   const uint32_t* words = reinterpret_cast<const uint32_t*>(smem);
@@ -36,6 +35,7 @@ __global__ void __launch_bounds__(kThreads) bf16_copies_kernel(const T* __restri
   const size_t slab = blockIdx.y;
   const size_t tok0 = static_cast<size_t>(blockIdx.x) * kTokens;
   const size_t first = (slab * N + tok0) * d;
+  sm100::griddep_begin();
 #pragma unroll 4
   for (int i = threadIdx.x; i < kTokens * groups; i += kThreads) {
     const int tok = i / groups, ch = i - tok * groups;
@@ -67,10 +67,8 @@ attn_status_t launch_copies_t(const void* src, int B, int H, int N, int d, void*
                               cudaStream_t stream) {
   const size_t smem = static_cast<size_t>(kTokens) * d * sizeof(__nv_bfloat16);        // at most 32 KB
   dim3 grid(N / kTokens, B * H);
-  bf16_copies_kernel<T><<<grid, kThreads, smem, stream>>>(static_cast<const T*>(src), N, d,
-                                                         static_cast<__nv_bfloat16*>(row_out),
-                                                         static_cast<__nv_bfloat16*>(col_out));
-  cudaError_t e = cudaGetLastError();
+  const cudaError_t e = launch_overlapped(bf16_copies_kernel<T>, grid, kThreads, smem, stream, 1, static_cast<const T*>(src), N, d,
+                                          static_cast<__nv_bfloat16*>(row_out), static_cast<__nv_bfloat16*>(col_out));
   if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "bf16 copies: launch: %s", cudaGetErrorString(e));
   return ATTN_OK;
 }

@@ -769,20 +769,16 @@ attn_status_t launch_kvmajor_t(const AttnShape& s, attn_qtensor_t q, attn_qtenso
   const size_t smem = sizeof(KvSmem<C>) + 1024;
   if ((st = allow_smem<kvmajor_kernel<C>>(smem, "bwd kv-major")) != ATTN_OK) return st;
   dim3 grid(s.Hkv, s.Nk / kTile, s.B);
+  // The first pass is launched behind whatever is ahead in the stream in the ordinary way: with programmatic
+  // serialisation there as well, the kernels behind this one no longer started beside it (dK, dV and dQ at head
+  // dim 256, 8/2 heads, one after the other: step 1065 -> 1257 us).
   cudaError_t e;
   if (behind) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid; cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, kvmajor_kernel<C>, p, tm_k, tm_v, tm_q, tm_dO, tm_qc, tm_dOc);
-    if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "bwd kv-major: launch: %s", cudaGetErrorString(e));
+    e = launch_overlapped(kvmajor_kernel<C>, grid, kThreads, smem, stream, 1, p, tm_k, tm_v, tm_q, tm_dO, tm_qc, tm_dOc);
   } else {
     kvmajor_kernel<C><<<grid, kThreads, smem, stream>>>(p, tm_k, tm_v, tm_q, tm_dO, tm_qc, tm_dOc);
+    e = cudaGetLastError();
   }
-  e = cudaGetLastError();
   if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "bwd kv-major: launch: %s", cudaGetErrorString(e));
   return ATTN_OK;
 }

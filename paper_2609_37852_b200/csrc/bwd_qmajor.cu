@@ -254,6 +254,10 @@ qmajor_kernel(const QmParams p, const __grid_constant__ CUtensorMap tm_q, const 
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
+  // (behind the key-major kernel of the same call there is nothing to wait for at the start: that kernel was ordered
+  // after what both read, and this one waits for it at its end)
+  if (!p.tail_wait) griddep_wait();
+  griddep_launch_dependents();
   const uint32_t tmem = sm.tmem_base;
 
   if (warp == 0) {
@@ -804,22 +808,9 @@ attn_status_t launch_qmajor_t(const AttnShape& s, attn_qtensor_t q, attn_qtensor
     if (items > 0x7fffffffLL) return fail(ATTN_ERR_UNSUPPORTED, "bwd q-major: %lld work items exceed 2^31 - 1", items);
     grid = dim3(static_cast<unsigned>(items < sms ? items : sms), 1, 1);
   }
-  cudaError_t e;
-  if (behind_dkdv) {
-    // the key-major kernel ahead in the stream reads what this one reads and writes other buffers:
-    // this grid may take the SMs that kernel's last wave leaves idle
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid; cfg.blockDim = dim3(C::kThreads); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, qmajor_kernel<C>, p, tm_q, tm_dO, tm_k, tm_v, tm_kc);
-    if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "bwd q-major: launch: %s", cudaGetErrorString(e));
-  } else {
-    qmajor_kernel<C><<<grid, C::kThreads, smem, stream>>>(p, tm_q, tm_dO, tm_k, tm_v, tm_kc);
-  }
-  e = cudaGetLastError();
+  // behind the key-major kernel, which reads what this one reads and writes other buffers, this grid takes the SMs
+  // that kernel's last wave leaves idle
+  const cudaError_t e = launch_overlapped(qmajor_kernel<C>, grid, C::kThreads, smem, stream, 1, p, tm_q, tm_dO, tm_k, tm_v, tm_kc);
   if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "bwd q-major: launch: %s", cudaGetErrorString(e));
   return ATTN_OK;
 }
@@ -849,10 +840,10 @@ attn_status_t launch_qmajor(const AttnShape& s, attn_qtensor_t q, attn_qtensor_t
 }
 
 // Stale delta: D_i = sum_c dO_ic O_ic from the BF16 tensors (paper Section 3.2).  One warp per row.
-__global__ void stale_delta_kernel(const __nv_bfloat16* __restrict__ dO, const __nv_bfloat16* __restrict__ o,
-                                   float* __restrict__ delta, size_t rows, int dv) {
+__global__ void stale_delta_kernel(const __nv_bfloat16* dO, const __nv_bfloat16* o, float* delta, size_t rows, int dv) {
   const size_t row = (static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
+  griddep_begin();
   if (row >= rows) return;
   float acc = 0.f;
   for (int c = lane * 2; c < dv; c += 64) {
@@ -869,11 +860,11 @@ __global__ void stale_delta_kernel(const __nv_bfloat16* __restrict__ dO, const _
 // Consistent dO (paper Section 3.3): the saved-output shortcut with dO replaced by the FP8 operand
 // the backward matmuls consume, D_i = sum_c dO^_ic O_ic with dO^ = code * 2^(byte - 127) from the
 // row-blocked copy.  One warp per row, four codes per lane and step.
-__global__ void consistent_delta_kernel(const uint8_t* __restrict__ dO_codes, const uint8_t* __restrict__ dO_scales,
-                                        const __nv_bfloat16* __restrict__ o, float* __restrict__ delta, size_t rows,
-                                        int N, int dv) {
+__global__ void consistent_delta_kernel(const uint8_t* dO_codes, const uint8_t* dO_scales, const __nv_bfloat16* o, float* delta,
+                                        size_t rows, int N, int dv) {
   const size_t row = (static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
+  griddep_begin();
   if (row >= rows) return;
   const size_t slab = row / N;
   const int r = static_cast<int>(row % N);
@@ -910,9 +901,8 @@ attn_status_t launch_consistent_delta(const AttnShape& s, attn_qtensor_t dO, con
   const size_t rows = static_cast<size_t>(s.B) * s.Hq * s.N;
   const int threads = 256;
   const size_t blocks = (rows * 32 + threads - 1) / threads;
-  consistent_delta_kernel<<<static_cast<unsigned>(blocks), threads, 0, stream>>>(
+  const cudaError_t e = launch_overlapped(consistent_delta_kernel, dim3(static_cast<unsigned>(blocks)), threads, 0, stream, 1,
       dO.row_codes, dO.row_scales, static_cast<const __nv_bfloat16*>(o_bf16), delta, rows, s.N, s.dv);
-  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "consistent delta: launch: %s", cudaGetErrorString(e));
   return ATTN_OK;
 }
@@ -935,9 +925,8 @@ attn_status_t launch_stale_delta(const AttnShape& s, const void* dO_bf16, const 
   const size_t rows = static_cast<size_t>(s.B) * s.Hq * s.N;
   const int threads = 256;
   const size_t blocks = (rows * 32 + threads - 1) / threads;
-  stale_delta_kernel<<<static_cast<unsigned>(blocks), threads, 0, stream>>>(
+  const cudaError_t e = launch_overlapped(stale_delta_kernel, dim3(static_cast<unsigned>(blocks)), threads, 0, stream, 1,
       static_cast<const __nv_bfloat16*>(dO_bf16), static_cast<const __nv_bfloat16*>(o_bf16), delta, rows, s.dv);
-  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "stale delta: launch: %s", cudaGetErrorString(e));
   return ATTN_OK;
 }

@@ -32,6 +32,26 @@ attn_status_t allow_smem(size_t bytes, const char* who) {
   return ATTN_OK;
 }
 
+// Launches `kernel` so that it may start while the kernel ahead of it in the stream is finishing (programmatic
+// stream serialisation): a kernel of the library sets itself up, executes griddepcontrol.wait before its first
+// access to global memory, and lets the next one start as soon as that has returned.  What overlaps is the
+// launch, barrier initialisation, tensor-memory allocation and descriptor fetch of one kernel and the tail of the
+// one ahead: a step of one head of 256 tokens went from 32.5 to 28 us, a padded forward of 24 heads of 1111 tokens
+// (five launches) from 69 to 62 us, an encoder step from 133 to 122 us.  `cluster`: CTAs per cluster along x.
+template <class... Params, class... Args>
+cudaError_t launch_overlapped(void (*kernel)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t stream, int cluster,
+                              Args&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid; cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr; cfg.numAttrs = cluster > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+
 // Bytes at the head of every workspace reserved for the device status word.
 constexpr size_t kWorkspaceHeaderBytes = ATTN_STATUS_WORKSPACE_BYTES;
 

@@ -161,6 +161,7 @@ fwd_kernel(const FwdParams p, const __grid_constant__ CUtensorMap tm_q, const __
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
+  griddep_begin();
   const uint32_t tmem = sm.tmem_base;
 
   if (warp == 0) {
@@ -475,8 +476,7 @@ attn_status_t launch_fwd_t(const AttnShape& s, attn_qtensor_t q, attn_qtensor_t 
   const size_t smem = sizeof(FwdSmem<C>) + 1024;
   if ((st = allow_smem<fwd_kernel<C>>(smem, "fwd")) != ATTN_OK) return st;
   dim3 grid(s.Hq, s.N / kTile, s.B);
-  fwd_kernel<C><<<grid, C::kThreads, smem, stream>>>(p, tm_q, tm_k, tm_v);
-  const cudaError_t e = cudaGetLastError();
+  const cudaError_t e = launch_overlapped(fwd_kernel<C>, grid, C::kThreads, smem, stream, 1, p, tm_q, tm_k, tm_v);
   if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "fwd: launch: %s", cudaGetErrorString(e));
   return ATTN_OK;
 }

@@ -198,6 +198,7 @@ fwd_il_kernel(const IlParams p, const __grid_constant__ CUtensorMap tm_q, const 
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
+  griddep_begin();
   const uint32_t tmem = sm.tmem_base;
 
   if (warp < 4) {
@@ -625,8 +626,7 @@ attn_status_t launch_fwd_il_t(const AttnShape& s, attn_qtensor_t q, attn_qtensor
   int dev = 0, sms = 0;
   if ((st = current_device(&dev, &sms)) != ATTN_OK) return st;
   dim3 grid(static_cast<unsigned>(items < sms ? items : sms), 1, 1);
-  fwd_il_kernel<C><<<grid, C::kThreads, smem, stream>>>(p, tm_q, tm_k, tm_v);
-  const cudaError_t e = cudaGetLastError();
+  const cudaError_t e = launch_overlapped(fwd_il_kernel<C>, grid, C::kThreads, smem, stream, 1, p, tm_q, tm_k, tm_v);
   if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "fwd: launch: %s", cudaGetErrorString(e));
   return ATTN_OK;
 }

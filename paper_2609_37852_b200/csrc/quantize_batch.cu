@@ -299,8 +299,10 @@ __global__ void __launch_bounds__(kThreads, 2) quantize_batch_kernel(const __gri
     for (int s = 0; s < n_ring; ++s) mbar_init(&full[s], 1);
     *abort_flag = 0;
     fence_mbar_init();
-    for (int i = 0; i < n_ring && i < my_tiles; ++i) issue(i);
   }
+  griddep_begin();
+  if (tid == 0)
+    for (int i = 0; i < n_ring && i < my_tiles; ++i) issue(i);
   __syncthreads();
 
   for (int i = 0; i < my_tiles; ++i) {
@@ -378,8 +380,7 @@ attn_status_t launch_batch_t(BatchParams& p, cudaStream_t stream) {
   const int per_sm = smem <= half_sm ? 2 : 1;        // two CTAs fit by registers (launch bounds): shared memory decides
   const int resident = sms * per_sm;
   const int grid = p.total_tiles < resident ? p.total_tiles : resident;
-  quantize_batch_kernel<T, kProd><<<grid, kThreads, smem, stream>>>(p);
-  const cudaError_t e = cudaGetLastError();
+  const cudaError_t e = launch_overlapped(quantize_batch_kernel<T, kProd>, dim3(grid), kThreads, smem, stream, 1, p);
   if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "quantize: launch: %s", cudaGetErrorString(e));
   return ATTN_OK;
 }

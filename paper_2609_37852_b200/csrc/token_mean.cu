@@ -46,9 +46,8 @@ constexpr int kMaxCluster = 8;
 constexpr int kMeanThreads = 512;
 
 template <typename T>
-__global__ void __launch_bounds__(kMeanThreads, 2) token_mean_kernel(const T* __restrict__ src, int N, int d,
-                                                              const float* __restrict__ cos, const float* __restrict__ sin,
-                                                              float* __restrict__ mean) {
+__global__ void __launch_bounds__(kMeanThreads, 2) token_mean_kernel(const T* src, int N, int d, const float* cos,
+                                                                     const float* sin, float* mean) {
   extern __shared__ __align__(16) uint8_t smem[];
   double* part = reinterpret_cast<double*>(smem);                   // [phases][d], then the CTA's sums in row 0
   cg::cluster_group cluster = cg::this_cluster();
@@ -59,6 +58,7 @@ __global__ void __launch_bounds__(kMeanThreads, 2) token_mean_kernel(const T* __
   const T* g = src + slab * N * d + pc;
   const int per = N / ranks;                                         // N is a multiple of 128
   const int n0 = rank * per, n1 = rank == ranks - 1 ? N : n0 + per;
+  sm100::griddep_begin();
   if (ph < phases) {
     double lo[4], hi[4];
 #pragma unroll
@@ -115,16 +115,8 @@ attn_status_t launch_mean_t(const void* src, int slabs, int N, int d, const floa
   while (ranks < kMaxCluster && slabs * ranks < 296 && 2 * ranks <= N / 128) ranks *= 2;
   const int chunks = d / 8;
   const size_t smem = static_cast<size_t>(kMeanThreads / chunks) * d * sizeof(double);   // 32 KB
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(static_cast<unsigned>(slabs) * ranks);
-  cfg.blockDim = dim3(kMeanThreads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = ranks; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr; cfg.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, token_mean_kernel<T>, static_cast<const T*>(src), N, d, cos, sin, mean);
+  const cudaError_t e = launch_overlapped(token_mean_kernel<T>, dim3(static_cast<unsigned>(slabs) * ranks), kMeanThreads, smem, stream,
+                                          ranks, static_cast<const T*>(src), N, d, cos, sin, mean);
   if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "token mean: launch: %s", cudaGetErrorString(e));
   return ATTN_OK;
 }

@@ -77,3 +77,33 @@ def test_captured_step_replays_bit_identically(name, kw):
         B.attn_fp8_read_status(bufs["ws"])
         for k in keys:
             assert torch.equal(bufs[k], eager[tag][k]), f"replay on input {tag}: {k} differs from the eager step"
+
+
+@pytest.mark.parametrize("name,kw", [
+    ("tiny", dict()),                                             # every kernel is launched while the one ahead runs
+    ("gqa4k", dict(batch=1, heads_q=8, heads_kv=2, seqlen=1152)),
+    ("gqa8k_d256", dict(heads_q=4, heads_kv=1, seqlen=512)),
+])
+def test_steps_back_to_back_equal_steps_waited_for(name, kw):
+    """The kernels of consecutive steps overlap at their edges: steps that alternate between two inputs through
+    the same operand and output buffers, with no wait between them, give the results of steps run alone."""
+    from paper_2609_37852_b200 import binding as B
+    w = workloads.WORKLOADS[name].scaled(**kw)
+    params = B.AttnParams(w.batch, w.seqlen, w.heads_q, w.heads_kv, w.head_dim_qk, w.head_dim_v, w.causal, w.softmax_scale)
+    keys = ("o", "lse", "delta", "dq", "dk", "dv")
+    inputs = [[x.cuda() for x in workloads.make_inputs(w.scaled(index=w.index + i))] for i in (0, 40)]
+    bufs, alone = _buffers(B, params, inputs[0]), []
+    for inp in inputs:
+        torch.cuda.synchronize()
+        _step(B, params, inp, bufs)
+        torch.cuda.synchronize()
+        alone.append({k: bufs[k].clone() for k in keys})
+    got = []
+    for i in range(12):
+        _step(B, params, inputs[i % 2], bufs)
+        if i >= 8:
+            got.append({k: bufs[k].clone() for k in keys})        # (copies of torch's, queued behind the step)
+    B.attn_fp8_read_status(bufs["ws"])
+    for i, g in enumerate(got):
+        for k in keys:
+            assert torch.equal(g[k], alone[i % 2][k]), (i, k)
