@@ -78,7 +78,7 @@ struct KvCfg {
   static constexpr int kRowBytes = (kCq + (kHasDk ? kCv : 0)) * kRowTok * 128;
   // (192,128) with both gradients in one pass (see kTight below): the Q^c stage holds the 192 rows it is
   // loaded with, not two full row tiles, which leaves room for a third row stage
-  static constexpr bool kTightDims = kMode_ == kBoth && ((kEB == 1 && kEBv == 1 && kCq == 2 && kCv == 1) || (kEB == 2 && kEBv == 2 && kCq == 3 && kCv == 2));
+  static constexpr bool kTightDims = kMode == kBoth && ((kFp8 && kFp8v && kCq == 2 && kCv == 1) || (kEB == 2 && kEBv == 2 && kCq == 3 && kCv == 2));
   static constexpr int kQcRows = kTightDims ? 192 : kRqAcc * kTile;
   static constexpr int kColBytes = ((kHasDk ? kQcRows : 0) + (kHasDv ? kRv * kTile : 0)) * 128;
   // rings shrink to one stage where two do not fit (wide heads in BF16 mode): loads and MMAs of
@@ -100,18 +100,25 @@ struct KvCfg {
   // (LSE arrives in the stage by a bulk copy), the preparation warp once it has read LSE out of the stage
   static constexpr int kRowReleases = !kEarly ? 1 : (kHasDk ? 2 : (kEB == 1 ? 1 : 2));
   static constexpr int kLseSlots = kEarly ? ((kRowStages + 4) & ~1) : kRowStages;
-  // tensor memory
-  // FP8 at (192, 128) with both gradients in one pass: dV 128 + dK 192 columns beside the score tiles
-  // fill tensor memory exactly when the P^ / dS^ operands and every scale-factor slot are single and the
-  // scale columns of the two gradient products are shared (they are used one after the other by one
-  // issuing thread): 64 + 64 + 16 + 16 + 128 + 192 + SF 32 = 512.
-  // (BF16 at the same head dims: no scale factors, 64 + 64 + 32 + 32 + 128 + 192 = 512 with single operand buffers)
-  static constexpr bool kTight = kMode == kBoth && ((kFp8 && kFp8v && kCq == 2 && kCv == 1) || (kEB == 2 && kEBv == 2 && kCq == 3 && kCv == 2));
-  static constexpr int kOpBufs = kTight ? 1 : 2;       // P^ / dS^ operand buffers
+  // Tensor memory.  BF16 mode has no scale factors, which leaves columns for a second S^T buffer (one per team) when
+  // P^ and dS^ keep one operand buffer each; S^T and dP^T are then released one by one (kApart: the softmax takes S,
+  // releases it, and takes dP after its exponentials), so that no team waits for the turnaround of a score buffer
+  // (issue, completion, wake-up, load, release) the other still uses: dK / dV of the 4K layer 297 -> 276 us.  FP8 at
+  // the same head dims fits as well with single scale slots, and loses (8K layer, 725 -> 770 us): its teams then are
+  // busy all the time, and an exponential loop apart from the dS arithmetic leaves the other pipes idle.
+  //   BF16, head dims 64 and 128:  2 x 64 + 64 + 32 + 32 + 128 + 128 = 512
+  // (192,128): dV 128 + dK 192 columns beside the score tiles fill tensor memory exactly when the P^ / dS^ operands and
+  // every scale-factor slot are single and the scale columns of the two gradient products are shared (one issuing
+  // thread uses them one after the other; its copies and MMAs run in the order issued):
+  //   FP8   64 + 64 + 16 + 16 + 128 + 192 + SF 32 = 512       BF16   64 + 64 + 32 + 32 + 128 + 192 = 512
+  static constexpr bool kTight = kTightDims;
+  static constexpr bool kApart = kMode == kBoth && kEB == 2 && !kTight;
+  static constexpr int kSBufs = kApart ? 2 : 1;
+  static constexpr int kOpBufs = kTight || kApart ? 1 : 2;   // P^ / dS^ operand buffers
   static constexpr int kSl = kTight ? 1 : 2;           // scale-factor slots per streamed stage
   static constexpr int kOpCols = 16 * kEB;             // columns of one P^ / dS^ buffer (64 queries)
   static constexpr uint32_t kColS = 0;
-  static constexpr uint32_t kColdP = 64;
+  static constexpr uint32_t kColdP = 64 * kSBufs;
   static constexpr uint32_t kColP = kColdP + (kHasDk ? 64 : 0);
   static constexpr uint32_t kColdS = kColP + (kHasDv ? kOpBufs * kOpCols : 0);
   static constexpr uint32_t kColdV = kColdS + (kHasDk ? kOpBufs * kOpCols : 0);
@@ -121,10 +128,10 @@ struct KvCfg {
   static constexpr uint32_t kColSFQ = kColSFV + (kHasDk && kFp8v ? 4 * kCv : 0);   // kSl slots
   static constexpr uint32_t kColSFdO = kColSFQ + 4 * kSl * kCq;                // kSl slots
   static constexpr uint32_t kColSFP = kColSFdO + (kHasDk && kFp8v ? 4 * kSl * kCv : 0);  // kOpBufs x 4
-  static constexpr uint32_t kColSFdS = kTight ? kColSFP : kColSFP + (kHasDv ? 8 : 0);   // kOpBufs x 4
-  static constexpr uint32_t kColSFdOc = kColSFdS + (kTight ? 4 : (kHasDk ? 8 : 0));     // kSl slots x row tiles
-  static constexpr uint32_t kColSFQc = kTight ? kColSFdOc : kColSFdOc + (kHasDv ? 8 * kRv : 0);   // kSl slots x row tiles
-  static constexpr uint32_t kColsUsed = kFp8 ? (kTight ? kColSFQc + 4 : kColSFQc + (kHasDk ? 8 * kRqAcc : 0)) : kColSFK;
+  static constexpr uint32_t kColSFdS = kTight ? kColSFP : kColSFP + (kHasDv ? 4 * kOpBufs : 0);   // kOpBufs x 4
+  static constexpr uint32_t kColSFdOc = kColSFdS + (kTight ? 4 : (kHasDk ? 4 * kOpBufs : 0));     // kSl slots x row tiles
+  static constexpr uint32_t kColSFQc = kTight ? kColSFdOc : kColSFdOc + (kHasDv ? 4 * kSl * kRv : 0);   // kSl slots x row tiles
+  static constexpr uint32_t kColsUsed = kFp8 ? (kTight ? kColSFQc + 4 : kColSFQc + (kHasDk ? 4 * kSl * kRqAcc : 0)) : kColSFK;
   static constexpr uint32_t kTmemCols = 512;
   static_assert(kColsUsed <= 512, "tensor memory exceeded");
 };
@@ -163,13 +170,16 @@ struct KvSmem {
   uint64_t lse_ready[C::kLseSlots];
   alignas(16) float lse_ring[C::kEarly ? C::kLseSlots : 1][kSub];     // kEarly: -LSE * log2(e) of a sub-tile
   alignas(16) float delta_ring[C::kEarly ? C::kLseSlots : 1][kSub];   // kEarly: -D
-  uint64_t sdp_full[kTeams], sdp_free[kTeams];
-  // P^ / dS^ hand-off.  "free" barriers are per softmax team (the team that writes the buffer next waits on its
-  // own: a team takes every other sub-tile, and a parity wait on a barrier that completes once per sub-tile
-  // would pass at once for a waiter a whole phase behind).  With a single operand buffer P^ and dS^ are handed
-  // over separately (p_full / p_free for P^), so that the next P^ is written while the dK MMAs still run.
-  uint64_t pds_full[2], pds_free[2];
+  // Hand-offs between the issuing threads and the softmax teams, per team: a team takes every other sub-tile, and a
+  // parity wait on a barrier that completes once per sub-tile would pass at once for a waiter a whole phase behind.
+  // s_full stands for S, LSE and (unless kApart) dP; dp_full / dp_free for dP taken apart.
+  uint64_t s_full[kTeams], s_free[kTeams];
+  uint64_t dp_full[kTeams], dp_free[kTeams];
+  // P^ and dS^ on their way back.  "free": the team that writes the buffer next waits on its own.  With a single
+  // operand buffer P^ and dS^ are handed over separately (p_full / p_free for P^), so that the next P^ is written
+  // while the dK MMAs still run.
   uint64_t p_full, p_free[2];
+  uint64_t op_full[2], op_free[2];
   uint64_t done;
   uint64_t drain[3];
   uint32_t tmem_base;
@@ -209,6 +219,8 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
   // (FP8 only: in BF16 mode the producer is not what paces the kernel, and the change cost 5 % there)
   constexpr bool kPrepLoads = kFp8 && C::kRowTok == kSub;
   constexpr bool kSplit = kOpBufs == 1;          // single operand buffer: P^ and dS^ are handed over separately
+  constexpr bool kApart = C::kApart;
+  constexpr int kSBufs = C::kSBufs;
   constexpr uint32_t kColS = C::kColS, kColdP = C::kColdP, kColP = C::kColP, kColdS = C::kColdS, kColdV = C::kColdV,
                      kColdK = C::kColdK, kColSFK = C::kColSFK, kColSFV = C::kColSFV, kColSFQ = C::kColSFQ,
                      kColSFdO = C::kColSFdO, kColSFP = C::kColSFP, kColSFdS = C::kColSFdS, kColSFdOc = C::kColSFdOc,
@@ -243,8 +255,11 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
     }
     for (int s = 0; s < C::kLseSlots; ++s) mbar_init(&sm.lse_ready[s], 1);   // one arrival by the prep warp
     for (int s = 0; s < kColStages; ++s) { mbar_init(&sm.col_full[s], 1); mbar_init(&sm.col_empty[s], 1); }
-    for (int t = 0; t < kTeams; ++t) { mbar_init(&sm.sdp_full[t], kHasDk ? 2 : 1); mbar_init(&sm.sdp_free[t], kTeamThreads); }
-    for (int i = 0; i < 2; ++i) { mbar_init(&sm.pds_full[i], kTeamThreads); mbar_init(&sm.pds_free[i], 1); mbar_init(&sm.p_free[i], 1); }
+    for (int t = 0; t < kTeams; ++t) { 
+      mbar_init(&sm.s_full[t], !kHasDk ? 1 : (kApart ? 2 : 3)); mbar_init(&sm.s_free[t], kTeamThreads);
+      mbar_init(&sm.dp_full[t], 1); mbar_init(&sm.dp_free[t], kTeamThreads);
+    }
+    for (int i = 0; i < 2; ++i) { mbar_init(&sm.op_full[i], kTeamThreads); mbar_init(&sm.op_free[i], 1); mbar_init(&sm.p_free[i], 1); }
     mbar_init(&sm.p_full, kTeamThreads);
     for (int i = 0; i < 3; ++i) mbar_init(&sm.drain[i], 1);
     mbar_init(&sm.done, 1);
@@ -344,15 +359,14 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ S^T issuer
-    // One tcgen05.mma can be issued per ~130 cycles from one warp whatever its size, so the
-    // products are spread over three issuing warps; orderings that a single issuer would give
-    // for free are carried by mbarriers instead.
-    {
+    // The products are spread over three issuing warps, so that none waits behind another's barriers;
+    // orderings that a single issuer would give for free are carried by mbarriers instead.
+    if (elect_one()) {
       const uint64_t desc_k = make_desc_sw128(smem_u32(sm.k[0]));
       bool ok = mbar_wait(&sm.kv_full, 0, abort_flag);
       if (ok && kFp8) {
         tc_fence_after_sync();
-        sf_copy_tiles<kCq>(tmem + kColSFK, sm.sf_k);
+        sf_copy_tiles<kCq, true>(tmem + kColSFK, sm.sf_k);
       }
       // the row ring is walked with a running (stage, phase) pair: a division by a ring depth of 3 in every
       // iteration is felt in the issue rate
@@ -366,35 +380,35 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
           ok = mbar_wait(&sm.row_full[s], s_phase, abort_flag);
           if (!ok) break;
           tc_fence_after_sync();
-          if (kFp8 && kSl == 2) sf_copy_tiles<kCq>(tmem + kColSFQ + 4 * kCq * slot, st.sf_q);
+          if (kFp8 && kSl == 2) sf_copy_tiles<kCq, true>(tmem + kColSFQ + 4 * kCq * slot, st.sf_q);
         }
-        if (u > 0) {
-          // the team of the previous sub-tile has pulled S and dP into registers
-          ok = mbar_wait(&sm.sdp_free[(u - 1) % kTeams], ((u - 1) / kTeams) & 1, abort_flag);
+        if (u >= kSBufs) {
+          // the team that had this buffer last has pulled S into registers
+          const int v = u - kSBufs;
+          ok = mbar_wait(&sm.s_free[v % kTeams], (v / kTeams) & 1, abort_flag);
           if (!ok) break;
           tc_fence_after_sync();
         }
-        // a single scale slot is rewritten only now that the product that read it has been consumed
-        if (kFp8 && kSl == 1 && sub_r == 0) sf_copy_tiles<kCq>(tmem + kColSFQ, st.sf_q);
+        if (kFp8 && kSl == 1 && sub_r == 0) sf_copy_tiles<kCq, true>(tmem + kColSFQ, st.sf_q);
         const uint64_t desc_q = make_desc_sw128(smem_u32(st.q[0])) + sub_r * (kSub * 128 / 16);
-        issue_ss<kFp8, kCq, kSub, kTile * 128 / 16, kRowTok * 128 / 16>(
-            tmem + kColS, desc_k, desc_q, nk_qk, tmem + kColSFK, tmem + kColSFQ + 4 * kCq * slot + 2 * half);
-        mma_commit_elect(&sm.sdp_full[u % kTeams]);
-        if (C::kEarly) mma_commit_elect(&sm.row_empty[s]);   // the row operands of this sub-tile have been read
+        issue_ss<kFp8, kCq, kSub, kTile * 128 / 16, kRowTok * 128 / 16, true>(
+            tmem + kColS + 64 * (u % kSBufs), desc_k, desc_q, nk_qk, tmem + kColSFK, tmem + kColSFQ + 4 * kCq * slot + 2 * half);
+        mma_commit(&sm.s_full[u % kTeams]);
+        if (C::kEarly) mma_commit(&sm.row_empty[s]);   // the row operands of this sub-tile have been read
       }
       if (!ok) {
         int dummy = 0;
-        mma_commit_elect(&sm.drain[0]);
+        mma_commit(&sm.drain[0]);
         mbar_wait(&sm.drain[0], 0, &dummy);
       }
     }
   } else if (warp == 2) {
     // ------------------------------------------------------------------ dP^T issuer + LSE preparation
     const uint64_t desc_v = make_desc_sw128(smem_u32(sm.v[0]));
-    bool ok = mbar_wait(&sm.kv_full, 0, abort_flag);
+    bool ok = __all_sync(0xffffffffu, mbar_wait(&sm.kv_full, 0, abort_flag));   // (one answer for the warp: elect_one needs it whole)
     if (ok && kFp8v && kHasDk) {
       tc_fence_after_sync();
-      sf_copy_tiles<kCv>(tmem + kColSFV, sm.sf_v);
+      if (elect_one()) sf_copy_tiles<kCv, true>(tmem + kColSFV, sm.sf_v);
     }
     int s = 0;                                        // running (stage, phase) of the row ring
     uint32_t s_phase = 0;
@@ -416,7 +430,7 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
       if (u > 0 && sub_r == 0 && ++s == kRowStages) { s = 0; s_phase ^= 1u; }
       KvRowStage<C>& st = sm.rst[s];
       if (sub_r == 0) {
-        ok = mbar_wait(&sm.row_full[s], s_phase, abort_flag);
+        ok = __all_sync(0xffffffffu, mbar_wait(&sm.row_full[s], s_phase, abort_flag));
         if (!ok) break;
         if (kPrepLoads) {
           if (4 * lane < kRowTok) {
@@ -437,107 +451,101 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
           }
         }
         if (C::kEarly && !kPrepLoads && !kHasDk) mbar_arrive_warp(&sm.row_empty[s]);   // LSE has been read out of the stage
-        mbar_arrive_warp(&sm.lse_ready[C::kEarly ? ls : s]);
+        if (!kHasDk) mbar_arrive_warp(&sm.lse_ready[C::kEarly ? ls : s]);
         if (++ls == C::kLseSlots) ls = 0;
         if (kFp8v && kHasDk && kSl == 2) {
           tc_fence_after_sync();
-          sf_copy_tiles<kCv>(tmem + kColSFdO + 4 * kCv * slot, st.sf_dO);
+          if (elect_one()) sf_copy_tiles<kCv, true>(tmem + kColSFdO + 4 * kCv * slot, st.sf_dO);
         }
       }
       if (kHasDk) {
+        // -LSE log2(e) and -D of this sub-tile are in place.  (The phase before has completed: its team released the
+        // score tile of sub-tile u - 2 before this warp went on to u - 1.)
+        mbar_arrive_warp(&sm.s_full[u % kTeams]);
         if (u > 0) {
-          ok = mbar_wait(&sm.sdp_free[(u - 1) % kTeams], ((u - 1) / kTeams) & 1, abort_flag);
+          // the team of the previous sub-tile has pulled dP into registers
+          ok = __all_sync(0xffffffffu, mbar_wait(kApart ? &sm.dp_free[(u - 1) % kTeams] : &sm.s_free[(u - 1) % kTeams], ((u - 1) / kTeams) & 1, abort_flag));
           if (!ok) break;
         }
         tc_fence_after_sync();
-        if (kFp8v && kSl == 1 && sub_r == 0) sf_copy_tiles<kCv>(tmem + kColSFdO, st.sf_dO);
-        const uint64_t desc_dO = make_desc_sw128(smem_u32(st.dO[0])) + sub_r * (kSub * 128 / 16);
-        issue_ss<kFp8v, kCv, kSub, kTile * 128 / 16, kRowTok * 128 / 16>(
-            tmem + kColdP, desc_v, desc_dO, nk_v, tmem + kColSFV, tmem + kColSFdO + 4 * kCv * slot + 2 * half);
-        mma_commit_elect(&sm.sdp_full[u % kTeams]);
-        if (C::kEarly) mma_commit_elect(&sm.row_empty[s]);
+        if (elect_one()) {
+          if (kFp8v && kSl == 1 && sub_r == 0) sf_copy_tiles<kCv, true>(tmem + kColSFdO, st.sf_dO);
+          const uint64_t desc_dO = make_desc_sw128(smem_u32(st.dO[0])) + sub_r * (kSub * 128 / 16);
+          issue_ss<kFp8v, kCv, kSub, kTile * 128 / 16, kRowTok * 128 / 16, true>(
+              tmem + kColdP, desc_v, desc_dO, nk_v, tmem + kColSFV, tmem + kColSFdO + 4 * kCv * slot + 2 * half);
+          mma_commit(kApart ? &sm.dp_full[u % kTeams] : &sm.s_full[u % kTeams]);
+          if (C::kEarly) mma_commit(&sm.row_empty[s]);
+        }
       }
     }
     if (!ok && kHasDk) {
       int dummy = 0;
-      mma_commit_elect(&sm.drain[1]);
+      if (elect_one()) mma_commit(&sm.drain[1]);
       mbar_wait(&sm.drain[1], 0, &dummy);
     }
   } else if (warp == 3) {
     // ------------------------------------------------------------------ dV / dK issuer
-    {
+    if (elect_one()) {
       bool ok = true;
       int rs_done = 0;                                // row stage whose queries go through the softmax next
       for (int u = 0; u < n_sub && ok; ++u) {
         const int buf = kOpBufs == 2 ? (u & 1) : 0, ci = u / kSubPerCol, s = ci % kColStages, slot = kSl == 2 ? (ci & 1) : 0, sub_c = u % kSubPerCol;
         KvColStage<C>& st = sm.cst[s];
+        const uint64_t desc_dOc = make_desc_sw128(smem_u32(st.dOc)), desc_qc = make_desc_sw128(smem_u32(st.qc));
         if (sub_c == 0) {
           ok = mbar_wait(&sm.col_full[s], (ci / kColStages) & 1, abort_flag);
           if (!ok) break;
           tc_fence_after_sync();
           if (kFp8 && !kTight) {
-            if (kHasDv) sf_copy_tiles<kRv>(tmem + kColSFdOc + 4 * kRv * slot, st.sf_dOc);
-            if (kHasDk) sf_copy_tiles<kRq>(tmem + kColSFQc + 4 * kRq * slot, st.sf_qc);
+            if (kHasDv) sf_copy_tiles<kRv, true>(tmem + kColSFdOc + 4 * kRv * slot, st.sf_dOc);
+            if (kHasDk) sf_copy_tiles<kRq, true>(tmem + kColSFQc + 4 * kRq * slot, st.sf_qc);
           }
         }
-        // (single operand buffer: P^ comes first, dS^ is waited for ahead of the dK product)
-        ok = kSplit ? mbar_wait(&sm.p_full, u & 1, abort_flag) : mbar_wait(&sm.pds_full[buf], (kOpBufs == 2 ? u >> 1 : u) & 1, abort_flag);
-        if (!ok) break;
-        // all queries of a row stage have been through the softmax: the stage (score operands,
-        // LSE, D) is no longer read
-        if (!C::kEarly && u % kSubPerRow == kSubPerRow - 1) {
-          if (lane == 0) mbar_arrive(&sm.row_empty[rs_done]);
-          if (++rs_done == kRowStages) rs_done = 0;
-        }
-        tc_fence_after_sync();
-        if (kFp8 && !kTight) {
-          if (kHasDv) sf_copy_elect(tmem + kColSFP + 4 * buf, make_desc_sf(smem_u32(sm.sf_p[buf])));
-          if (kHasDk) sf_copy_elect(tmem + kColSFdS + 4 * buf, make_desc_sf(smem_u32(sm.sf_ds[buf])));
-        }
-        if (kTight && kFp8) {
-          // One operand buffer, one pair of scale slots: the scales of P^ and dO^c, the dV product, then the
-          // scales of dS^ and of each row tile of Q^c in the same columns and the dK product of that tile.
-          // Copies and MMAs of one thread run in the order issued.
-          const uint64_t desc_qc = make_desc_sw128(smem_u32(st.qc));
-          sf_copy_elect(tmem + kColSFP, make_desc_sf(smem_u32(sm.sf_p[0])));
-          sf_copy_elect(tmem + kColSFdOc, make_desc_sf(smem_u32(st.sf_dOc)));
-          issue_ts<true, 1, 1>(tmem + kColdV, tmem + kColP, make_desc_sw128(smem_u32(st.dOc)), p.dv, sub_c, tmem + kColSFP,
-                               tmem + kColSFdOc, u > 0);
-          mma_commit_elect(&sm.p_free[(u + 1) & 1]);      // P^ and its scale bytes may be rewritten (by the other team)
-          ok = mbar_wait(&sm.pds_full[0], u & 1, abort_flag);
-          if (!ok) break;
-          tc_fence_after_sync();
-          sf_copy_elect(tmem + kColSFdS, make_desc_sf(smem_u32(sm.sf_ds[0])));
-#pragma unroll
-          for (int r = 0; r < 2; ++r) {
-            sf_copy_elect(tmem + kColSFQc, make_desc_sf(smem_u32(st.sf_qc + 512 * r)));
-            issue_ts<true, 1, 1>(tmem + kColdK + 128 * r, tmem + kColdS, desc_qc + r * (128 * 128 / 16), r == 0 ? 128 : dk_cols - 128,
-                                 sub_c, tmem + kColSFdS, tmem + kColSFQc, u > 0);
-          }
-        } else {
         // 64 queries = 2 (codes) or 4 (BF16) steps of 32 bytes; the B operands are taken 128 rows at a time
-        if (kHasDv)
-          issue_ts<kFp8, kEB, kRv>(tmem + kColdV, tmem + kColP + kOpCols * buf, make_desc_sw128(smem_u32(st.dOc)), p.dv,
-                                   sub_c, tmem + kColSFP + 4 * buf, tmem + kColSFdOc + 4 * kRv * slot, u > 0);
-        if (kSplit) {
-          mma_commit_elect(&sm.p_free[(u + 1) & 1]);
-          ok = mbar_wait(&sm.pds_full[0], u & 1, abort_flag);
+        if (kHasDv) {
+          ok = kSplit ? mbar_wait(&sm.p_full, u & 1, abort_flag) : mbar_wait(&sm.op_full[buf], (u >> 1) & 1, abort_flag);
           if (!ok) break;
           tc_fence_after_sync();
+          if (kFp8) sf_copy(tmem + kColSFP + 4 * buf, make_desc_sf(smem_u32(sm.sf_p[buf])));
+          if (kTight && kFp8) sf_copy(tmem + kColSFdOc, make_desc_sf(smem_u32(st.sf_dOc)));
+          issue_ts<kFp8, kEB, kRv, true>(tmem + kColdV, tmem + kColP + kOpCols * buf, desc_dOc, p.dv, sub_c, tmem + kColSFP + 4 * buf,
+                                         tmem + kColSFdOc + 4 * kRv * slot, u > 0);
+          if (kSplit) mma_commit(&sm.p_free[(u + 1) & 1]);      // P^ and its scale bytes may be rewritten (by the other team)
         }
-        if (kHasDk)
-          issue_ts<kFp8, kEB, kRq>(tmem + kColdK, tmem + kColdS + kOpCols * buf, make_desc_sw128(smem_u32(st.qc)), dk_cols,
-                                   sub_c, tmem + kColSFdS + 4 * buf, tmem + kColSFQc + 4 * kRq * slot, u > 0);
+        if (kHasDk) {
+          if (kSplit || !kHasDv) {
+            ok = mbar_wait(&sm.op_full[buf], (kOpBufs == 2 ? u >> 1 : u) & 1, abort_flag);
+            if (!ok) break;
+            tc_fence_after_sync();
+          }
+          if (kFp8) sf_copy(tmem + kColSFdS + 4 * buf, make_desc_sf(smem_u32(sm.sf_ds[buf])));
+          if (kTight && kFp8) {
+            // one pair of scale columns for both gradient products and both row tiles of Q^c, used one after the other
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+              sf_copy(tmem + kColSFQc, make_desc_sf(smem_u32(st.sf_qc + 512 * r)));
+              issue_ts<true, 1, 1, true>(tmem + kColdK + 128 * r, tmem + kColdS, desc_qc + r * (128 * 128 / 16),
+                                         r == 0 ? 128 : dk_cols - 128, sub_c, tmem + kColSFdS, tmem + kColSFQc, u > 0);
+            }
+          } else {
+            issue_ts<kFp8, kEB, kRq, true>(tmem + kColdK, tmem + kColdS + kOpCols * buf, desc_qc, dk_cols, sub_c,
+                                           tmem + kColSFdS + 4 * buf, tmem + kColSFQc + 4 * kRq * slot, u > 0);
+          }
+        }
+        // all queries of a row stage have been through the softmax: the stage (score operands, LSE, D) is no longer read
+        if (!C::kEarly && u % kSubPerRow == kSubPerRow - 1) {
+          mbar_arrive(&sm.row_empty[rs_done]);
+          if (++rs_done == kRowStages) rs_done = 0;
         }
         // operands and scale bytes of this buffer may be overwritten once these MMAs have run; the
         // col stage may be refilled after its last sub-tile
-        mma_commit_elect(&sm.pds_free[kOpBufs == 2 ? buf : ((u + 1) & 1)]);   // indexed by the team that writes next
-        if (sub_c == kSubPerCol - 1) mma_commit_elect(&sm.col_empty[s]);
-        if (u == n_sub - 1) mma_commit_elect(&sm.done);
+        mma_commit(&sm.op_free[kOpBufs == 2 ? buf : ((u + 1) & 1)]);   // indexed by the team that writes next
+        if (sub_c == kSubPerCol - 1) mma_commit(&sm.col_empty[s]);
+        if (u == n_sub - 1) mma_commit(&sm.done);
       }
       if (!ok) {
         int dummy = 0;
-        mma_commit_elect(&sm.drain[2]);
+        mma_commit(&sm.drain[2]);
         mbar_wait(&sm.drain[2], 0, &dummy);
       }
     }
@@ -565,33 +573,44 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
           if (++s == kRowStages) { s = 0; s_phase ^= 1u; }
         if ((ls += kTeams) >= C::kLseSlots) { ls -= C::kLseSlots; ls_phase ^= 1u; }
       }
-      ok = mbar_wait(&sm.sdp_full[team], (u / kTeams) & 1, abort_flag);
+      ok = mbar_wait(&sm.s_full[team], (u / kTeams) & 1, abort_flag);
       if (!ok) break;
       tc_fence_after_sync();
       uint32_t sr[32], dpr[32];                       // S then P; dP then dS (in place)
-      tmem_ld32(tmem + kColS + lane_addr + 32 * grp, sr);
-      if (kHasDk) tmem_ld32(tmem + kColdP + lane_addr + 32 * grp, dpr);
+      tmem_ld32(tmem + kColS + 64 * (u % kSBufs) + lane_addr + 32 * grp, sr);
+      if (kHasDk && !kApart) tmem_ld32(tmem + kColdP + lane_addr + 32 * grp, dpr);
       tmem_wait_ld();
       tc_fence_before_sync();
-      mbar_arrive(&sm.sdp_free[team]);
-      ok = C::kEarly ? mbar_wait(&sm.lse_ready[ls], ls_phase, abort_flag) : mbar_wait(&sm.lse_ready[s], s_phase, abort_flag);
-      if (!ok) break;
+      mbar_arrive(&sm.s_free[team]);
+      if (!kHasDk) {                                  // (otherwise s_full stands for LSE and D as well)
+        ok = C::kEarly ? mbar_wait(&sm.lse_ready[ls], ls_phase, abort_flag) : mbar_wait(&sm.lse_ready[s], s_phase, abort_flag);
+        if (!ok) break;
+      }
       const int col0 = half * kSub + 32 * grp;        // query row (inside the tile) of this thread's first column
       const int st0 = (u % kSubPerRow) * kSub + 32 * grp;   // the same inside the row stage
       const KvRowStage<C>& st = sm.rst[s];
-      float amax_p = 0.f, max_s = 0.f;
       const float* s_lse = C::kEarly ? &sm.lse_ring[ls][32 * grp] : &st.neg_lse2[st0];
       const float* s_delta = C::kEarly ? &sm.delta_ring[ls][32 * grp] : &st.delta[st0];
-      // two elements per instruction (fma / mul .f32x2) wherever the arithmetic allows: the loop is
-      // bound by instruction issue, not by a pipe
+      uint32_t words[8 * kEB];
+      // P = 2^(S scale log2e - LSE log2e), two elements per instruction (fma / mul .f32x2) wherever the arithmetic
+      // allows: the loop is bound by instruction issue, not by a pipe
+      float amax_p = 0.f, max_s = 0.f;
       const float2 sc2 = make_float2(p.scale_log2, p.scale_log2);
+      // dS = P (dP - D) of a pair of queries (dv2 holds -D)
+      auto gradient = [&](int c, const float2 p2, const float2 dv2) {
+        const float2 t2 = __fadd2_rn(make_float2(__uint_as_float(dpr[c]), __uint_as_float(dpr[c + 1])), dv2);
+        const float2 ds2 = __fmul2_rn(p2, t2);
+        dpr[c] = __float_as_uint(ds2.x);
+        dpr[c + 1] = __float_as_uint(ds2.y);
+        max_s = fmaxf(max_s, fmaxf(fabsf(ds2.x), fabsf(ds2.y)));
+      };
       auto body = [&](auto diag_tag) {
         constexpr bool kDiag = decltype(diag_tag)::value;
 #pragma unroll
         for (int c4 = 0; c4 < 32; c4 += 4) {
           const float4 l4 = lds_f4(&s_lse[c4]);
           float4 d4 = make_float4(0.f, 0.f, 0.f, 0.f);
-          if (kHasDk) d4 = lds_f4(&s_delta[c4]);
+          if (kHasDk && !kApart) d4 = lds_f4(&s_delta[c4]);
 #pragma unroll
           for (int e = 0; e < 4; e += 2) {
             const int c = c4 + e;
@@ -604,15 +623,8 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
             const float2 p2 = make_float2(ex2_approx(x2.x), ex2_approx(x2.y));
             sr[c] = __float_as_uint(p2.x);
             sr[c + 1] = __float_as_uint(p2.y);
-            amax_p = fmaxf(amax_p, fmaxf(p2.x, p2.y));
-            if (kHasDk) {
-              const float2 dv2 = e == 0 ? make_float2(d4.x, d4.y) : make_float2(d4.z, d4.w);
-              const float2 t2 = __fadd2_rn(make_float2(__uint_as_float(dpr[c]), __uint_as_float(dpr[c + 1])), dv2);   // dP - D (dv2 holds -D)
-              const float2 ds2 = __fmul2_rn(p2, t2);          // dS = P (dP - D)
-              dpr[c] = __float_as_uint(ds2.x);
-              dpr[c + 1] = __float_as_uint(ds2.y);
-              max_s = fmaxf(max_s, fmaxf(fabsf(ds2.x), fabsf(ds2.y)));
-            }
+            if (kFp8) amax_p = fmaxf(amax_p, fmaxf(p2.x, p2.y));
+            if (kHasDk && !kApart) gradient(c, p2, e == 0 ? make_float2(d4.x, d4.y) : make_float2(d4.z, d4.w));
           }
         }
       };
@@ -624,23 +636,24 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
         amax_p = 0.f;
         max_s = 0.f;
       }
-      uint32_t byte_p = 0, byte_s = 0;
-      float inv_p = 1.f, inv_s = 1.f;
-      if (kFp8) {
-        if (kHasDv) block_scale_finite(amax_p, byte_p, inv_p);
-        if (kHasDk) block_scale_finite(max_s, byte_s, inv_s);
+      if (kApart) {
+        ok = mbar_wait(&sm.dp_full[team], (u / kTeams) & 1, abort_flag);
+        if (!ok) break;
+        tc_fence_after_sync();
+        tmem_ld32(tmem + kColdP + lane_addr + 32 * grp, dpr);     // in flight while P is cast
       }
-      if (u >= kOpBufs) {
-        // the dV / dK MMAs of the sub-tile that last used this buffer have consumed its operands and scale bytes
-        // (single buffer: the dV MMAs have consumed P^; dS^ is waited for below)
-        ok = mbar_wait(kSplit ? &sm.p_free[team] : &sm.pds_free[team], ((u - kOpBufs) >> 1) & 1, abort_flag);
+      if (u >= kOpBufs && !kSplit) {
+        // the MMAs of the sub-tile that last used this buffer have consumed its operands and scale bytes
+        ok = mbar_wait(&sm.op_free[team], ((u - kOpBufs) >> 1) & 1, abort_flag);
         if (!ok) break;
         tc_fence_after_sync();
       }
-      uint32_t words[8 * kEB];
       if (kHasDv) {
+        uint32_t byte = 0;
         if (kFp8) {
-          const float2 inv2 = make_float2(inv_p, inv_p);
+          float inv;
+          block_scale_finite(amax_p, byte, inv);
+          const float2 inv2 = make_float2(inv, inv);
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
             const float2 a = __fmul2_rn(make_float2(__uint_as_float(sr[4 * i]), __uint_as_float(sr[4 * i + 1])), inv2);
@@ -652,25 +665,42 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
           for (int i = 0; i < 8 * kEB; ++i)
             words[i] = cvt_bf16x2(__uint_as_float(sr[(2 * i) & 31]), __uint_as_float(sr[(2 * i + 1) & 31]));
         }
-#pragma unroll
-        for (int i = 0; i < kEB; ++i) tmem_st8(tmem + kColP + kOpCols * buf + lane_addr + 8 * kEB * grp + 8 * i, words + 8 * i);
-      }
-      if (kSplit) {
-        // hand P^ over, then wait for the dK MMAs of the sub-tile before to have consumed dS^
-        if (kFp8) sts_u8(&sm.sf_p[0][(row & 31) * 16 + (row >> 5) * 4 + grp], byte_p);
-        tmem_wait_st();
-        fence_proxy_async_smem();
-        tc_fence_before_sync();
-        mbar_arrive(&sm.p_full);
-        if (u >= 1) {
-          ok = mbar_wait(&sm.pds_free[team], ((u - 1) >> 1) & 1, abort_flag);
+        if (kSplit && u >= 1) {
+          // the dV MMAs of the sub-tile before have consumed P^ and its scale bytes
+          ok = mbar_wait(&sm.p_free[team], ((u - 1) >> 1) & 1, abort_flag);
           if (!ok) break;
           tc_fence_after_sync();
         }
+#pragma unroll
+        for (int i = 0; i < kEB; ++i) tmem_st8(tmem + kColP + kOpCols * buf + lane_addr + 8 * kEB * grp + 8 * i, words + 8 * i);
+        if (kFp8) sts_u8(&sm.sf_p[buf][(row & 31) * 16 + (row >> 5) * 4 + grp], byte);
+        if (kSplit) {
+          tmem_wait_st();
+          fence_proxy_async_smem();
+          tc_fence_before_sync();
+          mbar_arrive(&sm.p_full);
+        }
+      }
+      if (kApart) {
+        tmem_wait_ld();
+        tc_fence_before_sync();
+        mbar_arrive(&sm.dp_free[team]);
+#pragma unroll
+        for (int c4 = 0; c4 < 32; c4 += 4) {
+          const float4 d4 = lds_f4(&s_delta[c4]);
+#pragma unroll
+          for (int e = 0; e < 4; e += 2) {
+            const int c = c4 + e;
+            gradient(c, make_float2(__uint_as_float(sr[c]), __uint_as_float(sr[c + 1])), e == 0 ? make_float2(d4.x, d4.y) : make_float2(d4.z, d4.w));
+          }
+        }
       }
       if (kHasDk) {
+        uint32_t byte = 0;
         if (kFp8) {
-          const float2 inv2 = make_float2(inv_s, inv_s);
+          float inv;
+          block_scale_finite(max_s, byte, inv);
+          const float2 inv2 = make_float2(inv, inv);
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
             const float2 a = __fmul2_rn(make_float2(__uint_as_float(dpr[4 * i]), __uint_as_float(dpr[4 * i + 1])), inv2);
@@ -682,18 +712,20 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
           for (int i = 0; i < 8 * kEB; ++i)
             words[i] = cvt_bf16x2(__uint_as_float(dpr[(2 * i) & 31]), __uint_as_float(dpr[(2 * i + 1) & 31]));
         }
+        if (kSplit && u >= 1) {
+          // the dK MMAs of the sub-tile before have consumed dS^ and its scale bytes
+          ok = mbar_wait(&sm.op_free[team], ((u - 1) >> 1) & 1, abort_flag);
+          if (!ok) break;
+          tc_fence_after_sync();
+        }
 #pragma unroll
         for (int i = 0; i < kEB; ++i) tmem_st8(tmem + kColdS + kOpCols * buf + lane_addr + 8 * kEB * grp + 8 * i, words + 8 * i);
-      }
-      if (kFp8) {
-        const int sf_at = (row & 31) * 16 + (row >> 5) * 4 + grp;
-        if (kHasDv && !kSplit) sts_u8(&sm.sf_p[buf][sf_at], byte_p);
-        if (kHasDk) sts_u8(&sm.sf_ds[buf][sf_at], byte_s);
+        if (kFp8) sts_u8(&sm.sf_ds[buf][(row & 31) * 16 + (row >> 5) * 4 + grp], byte);
       }
       tmem_wait_st();
       fence_proxy_async_smem();
       tc_fence_before_sync();
-      mbar_arrive(&sm.pds_full[buf]);
+      mbar_arrive(&sm.op_full[buf]);
       it = (it + 1 == tiles_n) ? it0 : it + 1;        // next tile of this head, or the first tile of the next head
     }
     // the epilogue is done by team 0 (group 0 stores dV, group 1 stores dK)
