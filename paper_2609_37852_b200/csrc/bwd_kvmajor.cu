@@ -231,10 +231,10 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
     return;
   }
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  // blocks are handed out x-fastest: KV heads vary fastest, key tiles in order, so the heaviest
-  // tiles (the earliest keys under the causal mask) of all heads go first
-  const int jt = blockIdx.y;
-  const int g = blockIdx.x, b = blockIdx.z;
+  // blocks are handed out x-fastest, z-slowest: key tiles in order, so the heaviest tiles (the earliest keys under
+  // the causal mask) of all heads and sequences go first
+  const int jt = blockIdx.z;
+  const int g = blockIdx.x, b = blockIdx.y;
   const int G = p.Hq / p.Hkv;
   const int tiles_n = p.N / kTile, tiles_nk = p.Nk / kTile;
   const int it0 = p.causal ? max(jt - p.q0t, 0) : 0;   // first query tile that sees these keys
@@ -800,7 +800,7 @@ attn_status_t launch_kvmajor_t(const AttnShape& s, attn_qtensor_t q, attn_qtenso
   p.tickets = clear_tickets ? ticket_counter(status) : nullptr;
   const size_t smem = sizeof(KvSmem<C>) + 1024;
   if ((st = allow_smem<kvmajor_kernel<C>>(smem, "bwd kv-major")) != ATTN_OK) return st;
-  dim3 grid(s.Hkv, s.Nk / kTile, s.B);
+  dim3 grid(s.Hkv, s.B, s.Nk / kTile);
   // The first pass is launched behind whatever is ahead in the stream in the ordinary way: with programmatic
   // serialisation there as well, the kernels behind this one no longer started beside it (dK, dV and dQ at head
   // dim 256, 8/2 heads, one after the other: step 1065 -> 1257 us).

@@ -187,8 +187,8 @@ qmajor_kernel(const QmParams p, const __grid_constant__ CUtensorMap tm_q, const 
     return;
   }
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  // Work items are numbered x-fastest over the grid (gx, gy, gz): heads vary fastest and the heaviest
-  // (latest) query tiles of all heads come first, so the light tiles fill the tail.  Without
+  // Work items are numbered over (head, batch, query tile), the tile slowest: the heaviest (latest) query tiles
+  // of all heads and sequences come first, so the light tiles fill the tail.  Without
   // persistence a CTA is its own item.  With a static list a persistent CTA takes the items c,
   // 2n-1-c, 2n+c, ... (n CTAs, c its index): alternate rounds run backwards, so that no CTA collects
   // the heavier item of every round.  In ticket mode the producer thread draws item numbers from a
@@ -217,11 +217,11 @@ qmajor_kernel(const QmParams p, const __grid_constant__ CUtensorMap tm_q, const 
     it.valid = true;
     return it;
   };
-  auto decode_linear = [&](int l) { return decode(l % p.gx, (l / p.gx) % p.gy, l / (p.gx * p.gy)); };
+  auto decode_linear = [&](int l) { return decode(l % p.gx, l / (p.gx * p.gz), (l / p.gx) % p.gz); };
   // the i-th item of this CTA (valid = false: no more; in ticket mode also when the wait gave up)
   auto item_at = [&](int i) {
     Item none; none.valid = false; none.qt = none.h = none.r_tile = none.b = none.g = none.n_tiles = 0;
-    if (!kPersist) return i == 0 ? decode(blockIdx.x, blockIdx.y, blockIdx.z) : none;
+    if (!kPersist) return i == 0 ? decode(blockIdx.x, blockIdx.z, blockIdx.y) : none;
     if (!kTicket) {
       if (i >= n_static) return none;
       const int pos = (i & 1) ? n_cta - 1 - static_cast<int>(blockIdx.x) : static_cast<int>(blockIdx.x);
@@ -798,8 +798,8 @@ attn_status_t launch_qmajor_t(const AttnShape& s, attn_qtensor_t q, attn_qtensor
   const size_t smem = sizeof(QmSmem<C>) + 1024;
   if ((st = allow_smem<qmajor_kernel<C>>(smem, "bwd q-major")) != ATTN_OK) return st;
   const int rq = (kDQ && !C::kWhole) ? (s.dqk + 127) / 128 : 1;
-  dim3 grid(s.Hq * rq, s.N / kTile, s.B);
-  p.gx = static_cast<int>(grid.x); p.gy = static_cast<int>(grid.y); p.gz = static_cast<int>(grid.z);
+  dim3 grid(s.Hq * rq, s.B, s.N / kTile);
+  p.gx = static_cast<int>(grid.x); p.gy = static_cast<int>(grid.z); p.gz = static_cast<int>(grid.y);
   if (C::kPersist) {
     // one CTA per SM (the kernel takes a whole SM's shared memory) walks the item list
     int dev = 0, sms = 0;

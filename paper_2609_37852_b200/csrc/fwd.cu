@@ -128,11 +128,9 @@ fwd_kernel(const FwdParams p, const __grid_constant__ CUtensorMap tm_q, const __
   constexpr uint32_t kColS = C::kColS, kColP = C::kColP, kColO = C::kColO, kColSFQ = C::kColSFQ, kColSFK = C::kColSFK,
                      kColSFV = C::kColSFV, kColSFP = C::kColSFP, kTmemCols = C::kTmemCols, kPCols = C::kPCols;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  // heavy (late) query tiles first
-  // blocks are handed out x-fastest: heads vary fastest and the heaviest (latest) query tiles of
-  // all heads go first, so the light tiles fill the tail of the launch
-  const int qt = p.causal ? (gridDim.y - 1 - blockIdx.y) : blockIdx.y;
-  const int h = blockIdx.x, b = blockIdx.z;
+  // blocks are handed out x-fastest, z-slowest: the heaviest (latest) query tiles of all heads and sequences go first, so the light tiles fill the tail of the launch
+  const int qt = p.causal ? (gridDim.z - 1 - blockIdx.z) : blockIdx.z;
+  const int h = blockIdx.x, b = blockIdx.y;
   const int g = h / (p.Hq / p.Hkv);
   const int n_tiles = p.causal ? qt + p.q0t + 1 : p.Nk / kTile;
   const int n_sub = 2 * n_tiles;
@@ -475,7 +473,7 @@ attn_status_t launch_fwd_t(const AttnShape& s, attn_qtensor_t q, attn_qtensor_t 
   p.scale_log2 = s.scale * kLog2e;
   const size_t smem = sizeof(FwdSmem<C>) + 1024;
   if ((st = allow_smem<fwd_kernel<C>>(smem, "fwd")) != ATTN_OK) return st;
-  dim3 grid(s.Hq, s.N / kTile, s.B);
+  dim3 grid(s.Hq, s.B, s.N / kTile);
   const cudaError_t e = launch_overlapped(fwd_kernel<C>, grid, C::kThreads, smem, stream, 1, p, tm_q, tm_k, tm_v);
   if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "fwd: launch: %s", cudaGetErrorString(e));
   return ATTN_OK;
