@@ -421,9 +421,10 @@ fwd_il_kernel(const IlParams p, const __grid_constant__ CUtensorMap tm_q, const 
       float lt = 0.f;
 #pragma unroll
       for (int j = 0; j < kWG * kSplit; ++j) {
-        const int first_u = (j / kSplit + kWG - G % kWG) % kWG;     // the team's first step of this item
+        // in the order of the item's steps, not of the teams: which team takes the first one depends on the items before
+        const int first_u = j / kSplit, at = ((first_u + G) % kWG) * kSplit + j % kSplit;
         if (first_u < it.n_steps)
-          lt += lds_f32(&sm.fin_l[i & 3][j][row]) * pow2_int(lds_f32(&sm.fin_m[i & 3][j][row]) - MO);   // M = -inf goes with l = 0
+          lt += lds_f32(&sm.fin_l[i & 3][at][row]) * pow2_int(lds_f32(&sm.fin_m[i & 3][at][row]) - MO);   // M = -inf goes with l = 0
       }
       const float inv_l = 1.f / lt;
       const size_t grow = static_cast<size_t>(it.b * p.Hq + it.h) * p.N + it.qt * kTile + row;

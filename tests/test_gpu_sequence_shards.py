@@ -150,3 +150,22 @@ def test_sharded_attention_on_a_one_rank_group():
         assert dk.dtype == torch.float32 and dk.shape == ref["dk"][:, :, rows].shape
         assert rel_fro(to_np(dk), to_np(ref["dk"][:, :, rows])) <= 4e-3
         assert rel_fro(to_np(dv), to_np(ref["dv"][:, :, rows])) <= 4e-3
+
+
+@pytest.mark.parametrize("name", ["gqa4k", "mla8k"])
+def test_forward_rows_do_not_depend_on_the_order_of_the_items(name):
+    """O and LSE of a (sequence, head) are the same bits alone and inside a batch: which items a CTA of the persistent
+    forward has behind it (and so which of its teams takes an item's first step) must not show."""
+    from paper_2609_37852_b200 import binding as B
+    kw = dict(batch=7, heads_q=12, heads_kv=12, seqlen=1152)               # 756 items of 1 ... 9 tiles on at most 148 CTAs
+    w = workloads.WORKLOADS[name].scaled(**kw)
+    q, k, v, _ = (x.cuda() for x in workloads.make_inputs(w))
+    run = lambda a, b, c, n, h: B.attn_fp8_fwd(
+        B.AttnParams(n, w.seqlen, h, h, w.head_dim_qk, w.head_dim_v, w.causal, w.softmax_scale),
+        *(B.attn_fp8_quantize(x.contiguous()) for x in (a, b, c)))
+    o, lse, ws = run(q, k, v, 7, 12)
+    for i, h in ((0, 0), (3, 5), (6, 11)):
+        one = lambda x: x[i:i + 1, h:h + 1]
+        o1, lse1, _ = run(one(q), one(k), one(v), 1, 1)
+        assert torch.equal(o1, one(o)) and torch.equal(lse1, one(lse))
+    B.attn_fp8_read_status(ws)
