@@ -197,10 +197,12 @@ struct KvParams {
   int kv_lim;               // without the causal mask: last real key of the last key tile (127: all real)
   int tail_wait;            // launched behind another key-major pass of the same call (see launch_kvmajor_t)
   int* tickets;             // the dQ kernel's ticket counter, to be cleared ahead of it; or null
+  int split;                // CTAs (a cluster) that share the query tiles of one key tile: 1, 2 or 4
   float scale, scale_log2;
 };
 
-template <class C>
+// kShared: a cluster of p.split CTAs shares the query tiles of a key tile (see split_of).
+template <class C, bool kShared>
 __global__ void __launch_bounds__(kThreads, 1)
 kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_dO,
@@ -234,12 +236,19 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
   // blocks are handed out x-fastest, z-slowest: key tiles in order, so the heaviest tiles (the earliest keys under
   // the causal mask) of all heads and sequences go first
   const int jt = blockIdx.z;
-  const int g = blockIdx.x, b = blockIdx.y;
+  // The walk of the list has a general form and, for one CTA per key tile, a simpler one.  They do the same; the softmax
+  // loop sits at its 96 registers, and the compiler keeps it free of spills with the one or the other (FP8 at head dims
+  // up to 128: 20 to 28 bytes with the simpler form, dK / dV of the 8K layer 1 % slower; (192,128): the reverse).
+  constexpr bool kGeneral = kShared || !kTight;
+  const int split = kShared ? p.split : 1, part = !kShared ? 0 : static_cast<int>(blockIdx.x) % split;
+  const int g = static_cast<int>(blockIdx.x) / split, b = blockIdx.y;
   const int G = p.Hq / p.Hkv;
   const int tiles_n = p.N / kTile, tiles_nk = p.Nk / kTile;
   const int it0 = p.causal ? max(jt - p.q0t, 0) : 0;   // first query tile that sees these keys
   const int tiles_per_head = tiles_n - it0;
-  const int n_qtiles = G * tiles_per_head;          // query tiles this CTA walks
+  // the query tiles of all heads of the group in one list; a CTA of a cluster walks every split-th of them
+  const int n_list = G * tiles_per_head;
+  const int n_qtiles = !kGeneral ? n_list : (part < n_list ? (n_list - part + split - 1) / split : 0);
   const int n_sub = 2 * n_qtiles;
   const int nk_qk = p.dqk * kEB / 32, nk_v = p.dv * C::kEBv / 32;   // 32-byte K steps of S^T and dP^T
   // columns of dK (rows of Q^c) this pass accumulates: all of them, or one tile of 128
@@ -283,6 +292,7 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
   // SMs that this grid's last wave leaves idle (nothing it does depends on this grid's output)
   griddep_launch_dependents();
   const uint32_t tmem = sm.tmem_base;
+  bool stores = false;                                // this thread takes part in the epilogue
 
   if (warp == 0) {
     // ------------------------------------------------------------------ producer
@@ -301,7 +311,7 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
       int issued_row = 0, issued_col = 0;
       bool ok = true;
       for (int u = 0; u < n_sub && ok; ++u) {
-        const int n = u >> 1, half = u & 1;
+        const int n = part + split * (u >> 1), half = u & 1;
         const int h = g * G + n / tiles_per_head, it = it0 + n % tiles_per_head;
         const int q_slab = b * p.Hq + h;
         const size_t sf_tile = static_cast<size_t>(q_slab) * tiles_n + it;
@@ -413,7 +423,7 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
     int s = 0;                                        // running (stage, phase) of the row ring
     uint32_t s_phase = 0;
     // kPrepLoads: LSE and D of the next row stage (= sub-tile), in flight while this one is handled
-    int pf_h = g * G, pf_it = it0;                    // (head, query tile) of the stage fetched next
+    int pf_h = g * G + (kShared ? part / tiles_per_head : 0), pf_it = it0 + (kShared ? part % tiles_per_head : 0);                    // (head, query tile) of the stage fetched next
     float4 pf_l = make_float4(0.f, 0.f, 0.f, 0.f), pf_d = make_float4(0.f, 0.f, 0.f, 0.f);
     auto prefetch = [&](int uu) {
       if (4 * lane < kRowTok) {
@@ -421,7 +431,12 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
         pf_l = *reinterpret_cast<const float4*>(p.lse + at);
         if (kHasDk) pf_d = *reinterpret_cast<const float4*>(p.delta + at);
       }
-      if ((uu & 1) && ++pf_it == tiles_n) { pf_it = it0; ++pf_h; }
+      if (uu & 1) {
+        if (kShared) {
+          pf_it += split;
+          while (pf_it >= tiles_n) { pf_it -= tiles_per_head; ++pf_h; }
+        } else if (++pf_it == tiles_n) { pf_it = it0; ++pf_h; }
+      }
     };
     if (kPrepLoads && n_sub > 0) prefetch(0);
     int ls = 0;                                       // kEarly: slot of the LSE / D ring (sub-tile u modulo its depth)
@@ -557,7 +572,7 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
     const int row = quad * 32 + lane;                 // key inside the tile == TMEM lane
     const uint32_t lane_addr = static_cast<uint32_t>(quad * 32) << 16;
     bool ok = true;
-    int it = it0;                                     // query tile of the current sub-tile (kTeams == 2: one tile per iteration)
+    int it = it0 + (kShared ? part % tiles_per_head : 0);             // query tile of the current sub-tile (kTeams == 2: one tile per iteration)
     static_assert(kTeams == 2, "a team advances by one query tile per iteration");
     // running (stage, phase) of the row ring: the team's first sub-tile is in row stage team / kSubPerRow and
     // it advances by kTeams / kSubPerRow stages per iteration
@@ -726,13 +741,19 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
       fence_proxy_async_smem();
       tc_fence_before_sync();
       mbar_arrive(&sm.op_full[buf]);
-      it = (it + 1 == tiles_n) ? it0 : it + 1;        // next tile of this head, or the first tile of the next head
+      if (kGeneral) {                                 // next tile of this CTA, of this head or of one that follows
+        it += split;
+        while (it >= tiles_n) it -= tiles_per_head;
+      } else {
+        it = (it + 1 == tiles_n) ? it0 : it + 1;
+      }
     }
-    // the epilogue is done by team 0 (group 0 stores dV, group 1 stores dK)
+    // The epilogue is done by team 0 (group 0 stores dV, group 1 stores dK).
     if (team != 0) ok = false;
     if (grp == 0 ? !kHasDv : !kHasDk) ok = false;
-    if (ok) ok = mbar_wait(&sm.done, 0, abort_flag);
-    if (ok) {
+    if (ok && (!kGeneral || n_sub > 0)) ok = mbar_wait(&sm.done, 0, abort_flag);
+    if (kShared) stores = ok;
+    else if (ok) {
       tc_fence_after_sync();
       const size_t grow = static_cast<size_t>(b * p.Hkv + g) * p.Nk + jt * kTile + row;
       const uint32_t col = grp == 0 ? kColdV : kColdK;
@@ -756,6 +777,66 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
       }
     }
   }
+  if constexpr (kShared) {
+    const int ep_grp = ((warp - 4) >> 2) & 1, ep_row = (warp & 3) * 32 + lane;
+    const uint32_t ep_col = tmem + (ep_grp == 0 ? kColdV : kColdK) + (static_cast<uint32_t>((warp & 3) * 32) << 16);
+    const int first = ep_grp == 0 ? 0 : dk_col0, count = ep_grp == 0 ? p.dv : dk_cols;   // columns this pass holds
+    const int slice = count / split;                    // columns this CTA stores (a multiple of 16)
+    // A cluster adds its partial sums column slice by column slice: each CTA sends the other CTAs their slices of its
+    // accumulators (FP32, into their operand stages, no longer in use), then adds the slices it got in the order of the
+    // ranks, so that the sum does not depend on timing.
+    float* const inbox = reinterpret_cast<float*>(smem_raw);
+    const int in_stride = ((kHasDv ? p.dv : 0) + (kHasDk ? dk_cols : 0)) / split * kTile;     // floats per sender
+    const int in_grp = (ep_grp == 1 && kHasDv ? p.dv / split : 0) * kTile;
+    __syncwarp();
+    cluster_sync();                                   // every CTA of the cluster has finished its main loop
+    if (stores && n_sub > 0) {
+      tc_fence_after_sync();
+      for (int to = 0; to < split; ++to) {
+        if (to == part) continue;
+        const uint32_t dst = cluster_map(smem_u32(inbox + (part < to ? part : part - 1) * in_stride + in_grp + ep_row), to);
+        for (int c0 = 0; c0 < slice; c0 += 16) {
+          uint32_t r[16];
+          tmem_ld16(ep_col + to * slice + c0, r);
+          tmem_wait_ld();
+#pragma unroll
+          for (int c = 0; c < 16; ++c) st_cluster_u32(dst + (c0 + c) * kTile * 4, r[c]);
+        }
+      }
+    }
+    __syncwarp();
+    cluster_sync();
+    if (stores) {
+      tc_fence_after_sync();
+      const size_t grow = static_cast<size_t>(b * p.Hkv + g) * p.Nk + jt * kTile + ep_row;
+      const float mul = ep_grp == 0 ? 1.f : p.scale;
+      __nv_bfloat16* out_row = (ep_grp == 0 ? p.dv_out : p.dk) + grow * (ep_grp == 0 ? p.dv : p.dqk) + first + part * slice;
+      for (int c0 = 0; c0 < slice; c0 += 16) {
+        uint32_t r[16];
+        if (n_sub > 0) {
+          tmem_ld16(ep_col + part * slice + c0, r);
+          tmem_wait_ld();
+        }
+        float sum[16];
+#pragma unroll
+        for (int c = 0; c < 16; ++c) sum[c] = 0.f;
+        for (int from = 0; from < split && from < n_list; ++from) {
+          const float* in = inbox + (from < part ? from : from - 1) * in_stride + in_grp + ep_row + c0 * kTile;
+#pragma unroll
+          for (int c = 0; c < 16; ++c) sum[c] += from == part ? __uint_as_float(r[c]) : lds_f32(in + c * kTile);
+        }
+        uint32_t packed[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          const __nv_bfloat162 v2 = __floats2bfloat162_rn(sum[2 * c] * mul, sum[2 * c + 1] * mul);
+          packed[c] = *reinterpret_cast<const uint32_t*>(&v2);
+        }
+        uint4* dst = reinterpret_cast<uint4*>(out_row + c0);
+        dst[0] = make_uint4(packed[0], packed[1], packed[2], packed[3]);
+        dst[1] = make_uint4(packed[4], packed[5], packed[6], packed[7]);
+      }
+    }
+  }
   __syncwarp();
   tc_fence_before_sync();
   __syncthreads();
@@ -768,16 +849,40 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
     griddep_wait();
 }
 
+// CTAs per key tile.  One CTA per key tile is the least work; but the first key tile's CTA walks G * N / 128 query tiles,
+// and with few heads it alone takes longer than an SM's share of everything the call does (`passes` key-major passes, and
+// the dQ kernel behind them, about three quarters of a pass, where there is one).  Then a cluster of two or four CTAs
+// shares the list, which costs a set-up and an exchange of the accumulators (about 8 us): taken where it saves more than
+// 12 query tiles (18 us) and a sixteenth of the share.  16 heads on 4 KV heads, 4096 tokens: dK / dV 204 -> 112 us, gradient call 211 -> 190 us (128 CTAs,
+// the longest 128 tiles, 57 on average); 2 x 16 on 4 heads, 1000 tokens without a mask: dK / dV 59 -> 39 us, but the gradient
+// call 64 -> 68 us, since the dQ kernel fills the idle SMs either way.
+int split_of(const AttnShape& s, int sms, int passes, bool dq_follows) {
+  const long long tiles = s.N / kTile, keys = s.Nk / kTile, G = s.Hq / s.Hkv;
+  // (query tile, key tile) pairs of a head: the first key tiles are seen by all query tiles, the last ones by fewer and fewer
+  const long long per_head = s.causal ? tiles * (keys - tiles) + tiles * (tiles + 1) / 2 : tiles * keys;
+  const long long longest = G * tiles, share = per_head * s.Hq * s.B * (4 * passes + (dq_follows ? 3 : 0)) / (4LL * sms);
+  int split = 1;
+  while (split < 4) {
+    const long long next = longest / (2 * split) > share ? longest / (2 * split) : share;
+    if (longest / split - next <= 12 + share / 16) break;
+    split *= 2;
+  }
+  return split;
+}
+
 // `behind`: the launch follows another key-major pass of the same call, which writes another output
 // (dV or dK, or another column tile of dK) from the same inputs.  With few KV heads a pass has fewer
 // CTAs than the GPU has SMs, or a long tail behind its heaviest CTAs; programmatic stream serialisation
 // lets this pass's CTAs take the SMs the pass ahead leaves idle (every key-major CTA executes
 // griddepcontrol.launch_dependents once set up).
-template <class C>
-attn_status_t launch_kvmajor_t(const AttnShape& s, attn_qtensor_t q, attn_qtensor_t k, attn_qtensor_t v, attn_qtensor_t dO,
+template <class C, bool kShared>
+attn_status_t launch_kvmajor_s(const AttnShape& s, attn_qtensor_t q, attn_qtensor_t k, attn_qtensor_t v, attn_qtensor_t dO,
                                const float* lse, const float* delta, void* dk, void* dv, int* status,
-                               cudaStream_t stream, bool behind = false, bool clear_tickets = false) {
+                               cudaStream_t stream, bool behind, bool clear_tickets, int split) {
   static_assert(sizeof(KvSmem<C>) + 1024 <= kSmemLimit, "shared memory exceeded");
+  // three quarters of the accumulators (a cluster of four) fit in the operand stages
+  static_assert(((C::kHasDv ? 128 * C::kRv : 0) + (C::kHasDk ? C::kQcRows : 0)) * kTile * 3 <=
+                    sizeof(KvSmem<C>::k) + sizeof(KvSmem<C>::rst) + sizeof(KvSmem<C>::cst), "inbox exceeds the operand stages");
   CUtensorMap tm_k, tm_v, tm_q, tm_dO, tm_qc, tm_dOc;
   attn_status_t st;
   const uint64_t eb = C::kEB, ebv = C::kEBv;
@@ -799,20 +904,25 @@ attn_status_t launch_kvmajor_t(const AttnShape& s, attn_qtensor_t q, attn_qtenso
   p.tail_wait = behind ? 1 : 0;
   p.tickets = clear_tickets ? ticket_counter(status) : nullptr;
   const size_t smem = sizeof(KvSmem<C>) + 1024;
-  if ((st = allow_smem<kvmajor_kernel<C>>(smem, "bwd kv-major")) != ATTN_OK) return st;
-  dim3 grid(s.Hkv, s.B, s.Nk / kTile);
+  if ((st = allow_smem<kvmajor_kernel<C, kShared>>(smem, "bwd kv-major")) != ATTN_OK) return st;
+  p.split = split;
+  dim3 grid(s.Hkv * split, s.B, s.Nk / kTile);
   // The first pass is launched behind whatever is ahead in the stream in the ordinary way: with programmatic
   // serialisation there as well, the kernels behind this one no longer started beside it (dK, dV and dQ at head
   // dim 256, 8/2 heads, one after the other: step 1065 -> 1257 us).
-  cudaError_t e;
-  if (behind) {
-    e = launch_overlapped(kvmajor_kernel<C>, grid, kThreads, smem, stream, 1, p, tm_k, tm_v, tm_q, tm_dO, tm_qc, tm_dOc);
-  } else {
-    kvmajor_kernel<C><<<grid, kThreads, smem, stream>>>(p, tm_k, tm_v, tm_q, tm_dO, tm_qc, tm_dOc);
-    e = cudaGetLastError();
-  }
+  const cudaError_t e = launch_kernel(kvmajor_kernel<C, kShared>, grid, kThreads, smem, stream, split, /*overlapped=*/behind, p, tm_k, tm_v,
+                                      tm_q, tm_dO, tm_qc, tm_dOc);
   if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "bwd kv-major: launch: %s", cudaGetErrorString(e));
   return ATTN_OK;
+}
+
+template <class C>
+attn_status_t launch_kvmajor_t(const AttnShape& s, attn_qtensor_t q, attn_qtensor_t k, attn_qtensor_t v, attn_qtensor_t dO,
+                               const float* lse, const float* delta, void* dk, void* dv, int* status, cudaStream_t stream,
+                               int split, bool behind = false, bool clear_tickets = false) {
+  if (split > 1)
+    return launch_kvmajor_s<C, true>(s, q, k, v, dO, lse, delta, dk, dv, status, stream, behind, clear_tickets, split);
+  return launch_kvmajor_s<C, false>(s, q, k, v, dO, lse, delta, dk, dv, status, stream, behind, clear_tickets, 1);
 }
 
 }  // namespace
@@ -821,37 +931,42 @@ attn_status_t launch_bwd_dkdv(const AttnShape& s, attn_qtensor_t q, attn_qtensor
                               const float* lse, const float* delta, void* dk, void* dv, int* status,
                               cudaStream_t stream, bool clear_tickets) {
   const int cq = (s.dqk * s.eb + 127) / 128, cv = (s.dv * s.ebv + 127) / 128;
+  int dev = 0, sms = 0;
+  const attn_status_t found = current_device(&dev, &sms);
+  if (found != ATTN_OK) return found;
+  const int passes = cq < 2 * s.eb || cv < 2 * s.eb ? 1 : (s.eb == 1 ? 2 : 3);    // (256,256) takes more than one
+  const int split = split_of(s, sms, passes, /*dq_follows=*/clear_tickets);
   if (s.eb == 1 && s.ebv == 2) {                     // protected dP: BF16 row copies of V and dO
     if (cq == 1 && cv == 1)
-      return launch_kvmajor_t<KvCfg<1, 1, 1, kBoth, 2>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream, false, clear_tickets);
+      return launch_kvmajor_t<KvCfg<1, 1, 1, kBoth, 2>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream, split, false, clear_tickets);
     if (cq == 1 && cv == 2)
-      return launch_kvmajor_t<KvCfg<1, 1, 2, kBoth, 2>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream, false, clear_tickets);
+      return launch_kvmajor_t<KvCfg<1, 1, 2, kBoth, 2>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream, split, false, clear_tickets);
     return fail(ATTN_ERR_UNSUPPORTED, "bwd kv-major: protected dP is built for head dims (64,64) and (128,128)");
   }
   if (s.eb == 1 && cq == 1 && cv == 1)
-    return launch_kvmajor_t<KvCfg<1, 1, 1, kBoth>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream, false, clear_tickets);
+    return launch_kvmajor_t<KvCfg<1, 1, 1, kBoth>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream, split, false, clear_tickets);
   if (s.eb == 2 && cq == 1 && cv == 1)
-    return launch_kvmajor_t<KvCfg<2, 1, 1, kBoth>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream, false, clear_tickets);
+    return launch_kvmajor_t<KvCfg<2, 1, 1, kBoth>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream, split, false, clear_tickets);
   if (s.eb == 2 && cq == 2 && cv == 2)
-    return launch_kvmajor_t<KvCfg<2, 2, 2, kBoth>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream, false, clear_tickets);
+    return launch_kvmajor_t<KvCfg<2, 2, 2, kBoth>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream, split, false, clear_tickets);
   // qk head dim above 128: dV and dK do not fit in tensor memory together; one pass each, the
   // heavier dK pass first and the dV pass launched behind it (see launch_kvmajor_t)
   // (at (192,128) both fit when every operand buffer and scale slot is single: KvCfg::kTight)
   if (s.eb == 1 && cq == 2 && cv == 1)
-    return launch_kvmajor_t<KvCfg<1, 2, 1, kBoth>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream, false, clear_tickets);
+    return launch_kvmajor_t<KvCfg<1, 2, 1, kBoth>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream, split, false, clear_tickets);
   if (s.eb == 1 && cq == 2 && cv == 2) {
-    attn_status_t st = launch_kvmajor_t<KvCfg<1, 2, 2, kDkOnly>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream, false, clear_tickets);
+    attn_status_t st = launch_kvmajor_t<KvCfg<1, 2, 2, kDkOnly>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream, split, false, clear_tickets);
     if (st != ATTN_OK) return st;
-    return launch_kvmajor_t<KvCfg<1, 2, 2, kDvOnly>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream, true);
+    return launch_kvmajor_t<KvCfg<1, 2, 2, kDvOnly>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream, split, true);
   }
   if (s.eb == 2 && cq == 3 && cv == 2)
-    return launch_kvmajor_t<KvCfg<2, 3, 2, kBoth>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream, false, clear_tickets);
+    return launch_kvmajor_t<KvCfg<2, 3, 2, kBoth>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream, split, false, clear_tickets);
   if (s.eb == 2 && cq == 4 && cv == 4) {
-    attn_status_t st = launch_kvmajor_t<KvCfg<2, 4, 4, kDkOnly, 2, 0>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream, false, clear_tickets);
+    attn_status_t st = launch_kvmajor_t<KvCfg<2, 4, 4, kDkOnly, 2, 0>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream, split, false, clear_tickets);
     if (st != ATTN_OK) return st;
-    st = launch_kvmajor_t<KvCfg<2, 4, 4, kDkOnly, 2, 1>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream, true);
+    st = launch_kvmajor_t<KvCfg<2, 4, 4, kDkOnly, 2, 1>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream, split, true);
     if (st != ATTN_OK) return st;
-    return launch_kvmajor_t<KvCfg<2, 4, 4, kDvOnly>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream, true);
+    return launch_kvmajor_t<KvCfg<2, 4, 4, kDvOnly>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream, split, true);
   }
   return fail(ATTN_ERR_UNSUPPORTED, "bwd kv-major: no kernel for head dims (%d, %d) at %d bytes per element", s.dqk, s.dv,
               s.eb);

@@ -307,3 +307,43 @@ def test_bench_residual_statistics_match_the_oracle_helpers():
     assert np.isclose(stats["kappa_mean"], np.mean(kappa), rtol=1e-9, atol=1e-18)
     assert np.isclose(stats["key_common_mode_median"], np.median(A.key_common_mode(to_np(dk))), rtol=1e-12, atol=0)
     assert np.isclose(stats["strict_ok_frac"], np.mean(r_pre <= 1e-5), rtol=0, atol=1e-12)
+
+
+@pytest.mark.parametrize("name,kw,bf16", [
+    ("gqa4k", dict(batch=1, heads_q=4, heads_kv=1, seqlen=3200), False),      # causal: the last key tile has a single query tile per head
+    ("tiny", dict(seqlen=2560, heads_q=1, heads_kv=1), False),                # one head, no mask, d = 64, lists of 20 tiles
+    ("gqa4k", dict(batch=1, heads_q=1, heads_kv=1, seqlen=4224), False),      # one head: CTAs of the last key tiles have no tile at all
+    ("mla8k", dict(heads_q=2, heads_kv=1, seqlen=2304), False),
+    ("gqa8k_d256", dict(heads_q=4, heads_kv=1, seqlen=2048), False),          # two passes
+    ("gqa4k", dict(batch=1, heads_q=4, heads_kv=1, seqlen=2048), True),
+])
+def test_key_tiles_shared_by_a_cluster(name, kw, bf16):
+    """Few heads: a cluster of CTAs shares a key tile and adds its partial sums (chosen by the launcher from the shape).
+    Against the same kernel on the same problem in a batch large enough for one CTA per key tile: the FP32 sums differ in
+    their order only, so the BF16 results differ by an ulp (2^-8) in few places; and the result does not depend on timing."""
+    from paper_2609_37852_b200 import binding
+    w = workloads.WORKLOADS[name].scaled(**kw)
+    tensors = [x.cuda() for x in workloads.make_inputs(w)]
+    if bf16:
+        tensors = [x.to(torch.bfloat16) for x in tensors]
+    prep = binding.attn_fp8_prepare_bf16 if bf16 else binding.attn_fp8_quantize
+    copies = 40
+
+    def grads(ts, batch):
+        params = binding.AttnParams(batch, w.seqlen, w.heads_q, w.heads_kv, w.head_dim_qk, w.head_dim_v, w.causal, w.softmax_scale,
+                                    precision=binding.ATTN_PREC_BF16 if bf16 else binding.ATTN_PREC_MXFP8)
+        q, k, v, dO = (prep(t) for t in ts)
+        _, lse, ws = binding.attn_fp8_fwd(params, q, k, v)
+        delta, _ = binding.attn_fp8_bwd_delta(params, q, k, v, dO, lse, workspace=ws)
+        out = [binding.attn_fp8_bwd_dkdv(params, q, k, v, dO, lse, delta, workspace=ws)[:2] for _ in range(3)]
+        binding.attn_fp8_read_status(ws)
+        for o in out[1:]:
+            assert torch.equal(o[0], out[0][0]) and torch.equal(o[1], out[0][1])
+        return out[0]
+
+    shared = grads(tensors, 1)
+    whole = grads([t.expand(copies, -1, -1, -1).contiguous() for t in tensors], copies)
+    for a, b in zip(shared, whole):
+        # one rounding to BF16 of FP32 sums that differ by ~1e-6: an ulp at a few elements, none elsewhere
+        assert rel_fro(to_np(a), to_np(b[:1])) <= 1e-3
+        assert worst_row_error(to_np(a), to_np(b[:1])) <= 4e-3
