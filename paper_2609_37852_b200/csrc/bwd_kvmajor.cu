@@ -274,12 +274,6 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
     mbar_init(&sm.done, 1);
     sm.abort_flag = 0;
     fence_mbar_init();
-    // The dQ kernel behind this grid starts once every CTA here has passed griddepcontrol.launch_dependents
-    // (below): it finds its counter cleared, without a memset of its own between the two launches.
-    if (p.tickets != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) {
-      atomicExch(p.tickets, 0);
-      __threadfence();
-    }
   }
   if (warp == 0) {
     tmem_alloc(&sm.tmem_base, kTmemCols);
@@ -288,8 +282,18 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
-  // the query-major kernel of the same call may be queued behind this grid: let its CTAs take the
-  // SMs that this grid's last wave leaves idle (nothing it does depends on this grid's output)
+  // The query-major kernel of the same call is queued behind this grid: its CTAs take the SMs that this grid's last
+  // wave leaves idle, and do not wait for this grid (nothing they do depends on its output).  So they must not start
+  // before what both read is complete, and their ticket counter is cleared: the wait comes first.  (A pass behind
+  // another key-major pass has nothing to wait for: that pass had waited when it let this one start.)
+  if (!p.tail_wait) griddep_wait();
+  if (p.tickets != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) {
+    if (tid == 0) {
+      atomicExch(p.tickets, 0);
+      __threadfence();
+    }
+    __syncthreads();
+  }
   griddep_launch_dependents();
   const uint32_t tmem = sm.tmem_base;
   bool stores = false;                                // this thread takes part in the epilogue
@@ -907,11 +911,15 @@ attn_status_t launch_kvmajor_s(const AttnShape& s, attn_qtensor_t q, attn_qtenso
   if ((st = allow_smem<kvmajor_kernel<C, kShared>>(smem, "bwd kv-major")) != ATTN_OK) return st;
   p.split = split;
   dim3 grid(s.Hkv * split, s.B, s.Nk / kTile);
-  // The first pass is launched behind whatever is ahead in the stream in the ordinary way: with programmatic
-  // serialisation there as well, the kernels behind this one no longer started beside it (dK, dV and dQ at head
-  // dim 256, 8/2 heads, one after the other: step 1065 -> 1257 us).
-  const cudaError_t e = launch_kernel(kvmajor_kernel<C, kShared>, grid, kThreads, smem, stream, split, /*overlapped=*/behind, p, tm_k, tm_v,
-                                      tm_q, tm_dO, tm_qc, tm_dOc);
+  // The first pass overlaps the kernel ahead like every other kernel only where its CTAs and those of the query-major
+  // kernel fit on the GPU together (one head of 256 tokens: step 28 -> 23 us).  On larger problems its CTAs would settle
+  // on whichever SMs the kernel ahead leaves first, and the kernels behind fill in worse: head dim 256, 8/2 heads, step
+  // 1046 -> 1113 us; 2 x 16/4 heads of 1000 tokens 119 -> 127 us; gqa4k 603 -> 611 us.
+  int dev = 0, sms = 0;
+  if ((st = current_device(&dev, &sms)) != ATTN_OK) return st;
+  const long long ctas = static_cast<long long>(s.B) * (s.Hkv * split * (s.Nk / kTile) + s.Hq * (s.N / kTile));
+  const cudaError_t e = launch_kernel(kvmajor_kernel<C, kShared>, grid, kThreads, smem, stream, split, behind || ctas <= sms, p,
+                                      tm_k, tm_v, tm_q, tm_dO, tm_qc, tm_dOc);
   if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "bwd kv-major: launch: %s", cudaGetErrorString(e));
   return ATTN_OK;
 }
