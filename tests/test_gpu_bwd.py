@@ -347,3 +347,18 @@ def test_key_tiles_shared_by_a_cluster(name, kw, bf16):
         # one rounding to BF16 of FP32 sums that differ by ~1e-6: an ulp at a few elements, none elsewhere
         assert rel_fro(to_np(a), to_np(b[:1])) <= 1e-3
         assert worst_row_error(to_np(a), to_np(b[:1])) <= 4e-3
+
+
+@pytest.mark.parametrize("dv,heads,seqlen", [(64, 1, 128), (64, 3, 384), (128, 2, 256), (256, 1, 128)])
+def test_stale_delta_every_head_dim(dv, heads, seqlen):
+    """delta = rowsum(dO o O) with 8, 16 and 32 lanes per row; FP32 sum of dv products: 2^-24 dv of the sum of magnitudes."""
+    from paper_2609_37852_b200 import binding
+    g = torch.Generator().manual_seed(dv)
+    dO, o = (torch.randn((1, heads, seqlen, dv), generator=g).to(torch.bfloat16).cuda() for _ in range(2))
+    lse = torch.zeros((1, heads, seqlen), device="cuda")
+    params = binding.AttnParams(1, seqlen, heads, heads, dv, dv, True, 0.1, delta_mode=binding.ATTN_DELTA_STALE)
+    none = binding.QTensor(shape=())
+    delta, ws = binding.attn_fp8_bwd_delta(params, none, none, none, none, lse, dO_bf16=dO, o_bf16=o)
+    binding.attn_fp8_read_status(ws)
+    prod = dO.double() * o.double()
+    assert bool(((delta.double() - prod.sum(-1)).abs() <= 2.0 ** -24 * dv * prod.abs().sum(-1)).all())
