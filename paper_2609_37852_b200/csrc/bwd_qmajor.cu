@@ -2,8 +2,8 @@
 // Eq. 4) and the query gradient (paper Appendix "Backward Correction and Gradient Computation").
 //
 // A work item is 128 query rows of one (batch, query head); the CTA that has it sweeps the key
-// tiles (128 keys) up to the causal diagonal.  Where shared memory allows, a CTA takes one item
-// after another (one CTA per SM; see QmCfg::kPersist for how the items are handed out).  For every
+// tiles (128 keys) up to the causal diagonal.  A CTA takes one item after another (one CTA per
+// SM; see QmCfg::kPersist for the exception and for how the items are handed out).  For every
 // key tile the tensor cores recompute
 //     S  = Q^ K^^T   (row-blocked FP8 copies, contraction over the qk channels)
 //     dP = dO^ V^^T  (row-blocked FP8 copies, contraction over the v channels)
@@ -60,10 +60,10 @@ struct QmCfg {
                                                         // 2 with kEB == 1 is the protected-dP ablation
   static constexpr bool kFp8 = kEB == 1;
   static constexpr bool kFp8v = kEBv == 1;
-  // Both kernels are persistent where shared memory allows: a CTA walks a list of query tiles, with
-  // the Q / dO tiles double-buffered and the K / V rings, the score buffers and their barriers
-  // running on across tile boundaries, so that set-up, pipeline fill and most of the drain are paid
-  // once per CTA instead of once per query tile.  The delta kernel takes a static list (all its CTAs
+  // Both kernels are persistent: a CTA walks a list of query tiles, with the Q / dO tiles double-buffered
+  // where shared memory allows and the K / V rings, the score buffers and their barriers running on across
+  // tile boundaries, so that set-up (4.6 us between two CTAs of an SM), pipeline fill and most of the drain
+  // are paid once per CTA instead of once per query tile.  The delta kernel takes a static list (all its CTAs
   // start together).  The dQ kernel is launched behind the key-major kernel, so its CTAs start at
   // different times: they draw their tiles from a ticket counter in the workspace instead.
   // FP8 at (256, 256) takes 64 keys per step: the whole dQ row (256 columns) then fits in tensor memory
@@ -82,10 +82,14 @@ struct QmCfg {
   static constexpr int kKcRows = kOneCta ? 192 : (kHalf ? 256 : 128);   // rows (dQ columns) of a K^c stage
   static constexpr int kDqCols = kKcRows;
   static constexpr int kKb = kStep * kEB / 32;          // 32-byte K steps of the dQ product per key step
-  static constexpr bool kPersist =
+  // (not dQ at head dim 256, whose eight softmax warps store 256 columns per item between two items: 232 us as one CTA
+  // per item, 243 persistent.  Gains elsewhere: dQ at (192,128) 320 -> 308 us, BF16 4K dQ 210 -> 195 and correction
+  // 166 -> 145, correction at head dim 256 123 -> 119)
+  static constexpr bool kPersist = !kHalf;
+  static constexpr bool kTwoQ = kPersist &&
       2 * (kCq + kCv) * kTile * 128 + 2 * ((kCq + kCv) * kStep * 128 + (kDQ ? kTile * 128 : 0)) <= 216 * 1024;
   static constexpr bool kTicket = kPersist && kDQ;
-  static constexpr int kQBufs = kPersist ? 2 : 1;       // Q / dO tile buffers (and scale-factor slots)
+  static constexpr int kQBufs = kTwoQ ? 2 : 1;          // Q / dO tile buffers (and scale-factor slots)
   static constexpr int kGroups = kStep / 32;            // 32-key column groups of a step
   static constexpr int kSoftmaxThreads = 128 * kGroups; // 4 TMEM lane quadrants x column groups
   static constexpr int kThreads = 128 + kSoftmaxThreads;
@@ -94,7 +98,7 @@ struct QmCfg {
   static constexpr int kFixedBytes = kQBufs * (kCq + kCv) * kTile * 128;
   static constexpr int kKvBytes = (kCq + kCv) * kStep * 128;
   static constexpr int kKcBytes = kDQ ? kKcRows * 128 : 0;
-  static constexpr int kRaw = ((kPersist ? 216 : 224) * 1024 - kFixedBytes - kKcBytes) / (kKvBytes + kKcBytes);
+  static constexpr int kRaw = ((kTwoQ ? 216 : 224) * 1024 - kFixedBytes - kKcBytes) / (kKvBytes + kKcBytes);
   // (BF16 at head dim 256: the Q / dO tiles alone take 128 KB and a K / V step 64 KB, so the ring is
   // a single stage there: loads and MMAs of successive steps no longer overlap)
   static constexpr bool kTwoFit = kFixedBytes + 2 * kKvBytes + kKcBytes <= 212 * 1024;
