@@ -209,6 +209,19 @@ attn_status_t attn_fp8_prepare_bf16(const void* src, int32_t src_dtype, int32_t 
 attn_status_t attn_fp8_pad_tokens(const void* src, int32_t elem_bytes, int32_t B, int32_t H, int32_t n, int32_t d,
                                   int32_t n_padded, void* dst, void* stream);
 
+/* One pitched copy: `rows` rows of `row_bytes` bytes, contiguous in src, `dst_pitch` bytes apart in dst. */
+typedef struct {
+  const void* src;
+  void* dst;
+  int64_t rows, row_bytes, dst_pitch;
+} attn_copy_job_t;
+#define ATTN_COPY_MAX_JOBS 64
+
+/* Up to ATTN_COPY_MAX_JOBS pitched copies in one launch (the chunks of a sequence, put together: every byte tensor of
+ * a quantised chunk is such a copy into that of the whole sequence).  Pointers, row_bytes and dst_pitch are multiples
+ * of 16; destinations must not overlap one another or a source.                                  */
+attn_status_t attn_fp8_copy_batch(const attn_copy_job_t* jobs, int32_t n_jobs, void* stream);
+
 /* Forward (paper Appendix "Forward Probability Encoding"): per query row, online softmax of
  * S = scale * Q^ K^^T over key tiles with a running INTEGER power-of-two shift, normaliser l
  * taken from the exponentials BEFORE the FP8 cast, probabilities quantised in-register in

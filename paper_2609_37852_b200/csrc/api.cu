@@ -271,6 +271,22 @@ attn_status_t attn_fp8_prepare_bf16(const void* src, int32_t src_dtype, int32_t 
   return launch_bf16_copies(src, src_dtype, B, H, N, d, out.row_codes, out.col_codes, static_cast<cudaStream_t>(stream));
 }
 
+attn_status_t attn_fp8_copy_batch(const attn_copy_job_t* jobs, int32_t n_jobs, void* stream) {
+  if (!jobs) return fail(ATTN_ERR_INVALID_ARG, "jobs is NULL");
+  if (n_jobs < 1 || n_jobs > ATTN_COPY_MAX_JOBS)
+    return fail(ATTN_ERR_INVALID_ARG, "n_jobs must be 1..%d (got %d)", ATTN_COPY_MAX_JOBS, n_jobs);
+  for (int j = 0; j < n_jobs; ++j) {
+    const attn_copy_job_t& c = jobs[j];
+    if (c.rows <= 0 || c.row_bytes <= 0 || c.dst_pitch < c.row_bytes)
+      return fail(ATTN_ERR_INVALID_ARG, "sizes must be positive and dst_pitch at least row_bytes");
+    if (c.row_bytes % 16 || c.dst_pitch % 16 || c.row_bytes / 16 > 0xffffffffLL)
+      return fail(ATTN_ERR_UNSUPPORTED, "row_bytes and dst_pitch must be multiples of 16");
+    CHECK(check_ptr(c.src, "src")); CHECK(check_ptr(c.dst, "dst"));
+  }
+  CHECK(check_device());
+  return launch_copy_batch(jobs, n_jobs, static_cast<cudaStream_t>(stream));
+}
+
 attn_status_t attn_fp8_pad_tokens(const void* src, int32_t elem_bytes, int32_t B, int32_t H, int32_t n, int32_t d,
                                   int32_t n_padded, void* dst, void* stream) {
   if (B <= 0 || H <= 0 || n <= 0 || d <= 0 || elem_bytes <= 0) return fail(ATTN_ERR_INVALID_ARG, "sizes must be positive");

@@ -91,6 +91,7 @@ attn_status_t launch_token_mean(const void* src, int src_dtype, int slabs, int N
 attn_status_t launch_quantize_batch(const attn_quantize_job_t* jobs, int n_jobs, int* status, cudaStream_t stream);
 attn_status_t launch_bf16_copies(const void* src, int src_dtype, int B, int H, int N, int d, void* row_out, void* col_out,
                                  cudaStream_t stream);
+attn_status_t launch_copy_batch(const attn_copy_job_t* jobs, int n, cudaStream_t stream);
 attn_status_t launch_pad_tokens(const void* src, long long slabs, long long row_bytes, int n, int n_out, void* dst, cudaStream_t stream);
 attn_status_t launch_fwd(const AttnShape& s, attn_qtensor_t q, attn_qtensor_t k, attn_qtensor_t v, void* o,
                          float* lse, int* status, cudaStream_t stream);

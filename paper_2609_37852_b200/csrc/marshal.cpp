@@ -349,10 +349,82 @@ PyObject* pad_tokens(PyObject*, PyObject* const* a, Py_ssize_t n) {
   });
 }
 
+// (parts): the buffers (row_codes, row_scales, col_codes, col_scales) of the QTensors of consecutive tokens put together,
+// or None where the kernel does not apply (the caller concatenates with torch then)
+PyObject* concat(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  return guarded(n, 1, [&]() -> PyObject* {
+    Attr parts(PySequence_Fast(a[0], "parts must be a sequence"));
+    const Py_ssize_t count = PySequence_Fast_GET_SIZE(parts.o);
+    PyObject* const field[4] = {names.row_codes, names.row_scales, names.col_codes, names.col_scales};
+    constexpr Py_ssize_t kMost = 256;
+    if (count < 1 || count > kMost) Py_RETURN_NONE;
+    int64_t b = 0, h = 0, d = 0, total = 0, tokens[kMost];
+    for (Py_ssize_t i = 0; i < count; ++i) {
+      Attr shape(PySequence_Fast_GET_ITEM(parts.o, i), names.shape);
+      Attr t(PySequence_Tuple(shape.o));
+      if (PyTuple_GET_SIZE(t.o) != 4) Py_RETURN_NONE;
+      const int64_t s[4] = {integer(PyTuple_GET_ITEM(t.o, 0)), integer(PyTuple_GET_ITEM(t.o, 1)), integer(PyTuple_GET_ITEM(t.o, 2)),
+                            integer(PyTuple_GET_ITEM(t.o, 3))};
+      if (i == 0) { b = s[0]; h = s[1]; d = s[3]; }
+      if (s[0] != b || s[1] != h || s[3] != d || s[2] <= 0 || s[2] % 128) Py_RETURN_NONE;
+      tokens[i] = s[2];
+      total += s[2];
+    }
+    // rows and bytes per row and token of the four byte tensors
+    const int64_t c = (d + 127) / 128, rows[4] = {b * h, b * h, b * h * d, b * h * c};
+    const auto width = [&](int f, int64_t n) { return f == 0 ? n * d : f == 1 ? n / 128 * c * 512 : f == 2 ? n : n / 128 * 512; };
+    if (b <= 0 || h <= 0 || d <= 0 || d % 16) Py_RETURN_NONE;
+    const int64_t dims[4][4] = {{b, h, total, d}, {}, {b, h, d, total}, {}};
+    at::Tensor out[4];
+    attn_copy_job_t jobs[ATTN_COPY_MAX_JOBS];
+    int n_jobs = 0;
+    void* const stream = c10::cuda::getCurrentCUDAStream().stream();
+    const auto flush = [&] {
+      if (n_jobs && attn_fp8_copy_batch(jobs, n_jobs, stream) != ATTN_OK) fail(PyExc_RuntimeError, attn_fp8_last_error());
+      n_jobs = 0;
+    };
+    // all tensors are looked at before the first launch
+    for (int pass = 0; pass < 2; ++pass) {
+      for (int f = 0; f < 4; ++f) {
+        int64_t at_bytes = 0;
+        for (Py_ssize_t i = 0; i < count; ++i) {
+          Attr o(PySequence_Fast_GET_ITEM(parts.o, i), field[f]);
+          if (o.o == Py_None) {
+            if (i && out[f].defined()) Py_RETURN_NONE;
+            continue;
+          }
+          if (!THPVariable_Check(o.o)) Py_RETURN_NONE;
+          const at::Tensor& x = THPVariable_Unpack(o.o);
+          const int64_t w = width(f, tokens[i]);
+          if (pass == 0) {
+            if (!x.is_cuda() || x.get_device() != c10::cuda::current_device() || x.scalar_type() != at::kByte || !x.is_contiguous() ||
+                x.numel() != rows[f] * w || reinterpret_cast<uintptr_t>(x.data_ptr()) % 16 || (i && !out[f].defined()))
+              Py_RETURN_NONE;
+            if (i == 0)
+              out[f] = f % 2 == 0 ? at::empty({dims[f][0], dims[f][1], dims[f][2], dims[f][3]}, x.options())
+                                  : at::empty({rows[f] * width(f, total)}, x.options());
+          } else {
+            jobs[n_jobs++] = attn_copy_job_t{x.data_ptr(), static_cast<uint8_t*>(out[f].data_ptr()) + at_bytes, rows[f], w, width(f, total)};
+            if (n_jobs == ATTN_COPY_MAX_JOBS) flush();
+            at_bytes += w;
+          }
+        }
+      }
+    }
+    flush();
+    PyObject* t[4];
+    for (int f = 0; f < 4; ++f) {
+      if (out[f].defined()) t[f] = THPVariable_Wrap(out[f]);
+      else { t[f] = Py_None; Py_INCREF(Py_None); }
+    }
+    return Py_BuildValue("(NNNN)", t[0], t[1], t[2], t[3]);
+  });
+}
+
 PyMethodDef methods[] = {
 #define ENTRY(name) {#name, reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(name)), METH_FASTCALL, nullptr}
     ENTRY(fwd), ENTRY(fwd_noalloc), ENTRY(bwd_delta), ENTRY(bwd), ENTRY(bwd_dq), ENTRY(bwd_dkdv), ENTRY(quantize),
-    ENTRY(quantize_batch), ENTRY(quantize_fused), ENTRY(prepare_bf16), ENTRY(new_operand), ENTRY(pad_tokens),
+    ENTRY(quantize_batch), ENTRY(quantize_fused), ENTRY(prepare_bf16), ENTRY(new_operand), ENTRY(pad_tokens), ENTRY(concat),
 #undef ENTRY
     {nullptr, nullptr, 0, nullptr}};
 

@@ -169,3 +169,20 @@ def test_forward_rows_do_not_depend_on_the_order_of_the_items(name):
         o1, lse1, _ = run(one(q), one(k), one(v), 1, 1)
         assert torch.equal(o1, one(o)) and torch.equal(lse1, one(lse))
     B.attn_fp8_read_status(ws)
+
+
+@pytest.mark.parametrize("lengths,d,row,col", [((128,), 64, True, True), ((128, 384, 256), 192, True, True), ((256, 128), 256, True, False),
+                                              ((128,) * 40, 128, True, True)])     # 160 copies: several launches
+def test_concat_chunks_gives_the_bytes_of_torch_cat(lengths, d, row, col):
+    from paper_2609_37852_b200 import binding as B
+    from paper_2609_37852_b200 import sequence_parallel as SP
+    g = torch.Generator().manual_seed(d)
+    parts = [SP.only(B.attn_fp8_quantize(torch.randn((2, 3, n, d), generator=g).cuda()), row, col) for n in lengths]
+    cpu = [B.QTensor(p.shape, *(None if t is None else t.cpu() for t in (p.row_codes, p.row_scales, p.col_codes, p.col_scales))) for p in parts]
+    got, want = SP.concat_chunks(parts), SP.concat_chunks(cpu)                  # CPU tensors: torch.cat
+    assert tuple(got.shape) == tuple(want.shape)
+    for f in ("row_codes", "row_scales", "col_codes", "col_scales"):
+        a, b = getattr(got, f), getattr(want, f)
+        assert (a is None) == (b is None)
+        if a is not None:
+            assert a.is_cuda and a.shape == b.shape and torch.equal(a.cpu(), b)
