@@ -171,3 +171,21 @@ def test_quantize_batch_random_job_mixes_bit_exact():
                 assert int(q.col_scales.to(torch.int64).sum()) == int(cs.astype(np.int64).sum())
             else:
                 assert q.col_codes is None
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("heads,wider", [(1, 0), (593, 0), (1185, 0), (5, 128)])
+def test_quantize_batch_of_head_dim_64_bit_exact(heads, wider, dtype):
+    # one tile; one more than four CTAs on each of 148 SMs; a third tile for one of them; next to a wider tensor
+    from paper_2609_37852_b200 import binding as B
+    g = torch.Generator().manual_seed(heads)
+    xs = [torch.randn(1, heads, 128, 64, generator=g).to(dtype)] + [torch.randn(1, 2, 128, wider, generator=g).to(dtype)] * (wider > 0)
+    outs, _ = B.attn_fp8_quantize_batch([x.cuda() for x in xs])
+    for x, qt in zip(xs, outs):
+        _, H, N, d = x.shape
+        rc, rs = mxfp8.quantize(to_np(x), axis=-1)
+        cc, cs = mxfp8.quantize(to_np(x), axis=-2)
+        assert np.array_equal(qt.row_codes.cpu().numpy(), rc)
+        assert np.array_equal(B.unpack_scales(qt.row_scales, 1, H, N, d).cpu().numpy(), rs)
+        assert np.array_equal(qt.col_codes.cpu().numpy(), np.swapaxes(cc, -1, -2))
+        assert np.array_equal(B.unpack_scales(qt.col_scales, 1, H, d, N).cpu().numpy(), np.swapaxes(cs, -1, -2))
