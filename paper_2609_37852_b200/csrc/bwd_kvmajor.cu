@@ -34,6 +34,7 @@
 #include "mma_issue.cuh"
 #include "mxfp8_device.cuh"
 #include "sm100_ptx.cuh"
+#include "work_order.cuh"
 
 namespace attnfp8 {
 
@@ -197,11 +198,16 @@ struct KvParams {
   int kv_lim;               // without the causal mask: last real key of the last key tile (127: all real)
   int tail_wait;            // launched behind another key-major pass of the same call (see launch_kvmajor_t)
   int* tickets;             // the dQ kernel's ticket counter, to be cleared ahead of it; or null
+  int slabs, group;         // (sequence, KV head) pairs, and how many of them run together (work_order.cuh)
   int split;                // CTAs (a cluster) that share the query tiles of one key tile: 1, 2 or 4
   float scale, scale_log2;
 };
 
 // kShared: a cluster of p.split CTAs shares the query tiles of a key tile (see split_of).
+__device__ __forceinline__ bool last_cta() {
+  return blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1 && blockIdx.z == gridDim.z - 1;
+}
+
 template <class C, bool kShared>
 __global__ void __launch_bounds__(kThreads, 1)
 kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
@@ -233,22 +239,23 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
     return;
   }
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  // blocks are handed out x-fastest, z-slowest: key tiles in order, so the heaviest tiles (the earliest keys under
-  // the causal mask) of all heads and sequences go first
-  const int jt = blockIdx.z;
-  // The walk of the list has a general form and, for one CTA per key tile, a simpler one.  They do the same; the softmax
-  // loop sits at its 96 registers, and the compiler keeps it free of spills with the one or the other (FP8 at head dims
-  // up to 128: 20 to 28 bytes with the simpler form, dK / dV of the 8K layer 1 % slower; (192,128): the reverse).
-  constexpr bool kGeneral = kShared || !kTight;
+  // The order of work_order.cuh, without its divisions, which cost the softmax loop registers: blocks are handed out
+  // x-fastest, z-slowest, (sequence, KV head) pairs within a group along x, key tiles along y (the earliest keys are the
+  // heaviest under the causal mask), groups along z.  The last group may be short of pairs.
+  const int jt = blockIdx.y;
   const int split = kShared ? p.split : 1, part = !kShared ? 0 : static_cast<int>(blockIdx.x) % split;
-  const int g = static_cast<int>(blockIdx.x) / split, b = blockIdx.y;
+  const int slab = static_cast<int>(blockIdx.z) * p.group + static_cast<int>(blockIdx.x) / split;
+  if (slab >= p.slabs) {                          // (all CTAs of a cluster)
+    if (p.tail_wait && tid == 0 && last_cta()) griddep_wait();
+    return;
+  }
   const int G = p.Hq / p.Hkv;
   const int tiles_n = p.N / kTile, tiles_nk = p.Nk / kTile;
   const int it0 = p.causal ? max(jt - p.q0t, 0) : 0;   // first query tile that sees these keys
   const int tiles_per_head = tiles_n - it0;
   // the query tiles of all heads of the group in one list; a CTA of a cluster walks every split-th of them
   const int n_list = G * tiles_per_head;
-  const int n_qtiles = !kGeneral ? n_list : (part < n_list ? (n_list - part + split - 1) / split : 0);
+  const int n_qtiles = part < n_list ? (n_list - part + split - 1) / split : 0;
   const int n_sub = 2 * n_qtiles;
   const int nk_qk = p.dqk * kEB / 32, nk_v = p.dv * C::kEBv / 32;   // 32-byte K steps of S^T and dP^T
   // columns of dK (rows of Q^c) this pass accumulates: all of them, or one tile of 128
@@ -303,21 +310,19 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
     if (lane == 0) {
       prefetch_tmap(&tm_k); prefetch_tmap(&tm_v); prefetch_tmap(&tm_q); prefetch_tmap(&tm_dO);
       prefetch_tmap(&tm_qc); prefetch_tmap(&tm_dOc);
-      const int kv_slab = b * p.Hkv + g;
       mbar_arrive_expect_tx(&sm.kv_full, kCq * (kTile * 128 + (kFp8 ? 512 : 0)) +
                                              (kHasDk ? kCv * (kTile * 128 + (kFp8v ? 512 : 0)) : 0));
-      for (int c = 0; c < kCq; ++c) tma_load_2d(sm.k[c], &tm_k, &sm.kv_full, 128 * c, kv_slab * p.Nk + jt * kTile);
-      if (kFp8) bulk_load_1d(sm.sf_k, p.k_sf + (static_cast<size_t>(kv_slab) * tiles_nk + jt) * kCq * 512, kCq * 512, &sm.kv_full);
+      for (int c = 0; c < kCq; ++c) tma_load_2d(sm.k[c], &tm_k, &sm.kv_full, 128 * c, slab * p.Nk + jt * kTile);
+      if (kFp8) bulk_load_1d(sm.sf_k, p.k_sf + (static_cast<size_t>(slab) * tiles_nk + jt) * kCq * 512, kCq * 512, &sm.kv_full);
       if (kHasDk) {
-        for (int c = 0; c < kCv; ++c) tma_load_2d(sm.v[c], &tm_v, &sm.kv_full, 128 * c, kv_slab * p.Nk + jt * kTile);
-        if (kFp8v) bulk_load_1d(sm.sf_v, p.v_sf + (static_cast<size_t>(kv_slab) * tiles_nk + jt) * kCv * 512, kCv * 512, &sm.kv_full);
+        for (int c = 0; c < kCv; ++c) tma_load_2d(sm.v[c], &tm_v, &sm.kv_full, 128 * c, slab * p.Nk + jt * kTile);
+        if (kFp8v) bulk_load_1d(sm.sf_v, p.v_sf + (static_cast<size_t>(slab) * tiles_nk + jt) * kCv * 512, kCv * 512, &sm.kv_full);
       }
       int issued_row = 0, issued_col = 0;
       bool ok = true;
       for (int u = 0; u < n_sub && ok; ++u) {
         const int n = part + split * (u >> 1), half = u & 1;
-        const int h = g * G + n / tiles_per_head, it = it0 + n % tiles_per_head;
-        const int q_slab = b * p.Hq + h;
+        const int q_slab = slab * G + n / tiles_per_head, it = it0 + n % tiles_per_head;
         const size_t sf_tile = static_cast<size_t>(q_slab) * tiles_n + it;
         if (u % kSubPerRow == 0) {
           const int ri = u / kSubPerRow, rs = ri % kRowStages;
@@ -427,11 +432,11 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
     int s = 0;                                        // running (stage, phase) of the row ring
     uint32_t s_phase = 0;
     // kPrepLoads: LSE and D of the next row stage (= sub-tile), in flight while this one is handled
-    int pf_h = g * G + (kShared ? part / tiles_per_head : 0), pf_it = it0 + (kShared ? part % tiles_per_head : 0);                    // (head, query tile) of the stage fetched next
+    int pf_h = slab * G + (kShared ? part / tiles_per_head : 0), pf_it = it0 + (kShared ? part % tiles_per_head : 0);                    // (head, query tile) of the stage fetched next
     float4 pf_l = make_float4(0.f, 0.f, 0.f, 0.f), pf_d = make_float4(0.f, 0.f, 0.f, 0.f);
     auto prefetch = [&](int uu) {
       if (4 * lane < kRowTok) {
-        const size_t at = static_cast<size_t>(b * p.Hq + pf_h) * p.N + pf_it * kTile + (uu & 1) * kSub + 4 * lane;
+        const size_t at = static_cast<size_t>(pf_h) * p.N + pf_it * kTile + (uu & 1) * kSub + 4 * lane;
         pf_l = *reinterpret_cast<const float4*>(p.lse + at);
         if (kHasDk) pf_d = *reinterpret_cast<const float4*>(p.delta + at);
       }
@@ -745,21 +750,17 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
       fence_proxy_async_smem();
       tc_fence_before_sync();
       mbar_arrive(&sm.op_full[buf]);
-      if (kGeneral) {                                 // next tile of this CTA, of this head or of one that follows
-        it += split;
-        while (it >= tiles_n) it -= tiles_per_head;
-      } else {
-        it = (it + 1 == tiles_n) ? it0 : it + 1;
-      }
+      it += split;                                    // next tile of this CTA, of this head or of one that follows
+      while (it >= tiles_n) it -= tiles_per_head;
     }
     // The epilogue is done by team 0 (group 0 stores dV, group 1 stores dK).
     if (team != 0) ok = false;
     if (grp == 0 ? !kHasDv : !kHasDk) ok = false;
-    if (ok && (!kGeneral || n_sub > 0)) ok = mbar_wait(&sm.done, 0, abort_flag);
+    if (ok && n_sub > 0) ok = mbar_wait(&sm.done, 0, abort_flag);
     if (kShared) stores = ok;
     else if (ok) {
       tc_fence_after_sync();
-      const size_t grow = static_cast<size_t>(b * p.Hkv + g) * p.Nk + jt * kTile + row;
+      const size_t grow = static_cast<size_t>(slab) * p.Nk + jt * kTile + row;
       const uint32_t col = grp == 0 ? kColdV : kColdK;
       const int width = grp == 0 ? p.dv : p.dqk;
       const int first = grp == 0 ? 0 : dk_col0, count = grp == 0 ? p.dv : dk_cols;   // columns this pass holds
@@ -812,7 +813,7 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
     cluster_sync();
     if (stores) {
       tc_fence_after_sync();
-      const size_t grow = static_cast<size_t>(b * p.Hkv + g) * p.Nk + jt * kTile + ep_row;
+      const size_t grow = static_cast<size_t>(slab) * p.Nk + jt * kTile + ep_row;
       const float mul = ep_grp == 0 ? 1.f : p.scale;
       __nv_bfloat16* out_row = (ep_grp == 0 ? p.dv_out : p.dk) + grow * (ep_grp == 0 ? p.dv : p.dqk) + first + part * slice;
       for (int c0 = 0; c0 < slice; c0 += 16) {
@@ -849,8 +850,7 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
   // This grid may have started while the pass ahead of it was draining.  One CTA, the last in launch
   // order, stays until that grid has completed, so that the completion of this grid implies the
   // completion of both for whatever follows in the stream.
-  if (p.tail_wait && tid == 0 && blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1 && blockIdx.z == gridDim.z - 1)
-    griddep_wait();
+  if (p.tail_wait && tid == 0 && last_cta()) griddep_wait();
 }
 
 // CTAs per key tile.  One CTA per key tile is the least work; but the first key tile's CTA walks G * N / 128 query tiles,
@@ -910,7 +910,12 @@ attn_status_t launch_kvmajor_s(const AttnShape& s, attn_qtensor_t q, attn_qtenso
   const size_t smem = sizeof(KvSmem<C>) + 1024;
   if ((st = allow_smem<kvmajor_kernel<C, kShared>>(smem, "bwd kv-major")) != ATTN_OK) return st;
   p.split = split;
-  dim3 grid(s.Hkv * split, s.B, s.Nk / kTile);
+  // bytes of Q and dO per (sequence, KV head): the copies this pass reads, of the heads of its group
+  const WorkOrder order = work_order(s.B * s.Hkv, 1, s.Nk / kTile,
+                                     static_cast<size_t>(s.Hq / s.Hkv) * s.N * (s.dqk * eb * (C::kHasDk ? 2 : 1) +
+                                                                                s.dv * ((C::kHasDk ? ebv : 0) + (C::kHasDv ? eb : 0))), false);
+  p.slabs = order.heads; p.group = order.group;
+  const dim3 grid = order.grid(split);
   // The first pass overlaps the kernel ahead like every other kernel only where its CTAs and those of the query-major
   // kernel fit on the GPU together (one head of 256 tokens: step 28 -> 23 us).  On larger problems its CTAs would settle
   // on whichever SMs the kernel ahead leaves first, and the kernels behind fill in worse: head dim 256, 8/2 heads, step

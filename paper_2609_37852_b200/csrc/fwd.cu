@@ -33,6 +33,7 @@
 #include "mma_issue.cuh"
 #include "mxfp8_device.cuh"
 #include "sm100_ptx.cuh"
+#include "work_order.cuh"
 
 namespace attnfp8 {
 
@@ -108,6 +109,7 @@ struct FwdParams {
   int N, Nk, q0t, Hq, Hkv, dqk, dv, causal;   // N query rows, Nk keys, q0t: tile offset of the causal diagonal
   int kv_lim;               // without the causal mask: last real key of the last key tile (127: all real)
   float scale_log2;         // softmax_scale * log2(e)
+  WorkOrder order;
 };
 
 template <class C>
@@ -128,10 +130,9 @@ fwd_kernel(const FwdParams p, const __grid_constant__ CUtensorMap tm_q, const __
   constexpr uint32_t kColS = C::kColS, kColP = C::kColP, kColO = C::kColO, kColSFQ = C::kColSFQ, kColSFK = C::kColSFK,
                      kColSFV = C::kColSFV, kColSFP = C::kColSFP, kTmemCols = C::kTmemCols, kPCols = C::kPCols;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  // blocks are handed out x-fastest, z-slowest: the heaviest (latest) query tiles of all heads and sequences go first, so the light tiles fill the tail of the launch
-  const int qt = p.causal ? (gridDim.z - 1 - blockIdx.z) : blockIdx.z;
-  const int h = blockIdx.x, b = blockIdx.y;
-  const int g = h / (p.Hq / p.Hkv);
+  int qt, q_slab;                                  // one item per CTA; the latest query tiles are the heaviest under the causal mask
+  if (!p.order.at_block(qt, q_slab)) return;
+  if (p.causal) qt = p.order.tiles - 1 - qt;
   const int n_tiles = p.causal ? qt + p.q0t + 1 : p.Nk / kTile;
   const int n_sub = 2 * n_tiles;
   const int n_stage_tiles = n_tiles * kEB;      // K / V stages to stream
@@ -166,13 +167,13 @@ fwd_kernel(const FwdParams p, const __grid_constant__ CUtensorMap tm_q, const __
     // ------------------------------------------------------------------ producer
     if (lane == 0) {
       prefetch_tmap(&tm_q); prefetch_tmap(&tm_k); prefetch_tmap(&tm_v);
-      const int q_row = (b * p.Hq + h) * p.N + qt * kTile;
+      const int q_row = q_slab * p.N + qt * kTile;
       const int tiles_n = p.N / kTile, tiles_nk = p.Nk / kTile;
       mbar_arrive_expect_tx(&sm.q_full, kCq * kTile * 128 + (kFp8 ? kCq * 512 : 0));
       for (int c = 0; c < kCq; ++c) tma_load_2d(sm.q[c], &tm_q, &sm.q_full, 128 * c, q_row);
       if (kFp8)
-        bulk_load_1d(sm.sf_q, p.q_sf + (static_cast<size_t>(b * p.Hq + h) * tiles_n + qt) * kCq * 512, kCq * 512, &sm.q_full);
-      const int kv_slab = b * p.Hkv + g;
+        bulk_load_1d(sm.sf_q, p.q_sf + (static_cast<size_t>(q_slab) * tiles_n + qt) * kCq * 512, kCq * 512, &sm.q_full);
+      const int kv_slab = p.order.slab_of(q_slab);
       int issued_k = 0, issued_v = 0;
       bool ok = true;
       for (int t = 0; t < n_stage_tiles && ok; ++t) {
@@ -425,7 +426,7 @@ fwd_kernel(const FwdParams p, const __grid_constant__ CUtensorMap tm_q, const __
     if (ok) {
       tc_fence_after_sync();
       const float inv_l = 1.f / l;
-      const size_t grow = static_cast<size_t>(b * p.Hq + h) * p.N + qt * kTile + row;
+      const size_t grow = static_cast<size_t>(q_slab) * p.N + qt * kTile + row;
       __nv_bfloat16* o_row = p.o + grow * p.dv;
       const int my_cols = p.dv / kSplit;              // each thread of a row stores its share of the row
       for (int c0 = grp * my_cols; c0 < (grp + 1) * my_cols; c0 += 32) {
@@ -473,8 +474,8 @@ attn_status_t launch_fwd_t(const AttnShape& s, attn_qtensor_t q, attn_qtensor_t 
   p.scale_log2 = s.scale * kLog2e;
   const size_t smem = sizeof(FwdSmem<C>) + 1024;
   if ((st = allow_smem<fwd_kernel<C>>(smem, "fwd")) != ATTN_OK) return st;
-  dim3 grid(s.Hq, s.B, s.N / kTile);
-  const cudaError_t e = launch_overlapped(fwd_kernel<C>, grid, C::kThreads, smem, stream, 1, p, tm_q, tm_k, tm_v);
+  p.order = work_order(s.B * s.Hkv, s.Hq / s.Hkv, s.N / kTile, static_cast<size_t>(s.Nk) * (s.dqk + s.dv) * eb, false);
+  const cudaError_t e = launch_overlapped(fwd_kernel<C>, p.order.grid(), C::kThreads, smem, stream, 1, p, tm_q, tm_k, tm_v);
   if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "fwd: launch: %s", cudaGetErrorString(e));
   return ATTN_OK;
 }

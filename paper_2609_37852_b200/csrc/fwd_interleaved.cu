@@ -27,6 +27,7 @@
 #include "mma_issue.cuh"
 #include "mxfp8_device.cuh"
 #include "sm100_ptx.cuh"
+#include "work_order.cuh"
 
 namespace attnfp8 {
 
@@ -126,7 +127,7 @@ struct IlParams {
   int* status;
   int N, Nk, q0t, Hq, Hkv, dqk, dv, causal;   // N query rows, Nk keys, q0t: tile offset of the causal diagonal
   int kv_lim;               // without the causal mask: last real key of the last key tile (127: all real)
-  int gx, gy, gz;           // the (head, query tile, batch) grid the work items are numbered in
+  WorkOrder order;
   float scale_log2;         // softmax_scale * log2(e)
 };
 
@@ -151,24 +152,20 @@ fwd_il_kernel(const IlParams p, const __grid_constant__ CUtensorMap tm_q, const 
   constexpr uint32_t kColS = C::kColS, kColO = C::kColO, kColP = C::kColP, kColSFQ = C::kColSFQ, kColSFK = C::kColSFK,
                      kColSFV = C::kColSFV, kColSFP = C::kColSFP;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  // Work items (128 query rows of one head) are numbered over (head, batch, query tile), the tile slowest, so that
-  // the heaviest (latest) query tiles of all heads and sequences come first.  (With the batch slowest, the second
-  // sequence's heaviest items came last: 2 x 16 heads x 4096 tokens, 118.7 us for 103.3 us of work per SM, now 105;
-  // 8 x 12 heads x 1024 tokens 38.4 us for 27.2, now 29.)  CTA c of n takes the items c, 2n-1-c, 2n+c, ...: alternate rounds run backwards, so that no CTA collects the
+  // Work items are numbered by p.order, the heaviest (latest) query tiles first.  CTA c of n takes the items c, 2n-1-c,
+  // 2n+c, ...: alternate rounds run backwards, so that no CTA collects the
   // heavier item of every round.  The K / V rings, the score and probability buffers and their
   // barriers run on across items; Q is double-buffered; the output accumulator is handed from the
   // unit keepers (who store the finished item) back to the P V issuer once per item.
   const int n_cta = static_cast<int>(gridDim.x), cta = static_cast<int>(blockIdx.x);
-  const int total_items = p.gx * p.gy * p.gz;
-  struct Item { int qt, h, b, g, n_tiles, n_steps; bool valid; };
+  const int total_items = p.order.heads * p.order.tiles;
+  struct Item { int qt, q_slab, n_tiles, n_steps; bool valid; };
   auto item_at = [&](int i) {
     Item it;
     const int l = i * n_cta + ((i & 1) ? n_cta - 1 - cta : cta);
     it.valid = l < total_items;
-    const int x = l % p.gx, z = (l / p.gx) % p.gz, y = l / (p.gx * p.gz);
-    it.qt = p.causal ? (p.gy - 1 - y) : y;
-    it.h = x; it.b = z;
-    it.g = it.h / (p.Hq / p.Hkv);
+    p.order.decode(it.valid ? l : 0, it.qt, it.q_slab);
+    if (p.causal) it.qt = p.order.tiles - 1 - it.qt;
     it.n_tiles = p.causal ? it.qt + p.q0t + 1 : p.Nk / kTile;
     it.n_steps = it.n_tiles * kSubPerTile;
     return it;
@@ -221,7 +218,7 @@ fwd_il_kernel(const IlParams p, const __grid_constant__ CUtensorMap tm_q, const 
             ok = mbar_wait(&sm.q_empty[qb], ((i >> 1) - 1) & 1, abort_flag);
             if (!ok) break;
           }
-          const int q_slab = it.b * p.Hq + it.h, kv_slab = it.b * p.Hkv + it.g;
+          const int q_slab = it.q_slab, kv_slab = p.order.slab_of(q_slab);
           mbar_arrive_expect_tx(&sm.q_full[qb], kCq * (kTile * 128 + 512));
           for (int c = 0; c < kCq; ++c) tma_load_2d(sm.q[qb][c], &tm_q, &sm.q_full[qb], 128 * c, q_slab * p.N + it.qt * kTile);
           bulk_load_1d(sm.sf_q[qb], p.q_sf + (static_cast<size_t>(q_slab) * tiles_n + it.qt) * kCq * 512, kCq * 512,
@@ -427,7 +424,7 @@ fwd_il_kernel(const IlParams p, const __grid_constant__ CUtensorMap tm_q, const 
           lt += lds_f32(&sm.fin_l[i & 3][at][row]) * pow2_int(lds_f32(&sm.fin_m[i & 3][at][row]) - MO);   // M = -inf goes with l = 0
       }
       const float inv_l = 1.f / lt;
-      const size_t grow = static_cast<size_t>(it.b * p.Hq + it.h) * p.N + it.qt * kTile + row;
+      const size_t grow = static_cast<size_t>(it.q_slab) * p.N + it.qt * kTile + row;
       __nv_bfloat16* o_row = p.o + grow * p.dv;
       for (int c0 = 0; c0 < p.dv; c0 += 16) {
         uint32_t r[16];
@@ -621,8 +618,8 @@ attn_status_t launch_fwd_il_t(const AttnShape& s, attn_qtensor_t q, attn_qtensor
   p.scale_log2 = s.scale * kLog2e;
   const size_t smem = sizeof(IlSmem<C>) + 1024;
   if ((st = allow_smem<fwd_il_kernel<C>>(smem, "fwd")) != ATTN_OK) return st;
-  p.gx = s.Hq; p.gy = s.N / kTile; p.gz = s.B;
-  const long long items = static_cast<long long>(p.gx) * p.gy * p.gz;
+  p.order = work_order(s.B * s.Hkv, s.Hq / s.Hkv, s.N / kTile, static_cast<size_t>(s.Nk) * (s.dqk + s.dv), true);
+  const long long items = p.order.items();
   if (items > 0x7fffffffLL) return fail(ATTN_ERR_UNSUPPORTED, "fwd: %lld work items exceed 2^31 - 1", items);
   // one CTA per SM (the kernel takes all of an SM's tensor memory) walks the item list
   int dev = 0, sms = 0;

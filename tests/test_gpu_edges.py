@@ -79,6 +79,32 @@ def test_shape_and_mode_combinations(name, kw, bf16):
     _check(w, tensors, _full_pass(w, tensors, bf16=bf16), prec="bf16" if bf16 else "mxfp8")
 
 
+@pytest.mark.parametrize("dims,heads_kv,per_kv,bf16", [
+    ((128, 128), 1030, 1, False),       # three groups of the work list, the last one short
+    ((128, 128), 520, 2, False),        # two query heads per KV head
+    ((192, 128), 420, 1, False),
+    ((256, 256), 260, 1, False),        # one CTA per item in the forward and the query-major kernels
+    ((128, 128), 260, 1, True),
+    ((256, 256), 131, 1, True),         # two dQ column tiles per head, three key-major passes
+])
+def test_heads_do_not_depend_on_their_group_of_the_work_list(dims, heads_kv, per_kv, bf16):
+    # 256 tokens, causal: K and V of all heads exceed the 32 MB of a group; 100 heads at a time they do not, and every
+    # head's results are the same bits
+    g = torch.Generator(device="cuda").manual_seed(heads_kv)
+    w = workloads.WORKLOADS["gqa4k"].scaled(batch=1, heads_q=heads_kv * per_kv, heads_kv=heads_kv, seqlen=256, head_dim_qk=dims[0],
+                                            head_dim_v=dims[1])
+    q, k, v, dO = (torch.randn(1, h, 256, d, generator=g, device="cuda", dtype=torch.bfloat16)
+                   for h, d in ((w.heads_q, dims[0]), (heads_kv, dims[0]), (heads_kv, dims[1]), (w.heads_q, dims[1])))
+    whole = _full_pass(w, (q, k, v, dO), bf16)
+    for a in range(0, heads_kv, 100):
+        b = min(a + 100, heads_kv)
+        qs = slice(a * per_kv, b * per_kv)
+        part = _full_pass(w.scaled(heads_q=(b - a) * per_kv, heads_kv=b - a), (q[:, qs], k[:, a:b], v[:, a:b], dO[:, qs]), bf16)
+        for n in ("o", "lse", "delta", "dq", "dk", "dv"):
+            heads = slice(a, b) if n in ("dk", "dv") else qs
+            assert torch.equal(whole[n][:, heads], part[n]), n
+
+
 def test_nearly_one_hot_rows_stress():
     """Outlier channels shared by a query head and its KV head: scores with a standard deviation of
     ~70, rows nearly one-hot, the running shift raised (and the output accumulator rescaled) often."""
