@@ -289,14 +289,12 @@ qmajor_kernel(const QmParams p, const __grid_constant__ CUtensorMap tm_q, const 
         }
         Item it;
         if (kTicket) {
-          // publish this CTA's i-th item (or the end of the list) to the other warps, and draw the
-          // next ticket now: its latency passes while this item's copies are issued
+          // publish this CTA's i-th item (or the end of the list) to the other warps
           const bool more = ticket < total_items;
           it = decode(more ? ticket : 0);
           *reinterpret_cast<int4*>(sm.item[i & 3]) = make_int4(it.qt, it.q_slab, it.r_tile, more ? it.n_tiles : 0);
           mbar_arrive(&sm.item_full[i & 3]);
           if (!more) break;
-          ticket = atomicAdd(p.sched, 1);
         } else {
           it = item_at(i);
           if (!it.valid) break;
@@ -310,6 +308,11 @@ qmajor_kernel(const QmParams p, const __grid_constant__ CUtensorMap tm_q, const 
         if (kFp8v)
           bulk_load_1d(sm.sf_dO[qb], p.dO_sf + (static_cast<size_t>(q_slab) * tiles_n + it.qt) * kCv * 512, kCv * 512, &sm.q_full[qb]);
         for (int t = 0; t < it.n_tiles && ok; ++t) {
+          // The next ticket is drawn one step before the last: its latency passes behind the copies of two steps, and
+          // the CTA holds no second item for the length of a first.  (Drawn when an item began, 4 heads of 2304 queries on
+          // 18432 keys at (192,128), 72 items: half of the CTAs took two items in a row and the others none, dK / dV and dQ
+          // 428 us, now 290; 8/2 heads x 3000 tokens, dQ 46 -> 36 us.)
+          if (kTicket && t == max(it.n_tiles - 2, 0)) ticket = atomicAdd(p.sched, 1);
           const int gt = T + t;                       // step index over all items of this CTA: the rings run on
           const int s = gt % kStages, u = gt / kStages;
           ok = mbar_wait(&sm.kv_empty[s], (u & 1) ^ 1, abort_flag);
