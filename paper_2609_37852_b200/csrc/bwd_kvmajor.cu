@@ -97,9 +97,12 @@ struct KvCfg {
   // taken S of u + 2, i.e. finished u); an even count keeps each slot with one team.
   // (not at (192,128) in BF16 mode, one pass: a single column stage paces that kernel and the change cost 5 %)
   static constexpr bool kEarly = kRowTok == kSub && !(kEB == 2 && kTightDims);
-  // arrivals that release a row stage: the commits behind the S^T and dP^T MMAs; without dP^T, in BF16 mode
-  // (LSE arrives in the stage by a bulk copy), the preparation warp once it has read LSE out of the stage
-  static constexpr int kRowReleases = !kEarly ? 1 : (kHasDk ? 2 : (kEB == 1 ? 1 : 2));
+  // arrivals that release a row stage: the commits behind the S^T and dP^T MMAs; without dP^T the preparation warp in
+  // the place of the latter, once it has seen the stage (and read LSE out of it, where LSE arrives in the stage).  It has
+  // to be one of them: the softmax releases S before it asks for LSE, so the S^T issuer can be three sub-tiles ahead of
+  // a preparation warp that waits for LSE from memory, and a stage filled anew in the meantime would complete the phase
+  // after the one that this warp has yet to see (FP8 dV pass at head dim 256: one call in about 600 waited for ever).
+  static constexpr int kRowReleases = !kEarly ? 1 : 2;
   static constexpr int kLseSlots = kEarly ? ((kRowStages + 4) & ~1) : kRowStages;
   // Tensor memory.  BF16 mode has no scale factors, which leaves columns for a second S^T buffer (one per team) when
   // P^ and dS^ keep one operand buffer each; S^T and dP^T are then released one by one (kApart: the softmax takes S,
@@ -457,6 +460,7 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
         ok = __all_sync(0xffffffffu, mbar_wait(&sm.row_full[s], s_phase, abort_flag));
         if (!ok) break;
         if (kPrepLoads) {
+          if (!kHasDk) mbar_arrive_warp(&sm.row_empty[s]);
           if (4 * lane < kRowTok) {
             *reinterpret_cast<float4*>(&sm.lse_ring[ls][4 * lane]) =
                 make_float4(-pf_l.x * kLog2e, -pf_l.y * kLog2e, -pf_l.z * kLog2e, -pf_l.w * kLog2e);

@@ -65,8 +65,8 @@ struct WorkOrder {
 
 // `slabs` (sequence, KV head) pairs of `per_slab` heads, `bytes` of operands per pair that its items share.
 // A group takes 32 MB of them (16 and 64 MB are 0 to 2 % behind where they differ), and not less than four rounds of items
-// on 148 SMs, since the CTAs drift apart where one group gives way to the next, unless that is more than 80 MB: beyond,
-// L2 (126 MB) may not hold it, and head dim 256 then fell into a state in which it took three times as long.
+// on 148 SMs, since the CTAs drift apart where one group gives way to the next, unless that is more than 80 MB, beyond
+// which L2 (126 MB) may not hold it.
 inline WorkOrder work_order(int slabs, int per_slab, int tiles, size_t bytes, bool flip) {
   const long long fits = (32LL << 20) / bytes, most = (80LL << 20) / bytes, per = static_cast<long long>(per_slab) * tiles;
   const long long enough = (4 * 148 + per - 1) / per;
