@@ -917,7 +917,7 @@ attn_status_t launch_kvmajor_s(const AttnShape& s, attn_qtensor_t q, attn_qtenso
   // bytes of Q and dO per (sequence, KV head): the copies this pass reads, of the heads of its group
   const WorkOrder order = work_order(s.B * s.Hkv, 1, s.Nk / kTile,
                                      static_cast<size_t>(s.Hq / s.Hkv) * s.N * (s.dqk * eb * (C::kHasDk ? 2 : 1) +
-                                                                                s.dv * ((C::kHasDk ? ebv : 0) + (C::kHasDv ? eb : 0))), false);
+                                                                                s.dv * ((C::kHasDk ? ebv : 0) + (C::kHasDv ? eb : 0))), s.causal, false);
   p.slabs = order.heads; p.group = order.group;
   const dim3 grid = order.grid(split);
   // The first pass overlaps the kernel ahead like every other kernel only where its CTAs and those of the query-major

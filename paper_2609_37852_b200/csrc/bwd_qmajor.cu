@@ -812,7 +812,7 @@ attn_status_t launch_qmajor_t(const AttnShape& s, attn_qtensor_t q, attn_qtensor
   const int rq = (kDQ && !C::kWhole) ? (s.dqk + 127) / 128 : 1;
   // bytes of K and V per (sequence, KV head): the row copies, and for dQ the column copy of K
   p.order = work_order(s.B * s.Hkv, s.Hq / s.Hkv * rq, s.N / kTile,
-                       static_cast<size_t>(s.Nk) * (s.dqk * eb * (kDQ ? 2 : 1) + s.dv * ebv), !C::kTicket);
+                       static_cast<size_t>(s.Nk) * (s.dqk * eb * (kDQ ? 2 : 1) + s.dv * ebv), s.causal, !C::kTicket);
   const long long items = p.order.items();
   if (items > 0x7fffffffLL) return fail(ATTN_ERR_UNSUPPORTED, "bwd q-major: %lld work items exceed 2^31 - 1", items);
   dim3 grid = p.order.grid();

@@ -474,7 +474,7 @@ attn_status_t launch_fwd_t(const AttnShape& s, attn_qtensor_t q, attn_qtensor_t 
   p.scale_log2 = s.scale * kLog2e;
   const size_t smem = sizeof(FwdSmem<C>) + 1024;
   if ((st = allow_smem<fwd_kernel<C>>(smem, "fwd")) != ATTN_OK) return st;
-  p.order = work_order(s.B * s.Hkv, s.Hq / s.Hkv, s.N / kTile, static_cast<size_t>(s.Nk) * (s.dqk + s.dv) * eb, false);
+  p.order = work_order(s.B * s.Hkv, s.Hq / s.Hkv, s.N / kTile, static_cast<size_t>(s.Nk) * (s.dqk + s.dv) * eb, s.causal, false);
   const cudaError_t e = launch_overlapped(fwd_kernel<C>, p.order.grid(), C::kThreads, smem, stream, 1, p, tm_q, tm_k, tm_v);
   if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "fwd: launch: %s", cudaGetErrorString(e));
   return ATTN_OK;

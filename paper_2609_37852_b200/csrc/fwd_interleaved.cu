@@ -618,7 +618,7 @@ attn_status_t launch_fwd_il_t(const AttnShape& s, attn_qtensor_t q, attn_qtensor
   p.scale_log2 = s.scale * kLog2e;
   const size_t smem = sizeof(IlSmem<C>) + 1024;
   if ((st = allow_smem<fwd_il_kernel<C>>(smem, "fwd")) != ATTN_OK) return st;
-  p.order = work_order(s.B * s.Hkv, s.Hq / s.Hkv, s.N / kTile, static_cast<size_t>(s.Nk) * (s.dqk + s.dv), true);
+  p.order = work_order(s.B * s.Hkv, s.Hq / s.Hkv, s.N / kTile, static_cast<size_t>(s.Nk) * (s.dqk + s.dv), s.causal, true);
   const long long items = p.order.items();
   if (items > 0x7fffffffLL) return fail(ATTN_ERR_UNSUPPORTED, "fwd: %lld work items exceed 2^31 - 1", items);
   // one CTA per SM (the kernel takes all of an SM's tensor memory) walks the item list
