@@ -657,7 +657,8 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
         }
       };
       if (p.causal && it + p.q0t == jt) body(std::true_type{}); else body(std::false_type{});
-      if (__builtin_expect(!p.causal && row > p.kv_lim && jt == p.Nk / kTile - 1, 0)) {
+      const bool padded = !p.causal && row > p.kv_lim && jt == p.Nk / kTile - 1;
+      if (__builtin_expect(padded, 0)) {
         // a padded key of a ragged sequence (no causal mask): its probabilities and score gradients are zero
 #pragma unroll
         for (int c = 0; c < 32; ++c) { sr[c] = 0u; dpr[c] = 0u; }
@@ -721,6 +722,10 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
             const int c = c4 + e;
             gradient(c, make_float2(__uint_as_float(sr[c]), __uint_as_float(sr[c + 1])), e == 0 ? make_float2(d4.x, d4.y) : make_float2(d4.z, d4.w));
           }
+        }
+        if (__builtin_expect(padded, 0)) {              // 0 * (dP - D) is not zero where dP or D is not finite
+#pragma unroll
+          for (int c = 0; c < 32; ++c) dpr[c] = 0u;
         }
       }
       if (kHasDk) {
