@@ -166,7 +166,8 @@ def pad_tokens(x: torch.Tensor, multiple: int = 128) -> torch.Tensor:
     pad = (-n) % multiple
     if pad == 0:
         return x.contiguous()
-    out = _marshal.pad_tokens(x, n + pad) if x.is_cuda else None
+    # (a compiler follows torch's operations only)
+    out = _marshal.pad_tokens(x, n + pad) if x.is_cuda and not torch.compiler.is_compiling() else None
     if out is not None:
         return out
     out = torch.zeros((x.shape[0], x.shape[1], n + pad, x.shape[3]), dtype=x.dtype, device=x.device)

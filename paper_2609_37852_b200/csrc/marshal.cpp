@@ -7,7 +7,9 @@
 
 #include <torch/csrc/autograd/python_variable.h>
 
+#include <ATen/PythonTorchFunctionTLS.h>
 #include <ATen/ops/empty.h>
+#include <c10/core/impl/LocalDispatchKeySet.h>
 #include <c10/cuda/CUDAFunctions.h>
 #include <c10/cuda/CUDAStream.h>
 
@@ -136,6 +138,19 @@ void check_shape(PyObject* qtensor, const attn_quantize_job_t& j, const char* me
   bool same = PyTuple_GET_SIZE(t.o) == 4;
   for (int i = 0; same && i < 4; ++i) same = integer(PyTuple_GET_ITEM(t.o, i)) == want[i];
   if (!same) fail(PyExc_ValueError, message);
+}
+
+// Whether a kernel launched here may stand in for torch operations on `o`: a plain CUDA tensor, with nothing that follows
+// or replaces the operations (a trace, a dispatch or function mode, a functorch level, a tensor subclass, a tangent, a
+// lazy conjugate, negative or zero).  Whatever does has to see torch's own operations.
+bool plain(PyObject* o) {
+  using c10::DispatchKey;
+  static constexpr c10::DispatchKeySet kTensor({DispatchKey::CUDA, DispatchKey::AutogradCUDA, DispatchKey::AutocastCUDA, DispatchKey::ADInplaceOrView});
+  static constexpr c10::DispatchKeySet kThread({DispatchKey::BackendSelect, DispatchKey::ADInplaceOrView});
+  if (!THPVariable_CheckExact(o)) return false;
+  const at::Tensor& x = THPVariable_Unpack(o);
+  return kTensor.has_all(x.key_set()) && kThread.has_all(c10::impl::tls_local_dispatch_key_set().included_) &&
+         !at::impl::torch_function_mode_enabled() && !x._fw_grad(0).defined();
 }
 
 template <class F>
@@ -332,10 +347,10 @@ PyObject* new_operand(PyObject*, PyObject* const* a, Py_ssize_t n) {
 // (x, n_padded): the padded tensor, or None where the kernel does not apply (the caller pads with torch then)
 PyObject* pad_tokens(PyObject*, PyObject* const* a, Py_ssize_t n) {
   return guarded(n, 2, [&]() -> PyObject* {
-    if (!THPVariable_Check(a[0])) Py_RETURN_NONE;
+    if (!plain(a[0])) Py_RETURN_NONE;
     const at::Tensor& x = THPVariable_Unpack(a[0]);
     const int64_t rows = integer(a[1]);
-    if (!x.is_cuda() || !x.is_contiguous() || x.dim() != 4 || x.requires_grad() || x.numel() == 0 || x.is_conj() || x.is_neg() ||
+    if (!x.is_contiguous() || x.dim() != 4 || x.requires_grad() || x.numel() == 0 ||
         (x.size(3) * x.element_size()) % 16 || reinterpret_cast<uintptr_t>(x.data_ptr()) % 16 || x.size(0) * x.size(1) > INT32_MAX ||
         x.get_device() != c10::cuda::current_device())
       Py_RETURN_NONE;

@@ -13,7 +13,7 @@ import torch
 
 from oracle import attention as A
 from paper_2609_37852_b200 import workloads
-from tests.util import rel_fro, to_np, worst_row_error
+from tests.util import followed_by_torch, rel_fro, to_np, worst_row_error
 
 pytestmark = pytest.mark.gpu
 
@@ -105,6 +105,22 @@ def test_pad_tokens_appends_zero_rows(shape, dtype):
         assert torch.equal(y[:, :, :n], x) and not y[:, :, n:].any()
     y = B.pad_tokens(x.clone().requires_grad_(True))                             # stays differentiable
     y.sum().backward()
+
+
+def test_pad_tokens_is_seen_by_whatever_follows_torch_operations():
+    """A trace or graph of it is a function of its input, tangents pass through, and fake and lazily zero tensors are taken."""
+    from paper_2609_37852_b200 import binding as B
+    import torch.autograd.forward_ad as fw
+    x, y = torch.randn((2, 1, 2, 100, 64), device="cuda")
+    want = torch.nn.functional.pad(y, (0, 0, 0, 28))
+    for how, got in followed_by_torch(B.pad_tokens, x, y):
+        assert torch.equal(got, want), how
+    with fw.dual_level():
+        p, t = fw.unpack_dual(B.pad_tokens(fw.make_dual(x, y)))
+        assert torch.equal(t, want) and torch.equal(p[:, :, :100], x)
+    p, t = torch.func.jvp(B.pad_tokens, (x,), (y,))
+    assert torch.equal(t, want)
+    assert not B.pad_tokens(torch._efficientzerotensor(1, 2, 100, 64, device="cuda")).any()
 
 
 def test_keys_valid_is_validated():

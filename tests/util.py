@@ -27,3 +27,27 @@ def worst_row_error(got, want) -> float:
         return 0.0
     sel &= ref > 0
     return float((err[sel] / ref[sel]).max())
+
+
+def followed_by_torch(f, x, y):
+    """Yields (name, f(y)) as each of torch's ways of following a function of a tensor gives it: recorded on `x` and played on
+    `y`, traced symbolically, or run under a mode."""
+    from torch._subclasses.fake_tensor import FakeTensorMode
+    from torch.fx.experimental.proxy_tensor import make_fx
+    yield "trace", torch.jit.trace(lambda a: f(a), (x,), check_trace=False)(y)
+    yield "make_fx", make_fx(lambda a: f(a))(x)(y)
+    yield "compile", torch.compile(lambda a: f(a), backend="eager", fullgraph=True)(y)
+    with FakeTensorMode(allow_non_fake_inputs=False) as mode:
+        fake = f(mode.from_tensor(y))
+    want = f(y)
+    assert type(fake).__name__ == "FakeTensor" and fake.shape == want.shape and fake.dtype == want.dtype
+    seen = []
+
+    class Mode(torch.overrides.TorchFunctionMode):
+        def __torch_function__(self, func, types, args=(), kwargs=None):
+            seen.append(func)
+            return func(*args, **(kwargs or {}))
+    with Mode():
+        got = f(y)
+    assert len(seen) > 1 and any("zeros" in str(s) or "cat" in str(s) for s in seen)
+    yield "function mode", got
