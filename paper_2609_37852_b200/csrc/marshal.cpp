@@ -408,11 +408,11 @@ PyObject* concat(PyObject*, PyObject* const* a, Py_ssize_t n) {
             if (i && out[f].defined()) Py_RETURN_NONE;
             continue;
           }
-          if (!THPVariable_Check(o.o)) Py_RETURN_NONE;
+          if (!plain(o.o)) Py_RETURN_NONE;
           const at::Tensor& x = THPVariable_Unpack(o.o);
           const int64_t w = width(f, tokens[i]);
           if (pass == 0) {
-            if (!x.is_cuda() || x.get_device() != c10::cuda::current_device() || x.scalar_type() != at::kByte || !x.is_contiguous() ||
+            if (x.get_device() != c10::cuda::current_device() || x.scalar_type() != at::kByte || !x.is_contiguous() ||
                 x.numel() != rows[f] * w || reinterpret_cast<uintptr_t>(x.data_ptr()) % 16 || (i && !out[f].defined()))
               Py_RETURN_NONE;
             if (i == 0)

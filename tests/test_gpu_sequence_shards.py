@@ -15,7 +15,7 @@ import torch
 
 from oracle import attention as A
 from paper_2609_37852_b200 import workloads
-from tests.util import rel_fro, to_np, worst_row_error
+from tests.util import followed_by_torch, rel_fro, to_np, worst_row_error
 
 pytestmark = pytest.mark.gpu
 
@@ -186,3 +186,12 @@ def test_concat_chunks_gives_the_bytes_of_torch_cat(lengths, d, row, col):
         assert (a is None) == (b is None)
         if a is not None:
             assert a.is_cuda and a.shape == b.shape and torch.equal(a.cpu(), b)
+
+
+def test_concat_chunks_is_seen_by_whatever_follows_torch_operations():
+    from paper_2609_37852_b200 import binding as B
+    from paper_2609_37852_b200 import sequence_parallel as SP
+    x, y = torch.randint(0, 256, (2, 2, 1, 2, 128, 64), dtype=torch.uint8, device="cuda")
+    f = lambda t: SP.concat_chunks([B.QTensor((1, 2, 128, 64), t[0]), B.QTensor((1, 2, 128, 64), t[1])]).row_codes
+    for how, got in followed_by_torch(f, x, y):
+        assert torch.equal(got, torch.cat([y[0], y[1]], dim=2)), how
