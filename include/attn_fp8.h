@@ -269,9 +269,12 @@ attn_status_t attn_fp8_bwd(const attn_params_t* p, attn_qtensor_t q, attn_qtenso
  *                      reads q.row_*, k.row_*, k.col_*, v.row_*, dO.row_*, lse, delta
  *   attn_fp8_bwd_dkdv  the key-major pass: dK and dV;
  *                      reads q.row_*, q.col_*, k.row_*, v.row_*, dO.row_*, dO.col_*, lse, delta
- * attn_fp8_bwd produces exactly their outputs with one call: it launches the key-major kernel first
+ * attn_fp8_bwd produces exactly their outputs (the same bits) with one call: it launches the key-major kernel first
  * and the query-major kernel behind it (the two are independent; the second starts on the SMs the
- * first one's last wave leaves idle), and both have completed when the stream reaches what follows. */
+ * first one's last wave leaves idle), and both have completed when the stream reaches what follows.
+ * Every output is bitwise reproducible.  dQ of a (sequence, head) does not depend on what else the call holds; dK and dV
+ * do in the last place: with few heads several CTAs share the queries of a key tile and add their FP32 sums in rank order,
+ * and how many they are follows from batch, head counts, lengths and the number of SMs.          */
 attn_status_t attn_fp8_bwd_dq(const attn_params_t* p, attn_qtensor_t q, attn_qtensor_t k, attn_qtensor_t v,
                               attn_qtensor_t dO, const float* lse, const float* delta, void* dq_bf16,
                               float* diag_rowsum_ds, float* diag_rowsum_abs_ds,

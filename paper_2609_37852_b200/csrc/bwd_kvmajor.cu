@@ -863,17 +863,20 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
 }
 
 // CTAs per key tile.  One CTA per key tile is the least work; but the first key tile's CTA walks G * N / 128 query tiles,
-// and with few heads it alone takes longer than an SM's share of everything the call does (`passes` key-major passes, and
-// the dQ kernel behind them, about three quarters of a pass, where there is one).  Then a cluster of two or four CTAs
+// and with few heads it alone takes longer than an SM's share of everything a gradient call does (`passes` key-major passes
+// and the dQ kernel behind them, about three quarters of a pass).  Then a cluster of two or four CTAs
 // shares the list, which costs a set-up and an exchange of the accumulators (about 8 us): taken where it saves more than
-// 12 query tiles (18 us) and a sixteenth of the share.  16 heads on 4 KV heads, 4096 tokens: dK / dV 204 -> 112 us, gradient call 211 -> 190 us (128 CTAs,
-// the longest 128 tiles, 57 on average); 2 x 16 on 4 heads, 1000 tokens without a mask: dK / dV 59 -> 39 us, but the gradient
-// call 64 -> 68 us, since the dQ kernel fills the idle SMs either way.
-int split_of(const AttnShape& s, int sms, int passes, bool dq_follows) {
+// 12 query tiles (18 us) and a sixteenth of the share.  Calls one after the other, with one CTA per key tile and by the rule:
+// 16 heads on 4 KV heads, 4096 tokens, two CTAs, dK / dV 194 -> 101 us, gradient call 199 -> 170 us; 8 on 2 heads, 2048
+// tokens, four CTAs, 99 -> 35 and 104 -> 38 us.  Left alone: 2 x 16 on 4 heads, 1000 tokens without a mask, where two CTAs
+// take dK / dV from 54 to 34 us but the call from 64 to 68 us, since the dQ kernel fills the idle SMs either way.
+// The dQ kernel counts whether it follows or not: the same sums in the same order with and without it, so that
+// attn_fp8_bwd and attn_fp8_bwd_dkdv give the same bits.
+int split_of(const AttnShape& s, int sms, int passes) {
   const long long tiles = s.N / kTile, keys = s.Nk / kTile, G = s.Hq / s.Hkv;
   // (query tile, key tile) pairs of a head: the first key tiles are seen by all query tiles, the last ones by fewer and fewer
   const long long per_head = s.causal ? tiles * (keys - tiles) + tiles * (tiles + 1) / 2 : tiles * keys;
-  const long long longest = G * tiles, share = per_head * s.Hq * s.B * (4 * passes + (dq_follows ? 3 : 0)) / (4LL * sms);
+  const long long longest = G * tiles, share = per_head * s.Hq * s.B * (4 * passes + 3) / (4LL * sms);
   int split = 1;
   while (split < 4) {
     const long long next = longest / (2 * split) > share ? longest / (2 * split) : share;
@@ -957,7 +960,7 @@ attn_status_t launch_bwd_dkdv(const AttnShape& s, attn_qtensor_t q, attn_qtensor
   const attn_status_t found = current_device(&dev, &sms);
   if (found != ATTN_OK) return found;
   const int passes = cq < 2 * s.eb || cv < 2 * s.eb ? 1 : (s.eb == 1 ? 2 : 3);    // (256,256) takes more than one
-  const int split = split_of(s, sms, passes, /*dq_follows=*/clear_tickets);
+  const int split = split_of(s, sms, passes);
   if (s.eb == 1 && s.ebv == 2) {                     // protected dP: BF16 row copies of V and dO
     if (cq == 1 && cv == 1)
       return launch_kvmajor_t<KvCfg<1, 1, 1, kBoth, 2>>(s, q, k, v, dO, lse, delta, dk, dv, status, stream, split, false, clear_tickets);

@@ -349,6 +349,27 @@ def test_key_tiles_shared_by_a_cluster(name, kw, bf16):
         assert worst_row_error(to_np(a), to_np(b[:1])) <= 4e-3
 
 
+@pytest.mark.parametrize("name,kw", [
+    ("gqa4k", dict(batch=2, heads_q=16, heads_kv=4, seqlen=1024, causal=False)),
+    ("gqa4k", dict(batch=1, heads_q=1, heads_kv=1, seqlen=7040)),             # clusters
+    ("gqa8k_d256", dict(heads_q=8, heads_kv=2, seqlen=2048)),                 # two key-major passes, clusters
+])
+def test_one_call_gives_the_bits_of_the_two_halves(name, kw):
+    """attn_fp8_bwd against attn_fp8_bwd_dq and attn_fp8_bwd_dkdv, at sizes where an SM's share of the work with and
+    without dQ lies on either side of the rule for sharing a key tile."""
+    from paper_2609_37852_b200 import binding
+    w = workloads.WORKLOADS[name].scaled(**kw)
+    q, k, v, dO = (binding.attn_fp8_quantize(x.cuda()) for x in workloads.make_inputs(w))
+    params = binding.AttnParams(w.batch, w.seqlen, w.heads_q, w.heads_kv, w.head_dim_qk, w.head_dim_v, w.causal, w.softmax_scale)
+    _, lse, ws = binding.attn_fp8_fwd(params, q, k, v)
+    delta, _ = binding.attn_fp8_bwd_delta(params, q, k, v, dO, lse, workspace=ws)
+    dq, dk, dv, _, _, _ = binding.attn_fp8_bwd(params, q, k, v, dO, lse, delta, workspace=ws)
+    dq2, _, _, _ = binding.attn_fp8_bwd_dq(params, q, k, v, dO, lse, delta, workspace=ws)
+    dk2, dv2, _ = binding.attn_fp8_bwd_dkdv(params, q, k, v, dO, lse, delta, workspace=ws)
+    binding.attn_fp8_read_status(ws)
+    assert torch.equal(dq, dq2) and torch.equal(dk, dk2) and torch.equal(dv, dv2)
+
+
 @pytest.mark.parametrize("dv,heads,seqlen", [(64, 1, 128), (64, 3, 384), (128, 2, 256), (256, 1, 128)])
 def test_stale_delta_every_head_dim(dv, heads, seqlen):
     """delta = rowsum(dO o O) with 8, 16 and 32 lanes per row; FP32 sum of dv products: 2^-24 dv of the sum of magnitudes."""
