@@ -386,7 +386,8 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
     if (elect_one()) {
       const uint64_t desc_k = make_desc_sw128(smem_u32(sm.k[0]));
       bool ok = mbar_wait(&sm.kv_full, 0, abort_flag);
-      if (ok && kFp8) {
+      // (a CTA of a cluster may have no query tile: no commit would follow its copies)
+      if (ok && kFp8 && (!kShared || n_sub > 0)) {
         tc_fence_after_sync();
         sf_copy_tiles<kCq, true>(tmem + kColSFK, sm.sf_k);
       }
@@ -428,7 +429,7 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
     // ------------------------------------------------------------------ dP^T issuer + LSE preparation
     const uint64_t desc_v = make_desc_sw128(smem_u32(sm.v[0]));
     bool ok = __all_sync(0xffffffffu, mbar_wait(&sm.kv_full, 0, abort_flag));   // (one answer for the warp: elect_one needs it whole)
-    if (ok && kFp8v && kHasDk) {
+    if (ok && kFp8v && kHasDk && (!kShared || n_sub > 0)) {
       tc_fence_after_sync();
       if (elect_one()) sf_copy_tiles<kCv, true>(tmem + kColSFV, sm.sf_v);
     }

@@ -313,6 +313,7 @@ def test_bench_residual_statistics_match_the_oracle_helpers():
     ("gqa4k", dict(batch=1, heads_q=4, heads_kv=1, seqlen=3200), False),      # causal: the last key tile has a single query tile per head
     ("tiny", dict(seqlen=2560, heads_q=1, heads_kv=1), False),                # one head, no mask, d = 64, lists of 20 tiles
     ("gqa4k", dict(batch=1, heads_q=1, heads_kv=1, seqlen=4224), False),      # one head: CTAs of the last key tiles have no tile at all
+    ("gqa4k", dict(batch=1, heads_q=2, heads_kv=1, seqlen=4608), False),      # four CTAs, of which two have no tile of the last keys
     ("mla8k", dict(heads_q=2, heads_kv=1, seqlen=2304), False),
     ("gqa8k_d256", dict(heads_q=4, heads_kv=1, seqlen=2048), False),          # two passes
     ("gqa4k", dict(batch=1, heads_q=4, heads_kv=1, seqlen=2048), True),
