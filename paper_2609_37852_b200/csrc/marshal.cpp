@@ -41,19 +41,28 @@ struct Attr {
 };
 
 int64_t integer(PyObject* o) {
-  long long v;
-  if (PyLong_Check(o)) {
-    v = PyLong_AsLongLong(o);
-  } else {
-    Attr n(PyNumber_Long(o));
-    v = PyLong_AsLongLong(n.o);
-  }
+  const long long v = PyLong_AsLongLong(o);
   if (v == -1 && PyErr_Occurred()) throw Failed{};
   return v;
 }
+// A field of a struct, as ctypes stores it: by __index__ (a float is refused, not truncated), the low 32 bits.
+int32_t int32(PyObject* o) {
+  const unsigned long v = PyLong_AsUnsignedLongMask(o);
+  if (v == static_cast<unsigned long>(-1) && PyErr_Occurred()) throw Failed{};
+  return static_cast<int32_t>(v);
+}
 int32_t int_field(PyObject* of, PyObject* name) {
   Attr a(of, name);
-  return static_cast<int32_t>(integer(a.o));
+  return int32(a.o);
+}
+// what int() and float() make of a value
+int32_t as_int(PyObject* o) {
+  Attr n(PyNumber_Long(o));
+  return int32(n.o);
+}
+float as_float(PyObject* o) {
+  Attr n(PyNumber_Float(o));
+  return static_cast<float>(PyFloat_AS_DOUBLE(n.o));
 }
 
 // Device pointer of a tensor (null for None).
@@ -93,11 +102,9 @@ attn_params_t parameters(PyObject* o) {
   p.heads_kv = int_field(o, names.heads_kv);
   p.head_dim_qk = int_field(o, names.head_dim_qk);
   p.head_dim_v = int_field(o, names.head_dim_v);
-  p.causal = int_field(o, names.causal);
-  Attr scale(o, names.softmax_scale);
-  const double s = PyFloat_AsDouble(scale.o);
-  if (s == -1.0 && PyErr_Occurred()) throw Failed{};
-  p.softmax_scale = static_cast<float>(s);
+  Attr causal(o, names.causal), scale(o, names.softmax_scale);
+  p.causal = as_int(causal.o);
+  p.softmax_scale = as_float(scale.o);
   p.precision = int_field(o, names.precision);
   p.delta_mode = int_field(o, names.delta_mode);
   p.seqlen_k = int_field(o, names.seqlen_k);
@@ -136,7 +143,12 @@ void check_shape(PyObject* qtensor, const attn_quantize_job_t& j, const char* me
   Attr t(PySequence_Tuple(shape.o));
   const int32_t want[4] = {j.B, j.H, j.N, j.d};
   bool same = PyTuple_GET_SIZE(t.o) == 4;
-  for (int i = 0; same && i < 4; ++i) same = integer(PyTuple_GET_ITEM(t.o, i)) == want[i];
+  for (int i = 0; same && i < 4; ++i) {
+    Attr n(PyLong_FromLong(want[i]));
+    const int equal = PyObject_RichCompareBool(PyTuple_GET_ITEM(t.o, i), n.o, Py_EQ);
+    if (equal < 0) throw Failed{};
+    same = equal;
+  }
   if (!same) fail(PyExc_ValueError, message);
 }
 
@@ -298,13 +310,12 @@ PyObject* quantize_fused(PyObject*, PyObject* const* a, Py_ssize_t n) {
         fail(PyExc_ValueError, "rotary tables must be contiguous float32 [N, d/2]");
     }
     const float *cos = static_cast<float*>(pointer(a[1])), *sin = static_cast<float*>(pointer(a[2]));
-    const double scale = PyFloat_AsDouble(a[3]);
-    if (scale == -1.0 && PyErr_Occurred()) throw Failed{};
+    const float scale = as_float(a[3]);
     float* mean = static_cast<float*>(pointer(a[4]));
     const attn_qtensor_t out = operand(a[5]);
     void* st = stream_of(a[6]);
     return status_of([&] {
-      return attn_fp8_quantize_fused(j.src, j.src_dtype, j.B, j.H, j.N, j.d, cos, sin, static_cast<float>(scale), mean, out, st);
+      return attn_fp8_quantize_fused(j.src, j.src_dtype, j.B, j.H, j.N, j.d, cos, sin, scale, mean, out, st);
     });
   });
 }

@@ -117,3 +117,25 @@ def test_batched_quantiser_and_workspace_validation_without_a_gpu(lib_path):
     import torch
     if not torch.cuda.is_available():
         assert lib.attn_fp8_read_status(None, None) == 6
+
+
+@pytest.mark.parametrize("field,value", [
+    ("batch", 2.0), ("batch", "2"), ("batch", np.int64(2)), ("batch", np.float32(2)), ("batch", 2 ** 32 + 2), ("batch", 2 ** 70),
+    ("seqlen", 100.5), ("seqlen", True), ("heads_kv", np.uint8(3)), ("precision", 7.0), ("keys_valid", None), ("q_start", -128),
+    ("causal", 1.0), ("causal", "1"), ("causal", "x"), ("causal", np.bool_(True)), ("causal", 2), ("causal", None),
+    ("softmax_scale", "0.5"), ("softmax_scale", np.float16(0.5)), ("softmax_scale", 1), ("softmax_scale", None), ("softmax_scale", 1e300),
+])
+def test_parameters_are_taken_as_the_c_struct_takes_them(lib_path, field, value):
+    """The marshalled call and the ctypes struct refuse the same values, and read the others alike."""
+    from paper_2609_37852_b200 import binding
+    p = binding.AttnParams(1, 256, 4, 2, 128, 128, True, 0.1)
+    setattr(p, field, value)
+    none, stream = binding.QTensor(shape=()), type("Stream", (), {"cuda_stream": 0})
+
+    def outcome(call):
+        try:
+            return call(), binding.attn_fp8_last_error()
+        except (TypeError, ValueError, OverflowError) as e:
+            return type(e), None
+    want = outcome(lambda: binding._lib.attn_fp8_fwd(ctypes.byref(p.c_struct()), *[none.c_struct()] * 3, None, None, None, 0, None))
+    assert outcome(lambda: binding._marshal.fwd(p, none, none, none, None, None, None, stream)) == want
