@@ -149,8 +149,8 @@ size_t attn_fp8_scale_bytes(int64_t B, int64_t H, int64_t rows, int64_t cols);
  *              orientation must both be given); all 16-byte aligned
  *   N % 128 == 0, d % 32 == 0, 32 <= d <= 256.
  * Non-finite inputs do not trap: NaN encodes as 0x7F, +-Inf saturates to +-448.
- * The first call on each device looks up the address of the library's built-in scratch (a
- * one-time runtime query): make that first call outside of any stream capture.                */
+ * The first call in a context looks up the address of the library's built-in scratch (a
+ * runtime query): make that first call outside of any stream capture.                          */
 attn_status_t attn_fp8_quantize(const void* src, int32_t src_dtype, int32_t B, int32_t H, int32_t N,
                                 int32_t d, attn_qtensor_t out, void* stream);
 
@@ -324,10 +324,9 @@ attn_status_t attn_fp8_bwd_dq_rowprobe(const attn_params_t* p, attn_qtensor_t q,
  *
  *   - Problems whose scratch need (attn_fp8_workspace_bytes(p, ATTN_WS_FWD)) exceeds 4096 bytes are
  *     rejected with ATTN_ERR_WORKSPACE and a message naming both sizes.
- *   - The first call on each device looks up the array's device address (a one-time runtime query
- *     made with that device current); make that first call outside of any stream capture.  The
- *     address is cached per device ordinal for the life of the process: it does not survive a
- *     cudaDeviceReset of that device (do not reset a device between calls of this library).
+ *   - The first call in a context looks up the array's device address (a runtime query made with
+ *     that context current; repeated where calls on a device alternate between contexts); make that
+ *     first call outside of any stream capture.
  *   - All calls on a device share the one array, and it keeps what earlier calls left; its
  *     status word is only ever set by a kernel that gave up, so nothing has to be cleared between
  *     calls and overlapping calls (different streams) do not disturb one another.

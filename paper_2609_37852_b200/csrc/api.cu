@@ -23,14 +23,22 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
+static void* driver_function(const char* name) {
+  void* p = nullptr;
+  cudaDriverEntryPointQueryResult q;
+  return cudaGetDriverEntryPoint(name, &p, cudaEnableDefault, &q) == cudaSuccess ? p : nullptr;
+}
+
 static EncodeTiledFn get_encode_fn() {
-  static EncodeTiledFn fn = []() -> EncodeTiledFn {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) != cudaSuccess) return nullptr;
-    return reinterpret_cast<EncodeTiledFn>(p);
-  }();
+  static EncodeTiledFn fn = reinterpret_cast<EncodeTiledFn>(driver_function("cuTensorMapEncodeTiled"));
   return fn;
+}
+
+uint64_t context_id() {
+  typedef CUresult (*CtxGetIdFn)(CUcontext, unsigned long long*);
+  static CtxGetIdFn fn = reinterpret_cast<CtxGetIdFn>(driver_function("cuCtxGetId"));
+  unsigned long long id = 0;
+  return fn && fn(nullptr, &id) == CUDA_SUCCESS ? id : 0;      // nullptr: the current context
 }
 
 attn_status_t encode_tmap_u8_sw128(CUtensorMap* out, const void* base, uint64_t row_bytes, uint64_t rows,
@@ -51,18 +59,17 @@ attn_status_t encode_tmap_u8_sw128(CUtensorMap* out, const void* base, uint64_t 
 static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
 attn_status_t current_device(int* dev, int* sms) {
-  constexpr int kKept = 64;
-  static std::atomic<uint32_t> kept[kKept];           // major << 16 | SM count; 0: not asked yet
+  static std::atomic<uint32_t> kept[kMaxDevices];     // major << 16 | SM count; 0: not asked yet
   cudaError_t e = cudaGetDevice(dev);
   if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "cudaGetDevice: %s", cudaGetErrorString(e));
-  uint32_t info = *dev < kKept ? kept[*dev].load(std::memory_order_relaxed) : 0;
+  uint32_t info = *dev < kMaxDevices ? kept[*dev].load(std::memory_order_relaxed) : 0;
   if (!info) {
     int major = 0, n = 0;
     e = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, *dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, *dev);
     if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "cudaDeviceGetAttribute: %s", cudaGetErrorString(e));
     info = static_cast<uint32_t>(major) << 16 | static_cast<uint32_t>(n);
-    if (*dev < kKept) kept[*dev].store(info, std::memory_order_relaxed);
+    if (*dev < kMaxDevices) kept[*dev].store(info, std::memory_order_relaxed);
   }
   if (info >> 16 != 10) return fail(ATTN_ERR_ARCH, "device compute capability %d.x is not 10.x (sm_100a)", static_cast<int>(info >> 16));
   *sms = static_cast<int>(info & 0xFFFF);
@@ -483,8 +490,8 @@ namespace attnfp8 {
 constexpr size_t kBuiltinScratchBytes = 4096;
 static __device__ __align__(256) unsigned char g_builtin_scratch[kBuiltinScratchBytes];
 
-constexpr int kMaxDevices = 64;
-static void* g_builtin_scratch_addr[kMaxDevices];   // device address of the array, per device ordinal
+// The address of the array per device ordinal, and the context in which it holds.
+static struct { uint64_t context; void* address; } g_builtin_scratch_at[kMaxDevices];
 static std::mutex g_builtin_scratch_mutex;
 
 static attn_status_t builtin_scratch_for_current_device(void** out) {
@@ -492,15 +499,18 @@ static attn_status_t builtin_scratch_for_current_device(void** out) {
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "cudaGetDevice: %s", cudaGetErrorString(e));
   if (dev < 0 || dev >= kMaxDevices) return fail(ATTN_ERR_UNSUPPORTED, "device ordinal %d is outside 0..%d", dev, kMaxDevices - 1);
+  const uint64_t id = context_id();
   std::lock_guard<std::mutex> lock(g_builtin_scratch_mutex);
-  if (!g_builtin_scratch_addr[dev]) {
+  auto& at = g_builtin_scratch_at[dev];
+  if (!id || at.context != id) {
     void* ptr = nullptr;
     e = cudaGetSymbolAddress(&ptr, g_builtin_scratch);
     if (e != cudaSuccess || !ptr)
       return fail(ATTN_ERR_CUDA, "cudaGetSymbolAddress(built-in scratch) on device %d: %s", dev, cudaGetErrorString(e));
-    g_builtin_scratch_addr[dev] = ptr;
+    at.context = context_id();                        // (the query made the context where the thread had none)
+    at.address = ptr;
   }
-  *out = g_builtin_scratch_addr[dev];
+  *out = at.address;
   return ATTN_OK;
 }
 

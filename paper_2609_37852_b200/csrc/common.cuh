@@ -17,18 +17,24 @@ attn_status_t fail(attn_status_t code, const char* fmt, ...);
 // says of a device is kept per ordinal: asked for on every call it was a quarter of a small call's host time.
 attn_status_t current_device(int* dev, int* sms);
 
-// Lets `kernel` ask for up to `bytes` of dynamic shared memory: one runtime call per kernel and device.
+// The id of the calling thread's context, never used again in the life of the process (a context that follows a reset has
+// another); 0 where the thread has none yet.
+uint64_t context_id();
+constexpr int kMaxDevices = 64;
+
+// Lets `kernel` ask for up to `bytes` of dynamic shared memory.  The limit belongs to a context: it is raised again where a
+// device's context is not the one of the call before, and one runtime call per launch is saved otherwise.
 template <auto kernel>
 attn_status_t allow_smem(size_t bytes, const char* who) {
-  static std::atomic<uint64_t> done{0};               // bit per device ordinal
+  static std::atomic<uint64_t> raised[kMaxDevices];   // per device ordinal: the context in which the limit is raised
   int dev = 0, sms = 0;
   const attn_status_t st = current_device(&dev, &sms);
   if (st != ATTN_OK) return st;
-  const uint64_t bit = dev < 64 ? uint64_t{1} << dev : 0;
-  if (done.load(std::memory_order_acquire) & bit) return ATTN_OK;
+  const uint64_t id = context_id();
+  if (id && dev < kMaxDevices && raised[dev].load(std::memory_order_acquire) == id) return ATTN_OK;
   const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
   if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "%s: cudaFuncSetAttribute: %s", who, cudaGetErrorString(e));
-  done.fetch_or(bit, std::memory_order_release);
+  if (id && dev < kMaxDevices) raised[dev].store(id, std::memory_order_release);
   return ATTN_OK;
 }
 
