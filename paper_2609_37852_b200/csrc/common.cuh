@@ -33,7 +33,10 @@ attn_status_t allow_smem(size_t bytes, const char* who) {
   const uint64_t id = context_id();
   if (id && dev < kMaxDevices && raised[dev].load(std::memory_order_acquire) == id) return ATTN_OK;
   const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
-  if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "%s: cudaFuncSetAttribute: %s", who, cudaGetErrorString(e));
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return fail(ATTN_ERR_CUDA, "%s: cudaFuncSetAttribute: %s", who, cudaGetErrorString(e));
+  }
   if (id && dev < kMaxDevices) raised[dev].store(id, std::memory_order_release);
   return ATTN_OK;
 }
@@ -59,7 +62,9 @@ cudaError_t launch_kernel(void (*kernel)(Params...), dim3 grid, int threads, siz
     attr[cfg.numAttrs].val.clusterDim.x = cluster; attr[cfg.numAttrs].val.clusterDim.y = 1; attr[cfg.numAttrs++].val.clusterDim.z = 1;
   }
   cfg.attrs = attr;
-  return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+  if (e != cudaSuccess) cudaGetLastError();            // reported here, and not again by the next call that asks
+  return e;
 }
 template <class... Params, class... Args>
 cudaError_t launch_overlapped(void (*kernel)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t stream, int cluster,

@@ -373,3 +373,17 @@ def test_measurement_aids():
     assert ms > 0 and nbytes == 4 * (8 * 9 // 2) * 2 * 64 * 128 * 4
     want = (torch.arange(1024, device="cuda") // 128 + 1).float()          # key tiles a causal row sees
     assert torch.equal(dq, want[None, None, :, None].expand_as(dq))
+
+
+def test_a_refused_launch_is_reported_once():
+    """The error of a launch that the runtime refuses (a grid of 65,536 rows of blocks) is not left for a later call."""
+    from paper_2609_37852_b200 import binding as B
+    ws = B.new_workspace(256, "cuda")
+    x = torch.zeros((65536, 1, 128, 32), dtype=torch.bfloat16, device="cuda")
+    with pytest.raises(B.AttnFp8Error) as e:
+        B.attn_fp8_prepare_bf16(x)
+    assert e.value.status == 6
+    B.attn_fp8_selftest_timeout(ws)                    # asks for the last error after its launch
+    with pytest.raises(B.AttnFp8Error) as e:
+        B.attn_fp8_read_status(ws)
+    assert e.value.status == 7
