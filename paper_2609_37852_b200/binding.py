@@ -15,6 +15,8 @@ from typing import Optional
 import numpy as np
 import torch
 
+from . import build as _build
+
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libattnfp8.so")
 
@@ -23,6 +25,10 @@ if not os.path.exists(LIB_PATH):
         f"{LIB_PATH} is missing: build the CUDA library first (python -m paper_2609_37852_b200.build); "
         "this package has no CPU or eager fallback")
 _lib = ctypes.CDLL(LIB_PATH)
+if _build.marshal_built_for() != _build.marshal_key():
+    raise ImportError(
+        f"{_build.MARSHAL} is built for '{_build.marshal_built_for()}' and this is '{_build.marshal_key()}': "
+        "build it again (python -m paper_2609_37852_b200.build)")
 from . import _marshal  # noqa: E402  (links against the library loaded above; built with it)
 
 ATTN_OK = 0

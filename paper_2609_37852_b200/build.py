@@ -76,10 +76,30 @@ def build(force=False, verbose=False):
     return OUT
 
 
+def marshal_key():
+    """The interpreter and torch build that a compiled marshalling module works with."""
+    import sysconfig
+    import torch
+    return "torch %s, C++11 ABI %d, %s" % (torch.__version__, int(torch.compiled_with_cxx11_abi()), sysconfig.get_config_var("EXT_SUFFIX"))
+
+
+def marshal_built_for(path=None):
+    """The key that the module at `path` was compiled for; None when there is no such file or it names none."""
+    mark = b"marshal built for: "
+    try:
+        with open(path or MARSHAL, "rb") as f:
+            data = f.read()
+    except OSError:
+        return None
+    at = data.find(mark)
+    return data[at + len(mark):data.index(b"\0", at)].decode() if at >= 0 else None
+
+
 def build_marshal(force=False, verbose=False):
     """Compile csrc/marshal.cpp into an extension module linked against the library and torch's own."""
     src = os.path.join(CSRC, "marshal.cpp")
-    if not force and not _stale(MARSHAL, [src, os.path.join(os.path.dirname(HERE), "include", "attn_fp8.h")]):
+    key = marshal_key()
+    if not force and marshal_built_for() == key and not _stale(MARSHAL, [src, os.path.join(os.path.dirname(HERE), "include", "attn_fp8.h")]):
         return
     import sysconfig
     import torch
@@ -88,7 +108,7 @@ def build_marshal(force=False, verbose=False):
                                            os.path.join(os.path.dirname(os.path.dirname(_nvcc())), "include")]
     lib = os.path.join(os.path.dirname(torch.__file__), "lib")
     cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
-           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch.compiled_with_cxx11_abi())]
+           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch.compiled_with_cxx11_abi()), '-DMARSHAL_BUILT_FOR="%s"' % key]
     for d in inc:
         cmd += ["-isystem", d]
     cmd += [src, "-o", MARSHAL, "-L" + HERE, "-lattnfp8", "-L" + lib, "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python",

@@ -15,6 +15,9 @@
 
 #include "../../include/attn_fp8.h"
 
+// What this file was compiled for, found in the module's bytes by build.py and binding.py before they load it.
+extern "C" __attribute__((used, visibility("default"))) const char attn_marshal_built_for[] = "marshal built for: " MARSHAL_BUILT_FOR;
+
 namespace {
 
 struct Names {

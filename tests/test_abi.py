@@ -2,6 +2,8 @@
 import ctypes
 import os
 import re
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -139,3 +141,20 @@ def test_parameters_are_taken_as_the_c_struct_takes_them(lib_path, field, value)
             return type(e), None
     want = outcome(lambda: binding._lib.attn_fp8_fwd(ctypes.byref(p.c_struct()), *[none.c_struct()] * 3, None, None, None, 0, None))
     assert outcome(lambda: binding._marshal.fwd(p, none, none, none, None, None, None, stream)) == want
+
+
+def test_a_module_of_another_torch_is_built_again_and_not_loaded(lib_path, monkeypatch):
+    """The marshalling module holds torch's C++ interface: one compiled for another build is stale, and refused by name."""
+    from paper_2609_37852_b200 import build
+    assert build.marshal_built_for() == build.marshal_key()
+    ran = []
+    monkeypatch.setattr(build.subprocess, "run", lambda cmd, **kw: ran.append(cmd) or subprocess.CompletedProcess(cmd, 0, "", ""))
+    build.build_marshal()
+    assert not ran
+    monkeypatch.setattr("torch.__version__", "0.0")
+    build.build_marshal()
+    assert len(ran) == 1
+    r = subprocess.Popen([sys.executable, "-c", "import torch; torch.__version__ = '0.0'; import paper_2609_37852_b200.binding"],
+                         cwd=ROOT, stderr=subprocess.PIPE, text=True)
+    err = r.communicate(timeout=300)[1]
+    assert r.returncode and "ImportError" in err and "built for" in err and "torch 0.0" in err
