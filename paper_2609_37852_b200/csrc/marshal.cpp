@@ -366,6 +366,7 @@ PyObject* pad_tokens(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const int64_t rows = integer(a[1]);
     if (!x.is_contiguous() || x.dim() != 4 || x.requires_grad() || x.numel() == 0 ||
         (x.size(3) * x.element_size()) % 16 || reinterpret_cast<uintptr_t>(x.data_ptr()) % 16 || x.size(0) * x.size(1) > INT32_MAX ||
+        rows > INT32_MAX || x.size(3) * x.element_size() / 16 * rows > INT32_MAX ||     // the kernel counts a slab's pieces in 32 bits
         x.get_device() != c10::cuda::current_device())
       Py_RETURN_NONE;
     at::Tensor out = at::empty({x.size(0), x.size(1), rows, x.size(3)}, x.options());

@@ -123,6 +123,27 @@ def test_pad_tokens_is_seen_by_whatever_follows_torch_operations():
     assert not B.pad_tokens(torch._efficientzerotensor(1, 2, 100, 64, device="cuda")).any()
 
 
+@pytest.mark.parametrize("n", [(1 << 31) - 100, (1 << 31) + 28, (1 << 32) + 1])
+def test_pad_tokens_leaves_slabs_beyond_32_bit_indices_to_torch(n, monkeypatch):
+    """A slab of 2^31 pieces of 16 bytes and more.  Nothing of it is allocated or read: the tensor only claims the size, and
+    the general path is stopped where it begins."""
+    from paper_2609_37852_b200 import binding as B
+    one = torch.zeros(16, dtype=torch.uint8, device="cuda")
+    claim = type("Claim", (), {"__cuda_array_interface__": dict(shape=(1, 1, n, 16), typestr="|u1", data=(one.data_ptr(), False),
+                                                                version=2, strides=None)})()
+    x = torch.as_tensor(claim, device="cuda")
+    assert x.is_contiguous() and x.shape[2] == n and x.data_ptr() == one.data_ptr()
+
+    class General(Exception):
+        pass
+
+    def zeros(*args, **kw):
+        raise General
+    monkeypatch.setattr(torch, "zeros", zeros)
+    with pytest.raises(General):
+        B.pad_tokens(x)
+
+
 def test_keys_valid_is_validated():
     from paper_2609_37852_b200 import binding as B
     w = workloads.WORKLOADS["gqa4k"].scaled(batch=1, heads_q=2, heads_kv=1, seqlen=256)
