@@ -191,9 +191,10 @@ __device__ __forceinline__ void quantize_tile(T* tile, int d_rt, const BatchJob&
   if (job.col_codes != nullptr) {
     if constexpr (sizeof(T) == 2) {
       // One pair of neighbouring channels x one block of 32 tokens per thread and step: 32-bit loads, packed maxima.
-      // A tile has 2 d such items: at head dims 64 and 192 they fill the CTA's threads half a time and one and a half
-      // times, so two lanes of a warp share an item there, 16 tokens each (four BF16 tensors of 8 x 12 heads x 1024 x 64: 28.7 -> 28.0 us).
-      constexpr int kShare = kD == 64 || kD == 192 ? 2 : 1, kTok = 32 / kShare;
+      // A tile has 2 d such items: at head dims up to 64 they fill at most half of the CTA's threads, so two lanes of a
+      // warp share an item there, 16 tokens each (four BF16 tensors of 8 x 12 heads x 1024 x 64: 28.7 -> 28.0 us; at head
+      // dim 192, where they fill the threads one and a half times, one of 2 x 16 x 4096 took 27.8 us shared, 27.2 not).
+      constexpr int kShare = kD == 32 || kD == 64 ? 2 : 1, kTok = 32 / kShare;
       const int pairs = d >> 1;
       for (int i = tid; i < pairs * 4 * kShare; i += kThreads) {
         const int item = kShare == 1 ? i : (i >> 5) * 16 + (i & 15), part = kShare == 1 ? 0 : (i >> 4) & 1;
@@ -269,12 +270,16 @@ __device__ __forceinline__ void quantize_tile(T* tile, int d_rt, const BatchJob&
   }
 }
 
-// kNarrow: every tensor has head dim 64.  A tile is then half as much work between the same barriers, and four CTAs per SM
-// (64 registers, at most 43 KB) cover each other's better than two: 28.0 -> 22.7 us on four BF16 tensors of 8 x 12 heads x
-// 1024 tokens, 24.6 -> 18.3 us on Q, dO of 2 x 16 and K, V of 2 x 4 heads x 4096.  A batch that also holds wider tensors
-// keeps two: their tiles need the registers.
-template <typename T, bool kProd, bool kNarrow>
-__global__ void __launch_bounds__(kThreads, kNarrow ? 4 : 2) quantize_batch_kernel(const __grid_constant__ BatchParams p) {
+// kOnly: the head dim that every tensor of the launch has, for the narrow ones (0: several, or a wide one).  A tile is then
+// less work between the same barriers, and four or three CTAs per SM (64 or 80 registers, at most 64 KB) cover each other's
+// better than two.  64: 28.0 -> 22.7 us on four BF16 tensors of 8 x 12 heads x 1024 tokens, 24.6 -> 18.3 us on Q, dO of
+// 2 x 16 and K, V of 2 x 4 heads x 4096.  32 and 96, one BF16 tensor of 2 x 16 x 4096, scaled: 13.5 -> 8.6 and 20.9 -> 16.2 us
+// (five CTAs at 32, 48 registers: 9.1).  A launch that also holds wider tensors keeps two: their tiles need the registers.
+template <int kOnly>
+constexpr int kCtas = kOnly == 0 ? 2 : kOnly == 32 ? 4 : kOnly == 64 ? 4 : 3;   // per SM
+
+template <typename T, bool kProd, int kOnly>
+__global__ void __launch_bounds__(kThreads, kCtas<kOnly>) quantize_batch_kernel(const __grid_constant__ BatchParams p) {
   extern __shared__ __align__(128) uint8_t smem[];
   const int tile_bytes_max = kTokens * p.d_max * static_cast<int>(sizeof(T));
   auto ring = [&](int slot) { return reinterpret_cast<T*>(smem + slot * tile_bytes_max); };
@@ -335,10 +340,11 @@ __global__ void __launch_bounds__(kThreads, kNarrow ? 4 : 2) quantize_batch_kern
     const bool landed = mbar_wait(&full[i % n_ring], (i / n_ring) & 1, abort_flag);
     if (__syncthreads_or(!landed)) break;        // all threads take the same way out
 
-    if constexpr (kNarrow) {
-      quantize_tile<T, 64, kProd>(tile, 64, job, p.prod, slab, tok0, s_row_sf, s_col_sf, s_col_codes, tid);
+    if constexpr (kOnly) {
+      quantize_tile<T, kOnly, kProd>(tile, kOnly, job, p.prod, slab, tok0, s_row_sf, s_col_sf, s_col_codes, tid);
     } else {
       switch (d) {                      // compile-time head dims: no integer division, constant strides
+                                        // (32 and 96 here too: 1 % of a step at head dim 128 that uses the producer, 338 -> 341 us)
         case 64:  quantize_tile<T, 64, kProd>(tile, d, job, p.prod, slab, tok0, s_row_sf, s_col_sf, s_col_codes, tid); break;
         case 128: quantize_tile<T, 128, kProd>(tile, d, job, p.prod, slab, tok0, s_row_sf, s_col_sf, s_col_codes, tid); break;
         case 192: quantize_tile<T, 192, kProd>(tile, d, job, p.prod, slab, tok0, s_row_sf, s_col_sf, s_col_codes, tid); break;
@@ -380,7 +386,7 @@ static size_t batch_smem_bytes(size_t elem, int d_max, int ring) {
          static_cast<size_t>(d_max) * kColPitch + 64;
 }
 
-template <typename T, bool kProd, bool kNarrow>
+template <typename T, bool kProd, int kOnly>
 attn_status_t launch_batch_n(BatchParams& p, cudaStream_t stream) {
   // two CTAs per SM come first (each covers the other's stalls), the deeper ring second: measured
   // at d = 192 one tile x two CTAs 0.078 ms against two tiles x one CTA 0.098 ms
@@ -388,26 +394,29 @@ attn_status_t launch_batch_n(BatchParams& p, cudaStream_t stream) {
   if (batch_smem_bytes(sizeof(T), p.d_max, kMaxRing) <= half_sm) p.ring = kMaxRing;
   else if (batch_smem_bytes(sizeof(T), p.d_max, 1) <= half_sm) p.ring = 1;
   else p.ring = batch_smem_bytes(sizeof(T), p.d_max, kMaxRing) <= whole_sm ? kMaxRing : 1;
-  if (kNarrow) p.ring = sizeof(T) == 2 ? kMaxRing : 1;
+  if (kOnly) p.ring = kCtas<kOnly> * (batch_smem_bytes(sizeof(T), p.d_max, kMaxRing) + 1024) <= whole_sm ? kMaxRing : 1;
   const size_t smem = batch_smem_bytes(sizeof(T), p.d_max, p.ring);
   int dev = 0, sms = 0;
   attn_status_t st = current_device(&dev, &sms);
-  if (st == ATTN_OK) st = allow_smem<quantize_batch_kernel<T, kProd, kNarrow>>(whole_sm, "quantize");
+  if (st == ATTN_OK) st = allow_smem<quantize_batch_kernel<T, kProd, kOnly>>(whole_sm, "quantize");
   if (st != ATTN_OK) return st;
   // the launch bounds let four or two CTAs fit by registers; shared memory decides between two and one
-  const int per_sm = kNarrow ? 4 : smem <= half_sm ? 2 : 1;
+  const int per_sm = kOnly ? kCtas<kOnly> : smem <= half_sm ? 2 : 1;
   const int resident = sms * per_sm;
   const int grid = p.total_tiles < resident ? p.total_tiles : resident;
-  const cudaError_t e = launch_overlapped(quantize_batch_kernel<T, kProd, kNarrow>, dim3(grid), kThreads, smem, stream, 1, p);
+  const cudaError_t e = launch_overlapped(quantize_batch_kernel<T, kProd, kOnly>, dim3(grid), kThreads, smem, stream, 1, p);
   if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "quantize: launch: %s", cudaGetErrorString(e));
   return ATTN_OK;
 }
 
 template <typename T, bool kProd>
 attn_status_t launch_batch_t(BatchParams& p, cudaStream_t stream) {
-  bool narrow = true;
-  for (int j = 0; j < p.n_jobs; ++j) narrow = narrow && p.job[j].d == 64;
-  return narrow ? launch_batch_n<T, kProd, true>(p, stream) : launch_batch_n<T, kProd, false>(p, stream);
+  bool one_dim = true;
+  for (int j = 0; j < p.n_jobs; ++j) one_dim = one_dim && p.job[j].d == p.d_max;
+  if (one_dim && p.d_max == 32) return launch_batch_n<T, kProd, 32>(p, stream);
+  if (one_dim && p.d_max == 64) return launch_batch_n<T, kProd, 64>(p, stream);
+  if (one_dim && p.d_max == 96) return launch_batch_n<T, kProd, 96>(p, stream);
+  return launch_batch_n<T, kProd, 0>(p, stream);
 }
 
 void fill_params(BatchParams& p, const attn_quantize_job_t* jobs, int n_jobs, int* status) {

@@ -189,3 +189,22 @@ def test_quantize_batch_of_head_dim_64_bit_exact(heads, wider, dtype):
         assert np.array_equal(B.unpack_scales(qt.row_scales, 1, H, N, d).cpu().numpy(), rs)
         assert np.array_equal(qt.col_codes.cpu().numpy(), np.swapaxes(cc, -1, -2))
         assert np.array_equal(B.unpack_scales(qt.col_scales, 1, H, d, N).cpu().numpy(), np.swapaxes(cs, -1, -2))
+
+
+@pytest.mark.parametrize("d,heads", [(32, 1), (32, 593), (96, 1), (96, 445)])
+def test_quantize_of_the_other_narrow_head_dims_bit_exact(d, heads):
+    # one tile; one more than four (head dim 32) or three (96) CTAs on each of 148 SMs; a mixed launch keeps two
+    from paper_2609_37852_b200 import binding as B
+    g = torch.Generator().manual_seed(heads + d)
+    xs = [torch.randn(1, heads, 128, d, generator=g), torch.randn(1, 2, 256, 160 - d, generator=g)]
+    for dtype in (torch.bfloat16, torch.float32):
+        for part in (xs[:1], xs):
+            outs, _ = B.attn_fp8_quantize_batch([x.to(dtype).cuda() for x in part])
+            for x, qt in zip(part, outs):
+                _, H, N, dd = x.shape
+                rc, rs = mxfp8.quantize(to_np(x.to(dtype)), axis=-1)
+                cc, cs = mxfp8.quantize(to_np(x.to(dtype)), axis=-2)
+                assert np.array_equal(qt.row_codes.cpu().numpy(), rc)
+                assert np.array_equal(B.unpack_scales(qt.row_scales, 1, H, N, dd).cpu().numpy(), rs)
+                assert np.array_equal(qt.col_codes.cpu().numpy(), np.swapaxes(cc, -1, -2))
+                assert np.array_equal(B.unpack_scales(qt.col_scales, 1, H, dd, N).cpu().numpy(), np.swapaxes(cs, -1, -2))
