@@ -921,20 +921,19 @@ attn_status_t launch_kvmajor_s(const AttnShape& s, attn_qtensor_t q, attn_qtenso
   p.tail_wait = behind ? 1 : 0;
   p.tickets = clear_tickets ? ticket_counter(status) : nullptr;
   const size_t smem = sizeof(KvSmem<C>) + 1024;
-  if ((st = allow_smem<kvmajor_kernel<C, kShared>>(smem, "bwd kv-major")) != ATTN_OK) return st;
+  int sms = 0;
+  if ((st = allow_smem<kvmajor_kernel<C, kShared>>(smem, "bwd kv-major", &sms)) != ATTN_OK) return st;
   p.split = split;
   // bytes of Q and dO per (sequence, KV head): the copies this pass reads, of the heads of its group
   const WorkOrder order = work_order(s.B * s.Hkv, 1, s.Nk / kTile,
                                      static_cast<size_t>(s.Hq / s.Hkv) * s.N * (s.dqk * eb * (C::kHasDk ? 2 : 1) +
-                                                                                s.dv * ((C::kHasDk ? ebv : 0) + (C::kHasDv ? eb : 0))), s.causal, false);
+                                                                                s.dv * ((C::kHasDk ? ebv : 0) + (C::kHasDv ? eb : 0))), s.causal, false, sms);
   p.slabs = order.heads; p.group = order.group;
   const dim3 grid = order.grid(split);
   // The first pass overlaps the kernel ahead like every other kernel only where its CTAs and those of the query-major
   // kernel fit on the GPU together (one head of 256 tokens: step 28 -> 23 us).  On larger problems its CTAs would settle
   // on whichever SMs the kernel ahead leaves first, and the kernels behind fill in worse: head dim 256, 8/2 heads, step
   // 1046 -> 1113 us; 2 x 16/4 heads of 1000 tokens 119 -> 127 us; gqa4k 603 -> 611 us.
-  int dev = 0, sms = 0;
-  if ((st = current_device(&dev, &sms)) != ATTN_OK) return st;
   const long long ctas = static_cast<long long>(s.B) * (s.Hkv * split * (s.Nk / kTile) + s.Hq * (s.N / kTile));
   const cudaError_t e = launch_kernel(kvmajor_kernel<C, kShared>, grid, kThreads, smem, stream, split, behind || ctas <= sms, p,
                                       tm_k, tm_v, tm_q, tm_dO, tm_qc, tm_dOc);

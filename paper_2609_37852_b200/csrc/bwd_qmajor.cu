@@ -808,18 +808,17 @@ attn_status_t launch_qmajor_t(const AttnShape& s, attn_qtensor_t q, attn_qtensor
   p.tail_wait = behind_dkdv ? 1 : 0;
   p.sched = ticket_counter(status);
   const size_t smem = sizeof(QmSmem<C>) + 1024;
-  if ((st = allow_smem<qmajor_kernel<C>>(smem, "bwd q-major")) != ATTN_OK) return st;
+  int sms = 0;
+  if ((st = allow_smem<qmajor_kernel<C>>(smem, "bwd q-major", &sms)) != ATTN_OK) return st;
   const int rq = (kDQ && !C::kWhole) ? (s.dqk + 127) / 128 : 1;
   // bytes of K and V per (sequence, KV head): the row copies, and for dQ the column copy of K
   p.order = work_order(s.B * s.Hkv, s.Hq / s.Hkv * rq, s.N / kTile,
-                       static_cast<size_t>(s.Nk) * (s.dqk * eb * (kDQ ? 2 : 1) + s.dv * ebv), s.causal, !C::kTicket);
+                       static_cast<size_t>(s.Nk) * (s.dqk * eb * (kDQ ? 2 : 1) + s.dv * ebv), s.causal, !C::kTicket, sms);
   const long long items = p.order.items();
   if (items > 0x7fffffffLL) return fail(ATTN_ERR_UNSUPPORTED, "bwd q-major: %lld work items exceed 2^31 - 1", items);
   dim3 grid = p.order.grid();
   if (C::kPersist) {
     // one CTA per SM (the kernel takes a whole SM's shared memory) walks the item list
-    int dev = 0, sms = 0;
-    if ((st = current_device(&dev, &sms)) != ATTN_OK) return st;
     grid = dim3(static_cast<unsigned>(items < sms ? items : sms), 1, 1);
   }
   // behind the key-major kernel, which reads what this one reads and writes other buffers, this grid takes the SMs

@@ -23,12 +23,13 @@ uint64_t context_id();
 constexpr int kMaxDevices = 64;
 
 // Lets `kernel` ask for up to `bytes` of dynamic shared memory.  The limit belongs to a context: it is raised again where a
-// device's context is not the one of the call before, and one runtime call per launch is saved otherwise.
+// device's context is not the one of the call before, and one runtime call per launch is saved otherwise.  Gives the
+// device's SM count as well.
 template <auto kernel>
-attn_status_t allow_smem(size_t bytes, const char* who) {
+attn_status_t allow_smem(size_t bytes, const char* who, int* sms) {
   static std::atomic<uint64_t> raised[kMaxDevices];   // per device ordinal: the context in which the limit is raised
-  int dev = 0, sms = 0;
-  const attn_status_t st = current_device(&dev, &sms);
+  int dev = 0;
+  const attn_status_t st = current_device(&dev, sms);
   if (st != ATTN_OK) return st;
   const uint64_t id = context_id();
   if (id && dev < kMaxDevices && raised[dev].load(std::memory_order_acquire) == id) return ATTN_OK;

@@ -473,8 +473,9 @@ attn_status_t launch_fwd_t(const AttnShape& s, attn_qtensor_t q, attn_qtensor_t 
   p.N = s.N; p.Nk = s.Nk; p.q0t = s.q0t; p.kv_lim = s.kv_lim; p.Hq = s.Hq; p.Hkv = s.Hkv; p.dqk = s.dqk; p.dv = s.dv; p.causal = s.causal;
   p.scale_log2 = s.scale * kLog2e;
   const size_t smem = sizeof(FwdSmem<C>) + 1024;
-  if ((st = allow_smem<fwd_kernel<C>>(smem, "fwd")) != ATTN_OK) return st;
-  p.order = work_order(s.B * s.Hkv, s.Hq / s.Hkv, s.N / kTile, static_cast<size_t>(s.Nk) * (s.dqk + s.dv) * eb, s.causal, false);
+  int sms = 0;
+  if ((st = allow_smem<fwd_kernel<C>>(smem, "fwd", &sms)) != ATTN_OK) return st;
+  p.order = work_order(s.B * s.Hkv, s.Hq / s.Hkv, s.N / kTile, static_cast<size_t>(s.Nk) * (s.dqk + s.dv) * eb, s.causal, false, sms);
   const cudaError_t e = launch_overlapped(fwd_kernel<C>, p.order.grid(), C::kThreads, smem, stream, 1, p, tm_q, tm_k, tm_v);
   if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "fwd: launch: %s", cudaGetErrorString(e));
   return ATTN_OK;

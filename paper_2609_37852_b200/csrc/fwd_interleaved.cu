@@ -635,13 +635,12 @@ attn_status_t launch_fwd_il_t(const AttnShape& s, attn_qtensor_t q, attn_qtensor
   p.N = s.N; p.Nk = s.Nk; p.q0t = s.q0t; p.kv_lim = s.kv_lim; p.Hq = s.Hq; p.Hkv = s.Hkv; p.dqk = s.dqk; p.dv = s.dv; p.causal = s.causal;
   p.scale_log2 = s.scale * kLog2e;
   const size_t smem = sizeof(IlSmem<C>) + 1024;
-  if ((st = allow_smem<fwd_il_kernel<C>>(smem, "fwd")) != ATTN_OK) return st;
-  p.order = work_order(s.B * s.Hkv, s.Hq / s.Hkv, s.N / kTile, static_cast<size_t>(s.Nk) * (s.dqk + s.dv), s.causal, true);
+  int sms = 0;
+  if ((st = allow_smem<fwd_il_kernel<C>>(smem, "fwd", &sms)) != ATTN_OK) return st;
+  p.order = work_order(s.B * s.Hkv, s.Hq / s.Hkv, s.N / kTile, static_cast<size_t>(s.Nk) * (s.dqk + s.dv), s.causal, true, sms);
   const long long items = p.order.items();
   if (items > 0x7fffffffLL) return fail(ATTN_ERR_UNSUPPORTED, "fwd: %lld work items exceed 2^31 - 1", items);
   // one CTA per SM (the kernel takes all of an SM's tensor memory) walks the item list
-  int dev = 0, sms = 0;
-  if ((st = current_device(&dev, &sms)) != ATTN_OK) return st;
   dim3 grid(static_cast<unsigned>(items < sms ? items : sms), 1, 1);
   const cudaError_t e = launch_overlapped(fwd_il_kernel<C>, grid, C::kThreads, smem, stream, 1, p, tm_q, tm_k, tm_v);
   if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "fwd: launch: %s", cudaGetErrorString(e));

@@ -1,6 +1,8 @@
 // Device-side pieces of the block quantiser shared by the quantiser kernel and by the attention
 // kernels that quantise probabilities and score gradients in registers.
 #pragma once
+#include <cuda_bf16.h>
+
 #include <cstdint>
 
 #include "sm100_ptx.cuh"
@@ -50,6 +52,15 @@ __device__ __forceinline__ uint32_t quantize_block32(const float* x, uint32_t* w
     words[i] = sm100::cvt_e4m3x4(a.x, a.y, b.x, b.y);
   }
   return byte;
+}
+
+// One rotated channel: x*cos -+ partner*sin with one rounding for the product and a fused
+// multiply-add, then BF16 (the order the header of attn_fp8_quantize_fused states).  The quantiser and the
+// token mean that it subtracts must agree on it bit for bit.
+__device__ __forceinline__ float rotate_bf16(float x, float partner, float c, float s, bool upper) {
+  const float t = __fmul_rn(partner, s);
+  const float r = __fmaf_rn(x, c, upper ? t : -t);
+  return __bfloat162float(__float2bfloat16_rn(r));
 }
 
 // offset of (row r of a 128-row tile, block k of 4) inside a 512-byte scale tile

@@ -67,13 +67,6 @@ __device__ __forceinline__ float2 unpack_bf16x2(uint32_t raw) {
   return make_float2(__uint_as_float(raw << 16), __uint_as_float(raw & 0xFFFF0000u));
 }
 
-// One rotated channel: x*cos -+ partner*sin with one rounding for the product and a fused
-// multiply-add, then BF16 (the order the header of attn_fp8_quantize_fused states).
-__device__ __forceinline__ float rotate_bf16(float x, float partner, float c, float s, bool upper) {
-  const float t = __fmul_rn(partner, s);
-  const float r = __fmaf_rn(x, c, upper ? t : -t);
-  return __bfloat162float(__float2bfloat16_rn(r));
-}
 // Eight consecutive values as FP32, and back (the values of a BF16 row are BF16-representable).
 __device__ __forceinline__ void load8(const __nv_bfloat16* p, float* x) {
   const uint4 raw = *reinterpret_cast<const uint4*>(p);
@@ -396,9 +389,8 @@ attn_status_t launch_batch_n(BatchParams& p, cudaStream_t stream) {
   else p.ring = batch_smem_bytes(sizeof(T), p.d_max, kMaxRing) <= whole_sm ? kMaxRing : 1;
   if (kOnly) p.ring = kCtas<kOnly> * (batch_smem_bytes(sizeof(T), p.d_max, kMaxRing) + 1024) <= whole_sm ? kMaxRing : 1;
   const size_t smem = batch_smem_bytes(sizeof(T), p.d_max, p.ring);
-  int dev = 0, sms = 0;
-  attn_status_t st = current_device(&dev, &sms);
-  if (st == ATTN_OK) st = allow_smem<quantize_batch_kernel<T, kProd, kOnly>>(whole_sm, "quantize");
+  int sms = 0;
+  const attn_status_t st = allow_smem<quantize_batch_kernel<T, kProd, kOnly>>(whole_sm, "quantize", &sms);
   if (st != ATTN_OK) return st;
   // the launch bounds let four or two CTAs fit by registers; shared memory decides between two and one
   const int per_sm = kOnly ? kCtas<kOnly> : smem <= half_sm ? 2 : 1;

@@ -12,9 +12,6 @@ namespace {
 
 namespace cg = cooperative_groups;
 
-__device__ __forceinline__ float to_f32(__nv_bfloat16 x) { return __bfloat162float(x); }
-__device__ __forceinline__ float to_f32(float x) { return x; }
-
 // Four consecutive values as FP32.
 __device__ __forceinline__ void load4(const __nv_bfloat16* p, float* x) {
   const uint2 raw = *reinterpret_cast<const uint2*>(p);
@@ -26,16 +23,9 @@ __device__ __forceinline__ void load4(const float* p, float* x) {
   x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w;
 }
 
-// One rotated channel, as the quantiser forms it (quantize_batch.cu).
-__device__ __forceinline__ float rotate_bf16(float x, float partner, float c, float s, bool upper) {
-  const float t = __fmul_rn(partner, s);
-  const float r = __fmaf_rn(x, c, upper ? t : -t);
-  return __bfloat162float(__float2bfloat16_rn(r));
-}
-
 // FP32 mean over tokens of the (rotated, BF16-rounded) tensor, per (batch, head, channel).  The
-// terms are BF16 values, so a double-precision sum is exact whatever its order, and the result is
-// the correctly rounded quotient: bitwise reproducible.
+// terms are BF16 values, so a double-precision sum is exact whatever its order while the largest
+// magnitude is at most 2^45 / N times the smallest, and the result is then the correctly rounded quotient; beyond that the order of the sum, which follows from the shape and the number of SMs, keeps it reproducible.
 //
 // Memory-bound work (the key tensor once, the tables from L2) on few slabs: a grouped-query layer has 4 to
 // 8, so a slab is shared by a cluster of up to eight CTAs, each summing a range of the tokens with vector
@@ -110,9 +100,11 @@ __global__ void __launch_bounds__(kMeanThreads, 2) token_mean_kernel(const T* sr
 template <typename T>
 attn_status_t launch_mean_t(const void* src, int slabs, int N, int d, const float* cos, const float* sin, float* mean,
                             cudaStream_t stream) {
-  // enough CTAs for two on every SM of the largest part, no fewer than 128 tokens each
-  int ranks = 1;
-  while (ranks < kMaxCluster && slabs * ranks < 296 && 2 * ranks <= N / 128) ranks *= 2;
+  // enough CTAs for two on every SM, no fewer than 128 tokens each
+  int dev = 0, sms = 0, ranks = 1;
+  const attn_status_t st = current_device(&dev, &sms);
+  if (st != ATTN_OK) return st;
+  while (ranks < kMaxCluster && slabs * ranks < 2 * sms && 2 * ranks <= N / 128) ranks *= 2;
   const int chunks = d / 8;
   const size_t smem = static_cast<size_t>(kMeanThreads / chunks) * d * sizeof(double);   // 32 KB
   const cudaError_t e = launch_overlapped(token_mean_kernel<T>, dim3(static_cast<unsigned>(slabs) * ranks), kMeanThreads, smem, stream,

@@ -65,13 +65,13 @@ struct WorkOrder {
 
 // `slabs` (sequence, KV head) pairs of `per_slab` heads, `bytes` of operands per pair that its items share.
 // A group takes 32 MB of them (16 and 64 MB are 0 to 2 % behind where they differ), and not less than four rounds of items
-// on 148 SMs under the causal mask, where a group ends in a tail of light tiles and the last one is the tail of the launch
+// on all SMs under the causal mask, where a group ends in a tail of light tiles and the last one is the tail of the launch
 // (BF16, 2 x 16 heads x 8192: step 2871 us with four rounds, 2925 with one); without it all items weigh the same and one
 // round will do (BF16 head dim 256, 8 heads x 12160: 12240 us with four, 11577 with one, 11500 with the batch slowest).  Not
 // for the rounds' sake more than 80 MB, beyond which L2 (126 MB) may not hold it.
-inline WorkOrder work_order(int slabs, int per_slab, int tiles, size_t bytes, bool causal, bool flip) {
+inline WorkOrder work_order(int slabs, int per_slab, int tiles, size_t bytes, bool causal, bool flip, int sms) {
   const long long fits = (32LL << 20) / bytes, most = (80LL << 20) / bytes, per = static_cast<long long>(per_slab) * tiles;
-  const long long enough = ((causal ? 4 : 1) * 148 + per - 1) / per;
+  const long long enough = ((causal ? 4 : 1) * static_cast<long long>(sms) + per - 1) / per;
   long long size = enough < most ? enough : most;
   if (size < fits) size = fits;
   if (size < 1) size = 1;
