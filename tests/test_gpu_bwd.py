@@ -5,7 +5,7 @@ import torch
 
 from oracle import attention as A
 from paper_2609_37852_b200 import workloads
-from tests.util import rel_fro, to_np, worst_row_error
+from tests.util import launched, rel_fro, to_np, worst_row_error
 
 pytestmark = pytest.mark.gpu
 
@@ -309,20 +309,26 @@ def test_bench_residual_statistics_match_the_oracle_helpers():
     assert np.isclose(stats["strict_ok_frac"], np.mean(r_pre <= 1e-5), rtol=0, atol=1e-12)
 
 
-@pytest.mark.parametrize("name,kw,bf16", [
-    ("gqa4k", dict(batch=1, heads_q=4, heads_kv=1, seqlen=3200), False),      # causal: the last key tile has a single query tile per head
-    ("tiny", dict(seqlen=2560, heads_q=1, heads_kv=1), False),                # one head, no mask, d = 64, lists of 20 tiles
-    ("gqa4k", dict(batch=1, heads_q=1, heads_kv=1, seqlen=4224), False),      # one head: CTAs of the last key tiles have no tile at all
-    ("gqa4k", dict(batch=1, heads_q=2, heads_kv=1, seqlen=4608), False),      # four CTAs, of which two have no tile of the last keys
-    ("mla8k", dict(heads_q=2, heads_kv=1, seqlen=2304), False),
-    ("gqa8k_d256", dict(heads_q=4, heads_kv=1, seqlen=2048), False),          # two passes
-    ("gqa4k", dict(batch=1, heads_q=4, heads_kv=1, seqlen=2048), True),
+@pytest.mark.parametrize("name,kw,bf16,split", [
+    ("gqa4k", dict(batch=1, heads_q=4, heads_kv=1, seqlen=3200), False, 4),   # causal: the last key tile has a single query tile per head
+    ("tiny", dict(seqlen=4096, heads_q=1, heads_kv=1), False, 2),             # one head, no mask, d = 64
+    ("tiny", dict(seqlen=2048, heads_q=4, heads_kv=1), False, 4),             # d = 64, slices of 16 columns
+    ("gqa4k", dict(batch=1, heads_q=1, heads_kv=1, seqlen=4224), False, 2),   # one head: CTAs of the last key tiles have no tile at all
+    ("gqa4k", dict(batch=1, heads_q=2, heads_kv=1, seqlen=4608), False, 4),   # four CTAs, of which two have no tile of the last keys
+    ("mla8k", dict(heads_q=2, heads_kv=1, seqlen=2304), False, 2),
+    ("mla8k", dict(heads_q=4, heads_kv=1, seqlen=2304), False, 4),            # slices of 32 and 48 columns
+    ("gqa8k_d256", dict(heads_q=4, heads_kv=1, seqlen=2048), False, 4),       # two passes
+    ("gqa4k", dict(batch=1, heads_q=4, heads_kv=1, seqlen=2048), True, 4),
+    ("gqa8k_d256", dict(heads_q=4, heads_kv=1, seqlen=2048), True, 4),        # three passes
+    ("gqa4k", dict(batch=1, heads_q=4, heads_kv=1, seqlen=1920, causal=False, keys_valid=1830), False, 4),   # ends inside the last key tile
 ])
-def test_key_tiles_shared_by_a_cluster(name, kw, bf16):
+def test_key_tiles_shared_by_a_cluster(name, kw, bf16, split):
     """Few heads: a cluster of CTAs shares a key tile and adds its partial sums (chosen by the launcher from the shape).
     Against the same kernel on the same problem in a batch large enough for one CTA per key tile: the FP32 sums differ in
     their order only, so the BF16 results differ by an ulp (2^-8) in few places; and the result does not depend on timing."""
     from paper_2609_37852_b200 import binding
+    kw = dict(kw)
+    keys_valid = kw.pop("keys_valid", 0)
     w = workloads.WORKLOADS[name].scaled(**kw)
     tensors = [x.cuda() for x in workloads.make_inputs(w)]
     if bf16:
@@ -332,7 +338,7 @@ def test_key_tiles_shared_by_a_cluster(name, kw, bf16):
 
     def grads(ts, batch):
         params = binding.AttnParams(batch, w.seqlen, w.heads_q, w.heads_kv, w.head_dim_qk, w.head_dim_v, w.causal, w.softmax_scale,
-                                    precision=binding.ATTN_PREC_BF16 if bf16 else binding.ATTN_PREC_MXFP8)
+                                    precision=binding.ATTN_PREC_BF16 if bf16 else binding.ATTN_PREC_MXFP8, keys_valid=keys_valid)
         q, k, v, dO = (prep(t) for t in ts)
         _, lse, ws = binding.attn_fp8_fwd(params, q, k, v)
         delta, _ = binding.attn_fp8_bwd_delta(params, q, k, v, dO, lse, workspace=ws)
@@ -340,10 +346,16 @@ def test_key_tiles_shared_by_a_cluster(name, kw, bf16):
         binding.attn_fp8_read_status(ws)
         for o in out[1:]:
             assert torch.equal(o[0], out[0][0]) and torch.equal(o[1], out[0][1])
+        for kernel, (x, _, z) in launched(lambda: binding.attn_fp8_bwd_dkdv(params, q, k, v, dO, lse, delta, workspace=ws)):
+            assert "kvmajor" in kernel                 # pairs along x, as often as CTAs share a key tile, in z groups
+            ctas = split if batch == 1 else 1
+            assert x * (z - 1) < batch * w.heads_kv * ctas <= x * z
         return out[0]
 
     shared = grads(tensors, 1)
     whole = grads([t.expand(copies, -1, -1, -1).contiguous() for t in tensors], copies)
+    if keys_valid:
+        assert not shared[0][:, :, keys_valid:].any() and not shared[1][:, :, keys_valid:].any()
     for a, b in zip(shared, whole):
         # one rounding to BF16 of FP32 sums that differ by ~1e-6: an ulp at a few elements, none elsewhere
         assert rel_fro(to_np(a), to_np(b[:1])) <= 1e-3

@@ -6,7 +6,7 @@ import torch
 from oracle import attention as A
 from oracle import mxfp8
 from paper_2609_37852_b200 import workloads
-from tests.util import rel_fro, to_np, worst_row_error
+from tests.util import launched, rel_fro, to_np, worst_row_error
 
 pytestmark = pytest.mark.gpu
 
@@ -81,20 +81,36 @@ def test_shape_and_mode_combinations(name, kw, bf16):
 
 @pytest.mark.parametrize("dims,heads_kv,per_kv,bf16", [
     ((128, 128), 1030, 1, False),       # three groups of the work list, the last one short
-    ((128, 128), 520, 2, False),        # two query heads per KV head
-    ((192, 128), 420, 1, False),
-    ((256, 256), 260, 1, False),        # one CTA per item in the forward and the query-major kernels
-    ((128, 128), 260, 1, True),
-    ((256, 256), 131, 1, True),         # two dQ column tiles per head, three key-major passes
+    ((128, 128), 521, 2, False),        # two query heads per KV head
+    ((192, 128), 421, 1, False),
+    ((256, 256), 601, 1, False),        # one CTA per item in the forward and the query-major kernel, two key-major passes
+    ((128, 128), 701, 1, True),
+    ((256, 256), 331, 1, True),         # two dQ column tiles per head, three key-major passes
 ])
 def test_heads_do_not_depend_on_their_group_of_the_work_list(dims, heads_kv, per_kv, bf16):
-    # 256 tokens, causal: K and V of all heads exceed the 32 MB of a group; 100 heads at a time they do not, and every
+    # 256 tokens, causal: K and V of all heads exceed a group's 32 to 80 MB; 100 heads at a time they do not, and every
     # head's results are the same bits
+    from paper_2609_37852_b200 import binding as B
     g = torch.Generator(device="cuda").manual_seed(heads_kv)
     w = workloads.WORKLOADS["gqa4k"].scaled(batch=1, heads_q=heads_kv * per_kv, heads_kv=heads_kv, seqlen=256, head_dim_qk=dims[0],
                                             head_dim_v=dims[1])
     q, k, v, dO = (torch.randn(1, h, 256, d, generator=g, device="cuda", dtype=torch.bfloat16)
                    for h, d in ((w.heads_q, dims[0]), (heads_kv, dims[0]), (heads_kv, dims[1]), (w.heads_q, dims[1])))
+    # kernels with one CTA per item have their groups along z: more than one, the last one short
+    params = B.AttnParams(1, 256, w.heads_q, heads_kv, *dims, w.causal, w.softmax_scale,
+                          precision=B.ATTN_PREC_BF16 if bf16 else B.ATTN_PREC_MXFP8)
+    ops = [(B.attn_fp8_prepare_bf16 if bf16 else B.attn_fp8_quantize)(x) for x in (q, k, v, dO)]
+    _, lse, ws = B.attn_fp8_fwd(params, *ops[:3])
+    grids = launched(lambda: (B.attn_fp8_fwd(params, *ops[:3], lse=lse, workspace=ws),
+                              B.attn_fp8_bwd(params, *ops, lse, torch.zeros_like(lse), workspace=ws)))
+    seen = set()
+    for kernel, (x, y, z) in grids:
+        if y > 1:
+            kind = next(n for n in ("fwd_kernel", "qmajor_kernel", "kvmajor_kernel") if n in kernel)
+            seen.add(kind)
+            assert z > 1 and x * z > (heads_kv if kind == "kvmajor_kernel" else w.heads_q), (kind, x, z)
+    assert seen == {"kvmajor_kernel"} | ({"fwd_kernel"} if bf16 or dims == (256, 256) else set()) | \
+        ({"qmajor_kernel"} if dims == (256, 256) and not bf16 else set())
     whole = _full_pass(w, (q, k, v, dO), bf16)
     for a in range(0, heads_kv, 100):
         b = min(a + 100, heads_kv)

@@ -51,3 +51,24 @@ def followed_by_torch(f, x, y):
         got = f(y)
     assert len(seen) > 1 and any("zeros" in str(s) or "cat" in str(s) for s in seen)
     yield "function mode", got
+
+
+def launched(f):
+    """[(kernel's mangled name, (grid x, y, z))] of the kernels that f() launches, read from a graph that captures the call."""
+    from cuda.bindings import driver
+
+    def got(result):
+        assert result[0] == driver.CUresult.CUDA_SUCCESS, result[0]
+        return result[1]
+    g = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(g):
+        f()
+    graph = driver.CUgraph(g.raw_cuda_graph())
+    _, _, count = driver.cuGraphGetNodes(graph, 0)
+    _, nodes, _ = driver.cuGraphGetNodes(graph, count)
+    found = []
+    for node in nodes[:count]:
+        if got(driver.cuGraphNodeGetType(node)) == driver.CUgraphNodeType.CU_GRAPH_NODE_TYPE_KERNEL:
+            p = got(driver.cuGraphKernelNodeGetParams(node))
+            found.append((got(driver.cuFuncGetName(p.func)).decode(), (p.gridDimX, p.gridDimY, p.gridDimZ)))
+    return found
