@@ -170,14 +170,6 @@ fwd_il_kernel(const IlParams p, const __grid_constant__ CUtensorMap tm_q, const 
     it.n_steps = it.n_tiles * kSubPerTile;
     return it;
   };
-  // The item after the one at hand, decoded before the steps of that one and not between the two, where every role would
-  // wait for it (the compiler moves the arithmetic down to its use unless it is pinned): (192,128), 8 x 32/8 heads x 384
-  // tokens without a mask, five items per CTA, 31.3 -> 28.4 us; (128,128), 64 x 8 heads x 256, 27.8 -> 24.8 us.
-  auto item_ahead = [&](int i) {
-    Item it = item_at(i);
-    asm volatile("" : "+r"(it.qt), "+r"(it.q_slab));
-    return it;
-  };
   constexpr int kStages = C::kStages, kVStages = C::kVStages, kCq = C::kCq;
   const int nk_qk = p.dqk / 32;                 // 32-byte K steps of the score MMA
   volatile int* abort_flag = &sm.abort_flag;
@@ -217,10 +209,8 @@ fwd_il_kernel(const IlParams p, const __grid_constant__ CUtensorMap tm_q, const 
         int issued_k = 0, issued_v = 0;
         int T = 0;                                    // key tiles of the items before this one
         bool ok = true;
-        Item nx = item_at(0);
         for (int i = 0; ok; ++i) {
-          const Item it = nx;
-          nx = item_ahead(i + 1);
+          const Item it = item_at(i);
           if (!it.valid) break;
           const int qb = i & 1;
           if (i >= 2) {
@@ -265,10 +255,8 @@ fwd_il_kernel(const IlParams p, const __grid_constant__ CUtensorMap tm_q, const 
       // ------------------------------------------------------------------ S = Q K^T issuer
       bool ok = true;
       int T = 0, G = 0;                               // key tiles and key steps of the items before this one
-      Item nx = item_at(0);
       for (int i = 0; ok; ++i) {
-        const Item it = nx;
-        nx = item_ahead(i + 1);
+        const Item it = item_at(i);
         if (!it.valid) break;
         const int qb = i & 1;
         const uint64_t desc_q = make_desc_sw128(smem_u32(sm.q[qb][0]));
@@ -312,10 +300,8 @@ fwd_il_kernel(const IlParams p, const __grid_constant__ CUtensorMap tm_q, const 
       bool ok = true;
       const uint32_t n_dv = static_cast<uint32_t>(p.dv);
       int T = 0, G = 0;
-      Item nx = item_at(0);
       for (int i = 0; ok; ++i) {
-        const Item it = nx;
-        nx = item_ahead(i + 1);
+        const Item it = item_at(i);
         if (!it.valid) break;
         for (int u = 0; u < it.n_steps && ok; ++u) {
           const int gu = G + u, gt = T + u / kSubPerTile;
@@ -364,10 +350,15 @@ fwd_il_kernel(const IlParams p, const __grid_constant__ CUtensorMap tm_q, const 
     const uint32_t lane_addr = static_cast<uint32_t>(quad * 32) << 16;
     bool ok = true;
     int G = 0;
+    // The item after the one at hand is decoded before the steps of that one, not between the two, where everybody waits
+    // for the accumulator (the compiler moves the arithmetic down to its use, and spills there, unless it is pinned):
+    // (192,128), 8 x 32/8 heads x 384 tokens without a mask, five items per CTA, 42.0 -> 38.1 us; (128,128), 64 x 8 heads
+    // x 256, 37.9 -> 35.2.  The other roles as well: no gain there, and 730 us for 722 with 8 heads, 8192 queries, 32768 keys.
     Item nx = item_at(0);
     for (int i = 0; ok; ++i) {
       const Item it = nx;
-      nx = item_ahead(i + 1);
+      nx = item_at(i + 1);
+      asm volatile("" : "+r"(nx.qt), "+r"(nx.q_slab));
       if (!it.valid) break;
       float MO = -INFINITY;                             // the accumulator row is expressed in units of 2^MO
       for (int u = 0; u < it.n_steps; ++u) {
@@ -473,10 +464,8 @@ fwd_il_kernel(const IlParams p, const __grid_constant__ CUtensorMap tm_q, const 
     const uint32_t lane_addr = static_cast<uint32_t>(quad * 32) << 16;
     bool ok = true;
     int G = 0;
-    Item nx = item_at(0);
     for (int i = 0; ok; ++i) {
-      const Item it = nx;
-      nx = item_ahead(i + 1);
+      const Item it = item_at(i);
       if (!it.valid) break;
       const int qt = it.qt;
       float M = -INFINITY;                              // private integer-valued shift (log2 units)
