@@ -307,6 +307,11 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
   griddep_launch_dependents();
   const uint32_t tmem = sm.tmem_base;
   bool stores = false;                                // this thread takes part in the epilogue
+  // kApart: a padded key of a ragged sequence (no causal mask) has a row of dV and dK of its own and nothing else, so its
+  // rows are stored as zeros, whatever its probabilities and score gradients came to (NaN behind an Inf in dO).  The other
+  // configurations make the latter zero in the loop: without that branch their loops come out 1 % slower (dK / dV and dQ
+  // of the 8K layer), with it the BF16 one does (dK / dV of the 4K layer 294 us, 290 without).
+  const int real_rows = kApart && !p.causal && jt == tiles_nk - 1 ? p.kv_lim + 1 : kTile;
 
   if (warp == 0) {
     // ------------------------------------------------------------------ producer
@@ -658,8 +663,7 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
         }
       };
       if (p.causal && it + p.q0t == jt) body(std::true_type{}); else body(std::false_type{});
-      const bool padded = !p.causal && row > p.kv_lim && jt == p.Nk / kTile - 1;
-      if (__builtin_expect(padded, 0)) {
+      if (!kApart && __builtin_expect(!p.causal && row > p.kv_lim && jt == p.Nk / kTile - 1, 0)) {
         // a padded key of a ragged sequence (no causal mask): its probabilities and score gradients are zero
 #pragma unroll
         for (int c = 0; c < 32; ++c) { sr[c] = 0u; dpr[c] = 0u; }
@@ -724,10 +728,6 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
             gradient(c, make_float2(__uint_as_float(sr[c]), __uint_as_float(sr[c + 1])), e == 0 ? make_float2(d4.x, d4.y) : make_float2(d4.z, d4.w));
           }
         }
-        if (__builtin_expect(padded, 0)) {              // 0 * (dP - D) is not zero where dP or D is not finite
-#pragma unroll
-          for (int c = 0; c < 32; ++c) dpr[c] = 0u;
-        }
       }
       if (kHasDk) {
         uint32_t byte = 0;
@@ -784,7 +784,7 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
 #pragma unroll
         for (int c = 0; c < 16; ++c) {
           __nv_bfloat162 v2 = __floats2bfloat162_rn(__uint_as_float(r[2 * c]) * mul, __uint_as_float(r[2 * c + 1]) * mul);
-          packed[c] = *reinterpret_cast<uint32_t*>(&v2);
+          packed[c] = !kApart || row < real_rows ? *reinterpret_cast<uint32_t*>(&v2) : 0u;
         }
         uint4* dst = reinterpret_cast<uint4*>(out_row + c0);
 #pragma unroll
@@ -844,7 +844,7 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
           const __nv_bfloat162 v2 = __floats2bfloat162_rn(sum[2 * c] * mul, sum[2 * c + 1] * mul);
-          packed[c] = *reinterpret_cast<const uint32_t*>(&v2);
+          packed[c] = !kApart || ep_row < real_rows ? *reinterpret_cast<const uint32_t*>(&v2) : 0u;
         }
         uint4* dst = reinterpret_cast<uint4*>(out_row + c0);
         dst[0] = make_uint4(packed[0], packed[1], packed[2], packed[3]);
