@@ -14,6 +14,7 @@ from typing import Optional
 
 import numpy as np
 import torch
+from torch.compiler import is_compiling
 
 from . import build as _build
 
@@ -168,14 +169,14 @@ def protect_dp_operand(qt: QTensor, src_bf16: torch.Tensor) -> QTensor:
 def pad_tokens(x: torch.Tensor, multiple: int = 128) -> torch.Tensor:
     """``x`` [B, H, N, d] with zero rows appended up to the next multiple of ``multiple`` tokens (the form in
     which a ragged sequence is handed to the library; see attn_params_t.keys_valid)."""
+    if not is_compiling():                             # (a compiler follows torch's operations only)
+        out = _marshal.pad_tokens(x, multiple)
+        if out is not None:
+            return out
     n = x.shape[2]
     pad = (-n) % multiple
     if pad == 0:
         return x.contiguous()
-    # (a compiler follows torch's operations only)
-    out = _marshal.pad_tokens(x, n + pad) if x.is_cuda and not torch.compiler.is_compiling() else None
-    if out is not None:
-        return out
     out = torch.zeros((x.shape[0], x.shape[1], n + pad, x.shape[3]), dtype=x.dtype, device=x.device)
     out[:, :, :n] = x
     return out

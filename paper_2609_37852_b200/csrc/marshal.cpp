@@ -358,13 +358,16 @@ PyObject* new_operand(PyObject*, PyObject* const* a, Py_ssize_t n) {
   });
 }
 
-// (x, n_padded): the padded tensor, or None where the kernel does not apply (the caller pads with torch then)
+// (x, multiple): the padded tensor, or None where there is nothing to pad or the kernel does not apply (the caller goes on
+// with torch then)
 PyObject* pad_tokens(PyObject*, PyObject* const* a, Py_ssize_t n) {
   return guarded(n, 2, [&]() -> PyObject* {
-    if (!plain(a[0])) Py_RETURN_NONE;
+    if (!plain(a[0]) || !PyLong_Check(a[1])) Py_RETURN_NONE;
     const at::Tensor& x = THPVariable_Unpack(a[0]);
-    const int64_t rows = integer(a[1]);
-    if (!x.is_contiguous() || x.dim() != 4 || x.requires_grad() || x.numel() == 0 ||
+    const int64_t multiple = integer(a[1]);
+    if (multiple <= 0 || multiple > INT32_MAX || !x.is_contiguous() || x.dim() != 4 || x.size(2) % multiple == 0) Py_RETURN_NONE;
+    const int64_t rows = (x.size(2) / multiple + 1) * multiple;
+    if (x.requires_grad() || x.numel() == 0 ||
         (x.size(3) * x.element_size()) % 16 || reinterpret_cast<uintptr_t>(x.data_ptr()) % 16 || x.size(0) * x.size(1) > INT32_MAX ||
         rows > INT32_MAX || x.size(3) * x.element_size() / 16 * rows > INT32_MAX ||     // the kernel counts a slab's pieces in 32 bits
         x.get_device() != c10::cuda::current_device())

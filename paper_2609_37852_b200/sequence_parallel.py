@@ -87,7 +87,7 @@ def concat_chunks(parts: Sequence[B.QTensor]) -> B.QTensor:
     Bn, H, _, d = parts[0].shape
     N = sum(p.shape[2] for p in parts)
     first = next((t for t in (parts[0].row_codes, parts[0].col_codes) if t is not None), None)
-    fast = B._marshal.concat(parts) if first is not None and first.is_cuda and not torch.compiler.is_compiling() else None
+    fast = B._marshal.concat(parts) if first is not None and first.is_cuda and not B.is_compiling() else None
     if fast is not None:                               # one launch for all byte tensors of all chunks
         return B.QTensor((Bn, H, N, d), *fast)
     views = [_views(p) for p in parts]

@@ -156,3 +156,16 @@ def test_keys_valid_is_validated():
     o_256, lse_256, ws = B.attn_fp8_fwd(B.AttnParams(1, 256, 2, 1, 128, 128, False, 0.1, keys_valid=256), qq, kq, vq)
     B.attn_fp8_read_status(ws)
     assert torch.equal(o_all, o_256) and torch.equal(lse_all, lse_256)
+
+
+def test_pad_tokens_of_other_multiples():
+    from paper_2609_37852_b200 import binding as B
+    x = torch.randn((1, 2, 100, 64), device="cuda")
+    for multiple in (1, 32, 64, 100, 300, True, np.int64(64)):
+        y = B.pad_tokens(x, multiple)
+        assert y.shape[2] == -(-100 // multiple) * multiple and torch.equal(y[:, :, :100], x) and not y[:, :, 100:].any()
+    assert B.pad_tokens(x, 50).data_ptr() == x.data_ptr()                        # nothing to pad: the tensor itself
+    with pytest.raises(ZeroDivisionError):
+        B.pad_tokens(x, 0)
+    for n in (0, 100):                                                           # no tokens, no heads
+        assert B.pad_tokens(torch.randn((1, 0 if n else 2, n, 64), device="cuda")).shape[2] == -(-n // 128) * 128
