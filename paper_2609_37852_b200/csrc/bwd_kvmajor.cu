@@ -1,8 +1,9 @@
 // Key-major backward kernel: dK and dV (paper Appendix "Backward Correction and Gradient
 // Computation", paragraph "Score-gradient quantization", merged with the GQA group reduction).
 //
-// One CTA owns 128 keys of one (batch, KV head).  It loops over the query heads of the group and,
-// for each, over the query tiles from the causal diagonal to the end, 64 query rows at a time.
+// One CTA, or a cluster of two or four (split_of), owns 128 keys of one (batch, KV head).  It loops over the query heads of
+// the group and, for each, over the query tiles from the causal diagonal to the end, 64 query rows at a time; the CTAs of
+// a cluster take every second or fourth query tile and add their sums at the end.
 // Per sub-tile the tensor cores recompute the TRANSPOSED products
 //     S^T  = K^ Q^^T    (128 keys x 64 queries; row-blocked FP8 copies)
 //     dP^T = V^ dO^^T
@@ -206,11 +207,11 @@ struct KvParams {
   float scale, scale_log2;
 };
 
-// kShared: a cluster of p.split CTAs shares the query tiles of a key tile (see split_of).
 __device__ __forceinline__ bool last_cta() {
   return blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1 && blockIdx.z == gridDim.z - 1;
 }
 
+// kShared: a cluster of p.split CTAs shares the query tiles of a key tile (see split_of).
 template <class C, bool kShared>
 __global__ void __launch_bounds__(kThreads, 1)
 kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
@@ -274,7 +275,7 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
     }
     for (int s = 0; s < C::kLseSlots; ++s) mbar_init(&sm.lse_ready[s], 1);   // one arrival by the prep warp
     for (int s = 0; s < kColStages; ++s) { mbar_init(&sm.col_full[s], 1); mbar_init(&sm.col_empty[s], 1); }
-    for (int t = 0; t < kTeams; ++t) { 
+    for (int t = 0; t < kTeams; ++t) {
       mbar_init(&sm.s_full[t], !kHasDk ? 1 : (kApart ? 2 : 3)); mbar_init(&sm.s_free[t], kTeamThreads);
       mbar_init(&sm.dp_full[t], 1); mbar_init(&sm.dp_free[t], kTeamThreads);
     }
@@ -441,7 +442,8 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
     int s = 0;                                        // running (stage, phase) of the row ring
     uint32_t s_phase = 0;
     // kPrepLoads: LSE and D of the next row stage (= sub-tile), in flight while this one is handled
-    int pf_h = slab * G + (kShared ? part / tiles_per_head : 0), pf_it = it0 + (kShared ? part % tiles_per_head : 0);                    // (head, query tile) of the stage fetched next
+    // (head, query tile) of the stage fetched next
+    int pf_h = slab * G + (kShared ? part / tiles_per_head : 0), pf_it = it0 + (kShared ? part % tiles_per_head : 0);
     float4 pf_l = make_float4(0.f, 0.f, 0.f, 0.f), pf_d = make_float4(0.f, 0.f, 0.f, 0.f);
     auto prefetch = [&](int uu) {
       if (4 * lane < kRowTok) {

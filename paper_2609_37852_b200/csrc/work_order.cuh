@@ -7,7 +7,6 @@
 // L2 holds the kernels are bound by DRAM: 8 x 12 heads, 6400 queries on 19200 keys, 470 MB of K and V, step 19.9 ms with
 // the batch slowest, 23.8 ms with the tile slowest.  So the tile is the slowest index within a GROUP of (sequence, KV head)
 // pairs whose operands stay in L2: 19.6 ms there; BF16 head dim 256, 4 x 12 heads x 9984, step 51.7 -> 58.6 -> 49.5 ms.
-// Over 50 problems of 0.4 to 25 ms the step takes 0.74 to 1.01 of what it took with the batch slowest.
 //
 // A CTA with a static list takes the items c, 2n-1-c, 2n+c, ... of n CTAs, which evens out where the weight of the items
 // falls steadily.  From group to group it would jump from the lightest to the heaviest tile, and CTAs on either side of the
