@@ -935,7 +935,7 @@ attn_status_t launch_kvmajor_s(const AttnShape& s, attn_qtensor_t q, attn_qtenso
   // The first pass overlaps the kernel ahead like every other kernel only where its CTAs and those of the query-major
   // kernel fit on the GPU together (one head of 256 tokens: step 28 -> 23 us).  On larger problems its CTAs would settle
   // on whichever SMs the kernel ahead leaves first, and the kernels behind fill in worse: head dim 256, 8/2 heads, step
-  // 1046 -> 1113 us; 2 x 16/4 heads of 1000 tokens 119 -> 127 us; gqa4k 603 -> 611 us.
+  // 1046 -> 1113 us; 2 x 16/4 heads of 1000 tokens 119 -> 127 us; 2 x 16/4 heads of 4096, steps in a row, 603 -> 611 us.
   const long long ctas = static_cast<long long>(s.B) * (s.Hkv * split * (s.Nk / kTile) + s.Hq * (s.N / kTile));
   const cudaError_t e = launch_kernel(kvmajor_kernel<C, kShared>, grid, kThreads, smem, stream, split, behind || ctas <= sms, p,
                                       tm_k, tm_v, tm_q, tm_dO, tm_qc, tm_dOc);
