@@ -111,6 +111,11 @@ struct QmCfg {
   // step, their completion, the wake-up, the load and the release ran one after the other: 1175 cycles a step in
   // the correction pass at head dim 128, 0.683 -> 0.598 ms on the 8K workload; the wide head dims gain nothing)
   static constexpr int kSBufs = (kEB == 2 && kEBv == 2 && kCq == 2 && kCv == 2) ? 2 : 1;
+  // The issuing warps as one elected thread each: only where a second S / dP pair lets them run ahead of the softmax (4K
+  // layer in BF16 mode, correction 153.9 -> 142.2 us, dQ 217.8 -> 215.6).  With one pair the softmax of all warps starts the
+  // sooner in step, and it costs 1 to 4 % (FP8 8K layer, correction 346 -> 359, dQ 551 -> 573; BF16 head dim 64, correction
+  // 17.6 -> 18.2; head dim 256, dQ 207 -> 213).
+  static constexpr bool kOne = kSBufs == 2;
   static constexpr uint32_t kSdp = 2 * kStep;           // columns of an S / dP pair
   static constexpr uint32_t kColS = 0, kColdP = kStep, kColdS = kSdp * kSBufs /* kDsBufs x 32 */, kColdQ = kColdS + 32 * kDsBufs;
   static constexpr uint32_t kColSFQ = kDQ ? kColdQ + kDqCols : kSdp * kSBufs;   // kQBufs slots (no dS^ / dQ columns without dQ)
@@ -180,7 +185,7 @@ qmajor_kernel(const QmParams p, const __grid_constant__ CUtensorMap tm_q, const 
   // declared with the alignment the swizzled operand tiles need, so that the compiler keeps the
   // shared state space of every access derived from it (checked below)
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  constexpr bool kDQ = C::kDQ, kFp8 = C::kFp8, kFp8v = C::kFp8v, kPersist = C::kPersist, kTicket = C::kTicket;
+  constexpr bool kDQ = C::kDQ, kFp8 = C::kFp8, kFp8v = C::kFp8v, kOne = C::kOne, kPersist = C::kPersist, kTicket = C::kTicket;
   constexpr int kStages = C::kStages, kKcStages = C::kKcStages, kEB = C::kEB, kCq = C::kCq, kCv = C::kCv;
   constexpr int kStep = C::kStep, kGroups = C::kGroups, kSoftmaxThreads = C::kSoftmaxThreads;
   constexpr uint32_t kColS = C::kColS, kColdP = C::kColdP, kColdS = C::kColdS, kColdQ = C::kColdQ, kColSFQ = C::kColSFQ,
@@ -359,7 +364,7 @@ qmajor_kernel(const QmParams p, const __grid_constant__ CUtensorMap tm_q, const 
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ S issuer
-    {
+    if (!kOne || elect_one()) {
       bool ok = true;
       int T = 0;
       for (int i = 0; ok; ++i) {
@@ -372,7 +377,7 @@ qmajor_kernel(const QmParams p, const __grid_constant__ CUtensorMap tm_q, const 
         if (!ok) break;
         if (kFp8) {
           tc_fence_after_sync();
-          sf_copy_tiles<kCq>(t_sfq, sm.sf_q[qb]);
+          sf_copy_tiles<kCq, kOne>(t_sfq, sm.sf_q[qb]);
         }
         for (int t = 0; t < it.n_tiles && ok; ++t) {
           const int gt = T + t;
@@ -380,7 +385,7 @@ qmajor_kernel(const QmParams p, const __grid_constant__ CUtensorMap tm_q, const 
           ok = mbar_wait(&sm.kv_full[s], (gt / kStages) & 1, abort_flag);
           if (!ok) break;
           tc_fence_after_sync();
-          if (kFp8 && kSfSlots == 2) sf_copy_tiles<kCq>(tmem + kColSFK + 4 * kCq * slot, sm.sf_k[s]);
+          if (kFp8 && kSfSlots == 2) sf_copy_tiles<kCq, kOne>(tmem + kColSFK + 4 * kCq * slot, sm.sf_k[s]);
           const int sb = kSBufs == 2 ? (gt & 1) : 0;   // S / dP pair of this step
           if (gt >= kSBufs) {
             // the softmax threads have pulled the S and dP that last used this pair into registers
@@ -389,26 +394,26 @@ qmajor_kernel(const QmParams p, const __grid_constant__ CUtensorMap tm_q, const 
             tc_fence_after_sync();
           }
           // a single scale slot is rewritten only now that the product that read it has been consumed
-          if (kFp8 && kSfSlots == 1) sf_copy_tiles<kCq>(tmem + kColSFK, sm.sf_k[s]);
+          if (kFp8 && kSfSlots == 1) sf_copy_tiles<kCq, kOne>(tmem + kColSFK, sm.sf_k[s]);
           const uint64_t desc_k = make_desc_sw128(smem_u32(sm.k[s][0]));
-          issue_ss<kFp8, kCq, kStep, kTile * 128 / 16, kStep * 128 / 16>(tmem + kColS + kSdp * sb, desc_q, desc_k, nk_qk, t_sfq,
+          issue_ss<kFp8, kCq, kStep, kTile * 128 / 16, kStep * 128 / 16, kOne>(tmem + kColS + kSdp * sb, desc_q, desc_k, nk_qk, t_sfq,
                                                                           tmem + kColSFK + 4 * kCq * slot + (kHalf ? 2 * (t & 1) : 0));
-          mma_commit_elect(&sm.sdp_full[sb]);
-          mma_commit_elect(&sm.kv_empty[s]);
+          commit<kOne>(&sm.sdp_full[sb]);
+          commit<kOne>(&sm.kv_empty[s]);
         }
-        if (kPersist && ok) mma_commit_elect(&sm.q_empty[qb]);     // this item's Q tile has been read
+        if (kPersist && ok) commit<kOne>(&sm.q_empty[qb]);     // this item's Q tile has been read
         T += it.n_tiles;
       }
       if (*abort_flag) ok = false;
       if (!ok) {
         int dummy = 0;
-        mma_commit_elect(&sm.drain[0]);
+        commit<kOne>(&sm.drain[0]);
         mbar_wait(&sm.drain[0], 0, &dummy);
       }
     }
   } else if (warp == 2) {
     // ------------------------------------------------------------------ dP issuer
-    {
+    if (!kOne || elect_one()) {
       bool ok = true;
       int T = 0;
       for (int i = 0; ok; ++i) {
@@ -421,7 +426,7 @@ qmajor_kernel(const QmParams p, const __grid_constant__ CUtensorMap tm_q, const 
         if (!ok) break;
         if (kFp8v) {
           tc_fence_after_sync();
-          sf_copy_tiles<kCv>(t_sfdO, sm.sf_dO[qb]);
+          sf_copy_tiles<kCv, kOne>(t_sfdO, sm.sf_dO[qb]);
         }
         for (int t = 0; t < it.n_tiles && ok; ++t) {
           const int gt = T + t;
@@ -429,33 +434,33 @@ qmajor_kernel(const QmParams p, const __grid_constant__ CUtensorMap tm_q, const 
           ok = mbar_wait(&sm.kv_full[s], (gt / kStages) & 1, abort_flag);
           if (!ok) break;
           tc_fence_after_sync();
-          if (kFp8v && kSfSlots == 2) sf_copy_tiles<kCv>(tmem + kColSFV + 4 * kCv * slot, sm.sf_v[s]);
+          if (kFp8v && kSfSlots == 2) sf_copy_tiles<kCv, kOne>(tmem + kColSFV + 4 * kCv * slot, sm.sf_v[s]);
           const int sb = kSBufs == 2 ? (gt & 1) : 0;
           if (gt >= kSBufs) {
             ok = mbar_wait(&sm.sdp_free[sb], (kSBufs == 2 ? (gt >> 1) - 1 : gt - 1) & 1, abort_flag);
             if (!ok) break;
             tc_fence_after_sync();
           }
-          if (kFp8v && kSfSlots == 1) sf_copy_tiles<kCv>(tmem + kColSFV, sm.sf_v[s]);
+          if (kFp8v && kSfSlots == 1) sf_copy_tiles<kCv, kOne>(tmem + kColSFV, sm.sf_v[s]);
           const uint64_t desc_v = make_desc_sw128(smem_u32(sm.v[s][0]));
-          issue_ss<kFp8v, kCv, kStep, kTile * 128 / 16, kStep * 128 / 16>(tmem + kColdP + kSdp * sb, desc_dO, desc_v, nk_v, t_sfdO,
+          issue_ss<kFp8v, kCv, kStep, kTile * 128 / 16, kStep * 128 / 16, kOne>(tmem + kColdP + kSdp * sb, desc_dO, desc_v, nk_v, t_sfdO,
                                                                           tmem + kColSFV + 4 * kCv * slot + (kHalf ? 2 * (t & 1) : 0));
-          mma_commit_elect(&sm.sdp_full[sb]);
-          mma_commit_elect(&sm.kv_empty[s]);
+          commit<kOne>(&sm.sdp_full[sb]);
+          commit<kOne>(&sm.kv_empty[s]);
         }
-        if (kPersist && ok) mma_commit_elect(&sm.q_empty[qb]);     // this item's dO tile has been read
+        if (kPersist && ok) commit<kOne>(&sm.q_empty[qb]);     // this item's dO tile has been read
         T += it.n_tiles;
       }
       if (*abort_flag) ok = false;
       if (!ok) {
         int dummy = 0;
-        mma_commit_elect(&sm.drain[1]);
+        commit<kOne>(&sm.drain[1]);
         mbar_wait(&sm.drain[1], 0, &dummy);
       }
     }
   } else if (warp == 3) {
     // ------------------------------------------------------------------ dQ issuer
-    if (kDQ) {
+    if (kDQ && (!kOne || elect_one())) {
       bool ok = true;
       int T = 0;
       for (int i = 0; ok; ++i) {
@@ -500,7 +505,7 @@ qmajor_kernel(const QmParams p, const __grid_constant__ CUtensorMap tm_q, const 
                                     make_idesc_mxf8(128, r == 0 ? 128 : n_dq - 128, kb, koff + kb), tmem + kColSFdS + 4 * buf,
                                     t_sfkc, (t > 0 || kb > 0));
                 else
-                  mma_bf16_ts_elect(tmem + kColdQ + 128 * r, tmem + kColdS + 32 * buf + 8 * kb,
+                  (kOne ? mma_bf16_ts : mma_bf16_ts_elect)(tmem + kColdQ + 128 * r, tmem + kColdS + 32 * buf + 8 * kb,
                                     desc_kc + (r * (128 * 128 / 16) + 2 * kb), make_idesc_bf16(128, r == 0 ? 128 : n_dq - 128),
                                     (t > 0 || kb > 0));
               }
@@ -513,19 +518,19 @@ qmajor_kernel(const QmParams p, const __grid_constant__ CUtensorMap tm_q, const 
                                 make_idesc_mxf8(128, n_dq, kb, kb), tmem + kColSFdS + 4 * buf, tmem + kColSFKc + 4 * slot,
                                 (t > 0 || kb > 0));
             else
-              mma_bf16_ts_elect(tmem + kColdQ, tmem + kColdS + 32 * buf + 8 * kb, desc_kc + 2 * kb,
+              (kOne ? mma_bf16_ts : mma_bf16_ts_elect)(tmem + kColdQ, tmem + kColdS + 32 * buf + 8 * kb, desc_kc + 2 * kb,
                                 make_idesc_bf16(128, n_dq), (t > 0 || kb > 0));
           }
-          mma_commit_elect(&sm.ds_free[buf]);            // operand and scale bytes of this buffer may be overwritten
-          mma_commit_elect(&sm.kc_empty[s]);
-          if (t == n_tiles - 1) mma_commit_elect(&sm.dq_done);
+          commit<kOne>(&sm.ds_free[buf]);            // operand and scale bytes of this buffer may be overwritten
+          commit<kOne>(&sm.kc_empty[s]);
+          if (t == n_tiles - 1) commit<kOne>(&sm.dq_done);
         }
         T += n_tiles;
       }
       if (*abort_flag) ok = false;
       if (!ok) {
         int dummy = 0;
-        mma_commit_elect(&sm.drain[2]);
+        commit<kOne>(&sm.drain[2]);
         mbar_wait(&sm.drain[2], 0, &dummy);
       }
     }

@@ -60,6 +60,9 @@ struct FwdCfg {
   static constexpr int kCq = kCq_;                      // 128-byte chunks per Q / K row
   static constexpr int kRv = kRv_;                      // 128-row tiles of the V^T operand (dv / 128, rounded up)
   static constexpr bool kFp8 = kEB == 1;
+  // The issuing warps of BF16 mode, whose 64-key steps take up to 16 MMAs a product, run as one elected thread each: 8/2 heads
+  // x 4096 x 256, 74.4 -> 65.3 us; 2 x 16/4 x 4096 x 128, 155.9 -> 153.7.  FP8 at head dim 256: 198.5 -> 200.5, so not there.
+  static constexpr bool kOne = !kFp8;
   static constexpr int kTileKeys = kTile / kEB;         // keys per K / V stage
   static constexpr int kSubPerTile = kTileKeys / kSub;  // 64-key steps per stage
   static constexpr int kPCols = 16 * kEB;               // columns of one probability buffer (64 keys)
@@ -124,7 +127,7 @@ fwd_kernel(const FwdParams p, const __grid_constant__ CUtensorMap tm_q, const __
     if (threadIdx.x == 0) atomicExch(p.status, static_cast<int>(ATTN_ERR_ALIGNMENT));
     return;
   }
-  constexpr bool kFp8 = C::kFp8;
+  constexpr bool kFp8 = C::kFp8, kOne = C::kOne;
   constexpr int kEB = C::kEB, kCq = C::kCq, kRv = C::kRv, kSubPerTile = C::kSubPerTile;
   constexpr int kSplit = C::kSplit, kBpt = C::kBpt, kSoftmaxThreads = C::kSoftmaxThreads;
   constexpr uint32_t kColS = C::kColS, kColP = C::kColP, kColO = C::kColO, kColSFQ = C::kColSFQ, kColSFK = C::kColSFK,
@@ -207,12 +210,12 @@ fwd_kernel(const FwdParams p, const __grid_constant__ CUtensorMap tm_q, const __
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ S = Q K^T issuer
-    {
+    if (!kOne || elect_one()) {
       const uint64_t desc_q = make_desc_sw128(smem_u32(sm.q[0]));
       bool ok = mbar_wait(&sm.q_full, 0, abort_flag);
       if (ok && kFp8) {
         tc_fence_after_sync();
-        sf_copy_tiles<kCq>(tmem + kColSFQ, sm.sf_q);
+        sf_copy_tiles<kCq, kOne>(tmem + kColSFQ, sm.sf_q);
       }
       for (int u = 0; u < n_sub && ok; ++u) {
         const int t = u / kSubPerTile, sub = u % kSubPerTile, s = t % kStages, slot = t & 1;
@@ -220,7 +223,7 @@ fwd_kernel(const FwdParams p, const __grid_constant__ CUtensorMap tm_q, const __
           ok = mbar_wait(&sm.k_full[s], (t / kStages) & 1, abort_flag);
           if (!ok) break;
           tc_fence_after_sync();
-          if (kFp8) sf_copy_tiles<kCq>(tmem + kColSFK + 4 * kCq * slot, sm.sf_k[s]);
+          if (kFp8) sf_copy_tiles<kCq, kOne>(tmem + kColSFK + 4 * kCq * slot, sm.sf_k[s]);
         }
         if (u > 0) {
           // the softmax threads have pulled the previous scores into registers
@@ -229,20 +232,20 @@ fwd_kernel(const FwdParams p, const __grid_constant__ CUtensorMap tm_q, const __
           tc_fence_after_sync();
         }
         const uint64_t desc_k = make_desc_sw128(smem_u32(sm.k[s][0])) + sub * (kSub * 128 / 16);
-        issue_ss<kFp8, kCq, kSub, kTile * 128 / 16, C::kTileKeys * 128 / 16>(
+        issue_ss<kFp8, kCq, kSub, kTile * 128 / 16, C::kTileKeys * 128 / 16, kOne>(
             tmem + kColS, desc_q, desc_k, nk_qk, tmem + kColSFQ, tmem + kColSFK + 4 * kCq * slot + 2 * sub);
-        mma_commit_elect(&sm.s_full);
-        if (sub == kSubPerTile - 1) mma_commit_elect(&sm.k_empty[s]);
+        commit<kOne>(&sm.s_full);
+        if (sub == kSubPerTile - 1) commit<kOne>(&sm.k_empty[s]);
       }
       if (!ok) {
         int dummy = 0;
-        mma_commit_elect(&sm.drain[0]);
+        commit<kOne>(&sm.drain[0]);
         mbar_wait(&sm.drain[0], 0, &dummy);
       }
     }
   } else if (warp == 2) {
     // ------------------------------------------------------------------ O += P V issuer
-    {
+    if (!kOne || elect_one()) {
       bool ok = true;
       for (int u = 0; u < n_sub && ok; ++u) {
         const int t = u / kSubPerTile, sub = u % kSubPerTile, s = t % kStages, slot = t & 1, buf = u & 1;
@@ -250,22 +253,22 @@ fwd_kernel(const FwdParams p, const __grid_constant__ CUtensorMap tm_q, const __
           ok = mbar_wait(&sm.v_full[s], (t / kStages) & 1, abort_flag);
           if (!ok) break;
           tc_fence_after_sync();
-          if (kFp8) sf_copy_tiles<kRv>(tmem + kColSFV + 4 * kRv * slot, sm.sf_v[s]);
+          if (kFp8) sf_copy_tiles<kRv, kOne>(tmem + kColSFV + 4 * kRv * slot, sm.sf_v[s]);
         }
         ok = mbar_wait(&sm.p_full[buf], (u >> 1) & 1, abort_flag);
         if (!ok) break;
         tc_fence_after_sync();
         if (kFp8) sf_copy_elect(tmem + kColSFP + 4 * buf, make_desc_sf(smem_u32(sm.sf_p[buf])));
         // 64 keys = 2 (codes) or 4 (BF16) steps of 32 bytes; the V^T operand is taken 128 rows at a time
-        issue_ts<kFp8, kEB, kRv>(tmem + kColO, tmem + kColP + kPCols * buf, make_desc_sw128(smem_u32(sm.v[s])), p.dv, sub,
+        issue_ts<kFp8, kEB, kRv, kOne>(tmem + kColO, tmem + kColP + kPCols * buf, make_desc_sw128(smem_u32(sm.v[s])), p.dv, sub,
                                  tmem + kColSFP + 4 * buf, tmem + kColSFV + 4 * kRv * slot, u > 0);
-        mma_commit_elect(&sm.p_free[buf]);              // operand (and scale bytes) of this buffer consumed; O updated
-        if (sub == kSubPerTile - 1) mma_commit_elect(&sm.v_empty[s]);
-        if (u == n_sub - 1) mma_commit_elect(&sm.o_done);
+        commit<kOne>(&sm.p_free[buf]);              // operand (and scale bytes) of this buffer consumed; O updated
+        if (sub == kSubPerTile - 1) commit<kOne>(&sm.v_empty[s]);
+        if (u == n_sub - 1) commit<kOne>(&sm.o_done);
       }
       if (!ok) {
         int dummy = 0;
-        mma_commit_elect(&sm.drain[1]);
+        commit<kOne>(&sm.drain[1]);
         mbar_wait(&sm.drain[1], 0, &dummy);
       }
     }
@@ -385,16 +388,16 @@ fwd_kernel(const FwdParams p, const __grid_constant__ CUtensorMap tm_q, const __
           const float bs0 = bs01.x + bs01.y, bs1 = bs23.x + bs23.y;
           l = fmaf(bs0 + bs1, __uint_as_float(bytes[bk] << 23), l);   // 2^e (0 for an all-masked block, whose sum is 0)
         } else {
-          float bs0 = 0.f, bs1 = 0.f;
+          const float2 sc2 = make_float2(p.scale_log2, p.scale_log2), nm2 = make_float2(neg_m, neg_m);
+          float2 bs = make_float2(0.f, 0.f);
 #pragma unroll
           for (int c = 0; c < 32; c += 2) {
-            const float p0 = ex2_approx(fmaf(x[c], p.scale_log2, neg_m));
-            const float p1 = ex2_approx(fmaf(x[c + 1], p.scale_log2, neg_m));
-            bs0 += p0;
-            bs1 += p1;
-            words[bk][c >> 1] = cvt_bf16x2(p0, p1);
+            const float2 a = __ffma2_rn(make_float2(x[c], x[c + 1]), sc2, nm2);
+            const float2 e = make_float2(ex2_approx(a.x), ex2_approx(a.y));
+            bs = __fadd2_rn(bs, e);
+            words[bk][c >> 1] = cvt_bf16x2(e.x, e.y);
           }
-          l += bs0 + bs1;
+          l += bs.x + bs.y;
         }
       }
       if (u >= 2) {

@@ -64,4 +64,9 @@ __device__ __forceinline__ void sf_copy_tiles(uint32_t tmem_dst, const uint8_t* 
   for (int c = 0; c < kTiles; ++c) (kOne ? sf_copy : sf_copy_elect)(tmem_dst + 4 * c, d + c * (512 / 16));
 }
 
+template <bool kOne>
+__device__ __forceinline__ void commit(uint64_t* bar) {
+  (kOne ? mma_commit : mma_commit_elect)(bar);
+}
+
 }  // namespace sm100
