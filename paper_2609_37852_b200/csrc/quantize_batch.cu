@@ -9,8 +9,12 @@
 // instruction per tile, completion counted on an mbarrier), so that the next tile is in flight
 // while the current one is quantised: the short tails and ramps of four separate launches
 // disappear and every SM always has loads outstanding.
-// Pass 1 walks the tile along channels (row copy), pass 2 along tokens (column copy, staged in
-// shared memory so that it leaves as full 128-byte rows).
+// Pass 1 walks the tile along channels (row copy), pass 2 along tokens (column copy).
+//
+// Bound by memory, nearly: Q, K, V, dO of 80 heads x 8192 x 128 in BF16 (341 MB) take 56.1 us, 6.1 TB/s or 0.93 of the measured
+// copy rate; before, with 8 values a thread in pass 1 and the transposed codes staged in shared memory and copied out
+// behind a third barrier, 63.3 (40.3 M instructions, now 32 M).  40 heads x 4096 x 128: 34.9 -> 30.8; 64 heads x 8192 x 192 / 128:
+// 72.8 -> 59.1; 20 heads x 8192 x 256: 36.6 -> 35.1.  Three CTAs per SM (80 registers, so fewer loads in flight) take 67.5 us on the first.
 //
 // Producer steps (kProd).  A pass ahead of the other two rotates the tile in place: a rotated channel is
 // a BF16 value, so it goes back into the slot it came from whatever the source type.  The FP32 steps
@@ -32,7 +36,6 @@ using namespace sm100;
 constexpr int kTokens = 128;
 constexpr int kThreads = 256;
 constexpr int kMaxRing = 2;
-constexpr int kColPitch = kTokens + 16;
 
 struct BatchJob {
   const void* src;
@@ -119,12 +122,22 @@ __device__ __forceinline__ float2 neg_mean2(const float* mean) {        // mean:
   return make_float2(-m.x, -m.y);
 }
 
+// 32 codes to global memory: one sector where the destination allows it, two 16-byte stores otherwise.
+__device__ __forceinline__ void store_codes32(uint8_t* p, const uint32_t* w, bool sector) {
+  if (sector)
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                 ::"l"(p), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
+  else {
+    reinterpret_cast<uint4*>(p)[0] = make_uint4(w[0], w[1], w[2], w[3]);
+    reinterpret_cast<uint4*>(p)[1] = make_uint4(w[4], w[5], w[6], w[7]);
+  }
+}
+
 // Both passes over one source tile in shared memory ([128 tokens][d], unpadded).  kD is the head
 // dim when it is one of the built ones (0: use the run-time value).
 template <typename T, int kD, bool kProd>
 __device__ __forceinline__ void quantize_tile(T* tile, int d_rt, const BatchJob& job, const Producer& prod, size_t slab,
-                                              size_t tok0, uint8_t* s_row_sf, uint8_t* s_col_sf, uint8_t* s_col_codes,
-                                              int tid) {
+                                              size_t tok0, uint8_t* s_row_sf, uint8_t* s_col_sf, int tid) {
   const int d = kD ? kD : d_rt;
   const int N = job.N;
   const float* mean = kProd && prod.mean != nullptr ? prod.mean + slab * d : nullptr;
@@ -133,55 +146,87 @@ __device__ __forceinline__ void quantize_tile(T* tile, int d_rt, const BatchJob&
     rotate_tile(tile, d, prod, tok0, tid);
     __syncthreads();
   }
-  // ---- pass 1: rows.  8 elements per thread per step, 4 lanes per block of 32 channels.
+  // ---- pass 1: rows.  32 bytes per thread and step, two (BF16) or four (FP32) lanes per block of 32 channels.  Every other
+  // group of four lanes takes its two 16-byte halves in the other order, so that eight lanes read from all 32 banks.
   if (job.row_codes != nullptr) {
     uint8_t* g_codes = job.row_codes + (slab * N + tok0) * d;
-    const int steps = kTokens * d / (8 * kThreads);
+    constexpr int kEl = 32 / static_cast<int>(sizeof(T)), kPr = kEl / 2;        // elements and pairs of a thread
+    // With producer steps a thread keeps its channels, so that their means stay in registers: whole tokens per step, some
+    // threads idle at head dim 192 (32 heads x 4096, rotated and centred, 75.4 us with the means loaded at every step, now 67.9).
+    constexpr bool kFixed = kProd && kD != 0;
+    constexpr int kLanes = kFixed ? kD / kEl : 1, kTokStep = kThreads / kLanes;
+    const int steps = kFixed ? (kTokens + kTokStep - 1) / kTokStep : kTokens * d / (kEl * kThreads);
+    const bool swapped = (tid >> 2) & 1;
+    const int off = swapped ? kEl / 2 : 0;
+    auto minus_mean = [&](int ch, int k) {            // of the pair held at place k
+      return neg_mean2(mean ? mean + ch + 2 * k + (k < kPr / 2 ? off : -off) : nullptr);
+    };
+    float2 nm[kPr];
+    if (kFixed)
+#pragma unroll
+      for (int k = 0; k < kPr; ++k) nm[k] = minus_mean((tid % kLanes) * kEl, k);
 #pragma unroll 4
     for (int s = 0; s < steps; ++s) {
-      const int e0 = (s * kThreads + tid) * 8;
-      const int tok = e0 / d, ch = e0 - tok * d;
-      float amax;
-      float2 v[4];
+      int e0 = (s * kThreads + tid) * kEl, tok = e0 / d, ch = e0 - tok * d;
+      bool mine = true;
+      if (kFixed) {
+        tok = s * kTokStep + tid / kLanes; ch = (tid % kLanes) * kEl;
+        mine = tid < kTokStep * kLanes && tok < kTokens;
+        e0 = mine ? tok * d + ch : 0;
+      }
+      const uint4 lo = *reinterpret_cast<const uint4*>(tile + e0 + off), hi = *reinterpret_cast<const uint4*>(tile + e0 + (kEl / 2 - off));
+      const uint32_t raw[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+      float amax = 0.f;
+      float2 v[kPr];
       if constexpr (sizeof(T) == 2) {
-        const uint4 raw = *reinterpret_cast<const uint4*>(tile + e0);
-        __nv_bfloat162 m = __float2bfloat162_rn(0.f);
-        if (!kProd) { m = absmax2(m, raw.x); m = absmax2(m, raw.y); m = absmax2(m, raw.z); m = absmax2(m, raw.w); }
-        amax = fmaxf(__low2float(m), __high2float(m));
-        v[0] = unpack_bf16x2(raw.x); v[1] = unpack_bf16x2(raw.y); v[2] = unpack_bf16x2(raw.z); v[3] = unpack_bf16x2(raw.w);
+        if (!kProd) {
+          const __nv_bfloat162 zero = __float2bfloat162_rn(0.f);
+          __nv_bfloat162 m = absmax2(absmax2(zero, raw[0]), raw[1]), n = absmax2(absmax2(zero, raw[2]), raw[3]);
+          m = absmax2(m, raw[4]); n = absmax2(n, raw[5]); m = absmax2(m, raw[6]); n = absmax2(n, raw[7]);
+          m = __hmax2(m, n);
+          m = __hmax2(m, __shfl_xor_sync(0xffffffffu, m, 1));
+          amax = fmaxf(__low2float(m), __high2float(m));
+        }
+#pragma unroll
+        for (int k = 0; k < kPr; ++k) v[k] = unpack_bf16x2(raw[k]);
       } else {
-        const float4 a = *reinterpret_cast<const float4*>(tile + e0);
-        const float4 b = *reinterpret_cast<const float4*>(tile + e0 + 4);
-        v[0] = make_float2(a.x, a.y); v[1] = make_float2(a.z, a.w); v[2] = make_float2(b.x, b.y); v[3] = make_float2(b.z, b.w);
-        amax = 0.f;
+#pragma unroll
+        for (int k = 0; k < kPr; ++k) v[k] = make_float2(__uint_as_float(raw[2 * k]), __uint_as_float(raw[2 * k + 1]));
       }
       if (kProd) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) v[k] = affine2(v[k], neg_mean2(mean ? mean + ch + 2 * k : nullptr), scale2);
+        for (int k = 0; k < kPr; ++k) v[k] = affine2(v[k], kFixed ? nm[k] : minus_mean(ch, k), scale2);
       }
       if (kProd || sizeof(T) == 4) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) amax = fmaxf(amax, fmaxf(fabsf(v[k].x), fabsf(v[k].y)));
+        for (int k = 0; k < kPr; ++k) amax = fmaxf(amax, fmaxf(fabsf(v[k].x), fabsf(v[k].y)));
+        amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 1));
+        if (sizeof(T) == 4) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 2));
       }
-      amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 1));
-      amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 2));
       uint32_t byte; float inv;
       block_scale(amax, byte, inv);
       const float2 inv2 = make_float2(inv, inv);
 #pragma unroll
-      for (int k = 0; k < 4; ++k) v[k] = __fmul2_rn(v[k], inv2);
-      uint2 codes;
-      codes.x = cvt_e4m3x4(v[0].x, v[0].y, v[1].x, v[1].y);
-      codes.y = cvt_e4m3x4(v[2].x, v[2].y, v[3].x, v[3].y);
-      *reinterpret_cast<uint2*>(g_codes + e0) = codes;
-      if ((tid & 3) == 0) {
+      for (int k = 0; k < kPr; ++k) v[k] = __fmul2_rn(v[k], inv2);
+      uint32_t w[kPr / 2];
+#pragma unroll
+      for (int k = 0; k < kPr; k += 2) w[k / 2] = cvt_e4m3x4(v[k].x, v[k].y, v[k + 1].x, v[k + 1].y);
+      if (kFixed && !mine) continue;
+      if constexpr (sizeof(T) == 2)
+        *reinterpret_cast<uint4*>(g_codes + e0) = swapped ? make_uint4(w[2], w[3], w[0], w[1]) : make_uint4(w[0], w[1], w[2], w[3]);
+      else
+        *reinterpret_cast<uint2*>(g_codes + e0) = swapped ? make_uint2(w[1], w[0]) : make_uint2(w[0], w[1]);
+      if ((tid & (32 / kEl - 1)) == 0) {
         const int blk = ch >> 5;
         s_row_sf[(blk >> 2) * 512 + sf_tile_offset(tok, blk & 3)] = static_cast<uint8_t>(byte);
       }
     }
   }
-  // ---- pass 2: columns.
+  // ---- pass 2: columns.  The 32 codes of a channel and token block leave from the thread that made them, one sector of
+  // the transposed copy; the other sectors of the line follow from other warps, before L2 lets go of it.
   if (job.col_codes != nullptr) {
+    uint8_t* g_col = job.col_codes + slab * d * N + tok0;
+    const bool sector = (reinterpret_cast<uintptr_t>(job.col_codes) & 31) == 0;
     if constexpr (sizeof(T) == 2) {
       // One pair of neighbouring channels x one block of 32 tokens per thread and step: 32-bit loads, packed maxima.
       // A tile has 2 d such items: at head dims up to 64 they fill at most half of the CTA's threads, so two lanes of a
@@ -226,11 +271,20 @@ __device__ __forceinline__ void quantize_tile(T* tile, int d_rt, const BatchJob&
           w_lo[t] = cvt_e4m3x4(a.x, b.x, e.x, f.x);
           w_hi[t] = cvt_e4m3x4(a.y, b.y, e.y, f.y);
         }
-        uint8_t* dst = s_col_codes + c * kColPitch + tb * 32 + part * kTok;
+        uint8_t* dst = g_col + static_cast<size_t>(c) * N + tb * 32;
+        if constexpr (kShare == 1) {
+          store_codes32(dst, w_lo, sector);
+          store_codes32(dst + N, w_hi, sector);
+        } else {
+          // the lanes that share an item swap halves, so that each has all 32 tokens of one of the channels
+          uint32_t w[8];
 #pragma unroll
-        for (int t = 0; t < kTok / 16; ++t) {
-          *reinterpret_cast<uint4*>(dst + 16 * t) = make_uint4(w_lo[4 * t], w_lo[4 * t + 1], w_lo[4 * t + 2], w_lo[4 * t + 3]);
-          *reinterpret_cast<uint4*>(dst + kColPitch + 16 * t) = make_uint4(w_hi[4 * t], w_hi[4 * t + 1], w_hi[4 * t + 2], w_hi[4 * t + 3]);
+          for (int t = 0; t < kTok / 4; ++t) {
+            const uint32_t other = __shfl_xor_sync(0xffffffffu, part ? w_lo[t] : w_hi[t], 16);
+            w[t] = part ? other : w_lo[t];
+            w[kTok / 4 + t] = part ? w_hi[t] : other;
+          }
+          store_codes32(dst + part * N, w, sector);
         }
         s_col_sf[(c >> 7) * 512 + sf_tile_offset(c & 127, tb)] = static_cast<uint8_t>(byte_lo);
         s_col_sf[(c >> 7) * 512 + sf_tile_offset((c + 1) & 127, tb)] = static_cast<uint8_t>(byte_hi);
@@ -254,9 +308,7 @@ __device__ __forceinline__ void quantize_tile(T* tile, int d_rt, const BatchJob&
 #pragma unroll
         for (int t = 0; t < 8; ++t)
           w[t] = cvt_e4m3x4(x[4 * t] * inv, x[4 * t + 1] * inv, x[4 * t + 2] * inv, x[4 * t + 3] * inv);
-        uint4* dst = reinterpret_cast<uint4*>(s_col_codes + c * kColPitch + tb * 32);
-        dst[0] = make_uint4(w[0], w[1], w[2], w[3]);
-        dst[1] = make_uint4(w[4], w[5], w[6], w[7]);
+        store_codes32(g_col + static_cast<size_t>(c) * N + tb * 32, w, sector);
         s_col_sf[(c >> 7) * 512 + sf_tile_offset(c & 127, tb)] = static_cast<uint8_t>(byte);
       }
     }
@@ -278,10 +330,9 @@ __global__ void __launch_bounds__(kThreads, kCtas<kOnly>) quantize_batch_kernel(
   auto ring = [&](int slot) { return reinterpret_cast<T*>(smem + slot * tile_bytes_max); };
   const int n_ring = p.ring;
   const int n_ct_max = (p.d_max / 32 + 3) / 4, n_rt_max = (p.d_max + 127) / 128;
-  uint8_t* s_row_sf = smem + n_ring * tile_bytes_max;
-  uint8_t* s_col_sf = s_row_sf + n_ct_max * 512;
-  uint8_t* s_col_codes = s_col_sf + n_rt_max * 512;                  // [d][128 + 16]
-  uint64_t* full = reinterpret_cast<uint64_t*>(s_col_codes + p.d_max * kColPitch);
+  const int sf_bytes = (n_ct_max + n_rt_max) * 512;                  // scale bytes of a tile, staged in two alternating buffers
+  uint8_t* s_sf = smem + n_ring * tile_bytes_max;
+  uint64_t* full = reinterpret_cast<uint64_t*>(s_sf + 2 * sf_bytes);
   int* abort_flag = reinterpret_cast<int*>(full + kMaxRing);
 
   const int tid = threadIdx.x;
@@ -328,21 +379,24 @@ __global__ void __launch_bounds__(kThreads, kCtas<kOnly>) quantize_batch_kernel(
     const bool want_row = job.row_codes != nullptr, want_col = job.col_codes != nullptr;
     T* tile = ring(i % n_ring);
 
-    for (int w = tid; w < (n_ct_max + n_rt_max) * 512 / 4; w += kThreads) reinterpret_cast<uint32_t*>(s_row_sf)[w] = 0;
+    uint8_t* s_row_sf = s_sf + (i & 1) * sf_bytes;
+    uint8_t* s_col_sf = s_row_sf + n_ct_max * 512;
+    if (d & 127)                       // the last scale tile has bytes that no block writes
+      for (int w = tid; w < sf_bytes / 4; w += kThreads) reinterpret_cast<uint32_t*>(s_row_sf)[w] = 0;
     // bounded wait: a copy that never lands ends the CTA with the time-out status, not a hang
     const bool landed = mbar_wait(&full[i % n_ring], (i / n_ring) & 1, abort_flag);
     if (__syncthreads_or(!landed)) break;        // all threads take the same way out
 
     if constexpr (kOnly) {
-      quantize_tile<T, kOnly, kProd>(tile, kOnly, job, p.prod, slab, tok0, s_row_sf, s_col_sf, s_col_codes, tid);
+      quantize_tile<T, kOnly, kProd>(tile, kOnly, job, p.prod, slab, tok0, s_row_sf, s_col_sf, tid);
     } else {
       switch (d) {                      // compile-time head dims: no integer division, constant strides
                                         // (32 and 96 here too: 1 % of a step at head dim 128 that uses the producer, 338 -> 341 us)
-        case 64:  quantize_tile<T, 64, kProd>(tile, d, job, p.prod, slab, tok0, s_row_sf, s_col_sf, s_col_codes, tid); break;
-        case 128: quantize_tile<T, 128, kProd>(tile, d, job, p.prod, slab, tok0, s_row_sf, s_col_sf, s_col_codes, tid); break;
-        case 192: quantize_tile<T, 192, kProd>(tile, d, job, p.prod, slab, tok0, s_row_sf, s_col_sf, s_col_codes, tid); break;
-        case 256: quantize_tile<T, 256, kProd>(tile, d, job, p.prod, slab, tok0, s_row_sf, s_col_sf, s_col_codes, tid); break;
-        default:  quantize_tile<T, 0, kProd>(tile, d, job, p.prod, slab, tok0, s_row_sf, s_col_sf, s_col_codes, tid); break;
+        case 64:  quantize_tile<T, 64, kProd>(tile, d, job, p.prod, slab, tok0, s_row_sf, s_col_sf, tid); break;
+        case 128: quantize_tile<T, 128, kProd>(tile, d, job, p.prod, slab, tok0, s_row_sf, s_col_sf, tid); break;
+        case 192: quantize_tile<T, 192, kProd>(tile, d, job, p.prod, slab, tok0, s_row_sf, s_col_sf, tid); break;
+        case 256: quantize_tile<T, 256, kProd>(tile, d, job, p.prod, slab, tok0, s_row_sf, s_col_sf, tid); break;
+        default:  quantize_tile<T, 0, kProd>(tile, d, job, p.prod, slab, tok0, s_row_sf, s_col_sf, tid); break;
       }
     }
     __syncthreads();
@@ -357,43 +411,33 @@ __global__ void __launch_bounds__(kThreads, kCtas<kOnly>) quantize_batch_kernel(
         reinterpret_cast<uint4*>(g)[w] = reinterpret_cast<const uint4*>(s_row_sf)[w];
     }
     if (want_col) {
-      for (int w = tid; w < d * 8; w += kThreads) {
-        const int c = w >> 3, chunk = w & 7;
-        *reinterpret_cast<uint4*>(job.col_codes + (slab * d + c) * N + tok0 + chunk * 16) =
-            *reinterpret_cast<const uint4*>(s_col_codes + c * kColPitch + chunk * 16);
-      }
       for (int rt = 0; rt < n_rt; ++rt) {
         uint8_t* g = job.col_scales + ((slab * n_rt + rt) * tiles_per_slab + tok_tile) * 512;
         for (int w = tid; w < 512 / 16; w += kThreads)
           reinterpret_cast<uint4*>(g)[w] = reinterpret_cast<const uint4*>(s_col_sf + rt * 512)[w];
       }
     }
-    __syncthreads();                 // staging buffers free for the next tile
   }
   if (tid == 0 && *abort_flag) atomicExch(p.status, static_cast<int>(ATTN_ERR_TIMEOUT));
 }
 
 static size_t batch_smem_bytes(size_t elem, int d_max, int ring) {
   const int n_ct = (d_max / 32 + 3) / 4, n_rt = (d_max + 127) / 128;
-  return ring * static_cast<size_t>(kTokens) * d_max * elem + (n_ct + n_rt) * 512 +
-         static_cast<size_t>(d_max) * kColPitch + 64;
+  return ring * static_cast<size_t>(kTokens) * d_max * elem + 2 * (n_ct + n_rt) * 512 + 64;
 }
 
 template <typename T, bool kProd, int kOnly>
 attn_status_t launch_batch_n(BatchParams& p, cudaStream_t stream) {
-  // two CTAs per SM come first (each covers the other's stalls), the deeper ring second: measured
-  // at d = 192 one tile x two CTAs 0.078 ms against two tiles x one CTA 0.098 ms
-  const size_t half_sm = 113 * 1024, whole_sm = 227 * 1024;
-  if (batch_smem_bytes(sizeof(T), p.d_max, kMaxRing) <= half_sm) p.ring = kMaxRing;
-  else if (batch_smem_bytes(sizeof(T), p.d_max, 1) <= half_sm) p.ring = 1;
-  else p.ring = batch_smem_bytes(sizeof(T), p.d_max, kMaxRing) <= whole_sm ? kMaxRing : 1;
-  if (kOnly) p.ring = kCtas<kOnly> * (batch_smem_bytes(sizeof(T), p.d_max, kMaxRing) + 1024) <= whole_sm ? kMaxRing : 1;
+  const size_t whole_sm = 227 * 1024;
+  auto fits = [&](int ctas, int ring) { return ctas * (batch_smem_bytes(sizeof(T), p.d_max, ring) + 1024) <= whole_sm; };
+  // as many CTAs per SM as the registers allow come first (they cover each other's stalls), the deeper ring second
+  int per_sm = kCtas<kOnly>;
+  while (per_sm > 1 && !fits(per_sm, 1)) --per_sm;
+  p.ring = fits(per_sm, kMaxRing) ? kMaxRing : 1;
   const size_t smem = batch_smem_bytes(sizeof(T), p.d_max, p.ring);
   int sms = 0;
   const attn_status_t st = allow_smem<quantize_batch_kernel<T, kProd, kOnly>>(whole_sm, "quantize", &sms);
   if (st != ATTN_OK) return st;
-  // the launch bounds let four or two CTAs fit by registers; shared memory decides between two and one
-  const int per_sm = kOnly ? kCtas<kOnly> : smem <= half_sm ? 2 : 1;
   const int resident = sms * per_sm;
   const int grid = p.total_tiles < resident ? p.total_tiles : resident;
   const cudaError_t e = launch_overlapped(quantize_batch_kernel<T, kProd, kOnly>, dim3(grid), kThreads, smem, stream, 1, p);

@@ -208,3 +208,41 @@ def test_quantize_of_the_other_narrow_head_dims_bit_exact(d, heads):
                 assert np.array_equal(B.unpack_scales(qt.row_scales, 1, H, N, dd).cpu().numpy(), rs)
                 assert np.array_equal(qt.col_codes.cpu().numpy(), np.swapaxes(cc, -1, -2))
                 assert np.array_equal(B.unpack_scales(qt.col_scales, 1, H, dd, N).cpu().numpy(), np.swapaxes(cs, -1, -2))
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("d", [32, 64, 96, 128, 160, 192, 256])
+def test_outputs_that_start_between_two_sectors(d, dtype):
+    """The 32 codes of a channel and token block leave as one 32-byte store where the copy starts on a sector, and as two
+    of 16 bytes where it starts in the middle of one (16-byte alignment is all that is asked for)."""
+    from paper_2609_37852_b200 import binding
+    x = torch.randn(1, 2, 384, d, device="cuda", dtype=dtype)
+    ref = binding.attn_fp8_quantize(x)
+    moved = binding.QTensor(shape=tuple(x.shape))
+    for name in ("row_codes", "row_scales", "col_codes", "col_scales"):
+        t = getattr(ref, name)
+        room = torch.full((t.numel() + 64,), 0xA5, dtype=torch.uint8, device="cuda")
+        assert room.data_ptr() % 32 == 0
+        setattr(moved, name, room[16:16 + t.numel()].view(t.shape))
+    binding.attn_fp8_quantize_batch([x], outs=[moved])
+    for name in ("row_codes", "row_scales", "col_codes", "col_scales"):
+        assert torch.equal(getattr(moved, name), getattr(ref, name)), name
+    _check(x.cpu())
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_a_nan_leaves_the_scale_to_the_other_values(dtype):
+    """A block's scale is that of its values that are numbers; a block of NaN alone has the scale of an all-zero one."""
+    from paper_2609_37852_b200 import binding
+    x = torch.randn(1, 1, 128, 128, device="cuda").to(dtype)
+    bad = torch.zeros_like(x, dtype=torch.bool)
+    bad[0, 0, 3, :] = True                          # four whole row blocks
+    bad[0, 0, 32:64, 9] = True                      # one whole column block
+    for t, c in ((5, 0), (6, 16), (7, 31), (70, 40), (127, 127)):
+        bad[0, 0, t, c] = True
+    qt = binding.attn_fp8_quantize(torch.where(bad, torch.nan, x))
+    ref = binding.attn_fp8_quantize(torch.where(bad, 0.0, x))
+    assert torch.equal(qt.row_scales, ref.row_scales) and torch.equal(qt.col_scales, ref.col_scales)
+    for got, want, m in ((qt.row_codes, ref.row_codes, bad), (qt.col_codes, ref.col_codes, bad.transpose(-1, -2))):
+        assert torch.equal(got[~m], want[~m])
+        assert ((got[m] & 0x7F) == 0x7F).all()
