@@ -1,9 +1,9 @@
 // Key-major backward kernel: dK and dV (paper Appendix "Backward Correction and Gradient
 // Computation", paragraph "Score-gradient quantization", merged with the GQA group reduction).
 //
-// One CTA, or a cluster of two or four (split_of), owns 128 keys of one (batch, KV head).  It loops over the query heads of
+// One CTA, or a cluster of two, four or eight (split_of), owns 128 keys of one (batch, KV head).  It loops over the query heads of
 // the group and, for each, over the query tiles from the causal diagonal to the end, 64 query rows at a time; the CTAs of
-// a cluster take every second or fourth query tile and add their sums at the end.
+// a cluster take every second, fourth or eighth query tile and add their sums at the end.
 // Per sub-tile the tensor cores recompute the TRANSPOSED products
 //     S^T  = K^ Q^^T    (128 keys x 64 queries; row-blocked FP8 copies)
 //     dP^T = V^ dO^^T
@@ -29,6 +29,7 @@
 // and accumulates dV, and a pass that rebuilds P and dS and accumulates dK.
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "common.cuh"
@@ -203,7 +204,7 @@ struct KvParams {
   int tail_wait;            // launched behind another key-major pass of the same call (see launch_kvmajor_t)
   int* tickets;             // the dQ kernel's ticket counter, to be cleared ahead of it; or null
   int slabs, group;         // (sequence, KV head) pairs, and how many of them run together (work_order.cuh)
-  int split;                // CTAs (a cluster) that share the query tiles of one key tile: 1, 2 or 4
+  int split;                // CTAs (a cluster) that share the query tiles of one key tile: 1, 2, 4 or 8
   float scale, scale_log2;
 };
 
@@ -866,27 +867,53 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
 }
 
 // CTAs per key tile.  One CTA per key tile is the least work; but the first key tile's CTA walks G * N / 128 query tiles,
-// and with few heads it alone takes longer than an SM's share of everything a gradient call does (`passes` key-major passes
-// and the dQ kernel behind them, about three quarters of a pass).  Then a cluster of two or four CTAs
-// shares the list, which costs a set-up and an exchange of the accumulators (about 8 us): taken where it saves more than
-// 12 query tiles (18 us) and a sixteenth of the share.  Calls one after the other, with one CTA per key tile and by the rule:
-// 16 heads on 4 KV heads, 4096 tokens, two CTAs, dK / dV 194 -> 101 us, gradient call 199 -> 170 us; 8 on 2 heads, 2048
-// tokens, four CTAs, 99 -> 35 and 104 -> 38 us.  Left alone: 2 x 16 on 4 heads, 1000 tokens without a mask, where two CTAs
-// take dK / dV from 54 to 34 us but the call from 64 to 68 us, since the dQ kernel fills the idle SMs either way.
+// and with few heads or short sequences it alone takes longer than the GPU takes for everything else.  Then a cluster of two,
+// four or eight CTAs shares the list, at the cost of more set-ups and of an exchange of the accumulators.  What a gradient
+// call takes with each is estimated (in us) from what its kernels were measured to take: per query tile of this kernel and per
+// key tile of the dQ kernel as in the tables, 6 per CTA of this kernel, 7.5 to 9 where CTAs share, 3 per item of the dQ kernel
+// and 4 until the first item of a CTA begins.  If all CTAs of both kernels fit on the GPU at once, the call takes as long as the longest of
+// them; if this kernel's do, dQ items fill the SMs it leaves, and what they do not get done waits for its CTAs to end; beyond
+// that the call takes the sum of the work, and the dQ kernel starts behind.  More CTAs only for 5 % and 1.5 us or more.
+// Gradient calls with one, two, four, eight CTAs and before: 8 heads on 2, 512 tokens, 30.5, 21.8, 17.2, 16.5, was 30.5 us; 4
+// on 1, 1024 tokens, 52.9, 33.1, 22.9, 19.1, was 33.1; one head of 2048, 29.9, 22.8, 22.8, 32.4, was 29.9; 2 x 16 on 4 x 512,
+// 32.8, 24.6, 29.1, -, was 32.8; 16 on 4 x 4096, 192.5, 172.3, 209.4, 289.9, was 172.4; BF16 at head dim 256, 8 on 2 x 1024,
+// 122.4, 67.7, 58.2, 88.3, was 67.7; one head of 9728, 118.7, 94.8, 135.6, 181.0, was 94.8.  Over 411 problems of up to 1.3 ms
+// (all head dims, both modes, chunks of sequences) the call takes 1.004 times as long as with the best number for each; with the
+// rule before this one (a longest CTA against the SMs' share of the work), which shared less, 1.165 times.
 // The dQ kernel counts whether it follows or not: the same sums in the same order with and without it, so that
 // attn_fp8_bwd and attn_fp8_bwd_dkdv give the same bits.
 int split_of(const AttnShape& s, int sms, int passes) {
-  const long long tiles = s.N / kTile, keys = s.Nk / kTile, G = s.Hq / s.Hkv;
+  const double tiles = s.N / kTile, keys = s.Nk / kTile, G = s.Hq / s.Hkv;
   // (query tile, key tile) pairs of a head: the first key tiles are seen by all query tiles, the last ones by fewer and fewer
-  const long long per_head = s.causal ? tiles * (keys - tiles) + tiles * (tiles + 1) / 2 : tiles * keys;
-  const long long longest = G * tiles, share = per_head * s.Hq * s.B * (4 * passes + 3) / (4LL * sms);
-  int split = 1;
-  while (split < 4) {
-    const long long next = longest / (2 * split) > share ? longest / (2 * split) : share;
-    if (longest / split - next <= 12 + share / 16) break;
-    split *= 2;
+  const double per_head = s.causal ? tiles * (keys - tiles) + tiles * (tiles + 1) / 2 : tiles * keys;
+  const double pairs = per_head * s.Hq * s.B;
+  const double items = tiles * s.Hq * s.B * (s.eb == 2 && s.dqk > 192 ? 2 : 1);             // (dQ columns in two items there)
+  static const double kPerQuery[2][3] = {{1.3, 1.5, 1.5}, {1.5, 2.5, 3.4}};     // FP8, BF16; qk head dim up to 128, 192, 256 (a pass)
+  static const double kPerKey[2][3] = {{0.9, 1.1, 1.5}, {1.0, 1.8, 2.6}};
+  const int mode = s.eb - 1, dims = s.dqk <= 128 ? 0 : s.dqk <= 192 ? 1 : 2;
+  const double t_pair = kPerQuery[mode][dims], t_dq = kPerKey[mode][dims], start = 4;
+  const double item = 3 + t_dq * per_head / tiles, last_dq = start + 3 + t_dq * keys;       // an average item, and the longest
+  auto estimate = [&](int split) {
+    const double cta = split == 1 ? 6 : split == 2 ? 7.5 : split == 4 ? 8.25 : 9;
+    const double list = G * tiles, longest = t_pair * static_cast<long long>((list + split - 1) / split) + cta;
+    const double ctas = s.B * s.Hkv * keys * split * passes, work = pairs * passes * t_pair + ctas * cta;
+    const double alone = longest > last_dq ? longest : last_dq;
+    if (ctas + items <= sms) return alone;
+    const double all = (work + items * item) / sms + start;
+    // a second round of CTAs (2 us); dQ begins once the last of them have, and the SMs that they leave are the sooner free the
+    // more the CTAs differ
+    if (ctas >= sms) return 2 + std::max(std::max(longest - 2, all), work / sms * (1 - sms / ctas) + work / ctas * per_head / (tiles * keys) + last_dq);
+    if (items * item <= (sms - ctas) * std::max(longest - start, 0.0)) return alone;
+    return std::max(std::max(alone, all), work / ctas + start + item);
+  };
+  int best = 1;
+  double least = estimate(1);
+  // (slices of the columns of dK and dV are multiples of 16)
+  for (int split = 2; split <= (s.dqk % 128 == 0 && s.dv % 128 == 0 ? 8 : 4); split *= 2) {
+    const double t = estimate(split);
+    if (t < 0.95 * least && least - t > 1.5) { best = split; least = t; }
   }
-  return split;
+  return best;
 }
 
 // `behind`: the launch follows another key-major pass of the same call, which writes another output
@@ -899,8 +926,8 @@ attn_status_t launch_kvmajor_s(const AttnShape& s, attn_qtensor_t q, attn_qtenso
                                const float* lse, const float* delta, void* dk, void* dv, int* status,
                                cudaStream_t stream, bool behind, bool clear_tickets, int split) {
   static_assert(sizeof(KvSmem<C>) + 1024 <= kSmemLimit, "shared memory exceeded");
-  // three quarters of the accumulators (a cluster of four) fit in the operand stages
-  static_assert(((C::kHasDv ? 128 * C::kRv : 0) + (C::kHasDk ? C::kQcRows : 0)) * kTile * 3 <=
+  // seven eighths of the accumulators (a cluster of eight) fit in the operand stages
+  static_assert(((C::kHasDv ? 128 * C::kRv : 0) + (C::kHasDk ? C::kQcRows : 0)) * kTile * 7 / 2 <=
                     sizeof(KvSmem<C>::k) + sizeof(KvSmem<C>::rst) + sizeof(KvSmem<C>::cst), "inbox exceeds the operand stages");
   CUtensorMap tm_k, tm_v, tm_q, tm_dO, tm_qc, tm_dOc;
   attn_status_t st;

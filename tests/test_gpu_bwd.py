@@ -321,6 +321,14 @@ def test_bench_residual_statistics_match_the_oracle_helpers():
     ("gqa4k", dict(batch=1, heads_q=4, heads_kv=1, seqlen=2048), True, 4),
     ("gqa8k_d256", dict(heads_q=4, heads_kv=1, seqlen=2048), True, 4),        # three passes
     ("gqa4k", dict(batch=1, heads_q=4, heads_kv=1, seqlen=1920, causal=False, keys_valid=1830), False, 4),   # ends inside the last key tile
+    ("gqa4k", dict(batch=1, heads_q=8, heads_kv=1, seqlen=640), False, 8),
+    ("gqa4k", dict(batch=1, heads_q=4, heads_kv=1, seqlen=1408, causal=False, keys_valid=1300), False, 8),
+    ("gqa4k", dict(batch=1, heads_q=4, heads_kv=1, seqlen=768), False, 8),                                   # CTAs of the last key tile without a query tile
+    ("gqa4k", dict(batch=1, heads_q=8, heads_kv=1, seqlen=512), True, 8),
+    ("gqa8k_d256", dict(heads_q=8, heads_kv=1, seqlen=256), False, 8),
+    ("gqa8k_d256", dict(heads_q=8, heads_kv=1, seqlen=256), True, 8),
+    ("tiny", dict(seqlen=384, heads_q=8, heads_kv=1), False, 4),              # d = 64: slices of 16 columns allow four
+    ("mla8k", dict(heads_q=8, heads_kv=1, seqlen=256), False, 4),
 ])
 def test_key_tiles_shared_by_a_cluster(name, kw, bf16, split):
     """Few heads: a cluster of CTAs shares a key tile and adds its partial sums (chosen by the launcher from the shape).
