@@ -198,6 +198,7 @@ struct KvParams {
   const float* delta;
   __nv_bfloat16* dk;
   __nv_bfloat16* dv_out;
+  int sectors;              // dk and dv_out start on 32-byte sectors
   int* status;
   int N, Nk, q0t, Hq, Hkv, dqk, dv, causal;   // N query rows, Nk keys, q0t: tile offset of the causal diagonal
   int kv_lim;               // without the causal mask: last real key of the last key tile (127: all real)
@@ -789,9 +790,9 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
           __nv_bfloat162 v2 = __floats2bfloat162_rn(__uint_as_float(r[2 * c]) * mul, __uint_as_float(r[2 * c + 1]) * mul);
           packed[c] = !kApart || row < real_rows ? *reinterpret_cast<uint32_t*>(&v2) : 0u;
         }
-        uint4* dst = reinterpret_cast<uint4*>(out_row + c0);
-#pragma unroll
-        for (int c = 0; c < 4; ++c) dst[c] = make_uint4(packed[4 * c], packed[4 * c + 1], packed[4 * c + 2], packed[4 * c + 3]);
+        // (16 bytes at a time: dK / dV of 8 x 12 heads x 1024 x 64 65.5 us, now 61.5; 16 heads x 8192 at (192,128) 489, now 469)
+        store_32b(out_row + c0, packed, p.sectors != 0);
+        store_32b(out_row + c0 + 16, packed + 8, p.sectors != 0);
       }
     }
   }
@@ -849,9 +850,7 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
           const __nv_bfloat162 v2 = __floats2bfloat162_rn(sum[2 * c] * mul, sum[2 * c + 1] * mul);
           packed[c] = !kApart || ep_row < real_rows ? *reinterpret_cast<const uint32_t*>(&v2) : 0u;
         }
-        uint4* dst = reinterpret_cast<uint4*>(out_row + c0);
-        dst[0] = make_uint4(packed[0], packed[1], packed[2], packed[3]);
-        dst[1] = make_uint4(packed[4], packed[5], packed[6], packed[7]);
+        store_32b(out_row + c0, packed, p.sectors != 0);
       }
     }
   }
@@ -944,7 +943,7 @@ attn_status_t launch_kvmajor_s(const AttnShape& s, attn_qtensor_t q, attn_qtenso
   p.k_sf = k.row_scales; p.v_sf = v.row_scales; p.q_sf = q.row_scales; p.dO_sf = dO.row_scales;
   p.qc_sf = q.col_scales; p.dOc_sf = dO.col_scales;
   p.lse = lse; p.delta = delta;
-  p.dk = static_cast<__nv_bfloat16*>(dk); p.dv_out = static_cast<__nv_bfloat16*>(dv); p.status = status;
+  p.dk = static_cast<__nv_bfloat16*>(dk); p.dv_out = static_cast<__nv_bfloat16*>(dv); p.sectors = starts_sector(dk) && starts_sector(dv); p.status = status;
   p.N = s.N; p.Nk = s.Nk; p.q0t = s.q0t; p.kv_lim = s.kv_lim; p.Hq = s.Hq; p.Hkv = s.Hkv; p.dqk = s.dqk; p.dv = s.dv; p.causal = s.causal;
   p.scale = s.scale; p.scale_log2 = s.scale * kLog2e;
   p.tail_wait = behind ? 1 : 0;

@@ -163,6 +163,7 @@ struct QmParams {
   const float* delta_in;
   float* delta_out;
   __nv_bfloat16* dq;
+  int dq_sector;            // dq starts on a 32-byte sector
   float* rowsum;
   float* rowabs;
   float* post_rowsum;       // optional: row sums of the CAST score gradient (the dQ operand) and of its magnitude
@@ -752,9 +753,9 @@ qmajor_kernel(const QmParams p, const __grid_constant__ CUtensorMap tm_q, const 
             __nv_bfloat162 v2 = __floats2bfloat162_rn(__uint_as_float(r[2 * c]) * p.scale, __uint_as_float(r[2 * c + 1]) * p.scale);
             packed[c] = *reinterpret_cast<uint32_t*>(&v2);
           }
-          uint4* dst = reinterpret_cast<uint4*>(out_row + c0);
-#pragma unroll
-          for (int c = 0; c < 4; ++c) dst[c] = make_uint4(packed[4 * c], packed[4 * c + 1], packed[4 * c + 2], packed[4 * c + 3]);
+          // (16 bytes at a time: dQ of 2 x 16/4 heads x 4096 145.6 us, now 143.7; 8 x 16 heads x 1024 61.5, now 59.4)
+          store_32b(out_row + c0, packed, p.dq_sector != 0);
+          store_32b(out_row + c0 + 16, packed + 8, p.dq_sector != 0);
         }
         if (kPersist) {
           // the accumulator may be overwritten by the next item's first dQ MMA
@@ -807,7 +808,7 @@ attn_status_t launch_qmajor_t(const AttnShape& s, attn_qtensor_t q, attn_qtensor
   p.q_sf = q.row_scales; p.dO_sf = dO.row_scales; p.k_sf = k.row_scales; p.v_sf = v.row_scales;
   p.kc_sf = kDQ ? k.col_scales : nullptr;
   p.lse = lse; p.delta_in = delta_in; p.delta_out = delta_out;
-  p.dq = static_cast<__nv_bfloat16*>(dq); p.rowsum = rowsum; p.rowabs = rowabs; p.post_rowsum = post_rowsum; p.post_rowabs = post_rowabs; p.p_abs_dp = p_abs_dp; p.status = status;
+  p.dq = static_cast<__nv_bfloat16*>(dq); p.dq_sector = starts_sector(dq); p.rowsum = rowsum; p.rowabs = rowabs; p.post_rowsum = post_rowsum; p.post_rowabs = post_rowabs; p.p_abs_dp = p_abs_dp; p.status = status;
   p.N = s.N; p.Nk = s.Nk; p.q0t = s.q0t; p.kv_lim = s.kv_lim; p.Hq = s.Hq; p.Hkv = s.Hkv; p.dqk = s.dqk; p.dv = s.dv; p.causal = s.causal;
   p.scale = s.scale; p.scale_log2 = s.scale * kLog2e;
   p.tail_wait = behind_dkdv ? 1 : 0;

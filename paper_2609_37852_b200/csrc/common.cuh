@@ -79,6 +79,9 @@ constexpr size_t kWorkspaceHeaderBytes = ATTN_STATUS_WORKSPACE_BYTES;
 // The ticket counter of the persistent dQ kernel: bytes 16..19 of the workspace header, whose first word is `status`.
 inline int* ticket_counter(int* status) { return status + 4; }
 
+// Whether rows of a multiple of 32 bytes from `p` on can be stored a sector at a time (pointers are 16-byte aligned).
+inline bool starts_sector(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 31) == 0; }
+
 // cuTensorMapEncodeTiled fetched through the runtime (no link-time dependency on libcuda).
 // Encodes a 2-D uint8 tensor [rows, row_bytes] (row pitch == row_bytes) with a
 // (box_rows x 128-byte) box and the 128-byte swizzle.

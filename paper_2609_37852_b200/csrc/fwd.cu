@@ -107,6 +107,7 @@ struct FwdParams {
   const uint8_t* k_sf;      // row scales of K
   const uint8_t* v_sf;      // col scales of V
   __nv_bfloat16* o;
+  int o_sector;             // o starts on a 32-byte sector
   float* lse;
   int* status;
   int N, Nk, q0t, Hq, Hkv, dqk, dv, causal;   // N query rows, Nk keys, q0t: tile offset of the causal diagonal
@@ -442,9 +443,8 @@ fwd_kernel(const FwdParams p, const __grid_constant__ CUtensorMap tm_q, const __
           __nv_bfloat162 v2 = __floats2bfloat162_rn(__uint_as_float(r[2 * c]) * inv_l, __uint_as_float(r[2 * c + 1]) * inv_l);
           packed[c] = *reinterpret_cast<uint32_t*>(&v2);
         }
-        uint4* dst = reinterpret_cast<uint4*>(o_row + c0);
-#pragma unroll
-        for (int c = 0; c < 4; ++c) dst[c] = make_uint4(packed[4 * c], packed[4 * c + 1], packed[4 * c + 2], packed[4 * c + 3]);
+        store_32b(o_row + c0, packed, p.o_sector != 0);
+        store_32b(o_row + c0 + 16, packed + 8, p.o_sector != 0);
       }
       // LSE = M ln2 + ln l with ln2 split so that M * ln2_hi is exact: one rounding at the end
       if (grp == 0) p.lse[grow] = fmaf(M, kLn2Hi, fmaf(M, kLn2Lo, logf(l)));
@@ -472,7 +472,7 @@ attn_status_t launch_fwd_t(const AttnShape& s, attn_qtensor_t q, attn_qtensor_t 
   if (st != ATTN_OK) return st;
   FwdParams p;
   p.q_sf = q.row_scales; p.k_sf = k.row_scales; p.v_sf = v.col_scales;
-  p.o = static_cast<__nv_bfloat16*>(o); p.lse = lse; p.status = status;
+  p.o = static_cast<__nv_bfloat16*>(o); p.o_sector = starts_sector(o); p.lse = lse; p.status = status;
   p.N = s.N; p.Nk = s.Nk; p.q0t = s.q0t; p.kv_lim = s.kv_lim; p.Hq = s.Hq; p.Hkv = s.Hkv; p.dqk = s.dqk; p.dv = s.dv; p.causal = s.causal;
   p.scale_log2 = s.scale * kLog2e;
   const size_t smem = sizeof(FwdSmem<C>) + 1024;

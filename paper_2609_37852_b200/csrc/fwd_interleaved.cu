@@ -123,6 +123,7 @@ struct IlParams {
   const uint8_t* k_sf;      // row scales of K
   const uint8_t* v_sf;      // col scales of V
   __nv_bfloat16* o;
+  int o_sector;             // o starts on a 32-byte sector
   float* lse;
   int* status;
   int N, Nk, q0t, Hq, Hkv, dqk, dv, causal;   // N query rows, Nk keys, q0t: tile offset of the causal diagonal
@@ -443,9 +444,8 @@ fwd_il_kernel(const IlParams p, const __grid_constant__ CUtensorMap tm_q, const 
           __nv_bfloat162 v2 = __floats2bfloat162_rn(__uint_as_float(r[2 * c]) * inv_l, __uint_as_float(r[2 * c + 1]) * inv_l);
           packed[c] = *reinterpret_cast<uint32_t*>(&v2);
         }
-        uint4* dst = reinterpret_cast<uint4*>(o_row + c0);
-        dst[0] = make_uint4(packed[0], packed[1], packed[2], packed[3]);
-        dst[1] = make_uint4(packed[4], packed[5], packed[6], packed[7]);
+        // (16 bytes at a time: 2 x 16/4 heads x 4096 103.1 us, now 100.2; 8 x 12 heads x 1024 x 64 27.7, now 26.7)
+        store_32b(o_row + c0, packed, p.o_sector != 0);
       }
       // the accumulator may be overwritten by the next item's first P V product
       tc_fence_before_sync();
@@ -620,7 +620,7 @@ attn_status_t launch_fwd_il_t(const AttnShape& s, attn_qtensor_t q, attn_qtensor
   if (st != ATTN_OK) return st;
   IlParams p;
   p.q_sf = q.row_scales; p.k_sf = k.row_scales; p.v_sf = v.col_scales;
-  p.o = static_cast<__nv_bfloat16*>(o); p.lse = lse; p.status = status;
+  p.o = static_cast<__nv_bfloat16*>(o); p.o_sector = starts_sector(o); p.lse = lse; p.status = status;
   p.N = s.N; p.Nk = s.Nk; p.q0t = s.q0t; p.kv_lim = s.kv_lim; p.Hq = s.Hq; p.Hkv = s.Hkv; p.dqk = s.dqk; p.dv = s.dv; p.causal = s.causal;
   p.scale_log2 = s.scale * kLog2e;
   const size_t smem = sizeof(IlSmem<C>) + 1024;

@@ -122,17 +122,6 @@ __device__ __forceinline__ float2 neg_mean2(const float* mean) {        // mean:
   return make_float2(-m.x, -m.y);
 }
 
-// 32 codes to global memory: one sector where the destination allows it, two 16-byte stores otherwise.
-__device__ __forceinline__ void store_codes32(uint8_t* p, const uint32_t* w, bool sector) {
-  if (sector)
-    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
-                 ::"l"(p), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
-  else {
-    reinterpret_cast<uint4*>(p)[0] = make_uint4(w[0], w[1], w[2], w[3]);
-    reinterpret_cast<uint4*>(p)[1] = make_uint4(w[4], w[5], w[6], w[7]);
-  }
-}
-
 // Both passes over one source tile in shared memory ([128 tokens][d], unpadded).  kD is the head
 // dim when it is one of the built ones (0: use the run-time value).
 template <typename T, int kD, bool kProd>
@@ -273,8 +262,8 @@ __device__ __forceinline__ void quantize_tile(T* tile, int d_rt, const BatchJob&
         }
         uint8_t* dst = g_col + static_cast<size_t>(c) * N + tb * 32;
         if constexpr (kShare == 1) {
-          store_codes32(dst, w_lo, sector);
-          store_codes32(dst + N, w_hi, sector);
+          store_32b(dst, w_lo, sector);
+          store_32b(dst + N, w_hi, sector);
         } else {
           // the lanes that share an item swap halves, so that each has all 32 tokens of one of the channels
           uint32_t w[8];
@@ -284,7 +273,7 @@ __device__ __forceinline__ void quantize_tile(T* tile, int d_rt, const BatchJob&
             w[t] = part ? other : w_lo[t];
             w[kTok / 4 + t] = part ? w_hi[t] : other;
           }
-          store_codes32(dst + part * N, w, sector);
+          store_32b(dst + part * N, w, sector);
         }
         s_col_sf[(c >> 7) * 512 + sf_tile_offset(c & 127, tb)] = static_cast<uint8_t>(byte_lo);
         s_col_sf[(c >> 7) * 512 + sf_tile_offset((c + 1) & 127, tb)] = static_cast<uint8_t>(byte_hi);
@@ -308,7 +297,7 @@ __device__ __forceinline__ void quantize_tile(T* tile, int d_rt, const BatchJob&
 #pragma unroll
         for (int t = 0; t < 8; ++t)
           w[t] = cvt_e4m3x4(x[4 * t] * inv, x[4 * t + 1] * inv, x[4 * t + 2] * inv, x[4 * t + 3] * inv);
-        store_codes32(g_col + static_cast<size_t>(c) * N + tb * 32, w, sector);
+        store_32b(g_col + static_cast<size_t>(c) * N + tb * 32, w, sector);
         s_col_sf[(c >> 7) * 512 + sf_tile_offset(c & 127, tb)] = static_cast<uint8_t>(byte);
       }
     }

@@ -146,6 +146,19 @@ __device__ __forceinline__ void sts_u8(void* p, uint32_t v) {
   asm volatile("st.shared.u8 [%0], %1;" ::"r"(smem_u32(p)), "r"(v) : "memory");
 }
 
+// 32 bytes of a row to global memory, one sector per lane where the row starts on one (`sector`), two 16-byte stores
+// otherwise.  A lane that stores its own row touches a line of its own, and the load / store unit takes the lines of an
+// instruction one after the other, so half as many instructions take half as long.
+__device__ __forceinline__ void store_32b(void* p, const uint32_t* w, bool sector) {
+  if (sector)
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                 ::"l"(p), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
+  else {
+    reinterpret_cast<uint4*>(p)[0] = make_uint4(w[0], w[1], w[2], w[3]);
+    reinterpret_cast<uint4*>(p)[1] = make_uint4(w[4], w[5], w[6], w[7]);
+  }
+}
+
 // ------------------------------------------------------------------ proxies / fences
 __device__ __forceinline__ void fence_proxy_async_smem() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");

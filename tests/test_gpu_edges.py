@@ -121,6 +121,38 @@ def test_heads_do_not_depend_on_their_group_of_the_work_list(dims, heads_kv, per
             assert torch.equal(whole[n][:, heads], part[n]), n
 
 
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("dims,heads", [((64, 64), (2, 2)), ((128, 128), (2, 2)), ((128, 128), (8, 1)), ((192, 128), (2, 1)), ((256, 256), (2, 2)),
+                                        ((256, 256), (8, 1))])
+def test_outputs_that_start_between_two_sectors(dims, heads, bf16):
+    """Rows leave in 32-byte stores where an output starts on a sector, and in 16-byte ones where it does not (16-byte
+    alignment is all that is asked for): the same bits, and nothing written beside them.  (8, 1) heads: key tiles shared by a
+    cluster, which stores slices of columns."""
+    from paper_2609_37852_b200 import binding as B
+    g = torch.Generator(device="cuda").manual_seed(sum(dims) + sum(heads))
+    n, (hq, hkv), (dqk, dv) = 384, heads, dims
+    q, k, v, dO = (torch.randn(1, h, n, d, generator=g, device="cuda", dtype=torch.bfloat16) for h, d in ((hq, dqk), (hkv, dqk), (hkv, dv), (hq, dv)))
+    params = B.AttnParams(1, n, hq, hkv, dqk, dv, True, dqk ** -0.5, precision=B.ATTN_PREC_BF16 if bf16 else B.ATTN_PREC_MXFP8)
+    ops = [(B.attn_fp8_prepare_bf16 if bf16 else B.attn_fp8_quantize)(x) for x in (q, k, v, dO)]
+    lse = torch.empty(1, hq, n, device="cuda")
+    delta = torch.empty_like(lse)
+
+    def run(offset):
+        rooms = [torch.full((x.numel() + 32,), 7.0, dtype=torch.bfloat16, device="cuda") for x in (dO, q, k, v)]
+        o, dq, dk, dv_ = (r[offset:offset + x.numel()].view(x.shape) for r, x in zip(rooms, (dO, q, k, v)))
+        assert o.data_ptr() % 32 == 2 * offset
+        _, _, ws = B.attn_fp8_fwd(params, *ops[:3], o=o, lse=lse)
+        B.attn_fp8_bwd_delta(params, *ops, lse, delta=delta, workspace=ws)
+        B.attn_fp8_bwd(params, *ops, lse, delta, dq=dq, dk=dk, dv=dv_, workspace=ws)
+        B.attn_fp8_read_status(ws)
+        for r, x in zip(rooms, (dO, q, k, v)):
+            assert (r[:offset] == 7.0).all() and (r[offset + x.numel():] == 7.0).all()
+        return [x.clone() for x in (o, dq, dk, dv_)]
+
+    for a, b in zip(run(0), run(8)):
+        assert torch.equal(a, b)
+
+
 def test_nearly_one_hot_rows_stress():
     """Outlier channels shared by a query head and its KV head: scores with a standard deviation of
     ~70, rows nearly one-hot, the running shift raised (and the output accumulator rescaled) often."""
