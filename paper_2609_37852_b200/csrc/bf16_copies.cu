@@ -23,10 +23,18 @@ __device__ __forceinline__ uint4 load8(const float* p) {
 // a channel.  The 16-byte groups of token t sit at group ^ (t / 8), so that the words the lanes of a warp
 // read (eight token groups x four channel pairs) fall into 32 different banks.  The four operands of a
 // layer with 2 x (16 + 4 + 4 + 16) heads of 4096 x 128 BF16 values: 54 us with 4-byte accesses and strided
-// 2-byte shared-memory reads, 32 us now (168 MB: 5.2 TB/s, 0.80 of the measured copy bandwidth).
-template <typename T>
-__global__ void __launch_bounds__(kThreads) bf16_copies_kernel(const T* src, int N, int d, __nv_bfloat16* row_out,
+// 2-byte shared-memory reads, 35.2 us with the loads and stores of this loop in turn, 32.4 us with every load of a thread
+// ahead of its first store (168 MB: 5.2 TB/s, 0.79 of the measured copy bandwidth).
+// kD is the head dim where it is one of the usual ones, which makes the index arithmetic constant and the loop one pass;
+// others (0: the run-time value) take passes of four groups a thread.  Four calls each, before and now: 8 x 12 heads x 1024 x
+// 64 23.3, 19.5 us; 16 x 8192 at (192, 128) 67.2, 56.9; 8/2 x 8192 x 256 43.9, 34.6; FP32 16/4 x 4096 x 256 76.2, 63.5; by the
+// general kernel 2 x 16/4 x 4096 x 96 30.4, 25.7 and 16 x 4096 at (160, 32) 22.0, 22.0.
+template <typename T, int kD>
+__global__ void __launch_bounds__(kThreads) bf16_copies_kernel(const T* src, int N, int d_rt, __nv_bfloat16* row_out,
                                                                __nv_bfloat16* col_out) {
+  constexpr int kBatch = kD ? kTokens * kD / 8 / kThreads : 4;        // 16-byte groups of a thread in flight
+  static_assert(kBatch * kThreads * 8 == kTokens * kD || kD == 0, "a thread's groups fill the tile");
+  const int d = kD ? kD : d_rt;
   extern __shared__ __align__(16) uint8_t smem[];
   uint4* tile = reinterpret_cast<uint4*>(smem);                       // [64][d / 8]
   const uint32_t* words = reinterpret_cast<const uint32_t*>(smem);
@@ -36,12 +44,20 @@ __global__ void __launch_bounds__(kThreads) bf16_copies_kernel(const T* src, int
   const size_t tok0 = static_cast<size_t>(blockIdx.x) * kTokens;
   const size_t first = (slab * N + tok0) * d;
   sm100::griddep_begin();
-#pragma unroll 4
-  for (int i = threadIdx.x; i < kTokens * groups; i += kThreads) {
-    const int tok = i / groups, ch = i - tok * groups;
-    const uint4 v = load8(src + first + static_cast<size_t>(i) * 8);
-    tile[tok * groups + (ch ^ ((tok >> 3) & mask))] = v;
-    if (row_out) *reinterpret_cast<uint4*>(row_out + first + static_cast<size_t>(i) * 8) = v;
+  const int total = kTokens * groups;
+  for (int i0 = threadIdx.x; i0 < total; i0 += kBatch * kThreads) {
+    uint4 v[kBatch];
+#pragma unroll
+    for (int k = 0; k < kBatch; ++k)
+      if (kD || i0 + k * kThreads < total) v[k] = load8(src + first + static_cast<size_t>(i0 + k * kThreads) * 8);
+#pragma unroll
+    for (int k = 0; k < kBatch; ++k) {
+      const int i = i0 + k * kThreads;
+      if (!kD && i >= total) break;
+      const int tok = i / groups, ch = i - tok * groups;
+      tile[tok * groups + (ch ^ ((tok >> 3) & mask))] = v[k];
+      if (row_out) *reinterpret_cast<uint4*>(row_out + first + static_cast<size_t>(i) * 8) = v[k];
+    }
   }
   if (!col_out) return;
   __syncthreads();
@@ -62,15 +78,26 @@ __global__ void __launch_bounds__(kThreads) bf16_copies_kernel(const T* src, int
   }
 }
 
-template <typename T>
-attn_status_t launch_copies_t(const void* src, int B, int H, int N, int d, void* row_out, void* col_out,
+template <typename T, int kD>
+attn_status_t launch_copies_d(const void* src, int B, int H, int N, int d, void* row_out, void* col_out,
                               cudaStream_t stream) {
   const size_t smem = static_cast<size_t>(kTokens) * d * sizeof(__nv_bfloat16);        // at most 32 KB
   dim3 grid(N / kTokens, B * H);
-  const cudaError_t e = launch_overlapped(bf16_copies_kernel<T>, grid, kThreads, smem, stream, 1, static_cast<const T*>(src), N, d,
+  const cudaError_t e = launch_overlapped(bf16_copies_kernel<T, kD>, grid, kThreads, smem, stream, 1, static_cast<const T*>(src), N, d,
                                           static_cast<__nv_bfloat16*>(row_out), static_cast<__nv_bfloat16*>(col_out));
   if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "bf16 copies: launch: %s", cudaGetErrorString(e));
   return ATTN_OK;
+}
+
+template <typename T>
+attn_status_t launch_copies_t(const void* src, int B, int H, int N, int d, void* row_out, void* col_out, cudaStream_t stream) {
+  switch (d) {
+    case 64: return launch_copies_d<T, 64>(src, B, H, N, d, row_out, col_out, stream);
+    case 128: return launch_copies_d<T, 128>(src, B, H, N, d, row_out, col_out, stream);
+    case 192: return launch_copies_d<T, 192>(src, B, H, N, d, row_out, col_out, stream);
+    case 256: return launch_copies_d<T, 256>(src, B, H, N, d, row_out, col_out, stream);
+    default: return launch_copies_d<T, 0>(src, B, H, N, d, row_out, col_out, stream);
+  }
 }
 
 }  // namespace

@@ -307,6 +307,16 @@ def test_prepare_bf16_transposes_every_head_dim(d):
         assert torch.equal(t.col_codes, x.to(torch.bfloat16).transpose(2, 3).contiguous())
 
 
+@pytest.mark.parametrize("d", [32, 64, 96, 128, 160, 192, 256])
+def test_prepare_bf16_transposes_bf16_sources(d):
+    """Head dims with a kernel of their own and those between them, whose last pass over a tile of 64 tokens is partial."""
+    from paper_2609_37852_b200 import binding as B
+    g = torch.Generator().manual_seed(d)
+    for n in (128, 640):
+        x = torch.randn((2, 3, n, d), generator=g).to(torch.bfloat16).cuda()
+        assert torch.equal(B.attn_fp8_prepare_bf16(x).col_codes, x.transpose(2, 3).contiguous())
+
+
 @pytest.mark.parametrize("d", [192, 256])
 def test_quantize_wide_heads_bit_exact(d):
     """Two 512-byte scale tiles per 128-row tile in both orientations."""
