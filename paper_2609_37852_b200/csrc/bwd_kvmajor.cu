@@ -234,6 +234,9 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
   constexpr bool kPrepLoads = kFp8 && C::kRowTok == kSub;
   constexpr bool kSplit = kOpBufs == 1;          // single operand buffer: P^ and dS^ are handed over separately
   constexpr bool kApart = C::kApart;
+  // BF16 mode at head dim 128 stores 16 bytes at a time: dK / dV of 2 x 16/4 heads x 4096 265.3 us by the sector, 259.9 so;
+  // 32/8 x 8192 1133 and 1114.  (Head dim 64 gains as FP8 does: 8 x 12 x 1024 89.3 -> 86.2.)
+  constexpr bool kSectors = !(C::kApart && C::kCq == 2);
   constexpr int kSBufs = C::kSBufs;
   constexpr uint32_t kColS = C::kColS, kColdP = C::kColdP, kColP = C::kColP, kColdS = C::kColdS, kColdV = C::kColdV,
                      kColdK = C::kColdK, kColSFK = C::kColSFK, kColSFV = C::kColSFV, kColSFQ = C::kColSFQ,
@@ -791,8 +794,8 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
           packed[c] = !kApart || row < real_rows ? *reinterpret_cast<uint32_t*>(&v2) : 0u;
         }
         // (16 bytes at a time: dK / dV of 8 x 12 heads x 1024 x 64 65.5 us, now 61.5; 16 heads x 8192 at (192,128) 489, now 469)
-        store_32b(out_row + c0, packed, p.sectors != 0);
-        store_32b(out_row + c0 + 16, packed + 8, p.sectors != 0);
+        store_32b(out_row + c0, packed, kSectors && p.sectors != 0);
+        store_32b(out_row + c0 + 16, packed + 8, kSectors && p.sectors != 0);
       }
     }
   }
