@@ -3,6 +3,8 @@
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "mxfp8_device.cuh"
 #include "sm100_ptx.cuh"
@@ -11,17 +13,6 @@ namespace attnfp8 {
 namespace {
 
 namespace cg = cooperative_groups;
-
-// Four consecutive values as FP32.
-__device__ __forceinline__ void load4(const __nv_bfloat16* p, float* x) {
-  const uint2 raw = *reinterpret_cast<const uint2*>(p);
-  x[0] = __uint_as_float(raw.x << 16); x[1] = __uint_as_float(raw.x & 0xFFFF0000u);
-  x[2] = __uint_as_float(raw.y << 16); x[3] = __uint_as_float(raw.y & 0xFFFF0000u);
-}
-__device__ __forceinline__ void load4(const float* p, float* x) {
-  const float4 a = *reinterpret_cast<const float4*>(p);
-  x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w;
-}
 
 // FP32 mean over tokens of the (rotated, BF16-rounded) tensor, per (batch, head, channel).  The
 // terms are BF16 values, so a double-precision sum is exact whatever its order while the largest
@@ -32,11 +23,28 @@ __device__ __forceinline__ void load4(const float* p, float* x) {
 // loads; the first CTA adds the others' sums from their shared memory.  With rotary embedding, BF16:
 // 4 x 4096 x 128 values 135 -> 13 us, 48 x 2816 x 128 97 -> 24 us against one CTA per slab with scalar loads
 // (four pairs per thread and 64 registers: with eight pairs and 88 registers the second took 40 us).
+// Where the CTAs fill no more than half of the SMs (kFew), the latency of a thread's loads is all that counts: it then takes
+// 128 registers and loads four tokens ahead of the arithmetic.  Mean and quantiser, before and so: 4 x 4096 x 128 18.4, 16.1
+// us; 8 x 8192 x 128 41.1, 27.6; 4 x 8192 x 192 47.7, 30.9; 4 x 16384 x 128 without rotation 35.1, 22.2.  With more CTAs, one
+// on an SM is too few and clusters of eight wait for one another: 16 x 8192 x 192 86.0, 88.3; 18 x 2048 x 128 19.2, 19.5.
 constexpr int kMaxCluster = 8;
 constexpr int kMeanThreads = 512;
+constexpr int kAhead = 4;                                            // tokens of a thread loaded ahead of the arithmetic
 
-template <typename T>
-__global__ void __launch_bounds__(kMeanThreads, 2) token_mean_kernel(const T* src, int N, int d, const float* cos,
+template <typename T> using Raw4 = typename std::conditional<sizeof(T) == 2, uint2, float4>::type;
+__device__ __forceinline__ void widen4(const uint2& raw, float* x) {
+  x[0] = __uint_as_float(raw.x << 16); x[1] = __uint_as_float(raw.x & 0xFFFF0000u);
+  x[2] = __uint_as_float(raw.y << 16); x[3] = __uint_as_float(raw.y & 0xFFFF0000u);
+}
+__device__ __forceinline__ void widen4(const float4& raw, float* x) {
+  x[0] = raw.x; x[1] = raw.y; x[2] = raw.z; x[3] = raw.w;
+}
+
+__device__ __forceinline__ void load4(const __nv_bfloat16* p, float* x) { widen4(*reinterpret_cast<const uint2*>(p), x); }
+__device__ __forceinline__ void load4(const float* p, float* x) { widen4(*reinterpret_cast<const float4*>(p), x); }
+
+template <typename T, bool kFew>
+__global__ void __launch_bounds__(kMeanThreads, kFew ? 1 : 2) token_mean_kernel(const T* src, int N, int d, const float* cos,
                                                                      const float* sin, float* mean) {
   extern __shared__ __align__(16) uint8_t smem[];
   double* part = reinterpret_cast<double*>(smem);                   // [phases][d], then the CTA's sums in row 0
@@ -53,8 +61,47 @@ __global__ void __launch_bounds__(kMeanThreads, 2) token_mean_kernel(const T* sr
     double lo[4], hi[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) lo[k] = hi[k] = 0.0;
+    int n = n0 + ph;
+    if constexpr (kFew) {
+      auto add = [&](float* x1, float* x2, const float* c, const float* s) {
+        if (cos != nullptr) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const float r = rotate_bf16(x1[k], x2[k], c[k], s[k], false);
+            x2[k] = rotate_bf16(x2[k], x1[k], c[k], s[k], true);
+            x1[k] = r;
+          }
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          lo[k] += static_cast<double>(x1[k]);
+          hi[k] += static_cast<double>(x2[k]);
+        }
+      };
+      for (; n + (kAhead - 1) * phases < n1; n += kAhead * phases) {
+        Raw4<T> r1[kAhead], r2[kAhead];
+        float4 c4[kAhead], s4[kAhead];
+#pragma unroll
+        for (int i = 0; i < kAhead; ++i) {
+          const size_t m = n + i * phases;
+          r1[i] = *reinterpret_cast<const Raw4<T>*>(g + m * d);
+          r2[i] = *reinterpret_cast<const Raw4<T>*>(g + m * d + half);
+          if (cos != nullptr) {
+            c4[i] = *reinterpret_cast<const float4*>(cos + m * half + pc);
+            s4[i] = *reinterpret_cast<const float4*>(sin + m * half + pc);
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < kAhead; ++i) {
+          float x1[4], x2[4], c[4], s[4];
+          widen4(r1[i], x1); widen4(r2[i], x2);
+          if (cos != nullptr) { widen4(c4[i], c); widen4(s4[i], s); }
+          add(x1, x2, c, s);
+        }
+      }
+    }
 #pragma unroll 4
-    for (int n = n0 + ph; n < n1; n += phases) {
+    for (; n < n1; n += phases) {
       float x1[4], x2[4];
       load4(g + static_cast<size_t>(n) * d, x1);
       load4(g + static_cast<size_t>(n) * d + half, x2);
@@ -85,13 +132,16 @@ __global__ void __launch_bounds__(kMeanThreads, 2) token_mean_kernel(const T* sr
   const int c = threadIdx.x;                                         // d <= 256: one channel per thread
   if (c < d) {
     double sum = 0.0;
+#pragma unroll (kFew ? 8 : 4)
     for (int i = 0; i < phases; ++i) sum += part[i * d + c];
     part[c] = sum;                                                   // only this thread reads column c
   }
   cluster.sync();
   if (rank == 0 && c < d) {
     double sum = part[c];
-    for (int r = 1; r < ranks; ++r) sum += *cluster.map_shared_rank(part + c, r);
+#pragma unroll
+    for (int r = 1; r < kMaxCluster; ++r)
+      if (r < ranks) sum += *cluster.map_shared_rank(part + c, r);
     mean[slab * d + c] = static_cast<float>(sum / static_cast<double>(N));
   }
   cluster.sync();                                                    // the sums stay until they have been read
@@ -107,7 +157,8 @@ attn_status_t launch_mean_t(const void* src, int slabs, int N, int d, const floa
   while (ranks < kMaxCluster && slabs * ranks < 2 * sms && 2 * ranks <= N / 128) ranks *= 2;
   const int chunks = d / 8;
   const size_t smem = static_cast<size_t>(kMeanThreads / chunks) * d * sizeof(double);   // 32 KB
-  const cudaError_t e = launch_overlapped(token_mean_kernel<T>, dim3(static_cast<unsigned>(slabs) * ranks), kMeanThreads, smem, stream,
+  const bool few = 2 * slabs * ranks <= sms;
+  const cudaError_t e = launch_overlapped(few ? token_mean_kernel<T, true> : token_mean_kernel<T, false>, dim3(static_cast<unsigned>(slabs) * ranks), kMeanThreads, smem, stream,
                                           ranks, static_cast<const T*>(src), N, d, cos, sin, mean);
   if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "token mean: launch: %s", cudaGetErrorString(e));
   return ATTN_OK;

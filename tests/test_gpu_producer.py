@@ -69,6 +69,20 @@ def test_fused_producer_shares_a_slab_between_ctas(H, N, d):
     _codes_match(qt, y, 1, H, N, d)
 
 
+@pytest.mark.parametrize("H,N,d", [(2, 4224, 128), (3, 640, 160), (80, 384, 64)])
+def test_token_mean_ahead_in_batches_and_single_tokens(H, N, d):
+    """Threads with four batches of tokens and one more or none, with less than a batch, and the kernel for many slabs."""
+    from paper_2609_37852_b200 import binding
+    g = torch.Generator().manual_seed(H + N + d)
+    x = (torch.randn((1, H, N, d), generator=g) + 0.5).to(torch.bfloat16)
+    cos, sin = P.rope_tables(N, d)
+    for rope in (True, False):
+        tables = (torch.from_numpy(cos).cuda(), torch.from_numpy(sin).cuda()) if rope else (None, None)
+        _, mean = binding.attn_fp8_quantize_fused(x.cuda(), *tables, center=True)
+        _, m = P.fused_operand(to_np(x), cos if rope else None, sin if rope else None, center=True)
+        assert np.array_equal(to_np(mean), m)
+
+
 def test_attention_from_fused_operands():
     """q, k before rotary embedding -> fused producer (tau folded, keys centered) -> forward and
     backward with softmax_scale = 1, against the oracle run on the producer oracle's tensors."""
