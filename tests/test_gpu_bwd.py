@@ -5,7 +5,7 @@ import torch
 
 from oracle import attention as A
 from paper_2609_37852_b200 import workloads
-from tests.util import launched, rel_fro, to_np, worst_row_error
+from tests.util import clusters, launched, rel_fro, to_np, worst_row_error
 
 pytestmark = pytest.mark.gpu
 
@@ -315,7 +315,8 @@ def test_bench_residual_statistics_match_the_oracle_helpers():
     ("tiny", dict(seqlen=2048, heads_q=4, heads_kv=1), False, 4),             # d = 64, slices of 16 columns
     ("gqa4k", dict(batch=1, heads_q=1, heads_kv=1, seqlen=4224), False, 2),   # one head: CTAs of the last key tiles have no tile at all
     ("gqa4k", dict(batch=1, heads_q=2, heads_kv=1, seqlen=4608), False, 4),   # four CTAs, of which two have no tile of the last keys
-    ("mla8k", dict(heads_q=2, heads_kv=1, seqlen=2304), False, 2),
+    ("mla8k", dict(heads_q=1, heads_kv=1, seqlen=1536), False, 2),
+    ("mla8k", dict(heads_q=2, heads_kv=1, seqlen=2304), False, 4),
     ("mla8k", dict(heads_q=4, heads_kv=1, seqlen=2304), False, 4),            # slices of 32 and 48 columns
     ("gqa8k_d256", dict(heads_q=4, heads_kv=1, seqlen=2048), False, 4),       # two passes
     ("gqa4k", dict(batch=1, heads_q=4, heads_kv=1, seqlen=2048), True, 4),
@@ -354,10 +355,12 @@ def test_key_tiles_shared_by_a_cluster(name, kw, bf16, split):
         binding.attn_fp8_read_status(ws)
         for o in out[1:]:
             assert torch.equal(o[0], out[0][0]) and torch.equal(o[1], out[0][1])
-        for kernel, (x, _, z) in launched(lambda: binding.attn_fp8_bwd_dkdv(params, q, k, v, dO, lse, delta, workspace=ws)):
-            assert "kvmajor" in kernel                 # pairs along x, as often as CTAs share a key tile, in z groups
-            ctas = split if batch == 1 else 1
-            assert x * (z - 1) < batch * w.heads_kv * ctas <= x * z
+        ctas = split if batch == 1 else 1
+        call = lambda: binding.attn_fp8_bwd_dkdv(params, q, k, v, dO, lse, delta, workspace=ws)
+        passes = clusters(call)
+        assert passes and all("kvmajor" in kernel and n == ctas for kernel, n in passes), passes
+        for kernel, (x, _, z) in launched(call):       # pairs along x, as often as CTAs share a key tile, in z groups
+            assert x % ctas == 0 and x * (z - 1) < batch * w.heads_kv * ctas <= x * z
         return out[0]
 
     shared = grads(tensors, 1)

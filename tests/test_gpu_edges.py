@@ -6,7 +6,7 @@ import torch
 from oracle import attention as A
 from oracle import mxfp8
 from paper_2609_37852_b200 import workloads
-from tests.util import launched, rel_fro, to_np, worst_row_error
+from tests.util import clusters, launched, rel_fro, to_np, worst_row_error
 
 pytestmark = pytest.mark.gpu
 
@@ -122,12 +122,12 @@ def test_heads_do_not_depend_on_their_group_of_the_work_list(dims, heads_kv, per
 
 
 @pytest.mark.parametrize("bf16", [False, True])
-@pytest.mark.parametrize("dims,heads", [((64, 64), (2, 2)), ((128, 128), (2, 2)), ((128, 128), (8, 1)), ((192, 128), (2, 1)), ((256, 256), (2, 2)),
-                                        ((256, 256), (8, 1))])
+@pytest.mark.parametrize("dims,heads", [((64, 64), (2, 2)), ((128, 128), (2, 2)), ((128, 128), (8, 1)), ((192, 128), (2, 2)), ((192, 128), (2, 1)),
+                                        ((256, 256), (2, 2)), ((256, 256), (8, 1))])
 def test_outputs_that_start_between_two_sectors(dims, heads, bf16):
     """Rows leave in 32-byte stores where an output starts on a sector, and in 16-byte ones where it does not (16-byte
-    alignment is all that is asked for): the same bits, and nothing written beside them.  (8, 1) heads: key tiles shared by a
-    cluster, which stores slices of columns."""
+    alignment is all that is asked for): the same bits, and nothing written beside them.  (8, 1) and (2, 1) heads: key tiles
+    shared by a cluster, which stores slices of columns; (2, 2): one CTA per key tile, which stores whole rows."""
     from paper_2609_37852_b200 import binding as B
     g = torch.Generator(device="cuda").manual_seed(sum(dims) + sum(heads))
     n, (hq, hkv), (dqk, dv) = 384, heads, dims
@@ -151,6 +151,9 @@ def test_outputs_that_start_between_two_sectors(dims, heads, bf16):
 
     for a, b in zip(run(0), run(8)):
         assert torch.equal(a, b)
+    _, _, ws = B.attn_fp8_fwd(params, *ops[:3], lse=lse)
+    ctas = [c for kernel, c in clusters(lambda: B.attn_fp8_bwd(params, *ops, lse, delta, workspace=ws)) if "kvmajor" in kernel]
+    assert ctas and all((c > 1) == (heads[1] == 1) for c in ctas), ctas
 
 
 def test_nearly_one_hot_rows_stress():

@@ -53,22 +53,38 @@ def followed_by_torch(f, x, y):
     yield "function mode", got
 
 
-def launched(f):
-    """[(kernel's mangled name, (grid x, y, z))] of the kernels that f() launches, read from a graph that captures the call."""
+def _kernel_nodes(f):
+    """(node, parameters) of the kernels that f() launches, from a graph that captures the call."""
     from cuda.bindings import driver
-
-    def got(result):
-        assert result[0] == driver.CUresult.CUDA_SUCCESS, result[0]
-        return result[1]
     g = torch.cuda.CUDAGraph(keep_graph=True)
     with torch.cuda.graph(g):
         f()
     graph = driver.CUgraph(g.raw_cuda_graph())
     _, _, count = driver.cuGraphGetNodes(graph, 0)
     _, nodes, _ = driver.cuGraphGetNodes(graph, count)
-    found = []
     for node in nodes[:count]:
-        if got(driver.cuGraphNodeGetType(node)) == driver.CUgraphNodeType.CU_GRAPH_NODE_TYPE_KERNEL:
-            p = got(driver.cuGraphKernelNodeGetParams(node))
-            found.append((got(driver.cuFuncGetName(p.func)).decode(), (p.gridDimX, p.gridDimY, p.gridDimZ)))
+        if _got(driver.cuGraphNodeGetType(node)) == driver.CUgraphNodeType.CU_GRAPH_NODE_TYPE_KERNEL:
+            yield node, _got(driver.cuGraphKernelNodeGetParams(node))
+
+
+def _got(result):
+    from cuda.bindings import driver
+    assert result[0] == driver.CUresult.CUDA_SUCCESS, result[0]
+    return result[1]
+
+
+def launched(f):
+    """[(kernel's mangled name, (grid x, y, z))] of the kernels that f() launches."""
+    from cuda.bindings import driver
+    return [(_got(driver.cuFuncGetName(p.func)).decode(), (p.gridDimX, p.gridDimY, p.gridDimZ)) for _, p in _kernel_nodes(f)]
+
+
+def clusters(f):
+    """[(kernel's mangled name, CTAs of a cluster)] of the kernels that f() launches (1: launched without clusters)."""
+    from cuda.bindings import driver
+    attr = driver.CUlaunchAttributeID.CU_LAUNCH_ATTRIBUTE_CLUSTER_DIMENSION
+    found = []
+    for node, p in _kernel_nodes(f):
+        dim = _got(driver.cuGraphKernelNodeGetAttribute(node, attr)).clusterDim
+        found.append((_got(driver.cuFuncGetName(p.func)).decode(), max(dim.x, 1) * max(dim.y, 1) * max(dim.z, 1)))
     return found
