@@ -17,6 +17,16 @@ __device__ __forceinline__ uint4 load8(const float* p) {
   return make_uint4(sm100::cvt_bf16x2(a.x, a.y), sm100::cvt_bf16x2(a.z, a.w), sm100::cvt_bf16x2(b.x, b.y), sm100::cvt_bf16x2(b.z, b.w));
 }
 
+// Groups of eight values that a thread loads ahead of its first store, and CTAs per SM that the registers have to allow.
+// FP32 values take twice the registers on their way; up to head dim 128 they are held to those of eight CTAs, and 32 and 96
+// have kernels of their own.  Without, one
+// call on 32 heads x 4096 that writes both took 13.7 us at 96 and 19.9 at 128, now 12.4 and 19.4, and the transposed copy of 128
+// heads x 8192 x 32 38.8, now 29.8.
+template <typename T, int kD>
+constexpr int kAhead = kD ? kTokens * kD / 8 / kThreads : 4;
+template <typename T, int kD>
+constexpr int kCtas = sizeof(T) == 4 && kD && kD <= 128 ? 8 : 0;        // (0: no demand)
+
 // Memory-bound: each value read once and written once or twice.  One CTA transposes 64 tokens x d channels
 // through shared memory, 16 bytes per access on both sides: a thread loads eight channels of a token, and
 // stores eight tokens of two neighbouring channels, eight threads of a warp covering one 128-byte line of
@@ -30,10 +40,10 @@ __device__ __forceinline__ uint4 load8(const float* p) {
 // 64 23.3, 19.5 us; 16 x 8192 at (192, 128) 67.2, 56.9; 8/2 x 8192 x 256 43.9, 34.6; FP32 16/4 x 4096 x 256 76.2, 63.5; by the
 // general kernel 2 x 16/4 x 4096 x 96 30.4, 25.7 and 16 x 4096 at (160, 32) 22.0, 22.0.
 template <typename T, int kD>
-__global__ void __launch_bounds__(kThreads) bf16_copies_kernel(const T* src, int N, int d_rt, __nv_bfloat16* row_out,
+__global__ void __launch_bounds__(kThreads, kCtas<T, kD>) bf16_copies_kernel(const T* src, int N, int d_rt, __nv_bfloat16* row_out,
                                                                __nv_bfloat16* col_out) {
-  constexpr int kBatch = kD ? kTokens * kD / 8 / kThreads : 4;        // 16-byte groups of a thread in flight
-  static_assert(kBatch * kThreads * 8 == kTokens * kD || kD == 0, "a thread's groups fill the tile");
+  constexpr int kBatch = kAhead<T, kD>;
+  static_assert(kD == 0 || kTokens * kD / 8 % (kBatch * kThreads) == 0, "a thread's groups fill the tile");
   const int d = kD ? kD : d_rt;
   extern __shared__ __align__(16) uint8_t smem[];
   uint4* tile = reinterpret_cast<uint4*>(smem);                       // [64][d / 8]
@@ -91,6 +101,10 @@ attn_status_t launch_copies_d(const void* src, int B, int H, int N, int d, void*
 
 template <typename T>
 attn_status_t launch_copies_t(const void* src, int B, int H, int N, int d, void* row_out, void* col_out, cudaStream_t stream) {
+  if constexpr (sizeof(T) == 4) {
+    if (d == 32) return launch_copies_d<T, 32>(src, B, H, N, d, row_out, col_out, stream);
+    if (d == 96) return launch_copies_d<T, 96>(src, B, H, N, d, row_out, col_out, stream);
+  }
   switch (d) {
     case 64: return launch_copies_d<T, 64>(src, B, H, N, d, row_out, col_out, stream);
     case 128: return launch_copies_d<T, 128>(src, B, H, N, d, row_out, col_out, stream);
