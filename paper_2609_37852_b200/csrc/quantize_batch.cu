@@ -142,7 +142,9 @@ __device__ __forceinline__ void quantize_tile(T* tile, int d_rt, const BatchJob&
     constexpr int kEl = 32 / static_cast<int>(sizeof(T)), kPr = kEl / 2;        // elements and pairs of a thread
     // With producer steps a thread keeps its channels, so that their means stay in registers: whole tokens per step, some
     // threads idle at head dim 192 (32 heads x 4096, rotated and centred, 75.4 us with the means loaded at every step, now 67.9).
-    constexpr bool kFixed = kProd && kD != 0;
+    // FP32 sources, which are not centred, gain by it from head dim 128 on (rotated and scaled, row copies of 32 heads x 4096:
+    // 27.7 -> 26.6 us at 128, 48.3 -> 46.7 at 192, 64.7 -> 63.2 at 256) and lose below (22.7 -> 24.3 at 96, where 4 of 256 threads idle).
+    constexpr bool kFixed = kProd && (sizeof(T) == 2 ? kD != 0 : kD >= 128);
     constexpr int kLanes = kFixed ? kD / kEl : 1, kTokStep = kThreads / kLanes;
     const int steps = kFixed ? (kTokens + kTokStep - 1) / kTokStep : kTokens * d / (kEl * kThreads);
     const bool swapped = (tid >> 2) & 1;
