@@ -36,6 +36,7 @@ using namespace sm100;
 constexpr int kTokens = 128;
 constexpr int kThreads = 256;
 constexpr int kMaxRing = 2;
+constexpr int kColPitch = kTokens + 16;
 
 struct BatchJob {
   const void* src;
@@ -123,10 +124,11 @@ __device__ __forceinline__ float2 neg_mean2(const float* mean) {        // mean:
 }
 
 // Both passes over one source tile in shared memory ([128 tokens][d], unpadded).  kD is the head
-// dim when it is one of the built ones (0: use the run-time value).
-template <typename T, int kD, bool kProd>
+// dim when it is one of the built ones (0: use the run-time value).  kCol: only the second pass, its codes staged in
+// s_col_codes (see launch_batch_o).
+template <typename T, int kD, bool kProd, bool kCol>
 __device__ __forceinline__ void quantize_tile(T* tile, int d_rt, const BatchJob& job, const Producer& prod, size_t slab,
-                                              size_t tok0, uint8_t* s_row_sf, uint8_t* s_col_sf, int tid) {
+                                              size_t tok0, uint8_t* s_row_sf, uint8_t* s_col_sf, uint8_t* s_col_codes, int tid) {
   const int d = kD ? kD : d_rt;
   const int N = job.N;
   const float* mean = kProd && prod.mean != nullptr ? prod.mean + slab * d : nullptr;
@@ -137,7 +139,7 @@ __device__ __forceinline__ void quantize_tile(T* tile, int d_rt, const BatchJob&
   }
   // ---- pass 1: rows.  32 bytes per thread and step, two (BF16) or four (FP32) lanes per block of 32 channels.  Every other
   // group of four lanes takes its two 16-byte halves in the other order, so that eight lanes read from all 32 banks.
-  if (job.row_codes != nullptr) {
+  if (!kCol && job.row_codes != nullptr) {
     uint8_t* g_codes = job.row_codes + (slab * N + tok0) * d;
     constexpr int kEl = 32 / static_cast<int>(sizeof(T)), kPr = kEl / 2;        // elements and pairs of a thread
     // With producer steps a thread keeps its channels, so that their means stay in registers: whole tokens per step, some
@@ -263,7 +265,14 @@ __device__ __forceinline__ void quantize_tile(T* tile, int d_rt, const BatchJob&
           w_hi[t] = cvt_e4m3x4(a.y, b.y, e.y, f.y);
         }
         uint8_t* dst = g_col + static_cast<size_t>(c) * N + tb * 32;
-        if constexpr (kShare == 1) {
+        if constexpr (kCol) {
+          uint8_t* staged = s_col_codes + c * kColPitch + tb * 32 + part * kTok;
+#pragma unroll
+          for (int t = 0; t < kTok / 16; ++t) {
+            *reinterpret_cast<uint4*>(staged + 16 * t) = make_uint4(w_lo[4 * t], w_lo[4 * t + 1], w_lo[4 * t + 2], w_lo[4 * t + 3]);
+            *reinterpret_cast<uint4*>(staged + kColPitch + 16 * t) = make_uint4(w_hi[4 * t], w_hi[4 * t + 1], w_hi[4 * t + 2], w_hi[4 * t + 3]);
+          }
+        } else if constexpr (kShare == 1) {
           store_32b(dst, w_lo, sector);
           store_32b(dst + N, w_hi, sector);
         } else {
@@ -299,7 +308,13 @@ __device__ __forceinline__ void quantize_tile(T* tile, int d_rt, const BatchJob&
 #pragma unroll
         for (int t = 0; t < 8; ++t)
           w[t] = cvt_e4m3x4(x[4 * t] * inv, x[4 * t + 1] * inv, x[4 * t + 2] * inv, x[4 * t + 3] * inv);
-        store_32b(g_col + static_cast<size_t>(c) * N + tb * 32, w, sector);
+        if constexpr (kCol) {
+          uint4* staged = reinterpret_cast<uint4*>(s_col_codes + c * kColPitch + tb * 32);
+          staged[0] = make_uint4(w[0], w[1], w[2], w[3]);
+          staged[1] = make_uint4(w[4], w[5], w[6], w[7]);
+        } else {
+          store_32b(g_col + static_cast<size_t>(c) * N + tb * 32, w, sector);
+        }
         s_col_sf[(c >> 7) * 512 + sf_tile_offset(c & 127, tb)] = static_cast<uint8_t>(byte);
       }
     }
@@ -314,7 +329,7 @@ __device__ __forceinline__ void quantize_tile(T* tile, int d_rt, const BatchJob&
 template <int kOnly>
 constexpr int kCtas = kOnly == 0 ? 2 : kOnly == 32 ? 4 : kOnly == 64 ? 4 : 3;   // per SM
 
-template <typename T, bool kProd, int kOnly>
+template <typename T, bool kProd, int kOnly, bool kCol>
 __global__ void __launch_bounds__(kThreads, kCtas<kOnly>) quantize_batch_kernel(const __grid_constant__ BatchParams p) {
   extern __shared__ __align__(128) uint8_t smem[];
   const int tile_bytes_max = kTokens * p.d_max * static_cast<int>(sizeof(T));
@@ -323,7 +338,8 @@ __global__ void __launch_bounds__(kThreads, kCtas<kOnly>) quantize_batch_kernel(
   const int n_ct_max = (p.d_max / 32 + 3) / 4, n_rt_max = (p.d_max + 127) / 128;
   const int sf_bytes = (n_ct_max + n_rt_max) * 512;                  // scale bytes of a tile, staged in two alternating buffers
   uint8_t* s_sf = smem + n_ring * tile_bytes_max;
-  uint64_t* full = reinterpret_cast<uint64_t*>(s_sf + 2 * sf_bytes);
+  uint8_t* s_col_codes = s_sf + 2 * sf_bytes;                        // kCol: [d][128 + 16]
+  uint64_t* full = reinterpret_cast<uint64_t*>(s_col_codes + (kCol ? p.d_max * kColPitch : 0));
   int* abort_flag = reinterpret_cast<int*>(full + kMaxRing);
 
   const int tid = threadIdx.x;
@@ -379,15 +395,15 @@ __global__ void __launch_bounds__(kThreads, kCtas<kOnly>) quantize_batch_kernel(
     if (__syncthreads_or(!landed)) break;        // all threads take the same way out
 
     if constexpr (kOnly) {
-      quantize_tile<T, kOnly, kProd>(tile, kOnly, job, p.prod, slab, tok0, s_row_sf, s_col_sf, tid);
+      quantize_tile<T, kOnly, kProd, kCol>(tile, kOnly, job, p.prod, slab, tok0, s_row_sf, s_col_sf, s_col_codes, tid);
     } else {
       switch (d) {                      // compile-time head dims: no integer division, constant strides
                                         // (32 and 96 here too: 1 % of a step at head dim 128 that uses the producer, 338 -> 341 us)
-        case 64:  quantize_tile<T, 64, kProd>(tile, d, job, p.prod, slab, tok0, s_row_sf, s_col_sf, tid); break;
-        case 128: quantize_tile<T, 128, kProd>(tile, d, job, p.prod, slab, tok0, s_row_sf, s_col_sf, tid); break;
-        case 192: quantize_tile<T, 192, kProd>(tile, d, job, p.prod, slab, tok0, s_row_sf, s_col_sf, tid); break;
-        case 256: quantize_tile<T, 256, kProd>(tile, d, job, p.prod, slab, tok0, s_row_sf, s_col_sf, tid); break;
-        default:  quantize_tile<T, 0, kProd>(tile, d, job, p.prod, slab, tok0, s_row_sf, s_col_sf, tid); break;
+        case 64:  quantize_tile<T, 64, kProd, kCol>(tile, d, job, p.prod, slab, tok0, s_row_sf, s_col_sf, s_col_codes, tid); break;
+        case 128: quantize_tile<T, 128, kProd, kCol>(tile, d, job, p.prod, slab, tok0, s_row_sf, s_col_sf, s_col_codes, tid); break;
+        case 192: quantize_tile<T, 192, kProd, kCol>(tile, d, job, p.prod, slab, tok0, s_row_sf, s_col_sf, s_col_codes, tid); break;
+        case 256: quantize_tile<T, 256, kProd, kCol>(tile, d, job, p.prod, slab, tok0, s_row_sf, s_col_sf, s_col_codes, tid); break;
+        default:  quantize_tile<T, 0, kProd, kCol>(tile, d, job, p.prod, slab, tok0, s_row_sf, s_col_sf, s_col_codes, tid); break;
       }
     }
     __syncthreads();
@@ -396,12 +412,18 @@ __global__ void __launch_bounds__(kThreads, kCtas<kOnly>) quantize_batch_kernel(
       fence_proxy_async_smem();
       issue(i + n_ring);
     }
-    if (want_row) {
+    if (!kCol && want_row) {
       uint8_t* g = job.row_scales + (slab * tiles_per_slab + tok_tile) * n_ct * 512;
       for (int w = tid; w < n_ct * 512 / 16; w += kThreads)
         reinterpret_cast<uint4*>(g)[w] = reinterpret_cast<const uint4*>(s_row_sf)[w];
     }
     if (want_col) {
+      if constexpr (kCol)
+        for (int w = tid; w < d * 8; w += kThreads) {
+          const int c = w >> 3, chunk = w & 7;
+          *reinterpret_cast<uint4*>(job.col_codes + (slab * d + c) * N + tok0 + chunk * 16) =
+              *reinterpret_cast<const uint4*>(s_col_codes + c * kColPitch + chunk * 16);
+        }
       for (int rt = 0; rt < n_rt; ++rt) {
         uint8_t* g = job.col_scales + ((slab * n_rt + rt) * tiles_per_slab + tok_tile) * 512;
         for (int w = tid; w < 512 / 16; w += kThreads)
@@ -412,38 +434,56 @@ __global__ void __launch_bounds__(kThreads, kCtas<kOnly>) quantize_batch_kernel(
   if (tid == 0 && *abort_flag) atomicExch(p.status, static_cast<int>(ATTN_ERR_TIMEOUT));
 }
 
-static size_t batch_smem_bytes(size_t elem, int d_max, int ring) {
+static size_t batch_smem_bytes(size_t elem, int d_max, int ring, bool col) {
   const int n_ct = (d_max / 32 + 3) / 4, n_rt = (d_max + 127) / 128;
-  return ring * static_cast<size_t>(kTokens) * d_max * elem + 2 * (n_ct + n_rt) * 512 + 64;
+  return ring * static_cast<size_t>(kTokens) * d_max * elem + 2 * (n_ct + n_rt) * 512 +
+         (col ? static_cast<size_t>(d_max) * kColPitch : 0) + 64;
 }
 
-template <typename T, bool kProd, int kOnly>
+template <typename T, bool kProd, int kOnly, bool kCol>
 attn_status_t launch_batch_n(BatchParams& p, cudaStream_t stream) {
   const size_t whole_sm = 227 * 1024;
-  auto fits = [&](int ctas, int ring) { return ctas * (batch_smem_bytes(sizeof(T), p.d_max, ring) + 1024) <= whole_sm; };
+  auto fits = [&](int ctas, int ring) { return ctas * (batch_smem_bytes(sizeof(T), p.d_max, ring, kCol) + 1024) <= whole_sm; };
   // as many CTAs per SM as the registers allow come first (they cover each other's stalls), the deeper ring second
   int per_sm = kCtas<kOnly>;
   while (per_sm > 1 && !fits(per_sm, 1)) --per_sm;
   p.ring = fits(per_sm, kMaxRing) ? kMaxRing : 1;
-  const size_t smem = batch_smem_bytes(sizeof(T), p.d_max, p.ring);
+  const size_t smem = batch_smem_bytes(sizeof(T), p.d_max, p.ring, kCol);
   int sms = 0;
-  const attn_status_t st = allow_smem<quantize_batch_kernel<T, kProd, kOnly>>(whole_sm, "quantize", &sms);
+  const attn_status_t st = allow_smem<quantize_batch_kernel<T, kProd, kOnly, kCol>>(whole_sm, "quantize", &sms);
   if (st != ATTN_OK) return st;
   const int resident = sms * per_sm;
   const int grid = p.total_tiles < resident ? p.total_tiles : resident;
-  const cudaError_t e = launch_overlapped(quantize_batch_kernel<T, kProd, kOnly>, dim3(grid), kThreads, smem, stream, 1, p);
+  const cudaError_t e = launch_overlapped(quantize_batch_kernel<T, kProd, kOnly, kCol>, dim3(grid), kThreads, smem, stream, 1, p);
   if (e != cudaSuccess) return fail(ATTN_ERR_CUDA, "quantize: launch: %s", cudaGetErrorString(e));
   return ATTN_OK;
+}
+
+// A launch that writes column copies only stages the codes of a tile in shared memory and copies them out in 128-byte lines:
+// without the row pass to hide behind, the stores of single sectors are what it waits for.  By the sector and staged, us, 32
+// heads x 4096 and 128 x 8192: BF16 6.8, 6.4 and 39.0, 37.1 at head dim 64; 14.1, 13.0 and 91.0, 84.7 at 160; 17.5, 16.8 and 122,
+// 115.6 at 224; 19.7, 19.7 and 128.8, 126.3 at 256; rotated and scaled 17.7, 15.6 and 107, 101 at 96; 28.7, 27.1 and 194, 188 at 192;
+// FP32 9.0, 8.4 and 76.9, 76.3 at 96.  By the sector: head dim 32 (5.0, 5.3 and 27.5, 29.0); BF16 without the producer at 96 (7.8, 7.3
+// but 48.0, 52.5), 128 (9.9, 9.3 but 62.6, 65.0) and 192 (14.1, 13.8 but 100, 103.5); FP32 from 192 on, where the staged codes
+// cost the second CTA of an SM or a tile of the ring (rotated and scaled 44.0, 46.4 and 270, 347 at 192).
+template <typename T, bool kProd, int kOnly>
+attn_status_t launch_batch_o(BatchParams& p, cudaStream_t stream) {
+  if constexpr (kOnly != 32 && (kOnly != 96 || kProd || sizeof(T) == 4)) {
+    bool col = sizeof(T) == 4 ? p.d_max < 192 : kProd || (p.d_max != 96 && p.d_max != 128 && p.d_max != 192);
+    for (int j = 0; j < p.n_jobs; ++j) col = col && p.job[j].row_codes == nullptr;
+    if (col) return launch_batch_n<T, kProd, kOnly, true>(p, stream);
+  }
+  return launch_batch_n<T, kProd, kOnly, false>(p, stream);
 }
 
 template <typename T, bool kProd>
 attn_status_t launch_batch_t(BatchParams& p, cudaStream_t stream) {
   bool one_dim = true;
   for (int j = 0; j < p.n_jobs; ++j) one_dim = one_dim && p.job[j].d == p.d_max;
-  if (one_dim && p.d_max == 32) return launch_batch_n<T, kProd, 32>(p, stream);
-  if (one_dim && p.d_max == 64) return launch_batch_n<T, kProd, 64>(p, stream);
-  if (one_dim && p.d_max == 96) return launch_batch_n<T, kProd, 96>(p, stream);
-  return launch_batch_n<T, kProd, 0>(p, stream);
+  if (one_dim && p.d_max == 32) return launch_batch_o<T, kProd, 32>(p, stream);
+  if (one_dim && p.d_max == 64) return launch_batch_o<T, kProd, 64>(p, stream);
+  if (one_dim && p.d_max == 96) return launch_batch_o<T, kProd, 96>(p, stream);
+  return launch_batch_o<T, kProd, 0>(p, stream);
 }
 
 void fill_params(BatchParams& p, const attn_quantize_job_t* jobs, int n_jobs, int* status) {

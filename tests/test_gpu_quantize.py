@@ -246,3 +246,21 @@ def test_a_nan_leaves_the_scale_to_the_other_values(dtype):
     for got, want, m in ((qt.row_codes, ref.row_codes, bad), (qt.col_codes, ref.col_codes, bad.transpose(-1, -2))):
         assert torch.equal(got[~m], want[~m])
         assert ((got[m] & 0x7F) == 0x7F).all()
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("d", [32, 64, 96, 128, 160, 192, 224, 256])
+def test_column_copies_alone(d, dtype):
+    """A launch that writes column copies only may stage them in shared memory: the bits of a launch that writes both, with more
+    tiles than the CTAs of the GPU take at once, with the producer in front, and for tensors of two head dims."""
+    from paper_2609_37852_b200 import binding as B
+    g = torch.Generator(device="cuda").manual_seed(d)
+    x = torch.randn(2, 5, 128 * 130, d, generator=g, device="cuda").to(dtype)
+    y = torch.randn(1, 3, 384, 128, generator=g, device="cuda").to(dtype)
+    angle = torch.rand(x.shape[2], d // 2, generator=g, device="cuda")
+    fused = lambda **want: B.attn_fp8_quantize_fused(x, angle.cos(), angle.sin(), scale=0.3, **want)[0]
+    for alone, both in ((B.attn_fp8_quantize(x, want_row=False), B.attn_fp8_quantize(x)),
+                        (fused(want_row=False), fused()),
+                        *zip(B.attn_fp8_quantize_batch([y, x], want=[(False, True)] * 2)[0], B.attn_fp8_quantize_batch([y, x])[0])):
+        assert alone.row_codes is None
+        assert torch.equal(alone.col_codes, both.col_codes) and torch.equal(alone.col_scales, both.col_scales)
