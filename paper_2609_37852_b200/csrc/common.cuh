@@ -101,7 +101,7 @@ struct AttnShape {
 // Kernel launchers (each validates nothing: the C-ABI layer has done so).
 attn_status_t launch_quantize_fused(const attn_quantize_job_t& job, const float* cos, const float* sin, float scale,
                                     float* mean, int* status, cudaStream_t stream);
-attn_status_t launch_token_mean(const void* src, int src_dtype, int slabs, int N, int d, const float* cos, const float* sin,
+attn_status_t launch_token_mean(const void* src, int slabs, int N, int d, const float* cos, const float* sin,
                                 float* mean, cudaStream_t stream);
 attn_status_t launch_quantize_batch(const attn_quantize_job_t* jobs, int n_jobs, int* status, cudaStream_t stream);
 attn_status_t launch_bf16_copies(const void* src, int src_dtype, int B, int H, int N, int d, void* row_out, void* col_out,

@@ -518,7 +518,7 @@ attn_status_t launch_quantize_fused(const attn_quantize_job_t& job, const float*
                                     float* mean, int* status, cudaStream_t stream) {
   if (cos == nullptr && mean == nullptr && scale == 1.f) return launch_quantize_batch(&job, 1, status, stream);
   if (mean != nullptr) {
-    const attn_status_t st = launch_token_mean(job.src, job.src_dtype, job.B * job.H, job.N, job.d, cos, sin, mean, stream);
+    const attn_status_t st = launch_token_mean(job.src, job.B * job.H, job.N, job.d, cos, sin, mean, stream);
     if (st != ATTN_OK) return st;
   }
   BatchParams p = {};
