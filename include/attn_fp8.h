@@ -274,7 +274,7 @@ attn_status_t attn_fp8_bwd(const attn_params_t* p, attn_qtensor_t q, attn_qtenso
  * first one's last wave leaves idle), and both have completed when the stream reaches what follows.
  * Every output is bitwise reproducible.  dQ of a (sequence, head) does not depend on what else the call holds; dK and dV
  * do in the last place: with few heads several CTAs share the queries of a key tile and add their FP32 sums in rank order,
- * and how many they are follows from batch, head counts, lengths and the number of SMs.          */
+ * and how many they are follows from batch, head counts, lengths, head dims, precision, causal mask and the number of SMs. */
 attn_status_t attn_fp8_bwd_dq(const attn_params_t* p, attn_qtensor_t q, attn_qtensor_t k, attn_qtensor_t v,
                               attn_qtensor_t dO, const float* lse, const float* delta, void* dq_bf16,
                               float* diag_rowsum_ds, float* diag_rowsum_abs_ds,

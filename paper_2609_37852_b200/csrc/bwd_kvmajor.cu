@@ -30,6 +30,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <cmath>
 #include <type_traits>
 
 #include "common.cuh"
@@ -870,18 +871,15 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
 
 // CTAs per key tile.  One CTA per key tile is the least work; but the first key tile's CTA walks G * N / 128 query tiles,
 // and with few heads or short sequences it alone takes longer than the GPU takes for everything else.  Then a cluster of two,
-// four or eight CTAs shares the list, at the cost of more set-ups and of an exchange of the accumulators.  What a gradient
-// call takes with each is estimated (in us) from what its kernels were measured to take: per query tile of this kernel and per
-// key tile of the dQ kernel as in the tables, 6 per CTA of this kernel, 7.5 to 9 where CTAs share, 3 per item of the dQ kernel
-// and 4 until the first item of a CTA begins.  If all CTAs of both kernels fit on the GPU at once, the call takes as long as the longest of
-// them; if this kernel's do, dQ items fill the SMs it leaves, and what they do not get done waits for its CTAs to end; beyond
-// that the call takes the sum of the work, and the dQ kernel starts behind.  More CTAs only for 5 % and 1.5 us or more.
-// Gradient calls with one, two, four, eight CTAs and before: 8 heads on 2, 512 tokens, 30.5, 21.8, 17.2, 16.5, was 30.5 us; 4
-// on 1, 1024 tokens, 52.9, 33.1, 22.9, 19.1, was 33.1; one head of 2048, 29.9, 22.8, 22.8, 32.4, was 29.9; 2 x 16 on 4 x 512,
-// 32.8, 24.6, 29.1, -, was 32.8; 16 on 4 x 4096, 192.5, 172.3, 209.4, 289.9, was 172.4; BF16 at head dim 256, 8 on 2 x 1024,
-// 122.4, 67.7, 58.2, 88.3, was 67.7; one head of 9728, 118.7, 94.8, 135.6, 181.0, was 94.8.  Over 411 problems of up to 1.3 ms
-// (all head dims, both modes, chunks of sequences) the call takes 1.004 times as long as with the best number for each; with the
-// rule before this one (a longest CTA against the SMs' share of the work), which shared less, 1.165 times.
+// four or eight CTAs shares the list, at the cost of more set-ups and of an exchange of the accumulators.  The gradient call is
+// estimated (us) from what calls that fit on the GPU at once were measured to take: a CTA of this kernel 6 and so much per
+// query tile as the first table says, and 1 per 40 columns of accumulators that it sends where CTAs share, the last pass of
+// several 2 later; an item of the dQ kernel 3 and so much per key tile as the second table says, the first of a CTA 3 later.
+//   All CTAs of both kernels fit at once: the call takes as long as the longest of them.
+//   This kernel's do: dQ items fill the SMs it leaves, and what they do not get done waits for its CTAs to end.
+//   They do not: the sum of the work, or a dQ item behind the rounds of this kernel.  In the last two, sharing costs 3 % per
+//   doubling, since a cluster waits for as many free SMs; clusters of eight leave a tenth of the SMs out.
+// More CTAs only for 5 % and 0.5 us or more.
 // The dQ kernel counts whether it follows or not: the same sums in the same order with and without it, so that
 // attn_fp8_bwd and attn_fp8_bwd_dkdv give the same bits.
 int split_of(const AttnShape& s, int sms, int passes) {
@@ -890,30 +888,30 @@ int split_of(const AttnShape& s, int sms, int passes) {
   const double per_head = s.causal ? tiles * (keys - tiles) + tiles * (tiles + 1) / 2 : tiles * keys;
   const double pairs = per_head * s.Hq * s.B;
   const double items = tiles * s.Hq * s.B * (s.eb == 2 && s.dqk > 192 ? 2 : 1);             // (dQ columns in two items there)
-  static const double kPerQuery[2][3] = {{1.3, 1.5, 1.5}, {1.5, 2.5, 3.4}};     // FP8, BF16; qk head dim up to 128, 192, 256 (a pass)
-  static const double kPerKey[2][3] = {{0.9, 1.1, 1.5}, {1.0, 1.8, 2.6}};
-  const int mode = s.eb - 1, dims = s.dqk <= 128 ? 0 : s.dqk <= 192 ? 1 : 2;
-  const double t_pair = kPerQuery[mode][dims], t_dq = kPerKey[mode][dims], start = 4;
+  // FP8 and BF16; qk head dim up to 64, 128, 192 and 256 (there for each pass)
+  static const double kPerQuery[2][4] = {{1.35, 1.42, 1.6, 1.55}, {1.55, 1.95, 3.0, 3.5}};
+  static const double kPerKey[2][4] = {{0.9, 0.9, 1.1, 1.5}, {1.0, 1.0, 1.8, 2.6}};
+  const int mode = s.eb - 1, dims = (s.dqk - 1) / 64;
+  const double t_pair = kPerQuery[mode][dims], t_dq = kPerKey[mode][dims], start = 3;
   const double item = 3 + t_dq * per_head / tiles, last_dq = start + 3 + t_dq * keys;       // an average item, and the longest
-  auto estimate = [&](int split) {
-    const double cta = split == 1 ? 6 : split == 2 ? 7.5 : split == 4 ? 8.25 : 9;
-    const double list = G * tiles, longest = t_pair * static_cast<long long>((list + split - 1) / split) + cta;
+  const double columns = passes > 1 ? 256 : s.dqk + s.dv;
+  auto estimate = [&](int split, double full) {
+    const double cta = 6 + columns * (split - 1) / split / 40;
+    const double longest = t_pair * std::ceil(G * tiles / split) + cta + (passes > 1 ? 2 : 0);
     const double ctas = s.B * s.Hkv * keys * split * passes, work = pairs * passes * t_pair + ctas * cta;
-    const double alone = longest > last_dq ? longest : last_dq;
-    if (ctas + items <= sms) return alone;
-    const double all = (work + items * item) / sms + start;
-    // a second round of CTAs (2 us); dQ begins once the last of them have, and the SMs that they leave are the sooner free the
-    // more the CTAs differ
-    if (ctas >= sms) return 2 + std::max(std::max(longest - 2, all), work / sms * (1 - sms / ctas) + work / ctas * per_head / (tiles * keys) + last_dq);
-    if (items * item <= (sms - ctas) * std::max(longest - start, 0.0)) return alone;
-    return std::max(std::max(alone, all), work / ctas + start + item);
+    const double alone = std::max(longest, last_dq), all = (work + items * item) / sms + start;
+    const double room = split == 8 ? 0.9 * sms : sms;
+    if (ctas + items <= room) return alone;
+    if (ctas >= room) return full * std::max(std::max(longest, all), work / room + last_dq);
+    if (items * item <= (room - ctas) * std::max(longest - start, 0.0)) return alone;
+    return full * std::max(std::max(alone, all), work / ctas + start + item);
   };
   int best = 1;
-  double least = estimate(1);
+  double least = estimate(1, 1.0), full = 1.03;
   // (slices of the columns of dK and dV are multiples of 16)
-  for (int split = 2; split <= (s.dqk % 128 == 0 && s.dv % 128 == 0 ? 8 : 4); split *= 2) {
-    const double t = estimate(split);
-    if (t < 0.95 * least && least - t > 1.5) { best = split; least = t; }
+  for (int split = 2; split <= (s.dqk % 128 == 0 && s.dv % 128 == 0 ? 8 : 4); split *= 2, full += 0.03) {
+    const double t = estimate(split, full);
+    if (t < 0.95 * least && least - t > 0.5) { best = split; least = t; }
   }
   return best;
 }

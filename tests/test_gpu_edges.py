@@ -122,12 +122,12 @@ def test_heads_do_not_depend_on_their_group_of_the_work_list(dims, heads_kv, per
 
 
 @pytest.mark.parametrize("bf16", [False, True])
-@pytest.mark.parametrize("dims,heads", [((64, 64), (2, 2)), ((128, 128), (2, 2)), ((128, 128), (8, 1)), ((192, 128), (2, 2)), ((192, 128), (2, 1)),
-                                        ((256, 256), (2, 2)), ((256, 256), (8, 1))])
+@pytest.mark.parametrize("dims,heads", [((64, 64), (12, 12)), ((128, 128), (2, 2)), ((128, 128), (8, 1)), ((192, 128), (2, 2)), ((192, 128), (8, 1)),
+                                        ((256, 256), (8, 8)), ((256, 256), (8, 1))])
 def test_outputs_that_start_between_two_sectors(dims, heads, bf16):
     """Rows leave in 32-byte stores where an output starts on a sector, and in 16-byte ones where it does not (16-byte
-    alignment is all that is asked for): the same bits, and nothing written beside them.  (8, 1) and (2, 1) heads: key tiles
-    shared by a cluster, which stores slices of columns; (2, 2): one CTA per key tile, which stores whole rows."""
+    alignment is all that is asked for): the same bits, and nothing written beside them.  (8, 1) heads: key tiles shared by a
+    cluster, which stores slices of columns; the others: one CTA per key tile, which stores whole rows."""
     from paper_2609_37852_b200 import binding as B
     g = torch.Generator(device="cuda").manual_seed(sum(dims) + sum(heads))
     n, (hq, hkv), (dqk, dv) = 384, heads, dims
