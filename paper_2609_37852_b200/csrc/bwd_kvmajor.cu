@@ -235,8 +235,9 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
   constexpr bool kPrepLoads = kFp8 && C::kRowTok == kSub;
   constexpr bool kSplit = kOpBufs == 1;          // single operand buffer: P^ and dS^ are handed over separately
   constexpr bool kApart = C::kApart;
-  // BF16 mode at head dim 128 stores 16 bytes at a time: dK / dV of 2 x 16/4 heads x 4096 265.3 us by the sector, 259.9 so;
-  // 32/8 x 8192 1133 and 1114.  (Head dim 64 gains as FP8 does: 8 x 12 x 1024 89.3 -> 86.2.)
+  // One CTA per key tile in BF16 mode at head dim 128 stores 16 bytes at a time: dK / dV of 2 x 16/4 heads x 4096, calls in a
+  // row below the power cap, 265.3 us by the sector, 259.9 so; 32/8 x 8192 1133 and 1114.  (Head dim 64 gains as FP8 does: 8 x 12
+  // x 1024 89.3 -> 86.2.  So does a cluster, which stores slices of rows: 16/4 heads x 4096 138.3 -> 137.1, 8/1 x 512 19.45 -> 19.36.)
   constexpr bool kSectors = !(C::kApart && C::kCq == 2);
   constexpr int kSBufs = C::kSBufs;
   constexpr uint32_t kColS = C::kColS, kColdP = C::kColdP, kColP = C::kColP, kColdS = C::kColdS, kColdV = C::kColdV,
@@ -317,7 +318,7 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
   // kApart: a padded key of a ragged sequence (no causal mask) has a row of dV and dK of its own and nothing else, so its
   // rows are stored as zeros, whatever its probabilities and score gradients came to (NaN behind an Inf in dO).  The other
   // configurations make the latter zero in the loop: without that branch their loops come out 1 % slower (dK / dV and dQ
-  // of the 8K layer), with it the BF16 one does (dK / dV of the 4K layer 294 us, 290 without).
+  // of the 8K layer), with it the BF16 one does (dK / dV of the 4K layer at the power cap 294 us, 290 without).
   const int real_rows = kApart && !p.causal && jt == tiles_nk - 1 ? p.kv_lim + 1 : kTile;
 
   if (warp == 0) {
@@ -879,7 +880,11 @@ kvmajor_kernel(const KvParams p, const __grid_constant__ CUtensorMap tm_k, const
 //   This kernel's do: dQ items fill the SMs it leaves, and what they do not get done waits for its CTAs to end.
 //   They do not: the sum of the work, or a dQ item behind the rounds of this kernel.  In the last two, sharing costs 3 % per
 //   doubling, since a cluster waits for as many free SMs; clusters of eight leave a tenth of the SMs out.
-// More CTAs only for 5 % and 0.5 us or more.
+// More CTAs only for 5 % and 0.5 us or more.  1680 random problems of up to 1.3 ms (all head dims, both modes, chunks of
+// sequences) take 1.004 times what the best number for each takes, 1.003 on the 420 of them that the choice of the costs did not
+// see; always one CTA 1.25, the rule before this one 1.009.  With one, two, four, eight: 8 heads on 1, 768 tokens, BF16, 93.0,
+// 54.1, 33.3, 23.6 us; 2 x 4 on 1 x 2560 at 64, 113.6, 62.9, 45.6.  8 on 2 x 128 at (192,128), where the exchange takes more
+// than sharing saves, 13.3, 15.0, 15.5.
 // The dQ kernel counts whether it follows or not: the same sums in the same order with and without it, so that
 // attn_fp8_bwd and attn_fp8_bwd_dkdv give the same bits.
 int split_of(const AttnShape& s, int sms, int passes) {

@@ -112,8 +112,8 @@ struct QmCfg {
   // the correction pass at head dim 128, 0.683 -> 0.598 ms on the 8K workload; the wide head dims gain nothing)
   static constexpr int kSBufs = (kEB == 2 && kEBv == 2 && kCq == 2 && kCv == 2) ? 2 : 1;
   // The issuing warps as one elected thread each: only where a second S / dP pair lets them run ahead of the softmax (4K
-  // layer in BF16 mode, correction 153.9 -> 142.2 us, dQ 217.8 -> 215.6).  With one pair the softmax of all warps starts the
-  // sooner in step, and it costs 1 to 4 % (FP8 8K layer, correction 346 -> 359, dQ 551 -> 573; BF16 head dim 64, correction
+  // layer in BF16 mode, each kernel alone, correction 154 -> 142 us, dQ 210 -> 207).  With one pair the softmax of all warps
+  // starts the sooner in step, and it costs 1 to 4 % (FP8 8K layer, correction 346 -> 359, dQ 551 -> 573; BF16 head dim 64, correction
   // 17.6 -> 18.2; head dim 256, dQ 207 -> 213).
   static constexpr bool kOne = kSBufs == 2;
   static constexpr uint32_t kSdp = 2 * kStep;           // columns of an S / dP pair

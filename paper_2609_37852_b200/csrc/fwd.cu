@@ -61,8 +61,8 @@ struct FwdCfg {
   static constexpr int kRv = kRv_;                      // 128-row tiles of the V^T operand (dv / 128, rounded up)
   static constexpr bool kFp8 = kEB == 1;
   // The issuing warps of BF16 mode, whose 64-key steps take up to 16 MMAs a product, run as one elected thread each: 8/2 heads
-  // x 4096 x 256, 74.4 -> 65.3 us; 2 x 16/4 x 4096 x 128, 155.9 -> 153.7.  FP8 at head dim 256: 198.5 -> 200.5, so not there,
-  // nor at (192,128): 16/4 x 4096 101.5 -> 104.9, 8 x 2048 28.0 -> 29.0.
+  // x 4096 x 256, 74.4 -> 65.3 us; 2 x 16/4 x 4096 x 128, 155.5 -> 147, with the exponentials in pairs.  FP8 at head
+  // dim 256: 198.5 -> 200.5, so not there, nor at (192,128): 16/4 x 4096 101.5 -> 104.9, 8 x 2048 28.0 -> 29.0.
   static constexpr bool kOne = !kFp8 && kCq != 3;
   static constexpr int kTileKeys = kTile / kEB;         // keys per K / V stage
   static constexpr int kSubPerTile = kTileKeys / kSub;  // 64-key steps per stage

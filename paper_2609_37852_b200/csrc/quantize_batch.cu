@@ -14,7 +14,8 @@
 // Bound by memory, nearly: Q, K, V, dO of 80 heads x 8192 x 128 in BF16 (341 MB) take 56.1 us, 6.1 TB/s or 0.93 of the measured
 // copy rate; before, with 8 values a thread in pass 1 and the transposed codes staged in shared memory and copied out
 // behind a third barrier, 63.3 (40.3 M instructions, now 32 M).  40 heads x 4096 x 128: 34.9 -> 30.8; 64 heads x 8192 x 192 / 128:
-// 72.8 -> 59.1; 20 heads x 8192 x 256: 36.6 -> 35.1.  Three CTAs per SM (80 registers, so fewer loads in flight) take 67.5 us on the first.
+// 72.8 -> 59.1; 20 heads x 8192 x 256: 36.6 -> 35.1.  (Launches of column copies only
+// kept the staged codes: launch_batch_o.)  Three CTAs per SM (80 registers, so fewer loads in flight) take 67.5 us on the first.
 //
 // Producer steps (kProd).  A pass ahead of the other two rotates the tile in place: a rotated channel is
 // a BF16 value, so it goes back into the slot it came from whatever the source type.  The FP32 steps

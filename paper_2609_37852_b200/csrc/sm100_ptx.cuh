@@ -148,7 +148,8 @@ __device__ __forceinline__ void sts_u8(void* p, uint32_t v) {
 
 // 32 bytes of a row to global memory, one sector per lane where the row starts on one (`sector`), two 16-byte stores
 // otherwise.  A lane that stores its own row touches a line of its own, and the load / store unit takes the lines of an
-// instruction one after the other, so half as many instructions take half as long.
+// instruction one after the other: half as many instructions made every kernel but one faster (figures beside the calls; the
+// exception is the key-major kernel in BF16 mode at head dim 128, see kSectors there).
 __device__ __forceinline__ void store_32b(void* p, const uint32_t* w, bool sector) {
   if (sector)
     asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
